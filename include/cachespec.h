@@ -178,8 +178,8 @@ cs_status cs_verify_attention(const cs_attn_dims* dims, const void* q, const voi
  *   out_n_accepted int32 [B]: a
  *   workspace      device scratch of at least cs_spec_accept_workspace_bytes(dims, k)
  *                  bytes, 256-byte aligned, any initial contents: every call
- *                  writes each scratch word it later reads (one pair per row
- *                  segment of the statistics pass).  Calls that share a
+ *                  writes each scratch word it later reads (the statistics of
+ *                  row segments, and what a long call's phases decide).  Calls that share a
  *                  workspace must be ordered (same stream or events).
  *
  * A logit of -inf marks a masked token (probability zero); NaN and +inf are

@@ -3,40 +3,34 @@
 // target and draft rows, the min(1, p/q) accept test, the residual
 // max(0, p - q) or bonus draw by inverse CDF, and the greedy variant.
 //
-// Two kernels per call, no atomics, no spin-waits and no scratch that has to
-// start at a known value:
-//   1. accept_stats_kernel streams every row of every request (target rows
-//      0..k, then draft rows 0..k-1; target rows only when greedy) once.  The
-//      rows are cut into 4 KB items and the flattened item sequence is split
-//      into one contiguous, equal range per warp of a grid that fills the
-//      device, so every SM reads the same number of bytes.  A warp keeps the
-//      next item in flight while it reduces the current one and writes one
-//      partial per row segment of its range: (max, sum 2^((z-max)c)) -- one
-//      exponential per logit -- or, greedy, (max, lowest id of the max).
-//      The partials of a row sit side by side in the order of the row, and
-//      the warp that holds a row's last item records how many there are.
-//   2. accept_draw_kernel runs one thread-block cluster per request and is
-//      launched as a programmatic dependent of kernel 1: it loads its inputs
-//      while kernel 1 finishes.  Every CTA folds the partials of the
-//      request's rows in the same fixed order (so all of them hold
-//      bit-identical statistics), runs the accept tests
-//      (one lane per position, the first rejection found by a ballot) and
-//      computes the draw mass of its slice of the vocabulary for the deciding
-//      row pair.  The CTAs swap their masses through distributed shared
-//      memory, fold them in rank order, and the CTA whose cell holds u_k * Z
-//      finds the token within its slice.
-//   Greedy mode replaces kernel 2 by accept_greedy_kernel (one warp per
-//   request: argmax agreement).
-// Token trees (multi-candidate verification) reuse kernel 1 over the target
-// rows of every node and the draft rows of the nodes that have children
-// (a leaf's draft row is not read), and walk the tree in tree_draw_kernel
-// (one cluster per request): the children of the current node are tested in
-// turn, each rejection turning the running distribution into the residual
-// max(p - kappa q, 0) / Z, whose mass Z takes one cluster-wide pass over the
-// row pair; the walk ends with the draw of section 2 at that kappa.  The
-// greedy walk is tree_greedy_kernel.
-// No probability is written to memory; the scratch holds the row-segment
-// pairs and one count per row.
+// Kernels of a call, each a programmatic dependent of the one before it (no
+// spin-waits, no scratch that has to start at a known value):
+//   1. accept_stats_kernel streams rows of every request (target rows, then
+//      draft rows; target rows only when greedy) once.  Rows are cut into 4 KB
+//      items and units of a few items; a warp keeps the next item in flight
+//      while it reduces the current one and writes one partial per unit: (max,
+//      sum 2^((z-max)c)) -- one exponential per logit -- or, greedy, (max,
+//      lowest id of the max).
+//   2. accept_walk_kernel, one thread-block cluster per request, folds the
+//      partials of the request's rows (every CTA in the same order, so all of
+//      them hold bit-identical statistics), runs the accept tests (one lane
+//      per position, the first rejection found by a ballot) and draws: the
+//      masses of the CTAs' slices of the deciding row pair are swapped through
+//      distributed shared memory, and one warp of the CTA whose cell holds
+//      u_k * Z finds the token.  Greedy: the arg max of the deciding row.
+// A chain's rows past its first rejection are not needed, so a call whose
+// positions take long to read (plan_accept) reads them in phases: kernel 1 for
+// the first positions of every request, accept_test_kernel for their tests,
+// kernel 1 for the next positions of the requests that are still undecided
+// (and for the draw masses of those just decided, whose rows are still in
+// L2), and so on; the walk then only draws.
+// Token trees (multi-candidate verification) walk likewise: the children of
+// the current node are tested in turn, each rejection turning the running
+// distribution into the residual max(p - kappa q, 0) / Z, whose mass Z takes
+// one cluster-wide pass over the row pair.  A large tree skips kernel 1: the
+// walk streams the rows of the nodes that it comes to.
+// No probability is written to memory; the scratch holds the units' partials,
+// draw masses and the phases' decisions.
 #include <limits.h>
 #include <math.h>
 
@@ -46,40 +40,60 @@
 namespace cs {
 namespace {
 
-constexpr int kThreads = 256;                  // kernel 1 and the greedy kernel
+constexpr int kThreads = 256;                  // the statistics kernel
 constexpr int kWarps = kThreads / 32;
-constexpr int kDrawThreads = 512;              // kernel 2
-constexpr int kDrawWarps = kDrawThreads / 32;
-constexpr int kVecs = 8;                       // kernel 1: 16-byte vectors per lane per item
+constexpr int kVecs = 8;                       // 16-byte vectors per lane per item
 constexpr int kItemBytes = 32 * kVecs * 16;    // 4 KB of one row
-constexpr int kRunVecs = 2;                    // kernel 2: 16-byte vectors per thread per row per pass
-constexpr int kMaxRows = 33;                   // 2k+1 rows of a request, k <= 16
-constexpr int kRowsPerDrawWarp = (kMaxRows + kDrawWarps - 1) / kDrawWarps;
-constexpr int kMaxPasses = 128;                // passes of one CTA over its vocabulary slice
 constexpr int kMaxCluster = 16;
 constexpr int kMaxTreeNodes = 64;
+constexpr int kMaxPhased = 4096;               // requests of a call whose positions are read in phases, at most
 
-struct AcceptParams {
-    const void* target;       // [B, n_t, V]: chain n_t = k+1, tree n_t = nodes
-    const void* draft;        // [B, d_rows, V]: chain d_rows = k, tree d_rows = nodes
-    const int32_t* tokens;    // chain [B, k]; tree [B, n_t] (node tokens)
-    const float* uniforms;    // chain [B, k+1]; tree [B, n_t]
-    int32_t* out_tokens;      // chain [B, k+1]; tree [B, n_t]
-    int32_t* out_n;           // [B], or null (the sampler)
-    const int32_t* parents;   // tree [B, n_t] (null for the chain)
-    int32_t* out_path;        // tree [B, n_t]: accepted nodes in walk order
-    int B, V, k;
-    int n_t, d_rows;          // target rows and draft rows per request
-    int R;                    // rows per request streamed by kernel 1: n_t + d_rows, or n_t (greedy)
+// x / d for 0 <= x by a multiplication whenever x < 2^31: with
+// s = ceil(log2 d) and mul = floor(2^(31+s) / d) + 1 < 2^32 + 1, the error of
+// x mul / 2^(31+s) over x / d is below x / 2^(31+s) < 1/d, too little to reach
+// the next whole number.
+struct FastDiv {
+    long long d;
+    unsigned long long mul;
+    int shift;
+    __host__ void set(long long by) {
+        if (by < 1) by = 1;
+        d = by;
+        shift = 31;
+        while ((1ll << (shift - 31)) < by) ++shift;
+        mul = (1ull << shift) / (unsigned long long)by + 1;
+    }
+    __device__ __forceinline__ long long div(long long x) const {
+        return x < 0x80000000ll ? (long long)((unsigned long long)x * mul >> shift) : x / d;
+    }
+};
+
+// The rows that one launch of the statistics kernel reads, and where their
+// partials are.  A chain's positions may be read in phases: phase 0 for every
+// request, later ones for the requests whose drafts were all accepted so far.
+struct Phase {
+    int p0;                   // first node (position) of the phase
+    int t_rows, R;            // target rows p0 .. p0+t_rows-1, then draft rows p0 .. p0+R-t_rows-1 of a request
+    int units, U;             // units of a row, items of a unit
+    const int* undecided;     // null: every request; else [B], < 0: the request takes part
+    float2* part;             // [B, R, units] partials of the rows' units
+    unsigned* ticket;         // a later phase's unit counter, 0 at its start
+};
+
+struct StatsParams {
+    const void* target;       // [B, n, V]
+    const void* draft;        // [B, d_rows, V] (null when greedy)
+    const int32_t* parents;   // tree [B, n] (null for the chain)
+    int B, V, n, d_rows;
     int I;                    // 4 KB items per row
-    long long N;              // B * R * I items in all
-    int W;                    // busy warps of kernel 1 (warp w owns items [w*N/W, (w+1)*N/W)), W <= N
-    int J;                    // partial slots per row (row segments a row can have)
-    int slice;                // kernel 2: logits of the vocabulary per CTA of a cluster
-    int b_base;               // kernel 2: first request of this launch
     float c_hi, c_lo;         // log2(e) / T as a float pair
-    float2* part;             // [B*R, J] row-segment partials, in row order
-    int* cnt;                 // [B*R] segments of each row
+    Phase ph;
+    // a later phase: for the requests that the phase before decided (at a position in
+    // [mass_lo, mass_hi)): the draw masses of the units of their row pair
+    int mass_lo, mass_hi;
+    const float4* stat;       // [B] statistics of the pair
+    float* mass;              // [B, units]
+    FastDiv by_units, by_R;
 };
 
 // ------------------------------------------------------------ small helpers
@@ -95,27 +109,74 @@ __device__ __forceinline__ float to_f(float v) { return v; }
 __device__ __forceinline__ float to_f(__nv_bfloat16 v) { return __bfloat162float(v); }
 
 template <typename T>
-__device__ __forceinline__ bool aligned16(const T* p) {
-    return (reinterpret_cast<uintptr_t>(p) & 15u) == 0;
-}
-
-template <typename T>
 union Vec16 {
     uint4 q;
     T t[16 / sizeof(T)];
 };
 
-// 16 bytes of row[start ..]; entries at or past `end` read as -inf.  `stream`
-// bypasses L1 (kernel 1 touches every byte once).
-template <typename T, bool kStream>
-__device__ __forceinline__ uint4 load16(const T* row, int start, int end, bool vec) {
+template <typename T>
+__device__ __forceinline__ int misaligned_by(const T* row) {   // elements past a 16-byte boundary
+    return (int)((reinterpret_cast<uintptr_t>(row) & 15u) / sizeof(T));
+}
+
+// row[start .. start + kPer) at any alignment; entries outside [0, V) read as
+// -inf.  Vectors that lie inside the row come as two aligned ones shifted
+// together (one when row + start is on a 16-byte boundary), the row's ends
+// element by element.
+template <typename T>
+__device__ __forceinline__ uint4 load16_any(const T* row, int start, int V) {
     constexpr int kPer = 16 / (int)sizeof(T);
-    if (vec && start + kPer <= end)
-        return kStream ? ld_stream(row + start) : __ldg(reinterpret_cast<const uint4*>(row + start));
-    Vec16<T> v;
+    const int off = (int)(reinterpret_cast<uintptr_t>(row + start) & 15u);   // bytes; the same in every lane
+    const int a = start - off / (int)sizeof(T);
+    if (a < 0 || a + (off ? 2 : 1) * kPer > V) {
+        Vec16<T> v;
 #pragma unroll
-    for (int e = 0; e < kPer; ++e) v.t[e] = start + e < end ? row[start + e] : (T)kNegInf;
-    return v.q;
+        for (int e = 0; e < kPer; ++e) v.t[e] = start + e >= 0 && start + e < V ? row[start + e] : (T)kNegInf;
+        return v.q;
+    }
+    const uint4 lo = __ldg(reinterpret_cast<const uint4*>(row + a));
+    if (off == 0) return lo;
+    const uint4 hi = __ldg(reinterpret_cast<const uint4*>(row + a) + 1);
+    uint32_t w[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+    if (off & 8) {
+#pragma unroll
+        for (int i = 0; i < 6; ++i) w[i] = w[i + 2];
+    }
+    if (off & 4) {
+#pragma unroll
+        for (int i = 0; i < 5; ++i) w[i] = w[i + 1];
+    }
+    const int sh = (off & 3) * 8;
+    return make_uint4(__funnelshift_r(w[0], w[1], sh), __funnelshift_r(w[1], w[2], sh),
+                      __funnelshift_r(w[2], w[3], sh), __funnelshift_r(w[3], w[4], sh));
+}
+
+// count vectors, the u-th at start + u * step.  Not inlined: a kernel holds
+// one copy of it for its row ends and odd rows, off the straight path (the
+// latency of a short call is mostly instruction fetches).
+template <typename T>
+__device__ __noinline__ void load_slow(const T* row, int start, int step, int count, int V, uint4* out) {
+#pragma unroll 1
+    for (int u = 0; u < count; ++u) out[u] = load16_any(row, start + u * step, V);
+}
+
+// Block j of a row (kN vectors per lane) into registers: lane l holds the
+// vectors u * 32 + l.  The blocks of a row start at the 16-byte boundary at
+// or before its first element, so rows of any alignment take vector loads.
+template <typename T, int kN>
+__device__ __forceinline__ void load_block(const T* row, int j, int V, int lane, uint4 (&v)[kN]) {
+    constexpr int kPer = 16 / (int)sizeof(T);
+    constexpr int kBlock = 32 * kN * kPer;
+    const int base = j * kBlock - misaligned_by(row);
+    if (base >= 0 && base + kBlock <= V) {
+#pragma unroll
+        for (int u = 0; u < kN; ++u) v[u] = ld_stream(row + base + (u * 32 + lane) * kPer);
+    } else {
+        uint4 t[kN];
+        load_slow(row, base + lane * kPer, 32 * kPer, kN, V, t);
+#pragma unroll
+        for (int u = 0; u < kN; ++u) v[u] = t[u];
+    }
 }
 
 // A pair (m, s) stands for sum_v 2^((z_v - m) c); empty is (-inf, 0).
@@ -132,11 +193,6 @@ __device__ __forceinline__ void fold(float& m, float& s, float m2, float s2, flo
 __device__ __forceinline__ void argmax_fold(float2& acc, float2 o) {
     if (o.x > acc.x || (o.x == acc.x && __float_as_int(o.y) < __float_as_int(acc.y))) acc = o;
 }
-
-// Unnormalised weight of one logit, 2^((z - m) c), with the same single-term
-// exponent the statistics summed (so that the weights of a row add up to its
-// normaliser S).  m is finite, so -inf weighs 2^-inf = 0.
-__device__ __forceinline__ float weight(float z, float m, float c_hi) { return ex2((z - m) * c_hi); }
 
 __device__ __forceinline__ float warp_incl_scan(float x, int lane) {
 #pragma unroll
@@ -177,14 +233,6 @@ __device__ __forceinline__ float2 warp_fold_argmax(float2 acc) {
     return acc;
 }
 
-// Row r of request b: target rows 0 .. n_t-1, then draft rows.
-template <typename T>
-__device__ __forceinline__ const T* row_ptr(const AcceptParams& p, int b, int r) {
-    const int V = p.V, nt = p.n_t;
-    return r < nt ? static_cast<const T*>(p.target) + ((size_t)b * nt + r) * V
-                  : static_cast<const T*>(p.draft) + ((size_t)b * p.d_rows + (r - nt)) * V;
-}
-
 // Bit u set iff tree node u of the parent array `par` (n <= 64 nodes) has a
 // child; every lane of the warp returns the same mask.
 __device__ __forceinline__ uint64_t tree_child_mask(const int32_t* par, int n, int lane) {
@@ -204,15 +252,10 @@ __device__ __forceinline__ uint64_t tree_child_mask(const int32_t* par, int n, i
 
 // x / d for x >= 0, d > 0: one 32-bit division whenever both fit (every
 // realistic problem), the 64-bit routine otherwise.
-__device__ __forceinline__ long long div_nn(long long x, long long d) {
+__device__ __noinline__ long long div_nn(long long x, long long d) {
     if ((unsigned long long)x <= 0xffffffffull && (unsigned long long)d <= 0xffffffffull)
         return (long long)((unsigned)x / (unsigned)d);
     return x / d;
-}
-
-// First item of warp w's range (kernel 1's balanced split).
-__device__ __forceinline__ long long range_lo(const AcceptParams& p, long long w) {
-    return div_nn(w * p.N, p.W);
 }
 
 // Programmatic dependent launch: each kernel may start while the one before
@@ -224,15 +267,16 @@ __device__ __forceinline__ void allow_dependent_launch() {
 }
 
 // ------------------------------------------------------------ kernel 1
-// Largest of the 8 * kVecs logits of one lane's item (bf16: packed maxima,
-// one instruction per pair).
-__device__ __forceinline__ float item_max(const uint4 (&v)[kVecs], __nv_bfloat16) {
+// Largest of the logits of one lane's vectors (bf16: packed maxima, one
+// instruction per pair).
+template <int kN>
+__device__ __forceinline__ float item_max(const uint4 (&v)[kN], __nv_bfloat16) {
     __nv_bfloat162 a = *reinterpret_cast<const __nv_bfloat162*>(&v[0].x);
     __nv_bfloat162 b = *reinterpret_cast<const __nv_bfloat162*>(&v[0].y);
     __nv_bfloat162 c = *reinterpret_cast<const __nv_bfloat162*>(&v[0].z);
     __nv_bfloat162 d = *reinterpret_cast<const __nv_bfloat162*>(&v[0].w);
 #pragma unroll
-    for (int u = 1; u < kVecs; ++u) {
+    for (int u = 1; u < kN; ++u) {
         a = __hmax2(a, *reinterpret_cast<const __nv_bfloat162*>(&v[u].x));
         b = __hmax2(b, *reinterpret_cast<const __nv_bfloat162*>(&v[u].y));
         c = __hmax2(c, *reinterpret_cast<const __nv_bfloat162*>(&v[u].z));
@@ -242,80 +286,254 @@ __device__ __forceinline__ float item_max(const uint4 (&v)[kVecs], __nv_bfloat16
     return fmaxf(__low2float(a), __high2float(a));
 }
 
-__device__ __forceinline__ float item_max(const uint4 (&v)[kVecs], float) {
+template <int kN>
+__device__ __forceinline__ float item_max(const uint4 (&v)[kN], float) {
     float a = kNegInf, b = kNegInf;
 #pragma unroll
-    for (int u = 0; u < kVecs; ++u) {
+    for (int u = 0; u < kN; ++u) {
         a = fmaxf(a, fmaxf(__uint_as_float(v[u].x), __uint_as_float(v[u].y)));
         b = fmaxf(b, fmaxf(__uint_as_float(v[u].z), __uint_as_float(v[u].w)));
     }
     return fmaxf(a, b);
 }
 
-// The logits of a 32-bit word: two bf16 (low half first) or one fp32.
-__device__ __forceinline__ float word_lo(uint32_t x, __nv_bfloat16) { return __uint_as_float(x << 16); }
-__device__ __forceinline__ float word_hi(uint32_t x, __nv_bfloat16) { return __uint_as_float(x & 0xffff0000u); }
-
-// sum over one lane's item of 2^((z - m) c_hi), four independent partial sums.
-template <typename T>
-__device__ __forceinline__ float item_sum(const uint4 (&v)[kVecs], float m, float c_hi) {
-    float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
+// The logits of a vector as fp32 pairs.
+__device__ __forceinline__ void to_pairs(const uint4& v, uint64_t (&z)[4], __nv_bfloat16) {
+    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-    for (int u = 0; u < kVecs; ++u) {
-        const uint32_t w[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
-        if constexpr (sizeof(T) == 2) {
-            s0 += ex2((word_lo(w[0], T()) - m) * c_hi);
-            s1 += ex2((word_hi(w[0], T()) - m) * c_hi);
-            s2 += ex2((word_lo(w[1], T()) - m) * c_hi);
-            s3 += ex2((word_hi(w[1], T()) - m) * c_hi);
-            s0 += ex2((word_lo(w[2], T()) - m) * c_hi);
-            s1 += ex2((word_hi(w[2], T()) - m) * c_hi);
-            s2 += ex2((word_lo(w[3], T()) - m) * c_hi);
-            s3 += ex2((word_hi(w[3], T()) - m) * c_hi);
-        } else {
-            s0 += ex2((__uint_as_float(w[0]) - m) * c_hi);
-            s1 += ex2((__uint_as_float(w[1]) - m) * c_hi);
-            s2 += ex2((__uint_as_float(w[2]) - m) * c_hi);
-            s3 += ex2((__uint_as_float(w[3]) - m) * c_hi);
-        }
-    }
-    return (s0 + s1) + (s2 + s3);
+    for (int i = 0; i < 4; ++i) z[i] = f2_pack(__uint_as_float(w[i] << 16), __uint_as_float(w[i] & 0xffff0000u));
+}
+__device__ __forceinline__ void to_pairs(const uint4& v, uint64_t (&z)[2], float) {
+    z[0] = f2_pack(__uint_as_float(v.x), __uint_as_float(v.y));
+    z[1] = f2_pack(__uint_as_float(v.z), __uint_as_float(v.w));
 }
 
-template <typename T, bool kGreedy>
-__global__ void __launch_bounds__(kThreads, 2) accept_stats_kernel(const AcceptParams p) {
+// The weights 2^((z - m) c_hi) of a pair: subtraction and product rounded one
+// after the other, in packed arithmetic (half the instructions of the scalar
+// form, bit for bit its results).
+__device__ __forceinline__ uint64_t weight2(uint64_t z, uint64_t m2, uint64_t c2) {
+    float a, b;
+    f2_unpack(f2_mul(f2_sub(z, m2), c2), a, b);
+    return f2_pack(ex2(a), ex2(b));
+}
+
+// sum over one lane's vectors of 2^((z - m) c_hi), four independent partial sums.
+template <typename T, int kN>
+__device__ __forceinline__ float item_sum(const uint4 (&v)[kN], float m, float c_hi) {
+    constexpr int kPairs = 8 / (int)sizeof(T);
+    const uint64_t m2 = f2_pack(m, m), c2 = f2_pack(c_hi, c_hi);
+    uint64_t s2[2] = {0ull, 0ull};   // +0.0f pairs
+#pragma unroll
+    for (int u = 0; u < kN; ++u) {
+        uint64_t z[kPairs];
+        to_pairs(v[u], z, T());
+#pragma unroll
+        for (int i = 0; i < kPairs; ++i) s2[i & 1] = f2_add(s2[i & 1], weight2(z[i], m2, c2));
+    }
+    float a, b, e, f;
+    f2_unpack(s2[0], a, b);
+    f2_unpack(s2[1], e, f);
+    return (a + b) + (e + f);
+}
+
+// Greedy: one lane's running (max, lowest id of it) over its item, whose
+// vector u holds the logits at0 + u * 32 * kPer ...
+template <typename T, int kN>
+__device__ __forceinline__ void item_argmax(const uint4 (&cur)[kN], int at0, float& m, int& id) {
+    constexpr int kPer = 16 / (int)sizeof(T);
+#pragma unroll
+    for (int u = 0; u < kN; ++u) {   // ascending ids: strict > keeps the lowest
+        Vec16<T> v;
+        v.q = cur[u];
+#pragma unroll
+        for (int e = 0; e < kPer; ++e) {
+            const float z = to_f(v.t[e]);
+            if (z > m) {
+                m = z;
+                id = at0 + u * 32 * kPer + e;
+            }
+        }
+    }
+}
+
+// The draw weights are p and max(p - kappa q, 0) scaled by S_t (the inverse
+// CDF does not depend on a common factor): 2^((zt - mt)c) and
+// max(2^((zt - mt)c) - rho 2^((zd - md)c), 0) with rho = kappa S_t / S_d.
+// p alone is rho = 0 with the target row in both places.
+template <typename T>
+struct DrawRow {
+    const T* rt;
+    const T* rd;
+    float mt, md, rho, c_hi;
+    bool same;   // both rows lie alike on 16-byte boundaries
+};
+
+// The pair's weights from its rows' statistics (a row without a finite entry,
+// outside the contract, weighs zero everywhere); kappa == 0: p alone.
+template <typename T>
+__device__ __forceinline__ void set_weights(DrawRow<T>& d, float2 st, float2 sd, float kappa, float c_hi) {
+    d.c_hi = c_hi;
+    d.mt = st.x == kNegInf ? 0.f : st.x;
+    d.md = sd.x == kNegInf ? 0.f : sd.x;
+    d.rho = sd.y > 0.f ? kappa * (st.y / sd.y) : 0.f;
+    if (!(kappa > 0.f)) {
+        d.rd = d.rt;
+        d.md = d.mt;
+        d.rho = 0.f;
+    }
+    d.same = misaligned_by(d.rt) == misaligned_by(d.rd);
+}
+
+// The weights of a vector of both rows.
+template <typename T>
+__device__ __forceinline__ void weigh(const DrawRow<T>& d, const uint4& t, const uint4& q, float* w) {
+    constexpr int kPairs = 8 / (int)sizeof(T);
+    const uint64_t mt = f2_pack(d.mt, d.mt), md = f2_pack(d.md, d.md), c2 = f2_pack(d.c_hi, d.c_hi);
+    const uint64_t nr = f2_pack(-d.rho, -d.rho);
+    uint64_t zt[kPairs], zd[kPairs];
+    to_pairs(t, zt, T());
+    to_pairs(q, zd, T());
+#pragma unroll
+    for (int i = 0; i < kPairs; ++i) {
+        float a, b;
+        f2_unpack(f2_fma(nr, weight2(zd[i], md, c2), weight2(zt[i], mt, c2)), a, b);
+        w[2 * i] = fmaxf(a, 0.f);
+        w[2 * i + 1] = fmaxf(b, 0.f);
+    }
+}
+
+// Draw mass of items [i0, i1) of the target row's items, by one warp: half an
+// item of both rows is in flight while the other half is summed.
+template <typename T>
+__device__ __forceinline__ float item_masses(const DrawRow<T>& d, int i0, int i1, int V, int lane) {
+    constexpr int kPer = 16 / (int)sizeof(T), kN = kVecs / 2, kHalf = 32 * kN * kPer;
+    const int mis = misaligned_by(d.rt);
+    auto load = [&](int h, uint4 (&t)[kN], uint4 (&q)[kN]) {
+        const int base = h * kHalf - mis, at = base + lane * kPer;
+        if (base >= 0 && base + kHalf <= V && d.same) {
+#pragma unroll
+            for (int u = 0; u < kN; ++u) {
+                t[u] = __ldg(reinterpret_cast<const uint4*>(d.rt + at + u * 32 * kPer));
+                q[u] = __ldg(reinterpret_cast<const uint4*>(d.rd + at + u * 32 * kPer));
+            }
+        } else {
+            uint4 x[2 * kN];
+            load_slow(d.rt, at, 32 * kPer, kN, V, x);
+            load_slow(d.rd, at, 32 * kPer, kN, V, x + kN);
+#pragma unroll
+            for (int u = 0; u < kN; ++u) {
+                t[u] = x[u];
+                q[u] = x[kN + u];
+            }
+        }
+    };
+    auto sum = [&](const uint4 (&t)[kN], const uint4 (&q)[kN]) {
+        float acc = 0.f;
+#pragma unroll
+        for (int u = 0; u < kN; ++u) {
+            float w[kPer];
+            weigh(d, t[u], q[u], w);
+            float s = 0.f;
+#pragma unroll
+            for (int e = 0; e < kPer; ++e) s += w[e];
+            acc += s;
+        }
+        return acc;
+    };
+    uint4 ta[kN], qa[kN], tb[kN], qb[kN];
+    float acc = 0.f;
+    load(2 * i0, ta, qa);
+#pragma unroll 1
+    for (int i = i0; i < i1; ++i) {
+        load(2 * i + 1, tb, qb);
+        acc += sum(ta, qa);
+        if (i + 1 < i1) load(2 * i + 2, ta, qa);
+        acc += sum(tb, qb);
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+    return acc;
+}
+
+// The grid fills the device once.  A unit is up to U items of one row and
+// leaves one partial, so the results do not depend on which warp takes it.
+// Phase 0 deals every warp an equal contiguous range of units.  kLater, the
+// phases after it: the requests still undecided, and one row of draw masses
+// for each that the phase before decided, are listed first; the last quarter
+// of the units goes to whichever warp is free, by a counter (a short phase
+// dealt out in equal shares ended 20-30% after its mean).  A warp keeps the next item in flight
+// while it reduces the current one, across units.
+template <typename T, bool kGreedy, bool kLater>
+__global__ void __launch_bounds__(kThreads, 2) accept_stats_kernel(const StatsParams p) {
     constexpr int kPer = 16 / (int)sizeof(T);
     constexpr int kItem = kItemBytes / (int)sizeof(T);
-    const int lane = threadIdx.x & 31;
-    const long long w = (long long)blockIdx.x * kWarps + (threadIdx.x >> 5);
+    constexpr bool kMass = kLater && !kGreedy;
+    __shared__ uint16_t s_list[kLater ? kMaxPhased : 1];   // undecided requests from the front, decided from the back
+    __shared__ int s_wcount[2][kWarps];
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     // launched as a programmatic dependent of the kernel before it: its
-    // inputs are read only past this wait, and the second kernel (which
+    // inputs are read only past this wait, and the next kernel (which
     // reads some inputs before its own wait) only starts after it
     wait_prior_grid();
     allow_dependent_launch();
-    if (w >= p.W) return;
-    const long long lo = range_lo(p, w), hi = range_lo(p, w + 1);
-    const int I = p.I, V = p.V, R = p.R;
-    // tree: the draft row of a node without children is never used; its
-    // items are skipped (read as -inf).  The child mask is cached per request.
-    long long kids_b = -1;
-    uint64_t kids = 0;
-    auto unused_row = [&](long long row) -> bool {
-        if (kGreedy || !p.parents) return false;
-        const int r = (int)(row % R);
-        if (r < p.n_t) return false;
-        const long long b = row / R;
-        if (b != kids_b) {
-            kids = tree_child_mask(p.parents + (size_t)b * p.n_t, p.n_t, lane);
-            kids_b = b;
+    const int I = p.I, V = p.V, R = p.ph.R, t_rows = p.ph.t_rows, p0 = p.ph.p0, units = p.ph.units, U = p.ph.U;
+    int requests = p.B, massed = 0;
+    if (kLater) {
+        requests = 0;
+        for (int b0 = 0; b0 < p.B; b0 += kThreads) {
+            const int a = b0 + tid < p.B ? __ldcg(p.ph.undecided + b0 + tid) : INT_MAX;
+            const bool in = a < 0, mass = kMass && a >= p.mass_lo && a < p.mass_hi;
+            const unsigned m0 = __ballot_sync(0xffffffffu, in), m1 = __ballot_sync(0xffffffffu, mass);
+            if (lane == 0) {
+                s_wcount[0][wid] = __popc(m0);
+                s_wcount[1][wid] = __popc(m1);
+            }
+            __syncthreads();
+            int at0 = requests + __popc(m0 & ((1u << lane) - 1u)), at1 = massed + __popc(m1 & ((1u << lane) - 1u));
+#pragma unroll 1
+            for (int i = 0; i < kWarps; ++i) {
+                const int n0 = s_wcount[0][i], n1 = s_wcount[1][i];
+                if (i < wid) {
+                    at0 += n0;
+                    at1 += n1;
+                }
+                requests += n0;
+                massed += n1;
+            }
+            if (in) s_list[at0] = (uint16_t)(b0 + tid);
+            if (mass) s_list[kMaxPhased - 1 - at1] = (uint16_t)(b0 + tid);
+            __syncthreads();
         }
-        return !((kids >> (r - p.n_t)) & 1ull);
-    };
+    }
+    // contiguous shares; of a later phase the last quarter goes by the counter
+    const int W = (int)gridDim.x * kWarps, w = (int)blockIdx.x * kWarps + wid;
+    const long long N = (long long)requests * R * units, fixed = kLater ? N - N / 4 : N;
+    long long unit = div_nn(w * fixed, W);
+    const long long hi = div_nn((w + 1) * fixed, W);
 
+    const T* rp = nullptr;   // row, items and partial of the unit whose items are being loaded
+    int item = 0, end = 0;
+    long long slot = 0;
+    bool skip = false;
+    auto open_unit = [&](long long x) {
+        const long long row = p.by_units.div(x);
+        const int u = (int)(x - row * units);
+        const int idx = (int)p.by_R.div(row), r = (int)(row - (long long)idx * R);
+        const int b = kLater ? s_list[idx] : idx;
+        const int at = p0 + (r < t_rows ? r : r - t_rows);   // the row's node
+        rp = r < t_rows ? static_cast<const T*>(p.target) + ((size_t)b * p.n + at) * V
+                        : static_cast<const T*>(p.draft) + ((size_t)b * p.d_rows + at) * V;
+        item = u * U;
+        end = min(item + U, I);
+        slot = ((long long)b * R + r) * units + u;
+        // tree: the draft row of a node without children is never used
+        if (!kLater && !kGreedy && p.parents)
+            skip = r >= t_rows && !((tree_child_mask(p.parents + (size_t)b * p.n, p.n, lane) >> at) & 1ull);
+    };
     // One item into registers: lane l holds vectors u*32 + l; entries past
-    // the row's end read as -inf.
-    auto load = [&](long long row, int item, uint4 (&v)[kVecs]) {
-        if (unused_row(row)) {
+    // the row's end, and skipped rows, read as -inf.
+    auto load = [&](uint4 (&v)[kVecs]) {
+        if (skip) {
             Vec16<T> ninf;
 #pragma unroll
             for (int e = 0; e < 16 / (int)sizeof(T); ++e) ninf.t[e] = (T)kNegInf;
@@ -323,47 +541,60 @@ __global__ void __launch_bounds__(kThreads, 2) accept_stats_kernel(const AcceptP
             for (int u = 0; u < kVecs; ++u) v[u] = ninf.q;
             return;
         }
-        const T* rp = row_ptr<T>(p, (int)(row / R), (int)(row % R));
-        const int e0 = item * kItem, e1 = min(V, e0 + kItem);
-        if (aligned16(rp) && e1 - e0 == kItem) {
-#pragma unroll
-            for (int u = 0; u < kVecs; ++u) v[u] = ld_stream(rp + e0 + (u * 32 + lane) * kPer);
-        } else {
-            const bool vec = aligned16(rp);
-#pragma unroll
-            for (int u = 0; u < kVecs; ++u) v[u] = load16<T, true>(rp, e0 + (u * 32 + lane) * kPer, e1, vec);
-        }
+        load_block(rp, item, V, lane, v);
     };
 
-    long long row = div_nn(lo, I);
-    int item = (int)(lo - row * I);
-    uint4 cur[kVecs], nxt[kVecs];
-    load(row, item, cur);
+    if (kMass) {
+        // draw masses first: their rows were read last, so they are in L2
+        const long long M = (long long)massed * units, m1 = div_nn((w + 1) * M, W);
+#pragma unroll 1
+        for (long long x = div_nn(w * M, W); x < m1; ++x) {
+            const long long i = p.by_units.div(x);
+            const int u = (int)(x - i * units), b = s_list[kMaxPhased - 1 - (int)i];
+            const int a = __ldcg(p.ph.undecided + b);
+            const float4 st = __ldcg(p.stat + b);
+            DrawRow<T> d;
+            d.rt = static_cast<const T*>(p.target) + ((size_t)b * p.n + a) * V;
+            d.rd = static_cast<const T*>(p.draft) + ((size_t)b * p.d_rows + a) * V;
+            set_weights(d, make_float2(st.x, st.y), make_float2(st.z, st.w), 1.f, p.c_hi);
+            const float acc = item_masses(d, u * U, min((u + 1) * U, I), V, lane);
+            if (lane == 0) p.mass[(size_t)b * units + u] = acc;
+        }
+    }
+    if (N == 0) return;
+    unsigned next = 0;   // the ticket taken ahead (lane 0)
+    if (kLater && unit + 1 >= hi && lane == 0) next = atomicAdd(p.ph.ticket, 1u);
+    if (unit >= hi) {
+        if (!kLater) return;
+        unit = fixed + __shfl_sync(0xffffffffu, next, 0);
+        if (unit >= N) return;
+        if (lane == 0) next = atomicAdd(p.ph.ticket, 1u);
+    }
+    open_unit(unit);
+
     float m = kNegInf, s = 0.f;            // sampling: lane's running (max, sum)
     int id = INT_MAX;                      // greedy: lane's lowest id of the max (m)
-    for (long long f = lo; f < hi; ++f) {
-        long long nrow = row;
-        int nitem = item + 1;
-        if (nitem == I) {
-            nrow = row + 1;
-            nitem = 0;
-        }
-        if (f + 1 < hi) load(nrow, nitem, nxt);
-        if (kGreedy) {
-            const int base = item * kItem;
-#pragma unroll
-            for (int u = 0; u < kVecs; ++u) {   // ascending ids: strict > keeps the lowest
-                Vec16<T> v;
-                v.q = cur[u];
-#pragma unroll
-                for (int e = 0; e < kPer; ++e) {
-                    const float z = to_f(v.t[e]);
-                    if (z > m) {
-                        m = z;
-                        id = base + (u * 32 + lane) * kPer + e;
-                    }
-                }
+    bool more = true;
+    // reduces the item in `cur` while the next one lands in `nxt`
+    auto step = [&](uint4 (&cur)[kVecs], uint4 (&nxt)[kVecs]) {
+        const int at0 = kGreedy ? item * kItem - misaligned_by(rp) + lane * kPer : 0;
+        const long long done = slot;
+        const bool unit_end = ++item == end;
+        if (unit_end) {
+            ++unit;
+            if (kLater && unit >= hi) {
+                unit = fixed + __shfl_sync(0xffffffffu, next, 0);
+                more = unit < N;
+            } else {
+                more = unit < hi;
             }
+            if (more) open_unit(unit);
+        }
+        if (more) load(nxt);
+        // a ticket ahead from the share's last unit on
+        if (kLater && unit_end && more && unit + 1 >= hi && lane == 0) next = atomicAdd(p.ph.ticket, 1u);
+        if (kGreedy) {
+            item_argmax<T>(cur, at0, m, id);
         } else {
             const float mi = item_max(cur, T());
             if (mi > m) {
@@ -372,66 +603,49 @@ __global__ void __launch_bounds__(kThreads, 2) accept_stats_kernel(const AcceptP
             }
             if (m != kNegInf) s += item_sum<T>(cur, m, p.c_hi);
         }
-        if (nitem == 0 || f + 1 == hi) {
-            // the row segment ends: fold the lanes and publish the pair in
-            // slot w - (owner of the row's first item) of the row
+        if (unit_end) {
+            // fold the lanes and publish the pair
             const float2 acc = kGreedy ? warp_fold_argmax(make_float2(m, __int_as_float(id)))
                                        : warp_fold_sum(m, s, p.c_hi, p.c_lo);
-            if (lane == 0) {
-                const long long first_owner = div_nn((row * I + 1) * p.W - 1, p.N);
-                const int j = (int)(w - first_owner);
-                p.part[row * p.J + j] = acc;
-                if (nitem == 0) p.cnt[row] = j + 1;   // this warp holds the row's last item
-            }
+            if (lane == 0) p.ph.part[done] = acc;
             m = kNegInf;
             s = 0.f;
             id = INT_MAX;
         }
-        row = nrow;
-        item = nitem;
-#pragma unroll
-        for (int u = 0; u < kVecs; ++u) cur[u] = nxt[u];
+    };
+    uint4 va[kVecs], vb[kVecs];
+    load(va);
+    for (;;) {
+        step(va, vb);
+        if (!more) break;
+        step(vb, va);
+        if (!more) break;
     }
 }
 
-// ------------------------------------------------- row statistics (kernel 2)
-// Row g's partials are part[g*J .. g*J + cnt[g]), in the order of the row.
-// Lane l folds slots l, l+32, ... in order, then the lanes are folded; the
-// result is the same in every lane and in every CTA that folds row g.
-// The rows of one call are folded kBatch at a time, with the loads of a
-// whole batch in flight together.
+// Statistics of kBatch rows (r0, r0 + step, ... below R) of request b: lane l
+// folds units l, l + 32, ... in order, then the lanes; the same numbers in
+// every warp that folds the row.  The rows' loads are in flight together.
 template <bool kGreedy, int kBatch>
-__device__ __forceinline__ void fold_rows(const AcceptParams& p, int b, int first_row, int row_step,
-                                          int n_rows, int lane, float2* s_stat) {
+__device__ __forceinline__ void fold_rows(const Phase& ph, int b, int r0, int step, int lane, float c_hi, float c_lo,
+                                          float2 (&f)[kBatch]) {
     const float2 empty = make_float2(kNegInf, kGreedy ? __int_as_float(INT_MAX) : 0.f);
-    for (int r0 = first_row; r0 < n_rows; r0 += kBatch * row_step) {
-        float2 pre[kBatch];
-        int n[kBatch];
+    const float2* const part = ph.part + (size_t)b * ph.R * ph.units;
 #pragma unroll
-        for (int j = 0; j < kBatch; ++j) {
-            const int r = r0 + j * row_step;
-            pre[j] = empty;
-            n[j] = 0;
-            if (r < n_rows) {
-                const long long g = (long long)b * p.R + r;
-                n[j] = __ldcg(p.cnt + g);
-                if (lane < p.J) pre[j] = __ldcg(p.part + g * p.J + lane);
-            }
-        }
+    for (int i = 0; i < kBatch; ++i) {
+        const int r = r0 + i * step;
+        f[i] = r < ph.R && lane < ph.units ? __ldcg(part + (size_t)r * ph.units + lane) : empty;
+    }
 #pragma unroll
-        for (int j = 0; j < kBatch; ++j) {
-            const int r = r0 + j * row_step;
-            if (r >= n_rows) break;
-            const long long g = (long long)b * p.R + r;
-            float2 f = lane < n[j] ? pre[j] : empty;
-            for (int l = lane + 32; l < n[j]; l += 32) {
-                const float2 o = __ldcg(p.part + g * p.J + l);
-                if (kGreedy) argmax_fold(f, o);
-                else fold(f.x, f.y, o.x, o.y, p.c_hi, p.c_lo);
-            }
-            f = kGreedy ? warp_fold_argmax(f) : warp_fold_sum(f.x, f.y, p.c_hi, p.c_lo);
-            if (lane == 0) s_stat[r] = f;
+    for (int i = 0; i < kBatch; ++i) {
+        const int r = r0 + i * step;
+#pragma unroll 1
+        for (int l = lane + 32; r < ph.R && l < ph.units; l += 32) {
+            const float2 o = __ldcg(part + (size_t)r * ph.units + l);
+            if (kGreedy) argmax_fold(f[i], o);
+            else fold(f[i].x, f[i].y, o.x, o.y, c_hi, c_lo);
         }
+        f[i] = kGreedy ? warp_fold_argmax(f[i]) : warp_fold_sum(f[i].x, f[i].y, c_hi, c_lo);
     }
 }
 
@@ -455,10 +669,84 @@ __device__ __forceinline__ float accept_ratio(bool valid, float zt, float zd, fl
     return ex2(H) * fmaf(E, kLn2, 1.f);
 }
 
-// Whether position i rejects: u_i < p_i(x_i) / q_i(x_i) fails.
-__device__ __forceinline__ bool rejects(bool valid, float zt, float zd, float2 st, float2 sd, float u,
-                                        float c_hi, float c_lo) {
-    return !(u < accept_ratio(valid, zt, zd, st, sd, c_hi, c_lo));
+// ------------------------------------------------------------ test kernel
+// What a phase decides: per request the accepted count a, or -1 while every
+// position so far is accepted, and the statistics of the deciding row pair
+// (greedy: the emitted token's bits in x).
+struct Decided {
+    int* a;        // [B]
+    float4* stat;  // [B]
+};
+
+struct TestParams {
+    const void* target;
+    const void* draft;
+    const int32_t* tokens;    // [B, n-1]
+    const float* uniforms;    // [B, n]
+    int B, V, n;
+    float c_hi, c_lo;
+    Phase ph;
+    Decided dec;
+};
+
+// One warp per request tests the positions of a phase (a single phase's are
+// tested by the walk kernel).
+template <typename T, bool kGreedy>
+__global__ void __launch_bounds__(kThreads) accept_test_kernel(const TestParams p) {
+    constexpr int kBatch = 4;
+    __shared__ float2 s_stat[kWarps][2 * kMaxTreeNodes];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int b = blockIdx.x * kWarps + wid;
+    const int p0 = p.ph.p0, g = p.ph.t_rows, R = p.ph.R;
+    const int tests = min(g, p.n - 1 - p0);   // positions with a draft (all but a chain's last)
+    int x = -1;
+    float zt = kNegInf, zd = 0.f, u = 1.f;
+    if (b < p.B && lane < tests) {
+        x = __ldg(p.tokens + (size_t)b * (p.n - 1) + p0 + lane);
+        if (!kGreedy) {
+            u = __ldg(p.uniforms + (size_t)b * p.n + p0 + lane);
+            if (x >= 0 && x < p.V) {
+                zt = to_f(static_cast<const T*>(p.target)[((size_t)b * p.n + p0 + lane) * p.V + x]);
+                zd = to_f(static_cast<const T*>(p.draft)[((size_t)b * (p.n - 1) + p0 + lane) * p.V + x]);
+            }
+        }
+    }
+    wait_prior_grid();
+    allow_dependent_launch();
+    if (blockIdx.x == 0 && threadIdx.x == 0) *p.ph.ticket = 0;   // for the next phase
+    if (b >= p.B) return;
+    if (p.ph.undecided && __ldcg(p.ph.undecided + b) >= 0) return;
+#pragma unroll 1
+    for (int r0 = 0; r0 < R; r0 += kBatch) {
+        float2 f[kBatch];
+        fold_rows<kGreedy, kBatch>(p.ph, b, r0, 1, lane, p.c_hi, p.c_lo, f);
+#pragma unroll
+        for (int i = 0; i < kBatch; ++i)
+            if (lane == i && r0 + i < R) s_stat[wid][r0 + i] = f[i];
+    }
+    __syncwarp();
+    bool rej = false;
+    int top = 0;
+    float2 st = make_float2(0.f, 0.f), sd = st;
+    if (lane < g) {
+        st = s_stat[wid][lane];
+        if (kGreedy) {
+            top = __float_as_int(st.y);
+            if (top == INT_MAX) top = 0;   // a row with no finite entry
+            rej = lane < tests && x != top;
+        } else if (lane < tests) {
+            sd = s_stat[wid][g + lane];
+            rej = !(u < accept_ratio(zt != kNegInf, zt, zd, st, sd, p.c_hi, p.c_lo));
+        }
+    }
+    const unsigned m = __ballot_sync(0xffffffffu, rej);
+    const int at = m ? __ffs(m) - 1 : tests;   // the deciding position
+    if (at == g) {
+        if (lane == 0) p.dec.a[b] = -1;
+    } else if (lane == at) {
+        p.dec.a[b] = p0 + lane;
+        p.dec.stat[b] = kGreedy ? make_float4(__int_as_float(top), 0.f, 0.f, 0.f) : make_float4(st.x, st.y, sd.x, sd.y);
+    }
 }
 
 // ------------------------------------------------------------ cluster PTX
@@ -482,677 +770,34 @@ __device__ __forceinline__ void cluster_wait() {
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-// Reads a float2 at the same shared-memory offset in CTA `rank` of the cluster.
-__device__ __forceinline__ float2 ld_cluster_f2(const float2* local, uint32_t rank) {
-    uint32_t remote;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(smem_u32(local)), "r"(rank));
-    float2 v;
-    asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(remote) : "memory");
-    return v;
-}
-
-// ------------------------------------------------------------ draw weights
-// Weights of thread-run [start, start + kRun) of the draw row pair (entries at
-// or past `end` weigh zero): max(p - q, 0), or p alone when !residual.
-template <typename T>
-// The draw weights are p and max(p - q, 0) scaled by S_t (the inverse CDF
-// does not depend on a common factor): 2^((zt - mt)c) and
-// max(2^((zt - mt)c) - rho 2^((zd - md)c), 0) with rho = S_t / S_d.
-struct DrawRow {
-    const T* rt;
-    const T* rd;
-    float mt, md, rho, c_hi;
-    bool at, ad;
-};
-
-template <typename T, bool kResidual>
-__device__ __forceinline__ void run_weights(const DrawRow<T>& d, int start, int end,
-                                            float (&w)[kRunVecs * 16 / sizeof(T)]) {
-    constexpr int kPer = 16 / (int)sizeof(T);
-    uint4 vt[kRunVecs], vd[kRunVecs];
-    if (d.at && (!kResidual || d.ad) && start + kRunVecs * kPer <= end) {
-#pragma unroll
-        for (int u = 0; u < kRunVecs; ++u) {
-            vt[u] = __ldg(reinterpret_cast<const uint4*>(d.rt + start + u * kPer));
-            if (kResidual) vd[u] = __ldg(reinterpret_cast<const uint4*>(d.rd + start + u * kPer));
-        }
-    } else {
-#pragma unroll
-        for (int u = 0; u < kRunVecs; ++u) {
-            vt[u] = load16<T, false>(d.rt, start + u * kPer, end, d.at);
-            if (kResidual) vd[u] = load16<T, false>(d.rd, start + u * kPer, end, d.ad);
-        }
-    }
-#pragma unroll
-    for (int u = 0; u < kRunVecs; ++u) {
-        Vec16<T> a, b;
-        a.q = vt[u];
-        if (kResidual) b.q = vd[u];
-#pragma unroll
-        for (int e = 0; e < kPer; ++e) {
-            const float pt = weight(to_f(a.t[e]), d.mt, d.c_hi);
-            if (kResidual) w[u * kPer + e] = fmaxf(fmaf(-d.rho, weight(to_f(b.t[e]), d.md, d.c_hi), pt), 0.f);
-            else w[u * kPer + e] = pt;
-        }
-    }
-}
-
-// One pass of a CTA over logits [pass_start, pass_start + kDrawThreads*kRun):
-// every thread's weights, its inclusive scan position and the pass total.
-// The warp totals are folded in warp order, so the pass total and every
-// thread's prefix are the same numbers whenever the pass is recomputed.
-struct PassScan {
-    float incl;    // mass of the pass up to and including this thread's run
-    float excl;    // incl less the thread's own run (the start of its walk)
-    float own;     // mass of this thread's run
-    float total;   // mass of the pass
-    int last;      // largest id of the pass with positive weight, -1 if none
-};
-
-template <typename T, bool kResidual>
-__device__ __forceinline__ PassScan pass_scan_t(const DrawRow<T>& d, int pass_start, int end,
-                                              float (&w)[kRunVecs * 16 / sizeof(T)], float (&s_wsum)[kDrawWarps],
-                                              int (&s_wlast)[kDrawWarps]) {
-    constexpr int kRun = kRunVecs * 16 / (int)sizeof(T);
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    const int start = pass_start + tid * kRun;
-    run_weights<T, kResidual>(d, start, end, w);
-    float ls = 0.f;
-    int lp = -1;
-#pragma unroll
-    for (int e = 0; e < kRun; ++e) {
-        ls += w[e];
-        if (w[e] > 0.f) lp = start + e;
-    }
-    const float incl = warp_incl_scan(ls, lane);
-    lp = warp_max_int(lp);
-    if (lane == 31) s_wsum[wid] = incl;
-    if (lane == 0) s_wlast[wid] = lp;
-    __syncthreads();
-    PassScan r;
-    float off = 0.f, tot = 0.f;
-    int last = -1;
-#pragma unroll
-    for (int j = 0; j < kDrawWarps; ++j) {
-        if (j == wid) off = tot;
-        tot += s_wsum[j];
-        last = max(last, s_wlast[j]);
-    }
-    __syncthreads();   // s_wsum / s_wlast are reused by the next pass
-    // the last thread's incl is the pass total bit for bit (same additions)
-    r.incl = off + incl;
-    r.excl = r.incl - ls;
-    r.own = ls;
-    r.total = tot;
-    r.last = last;
-    return r;
-}
-
-template <typename T>
-__device__ __forceinline__ PassScan pass_scan(const DrawRow<T>& d, bool residual, int pass_start, int end,
-                                              float (&w)[kRunVecs * 16 / sizeof(T)], float (&s_wsum)[kDrawWarps],
-                                              int (&s_wlast)[kDrawWarps]) {
-    return residual ? pass_scan_t<T, true>(d, pass_start, end, w, s_wsum, s_wlast)
-                    : pass_scan_t<T, false>(d, pass_start, end, w, s_wsum, s_wlast);
-}
-
-// Per-warp pass totals of a slice (one block-wide buffer per kernel).
-__device__ __forceinline__ float* draw_warp_pass_totals() {
-    __shared__ float s_wpass[kDrawWarps * kMaxPasses];
-    return s_wpass;
-}
-
-struct SliceMass {
-    float mass;   // the slice's mass: the pass totals added in pass order
-    int last;     // largest id of the slice with positive weight, -1 if none
-};
-
-// All n_pass passes of this CTA's slice [c0, c1), streamed without a block
-// barrier per pass: each warp folds its runs with the warp scan of pass_scan
-// and leaves its total for the pass; one barrier at the end, then every pass
-// total is the warp totals added in warp order, bit for bit the total that
-// pass_scan computes when the pass is walked again.  s_pass[ps] receives
-// them.
-template <typename T, bool kResidual>
-__device__ __forceinline__ SliceMass slice_passes_t(const DrawRow<T>& d, int c0, int c1, int n_pass, float* s_pass,
-                                                    int (&s_wlast)[kDrawWarps]) {
-    constexpr int kRun = kRunVecs * 16 / (int)sizeof(T);
-    constexpr int kPass = kDrawThreads * kRun;
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    float* s_wpass = draw_warp_pass_totals();
-    float w[kRun];
-    int last = -1;
-    for (int ps = 0; ps < n_pass; ++ps) {
-        const int nx = c0 + (ps + 1) * kPass + tid * kRun;
-        if (ps + 1 < n_pass && (tid & 3) == 0 && nx < c1) {
-            // the next pass into L1 while this one is reduced (a 128-byte
-            // line holds the runs of four threads); only addresses inside the
-            // slice are touched
-            asm volatile("prefetch.global.L1 [%0];" ::"l"(d.rt + nx));
-            if (kResidual) asm volatile("prefetch.global.L1 [%0];" ::"l"(d.rd + nx));
-        }
-        const int start = c0 + ps * kPass + tid * kRun;
-        run_weights<T, kResidual>(d, start, c1, w);
-        float ls = 0.f;
-#pragma unroll
-        for (int e = 0; e < kRun; ++e) {
-            ls += w[e];
-            if (w[e] > 0.f) last = start + e;
-        }
-        const float incl = warp_incl_scan(ls, lane);
-        if (lane == 31) s_wpass[wid * kMaxPasses + ps] = incl;
-    }
-    last = warp_max_int(last);
-    if (lane == 0) s_wlast[wid] = last;
-    __syncthreads();
-    if (tid < n_pass) {
-        float tot = 0.f;
-#pragma unroll
-        for (int j = 0; j < kDrawWarps; ++j) tot += s_wpass[j * kMaxPasses + tid];
-        s_pass[tid] = tot;
-    }
-    SliceMass r{0.f, -1};
-#pragma unroll
-    for (int j = 0; j < kDrawWarps; ++j) r.last = max(r.last, s_wlast[j]);
-    __syncthreads();
-    for (int ps = 0; ps < n_pass; ++ps) r.mass += s_pass[ps];
-    __syncthreads();   // s_wlast / s_pass stay unchanged until every thread has read them
-    return r;
-}
-
-template <typename T>
-__device__ __forceinline__ SliceMass slice_passes(const DrawRow<T>& d, bool residual, int c0, int c1, int n_pass,
-                                                  float* s_pass, int (&s_wlast)[kDrawWarps]) {
-    return residual ? slice_passes_t<T, true>(d, c0, c1, n_pass, s_pass, s_wlast)
-                    : slice_passes_t<T, false>(d, c0, c1, n_pass, s_pass, s_wlast);
-}
-
-// ------------------------------------------------------------ the draw
-// Inverse-CDF draw of one token from the weights of row pair d -- p, or
-// max(p - rho q, 0) when `residual` (rho as folded into d) -- over the
-// vocabulary slices of the cluster: this CTA owns [c0, c1) in n_pass passes.
-// Round 0 sums the slice masses and swaps them through distributed shared
-// memory; a residual without positive mass falls back to p in round 1.  On
-// return `writer` is the thread of this CTA that stores `token` (-1: another
-// CTA does).  Exchange slots alternate with the round counter xr, so one
-// cluster barrier per round keeps a slot from being rewritten while a peer
-// may still read it.
-template <typename T>
-__device__ __forceinline__ void cluster_draw(const DrawRow<T>& d, bool residual, float uk, int c0, int c1,
-                                             int n_pass, uint32_t rank, uint32_t n_ranks, float* s_pass,
-                                             float (&s_wsum)[kDrawWarps], int (&s_wlast)[kDrawWarps],
-                                             int (&s_first)[kDrawWarps], float2* s_x, int& xr, int& token,
-                                             int& writer) {
-    constexpr int kPer = 16 / (int)sizeof(T);
-    constexpr int kRun = kRunVecs * kPer;
-    constexpr int kPass = kDrawThreads * kRun;
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    float w[kRun];
-    token = 0;
-    writer = -1;
-    for (int round = 0; round < 2; ++round) {
-        // one pass: scanned at once, its weights and prefixes kept for the
-        // walk; several: streamed, and the owning pass walked again
-        PassScan kept{0.f, 0.f, 0.f, 0.f, -1};
-        SliceMass sm{0.f, -1};
-        if (n_pass == 1) {
-            kept = pass_scan<T>(d, residual, c0, c1, w, s_wsum, s_wlast);
-            if (tid == 0) s_pass[0] = kept.total;
-            sm.mass = kept.total;
-            sm.last = kept.last;
-        } else {
-            sm = slice_passes<T>(d, residual, c0, c1, n_pass, s_pass, s_wlast);
-        }
-        const float mass = sm.mass;
-        const int last = sm.last;
-        const int slot = xr & 1;
-        ++xr;
-        if (tid == 0) s_x[slot] = make_float2(mass, __int_as_float(last));
-        cluster_arrive();
-        cluster_wait();
-        // every CTA folds the masses of ranks 0..n-1 in the same order
-        float2 x = make_float2(0.f, __int_as_float(-1));
-        if (lane < (int)n_ranks) x = ld_cluster_f2(&s_x[slot], lane);
-        const float incl = warp_incl_scan(x.x, lane);
-        const float Z = __shfl_sync(0xffffffffu, incl, 31);
-        if (!(Z > 0.f) && residual && round == 0) {
-            // no positive residual (p == q up to rounding): draw from p instead
-            residual = false;
-            continue;
-        }
-        const float t = uk * Z;
-        const float before = incl - x.x;
-        const unsigned own = __ballot_sync(0xffffffffu, lane < (int)n_ranks && x.x > 0.f && incl > t);
-        if (!own) {
-            // u_k * Z at or past the total through rounding: the last positive weight
-            const int lp = warp_max_int(__float_as_int(x.y));
-            token = lp >= 0 ? lp : 0;
-            if (rank == 0) writer = 0;
-            break;
-        }
-        const int owner = __ffs(own) - 1;
-        if ((int)rank != owner) break;
-        float tt = t - __shfl_sync(0xffffffffu, before, owner);   // position within this slice
-        // the pass that holds the cell, in the order the mass was summed
-        int pj = -1;
-        float cum = 0.f;
-        for (int ps = 0; ps < n_pass; ++ps) {
-            const float m = s_pass[ps];
-            if (m > 0.f && cum + m > tt) {
-                pj = ps;
-                break;
-            }
-            cum += m;
-        }
-        if (pj < 0) {   // rounding: the slice's last positive weight
-            token = last;
-            writer = 0;
-            break;
-        }
-        tt -= cum;
-        // walked again, the pass's scan reproduces its total bit for bit
-        const PassScan sc = n_pass == 1 ? kept : pass_scan<T>(d, residual, c0 + pj * kPass, c1, w, s_wsum, s_wlast);
-        // the first run with positive mass whose prefix passes tt (a run of
-        // zero weights can come first through rounding; it never owns the draw)
-        const unsigned cross = __ballot_sync(0xffffffffu, sc.own > 0.f && sc.incl > tt);
-        if (lane == 0) s_first[wid] = cross ? wid * 32 + __ffs(cross) - 1 : INT_MAX;
-        __syncthreads();
-        int first = INT_MAX;
-#pragma unroll
-        for (int j = 0; j < kDrawWarps; ++j) first = min(first, s_first[j]);
-        if (first == INT_MAX) {   // rounding: the pass's last positive weight
-            token = sc.last;
-            writer = 0;
-            break;
-        }
-        if (tid == first) {
-            const int start = c0 + pj * kPass + tid * kRun;
-            float c = sc.excl;
-            int pick = -1, lastp = -1;
-#pragma unroll
-            for (int e = 0; e < kRun; ++e) {
-                c += w[e];
-                if (w[e] > 0.f) {   // only a token with positive weight can be drawn
-                    lastp = start + e;
-                    if (pick < 0 && c > tt) pick = start + e;
-                }
-            }
-            token = pick >= 0 ? pick : lastp;   // the run has a positive weight
-        }
-        writer = first;
-        break;
-    }}
-
-// ------------------------------------------------------------ kernel 2
-template <typename T>
-__global__ void __launch_bounds__(kDrawThreads, 2) accept_draw_kernel(const AcceptParams p) {
-    constexpr int kPer = 16 / (int)sizeof(T);
-    constexpr int kRun = kRunVecs * kPer;
-    constexpr int kPass = kDrawThreads * kRun;
-    __shared__ float2 s_stat[kMaxRows];
-    __shared__ float s_pass[kMaxPasses];
-    __shared__ float s_wsum[kDrawWarps];
-    __shared__ int s_wlast[kDrawWarps];
-    __shared__ int s_first[kDrawWarps];
-    __shared__ int s_a;
-    __shared__ float2 s_x[2];   // (slice mass, last positive id) per exchange round
-
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    const uint32_t rank = cluster_rank(), n_ranks = cluster_size();
-    const int b = p.b_base + blockIdx.y;
-    const int k = p.k, V = p.V;
-
-    // ---- the accept-test inputs of lane i < k of warp 0, loaded first
-    bool valid = false;
-    float zt = 0.f, zd = 0.f, ui = 1.f;
-    int xi = -1;
-    if (wid == 0 && lane < k) {
-        xi = __ldg(p.tokens + (size_t)b * k + lane);
-        ui = __ldg(p.uniforms + (size_t)b * (k + 1) + lane);
-        valid = xi >= 0 && xi < V;
-        if (valid) {
-            zt = to_f(row_ptr<T>(p, b, lane)[xi]);
-            zd = to_f(row_ptr<T>(p, b, k + 1 + lane)[xi]);
-        }
-    }
-    const float uk = __ldg(p.uniforms + (size_t)b * (k + 1) + k);
-
-    // ---- row statistics of the request (kernel 1's output), then the tests
-    wait_prior_grid();
-    allow_dependent_launch();   // the next call's first kernel may start
-    fold_rows<false, kRowsPerDrawWarp>(p, b, wid, kDrawWarps, p.R, lane, s_stat);
-    __syncthreads();
-    if (wid == 0) {
-        bool rej = false;
-        if (lane < k) rej = rejects(valid, zt, zd, s_stat[lane], s_stat[k + 1 + lane], ui, p.c_hi, p.c_lo);
-        const unsigned m = __ballot_sync(0xffffffffu, rej);
-        if (lane == 0) s_a = m ? __ffs(m) - 1 : k;
-    }
-    __syncthreads();
-    const int a = s_a;
-
-    // ---- the draw: this CTA's slice [c0, c1) of row pair a
-    const int c0 = min(V, (int)rank * p.slice), c1 = min(V, c0 + p.slice);
-    const int n_pass = (c1 - c0 + kPass - 1) / kPass;
-    DrawRow<T> d;
-    d.rt = row_ptr<T>(p, b, a);
-    d.rd = a < k ? row_ptr<T>(p, b, k + 1 + a) : d.rt;
-    // a row without a finite entry (outside the contract) weighs zero everywhere
-    const float2 st = s_stat[a], sd = a < k ? s_stat[k + 1 + a] : make_float2(0.f, 0.f);
-    d.mt = st.x == kNegInf ? 0.f : st.x;
-    d.md = sd.x == kNegInf ? 0.f : sd.x;
-    d.rho = sd.y > 0.f ? st.y / sd.y : 0.f;
-    d.c_hi = p.c_hi;
-    d.at = aligned16(d.rt);
-    d.ad = aligned16(d.rd);
-
-    if (n_pass > 1) {
-        // several passes: ask L2 for the whole slice of the row pair now, so
-        // that the passes below find it there instead of waiting on DRAM
-        const char* bt = reinterpret_cast<const char*>(d.rt + c0);
-        const char* bd = reinterpret_cast<const char*>(d.rd + c0);
-        const int bytes = (c1 - c0) * (int)sizeof(T);
-        for (int off = tid * 128; off < bytes; off += kDrawThreads * 128) {
-            asm volatile("prefetch.global.L2 [%0];" ::"l"(bt + off));
-            if (a < k) asm volatile("prefetch.global.L2 [%0];" ::"l"(bd + off));
-        }
-    }
-    int token = 0;
-    int writer = -1;   // the thread of this CTA that writes the emitted token
-    int xr = 0;
-    cluster_draw<T>(d, a < k, uk, c0, c1, n_pass, rank, n_ranks, s_pass, s_wsum, s_wlast, s_first, s_x, xr,
-                    token, writer);
-    if (tid == writer) p.out_tokens[(size_t)b * (k + 1) + a] = token >= 0 ? token : 0;
-    if (rank == 0 && tid <= k && tid != a) {
-        const int32_t x = tid < a ? __ldg(p.tokens + (size_t)b * k + tid) : -1;
-        p.out_tokens[(size_t)b * (k + 1) + tid] = x;
-    }
-    if (rank == 0 && tid == 0 && p.out_n) p.out_n[b] = a;
-    // no CTA leaves while another may still read its exchange slots
-    cluster_arrive();
-    cluster_wait();
-}
-
-// ------------------------------------------------------------ greedy
-template <typename T>
-__global__ void __launch_bounds__(kThreads) accept_greedy_kernel(const AcceptParams p) {
-    __shared__ float2 s_stat[kWarps][kMaxRows];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int b = blockIdx.x * kWarps + wid;
-    const int k = p.k;
-    wait_prior_grid();
-    allow_dependent_launch();   // the next call's first kernel may start
-    if (b >= p.B) return;
-    fold_rows<true, 4>(p, b, 0, 1, k + 1, lane, s_stat[wid]);
-    __syncwarp();
-    int g = 0, x = -1;
-    if (lane <= k) {
-        g = __float_as_int(s_stat[wid][lane].y);
-        if (g == INT_MAX) g = 0;   // a row with no finite entry
-    }
-    if (lane < k) x = __ldg(p.tokens + (size_t)b * k + lane);
-    const unsigned miss = __ballot_sync(0xffffffffu, lane < k && x != g);
-    const int a = miss ? __ffs(miss) - 1 : k;
-    const int emit = __shfl_sync(0xffffffffu, g, a);
-    if (lane <= k) p.out_tokens[(size_t)b * (k + 1) + lane] = lane < a ? x : (lane == a ? emit : -1);
-    if (lane == 0 && p.out_n) p.out_n[b] = a;
-}
-
-// ------------------------------------------------------------ token trees
-// Cluster-wide mass of the draw weights of row pair d (p scaled by S_t, or
-// max(p - kappa q, 0) scaled by S_t when `residual`): every CTA sums its
-// slice, the slice masses are swapped through distributed shared memory and
-// folded in rank order, so every CTA holds the same total.
-template <typename T>
-__device__ __forceinline__ float cluster_mass(const DrawRow<T>& d, bool residual, int c0, int c1, int n_pass,
-                                              uint32_t n_ranks, float (&s_wsum)[kDrawWarps],
-                                              int (&s_wlast)[kDrawWarps], float2* s_x, int& xr) {
-    __shared__ float s_tpass[kMaxPasses];
-    const float mass = slice_passes<T>(d, residual, c0, c1, n_pass, s_tpass, s_wlast).mass;
-    (void)s_wsum;
-    const int slot = xr & 1;
-    ++xr;
-    if (threadIdx.x == 0) s_x[slot] = make_float2(mass, 0.f);
-    cluster_arrive();
-    cluster_wait();
-    const int lane = threadIdx.x & 31;
-    float2 x = make_float2(0.f, 0.f);
-    if (lane < (int)n_ranks) x = ld_cluster_f2(&s_x[slot], lane);
-    return __shfl_sync(0xffffffffu, warp_incl_scan(x.x, lane), 31);
-}
-
-// One cluster per request walks its tree (multi-candidate speculative
-// sampling).  At node u the running distribution is r = max(p_u - kappa q_u,
-// 0) / Z (kappa = 0, Z = 1: r = p_u); child c with token x is accepted iff
-// u_{c-1} < r(x) / q_u(x) = max(p(x)/q(x) - kappa, 0) / Z.  A rejection
-// makes r the residual max(0, r - q_u) normalised, which is the same form
-// with kappa + Z in place of kappa; its mass is one cluster pass over the
-// row pair, needed only when another sibling is still to be tested (the
-// draw sums its own weights).  A residual without positive mass ends the
-// tests and the draw falls back to p_u.
-template <typename T>
-__global__ void __launch_bounds__(kDrawThreads, 2) tree_draw_kernel(const AcceptParams p) {
-    constexpr int kPer = 16 / (int)sizeof(T);
-    constexpr int kRun = kRunVecs * kPer;
-    constexpr int kPass = kDrawThreads * kRun;
-    __shared__ float2 s_stat[2 * kMaxTreeNodes];
-    __shared__ float2 s_z[kMaxTreeNodes];      // target / draft logit of node c's token in its parent's rows
-    __shared__ int s_par[kMaxTreeNodes];
-    __shared__ int s_tok[kMaxTreeNodes];
-    __shared__ float s_u[kMaxTreeNodes];
-    __shared__ unsigned long long s_kids[kMaxTreeNodes];
-    __shared__ int s_path[kMaxTreeNodes];
-    __shared__ float s_pass[kMaxPasses];
-    __shared__ float s_wsum[kDrawWarps];
-    __shared__ int s_wlast[kDrawWarps];
-    __shared__ int s_first[kDrawWarps];
-    __shared__ float2 s_x[2];
-
-    const int tid = threadIdx.x, lane = tid & 31;
-    const uint32_t rank = cluster_rank(), n_ranks = cluster_size();
-    const int b = p.b_base + blockIdx.y;
-    const int n = p.n_t, V = p.V;
-
-    // ---- the tree and every accept-test input, loaded before the statistics
-    for (int c = tid; c < n; c += kDrawThreads) {
-        int par = -1;
-        if (c > 0) {
-            const int q = __ldg(p.parents + (size_t)b * n + c);
-            par = (q >= 0 && q < c) ? q : -1;
-        }
-        const int x = __ldg(p.tokens + (size_t)b * n + c);
-        s_par[c] = par;
-        s_tok[c] = x;
-        s_u[c] = __ldg(p.uniforms + (size_t)b * n + c);
-        float2 z = make_float2(kNegInf, 0.f);    // an invalid token tests as ratio 0
-        if (par >= 0 && x >= 0 && x < V)
-            z = make_float2(to_f(row_ptr<T>(p, b, par)[x]), to_f(row_ptr<T>(p, b, n + par)[x]));
-        s_z[c] = z;
-    }
-    __syncthreads();
-    for (int u = tid; u < n; u += kDrawThreads) {
-        unsigned long long m = 0;
-        for (int c = u + 1; c < n; ++c)
-            if (s_par[c] == u) m |= 1ull << c;
-        s_kids[u] = m;
-    }
-    wait_prior_grid();
-    allow_dependent_launch();   // the next call's first kernel may start
-    fold_rows<false, 8>(p, b, tid >> 5, kDrawWarps, p.R, lane, s_stat);
-    __syncthreads();
-
-    // ---- the walk: every thread takes the same decisions from shared data
-    const int c0 = min(V, (int)rank * p.slice), c1 = min(V, c0 + p.slice);
-    const int n_pass = (c1 - c0 + kPass - 1) / kPass;
-    int node = 0, depth = 0, xr = 0;
-    float kappa = 0.f;
-    DrawRow<T> d;
-    d.c_hi = p.c_hi;
-    for (;;) {
-        const float2 st = s_stat[node], sd = s_stat[n + node];
-        d.rt = row_ptr<T>(p, b, node);
-        d.rd = row_ptr<T>(p, b, n + node);
-        d.mt = st.x == kNegInf ? 0.f : st.x;
-        d.md = sd.x == kNegInf ? 0.f : sd.x;
-        d.at = aligned16(d.rt);
-        d.ad = aligned16(d.rd);
-        const float rho1 = sd.y > 0.f ? st.y / sd.y : 0.f;
-        unsigned long long kids = s_kids[node];
-        float kap = 0.f, Z = 1.f;
-        int next = -1;
-        while (kids) {
-            const int c = __ffsll((long long)kids) - 1;
-            kids &= kids - 1;
-            const float2 z = s_z[c];
-            float ratio = accept_ratio(z.x != kNegInf, z.x, z.y, st, sd, p.c_hi, p.c_lo);
-            if (kap > 0.f) ratio = fmaxf(ratio - kap, 0.f) / Z;
-            if (s_u[c - 1] < ratio) {
-                next = c;
-                break;
-            }
-            kap += Z;               // the residual of this rejection
-            if (!kids) break;       // no sibling left: the draw sums its own weights
-            d.rho = kap * rho1;
-            Z = cluster_mass<T>(d, true, c0, c1, n_pass, n_ranks, s_wsum, s_wlast, s_x, xr) / st.y;
-            if (!(Z > 0.f)) {       // no positive residual (p == kappa q up to rounding): draw from p
-                kap = 0.f;
-                break;
-            }
-        }
-        if (next < 0) {
-            kappa = kap;
-            break;
-        }
-        if (tid == 0) s_path[depth] = next;
-        ++depth;
-        node = next;
-    }
-
-    // ---- the draw at the final node
-    d.rho = kappa * (s_stat[n + node].y > 0.f ? s_stat[node].y / s_stat[n + node].y : 0.f);
-    if (!(kappa > 0.f)) d.rd = d.rt;
-    if (n_pass > 1) {
-        const char* bt = reinterpret_cast<const char*>(d.rt + c0);
-        const char* bd = reinterpret_cast<const char*>(d.rd + c0);
-        const int bytes = (c1 - c0) * (int)sizeof(T);
-        for (int off = tid * 128; off < bytes; off += kDrawThreads * 128) {
-            asm volatile("prefetch.global.L2 [%0];" ::"l"(bt + off));
-            if (kappa > 0.f) asm volatile("prefetch.global.L2 [%0];" ::"l"(bd + off));
-        }
-    }
-    int token = 0, writer = -1;
-    cluster_draw<T>(d, kappa > 0.f, s_u[n - 1], c0, c1, n_pass, rank, n_ranks, s_pass, s_wsum, s_wlast, s_first,
-                    s_x, xr, token, writer);
-    __syncthreads();
-    int32_t* out = p.out_tokens + (size_t)b * n;
-    if (tid == writer) out[depth] = token >= 0 ? token : 0;
-    if (rank == 0) {
-        for (int i = tid; i < n; i += kDrawThreads) {
-            if (i < depth) {
-                out[i] = s_tok[s_path[i]];
-                p.out_path[(size_t)b * n + i] = s_path[i];
-            } else {
-                if (i > depth) out[i] = -1;
-                p.out_path[(size_t)b * n + i] = -1;
-            }
-        }
-        if (tid == 0) p.out_n[b] = depth;
-    }
-    // no CTA leaves while another may still read its exchange slots
-    cluster_arrive();
-    cluster_wait();
-}
-
-// Greedy tree walk, one warp per request: at node u the first child whose
-// token is the arg max of u's target row is accepted, else that arg max is
-// emitted.
-template <typename T>
-__global__ void __launch_bounds__(kThreads) tree_greedy_kernel(const AcceptParams p) {
-    __shared__ float2 s_stat[kWarps][kMaxTreeNodes];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int b = blockIdx.x * kWarps + wid;
-    if (b >= p.B) return;
-    const int n = p.n_t;
-    int par[2], tok[2];
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        const int c = lane + 32 * h;
-        par[h] = -1;
-        tok[h] = -1;
-        if (c < n) {
-            tok[h] = __ldg(p.tokens + (size_t)b * n + c);
-            if (c > 0) {
-                const int q = __ldg(p.parents + (size_t)b * n + c);
-                par[h] = (q >= 0 && q < c) ? q : -1;
-            }
-        }
-    }
-    wait_prior_grid();
-    allow_dependent_launch();   // the next call's first kernel may start
-    fold_rows<true, 4>(p, b, 0, 1, n, lane, s_stat[wid]);
-    __syncwarp();
-    int32_t* out = p.out_tokens + (size_t)b * n;
-    int32_t* path = p.out_path + (size_t)b * n;
-    int node = 0, depth = 0, g = 0;
-    for (;;) {
-        g = __float_as_int(s_stat[wid][node].y);
-        if (g == INT_MAX) g = 0;   // a row with no finite entry
-        const unsigned m0 = __ballot_sync(0xffffffffu, par[0] == node && tok[0] == g);
-        const unsigned m1 = __ballot_sync(0xffffffffu, par[1] == node && tok[1] == g);
-        if (!m0 && !m1) break;
-        const int next = m0 ? __ffs(m0) - 1 : 32 + __ffs(m1) - 1;
-        if (lane == 0) {
-            out[depth] = g;
-            path[depth] = next;
-        }
-        ++depth;
-        node = next;
-    }
-    for (int i = lane; i < n; i += 32) {
-        if (i == depth) out[i] = g;
-        else if (i > depth) out[i] = -1;
-        if (i >= depth) path[i] = -1;
-    }
-    if (lane == 0) p.out_n[b] = depth;
-}
+#include "spec_accept_walk.cuh"
 
 // ------------------------------------------------------------------- host
-// Resident CTAs of `kern` on the current device (cached per device and slot).
-template <typename K>
-int resident_ctas(K kern, int slot, int threads, int smem) {
-    static int cache[64][8] = {};
-    int dev = 0;
-    cudaGetDevice(&dev);
-    int occ = (dev >= 0 && dev < 64) ? cache[dev][slot] : 0;
-    if (!occ) {
-        if (smem > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, threads, smem) != cudaSuccess || occ <= 0)
-            occ = 2;
-        cudaGetLastError();
-        if (dev >= 0 && dev < 64) cache[dev][slot] = occ;
-    }
-    return occ * current_sm_count();
-}
-
 int g_max_cluster[64] = {0};
 
 // The largest cluster (16, non-portable, or 8) the device schedules for the
-// draw kernel.
+// walk kernel.
 int max_cluster_size() {
     int dev = 0;
     cudaGetDevice(&dev);
     if (dev < 0 || dev >= 64) return 8;
     if (g_max_cluster[dev]) return g_max_cluster[dev];
     int best = 8;
-    void (*kerns[4])(const AcceptParams) = {accept_draw_kernel<__nv_bfloat16>, accept_draw_kernel<float>,
-                                            tree_draw_kernel<__nv_bfloat16>, tree_draw_kernel<float>};
+    const void* kerns[8] = {(const void*)accept_walk_kernel<__nv_bfloat16, false, false>,
+                            (const void*)accept_walk_kernel<float, false, false>,
+                            (const void*)accept_walk_kernel<__nv_bfloat16, true, false>,
+                            (const void*)accept_walk_kernel<float, true, false>,
+                            (const void*)accept_walk_kernel<__nv_bfloat16, false, true>,
+                            (const void*)accept_walk_kernel<float, false, true>,
+                            (const void*)accept_walk_kernel<__nv_bfloat16, true, true>,
+                            (const void*)accept_walk_kernel<float, true, true>};
     bool attrs_ok = true;
     for (auto k : kerns)
         attrs_ok = attrs_ok && cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
     if (attrs_ok) {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(kMaxCluster, 1, 1);
-        cfg.blockDim = dim3(kDrawThreads, 1, 1);
+        cfg.blockDim = dim3(kWalkMaxThreads, 1, 1);
         cudaLaunchAttribute attr;
         attr.id = cudaLaunchAttributeClusterDimension;
         attr.val.clusterDim.x = kMaxCluster;
@@ -1172,132 +817,239 @@ int max_cluster_size() {
     return best;
 }
 
+constexpr int kMaxPhases = 4;
+
 struct AcceptPlan {
-    int R, I, W, J, grid1;
-    long long N;
-    int cluster, slice;
-    size_t off_cnt, bytes;
+    int I;                                     // items of a row
+    int phases, start[kMaxPhases + 1];         // nodes [start[i], start[i+1]) are read in phase i (0: the walk streams)
+    int units, U;                              // units of a row, items of a unit
+    int cluster, threads, blocks, per, look;   // the walk
+    size_t off_mass, off_stat, off_a, off_ticket, bytes;
 };
 
-template <typename T, bool G>
-int stats_resident() {
-    const int slot = (G ? 1 : 0) + (sizeof(T) == 4 ? 2 : 0);
-    return resident_ctas(accept_stats_kernel<T, G>, slot, kThreads, 0);
-}
-
-// n_t target rows and d_rows draft rows per request (chain: k+1 and k;
-// tree: the node count twice).
-AcceptPlan plan_accept_rows(const cs_accept_dims& d, int n_t, int d_rows, bool greedy, bool with_cluster) {
+// n nodes per request (chain: k + 1; tree), on rows at 16-byte boundaries or not.
+AcceptPlan plan_accept(const cs_accept_dims& d, int n, bool tree, bool greedy, bool aligned) {
     const bool f32 = d.logit_dtype == CS_F32;
+    const int esz = f32 ? 4 : 2, item = kItemBytes / esz, sms = current_sm_count();
     AcceptPlan P{};
-    P.R = greedy ? n_t : n_t + d_rows;
-    const int item = kItemBytes / (f32 ? 4 : 2);
-    P.I = (d.vocab + item - 1) / item;
-    P.N = (long long)d.batch * P.R * P.I;
-    const int resident = f32 ? (greedy ? stats_resident<float, true>() : stats_resident<float, false>())
-                             : (greedy ? stats_resident<__nv_bfloat16, true>()
-                                       : stats_resident<__nv_bfloat16, false>());
-    long long g = (P.N + kWarps - 1) / kWarps;
-    if (g > resident) g = resident;
-    P.grid1 = (int)(g > 0 ? g : 1);
-    // every busy warp owns at least one item, so a row's segments come from
-    // consecutive warps
-    const long long warps = (long long)P.grid1 * kWarps;
-    P.W = (int)(warps < P.N ? warps : (P.N > 0 ? P.N : 1));
-    // a row meets at most (I-1)/q + 2 ranges of q >= 1 items, and at most I
-    const long long q = P.N / P.W > 0 ? P.N / P.W : 1;
-    const long long J = (P.I - 1) / q + 2;
-    P.J = (int)(J < P.I ? J : P.I);
-    const size_t rows = (size_t)d.batch * P.R;
-    P.off_cnt = (rows * P.J * sizeof(float2) + 255) / 256 * 256;
-    P.bytes = P.off_cnt + (rows * sizeof(int) + 255) / 256 * 256;
-    if (!greedy && with_cluster) {
-        // All clusters in one wave (two CTAs per SM), no CTA with an empty
-        // slice, at most kMaxPasses passes per CTA.
-        const int pass = kDrawThreads * kRunVecs * (f32 ? 4 : 8);
-        const int sms = current_sm_count();
-        int c = 2 * sms / (d.batch > 0 ? d.batch : 1);
-        const int by_vocab = (d.vocab + pass - 1) / pass;
-        if (c > by_vocab) c = by_vocab;
-        const int cmax = max_cluster_size();
-        if (c > cmax) c = cmax;
-        const int need = (int)(((long long)d.vocab + (long long)kMaxPasses * pass - 1) / ((long long)kMaxPasses * pass));
-        if (c < need) c = need;
-        if (c < 1) c = 1;
-        P.cluster = c;
-        const int per = (d.vocab + c - 1) / c;
-        P.slice = (per + 7) / 8 * 8;
+    P.I = (int)(((long long)d.vocab + (aligned ? 0 : 16 / esz - 1) + item - 1) / item);
+    // one position of every request, in us at the copy bandwidth
+    const double pos_us = (double)d.batch * d.vocab * esz * (greedy || n == 1 ? 1 : 2) / 6.5e6;
+    // A tree whose nodes' rows take longer than a few rounds of the walk is
+    // streamed by it: 34 nodes, V = 128256, bf16: 31 us (B = 8), against 50
+    // when every row is read first; 7 nodes in a chain: 35 against 17.
+    const bool stream = tree && n * pos_us >= 8.0;
+    if (!stream) {
+        // The first phase takes the positions of about 30 us, every later one
+        // twice as many as were read before it, and what is left over when it
+        // is less than 15 us joins the last.  A phase costs about 8 us (its
+        // test, two hand-offs, an uneven end), so a call under 45 us is read
+        // at once.  B = 256, k = 8, V = 128256, bf16: 140 us with 1.9 of 8
+        // drafts accepted and 198 with 7.5 (at once: 208 and 201); B = 64,
+        // k = 4, V = 151936 at once 46 us, in two phases 58.
+        constexpr double kPhaseUs = 30.0;
+        P.phases = 1;
+        long long g = (long long)(kPhaseUs / pos_us) + 1;
+        while (!tree && d.batch <= kMaxPhased && P.phases < kMaxPhases && g < n && (n - g) * pos_us >= kPhaseUs / 2) {
+            P.start[P.phases++] = (int)g;
+            g *= 2;
+        }
+        P.start[P.phases] = n;
+    }
+    // The cluster: the CTAs of all requests in one wave (two an SM), a power
+    // of two (they pack a GPC; nine CTAs a request took 40 us where eight took
+    // 35, B = 32); a streamed tree's at least four, for its rounds' latency.
+    // Decided requests, the sampler and greedy calls have no slices to share.
+    int c = 1;
+    while (2 * c <= max_cluster_size() && 2 * c * d.batch <= 2 * sms) c *= 2;
+    P.threads = kWalkMaxThreads;
+    if (stream) {
+        if (c < 4) c = 4;
+    } else if (P.phases > 1 || greedy || n == 1) {
+        c = 1;
+        if (n > 1) P.threads = 64;
+    }
+    P.look = 1;
+    const int block = 32 * kWalkVecs * 16 / esz, most = kWalkSegs * kRunVecs / kWalkVecs;
+    P.blocks = (int)(((long long)d.vocab + (aligned ? 0 : 16 / esz - 1) + block - 1) / block);
+    const int need = (P.blocks + most - 1) / most;
+    if (c < need) c = need;
+    if (c > P.blocks) c = P.blocks;
+    P.cluster = c;
+    P.per = (P.blocks + c - 1) / c;
+    if (!stream && !greedy)
+        while (P.threads > 64 && P.threads / 64 >= P.per && (long long)d.batch * c > sms) P.threads /= 2;   // tiny rows
+    P.bytes = 256;
+    if (P.phases > 0) {
+        int g = 0;
+        for (int i = 0; i < P.phases; ++i)
+            if (P.start[i + 1] - P.start[i] > g) g = P.start[i + 1] - P.start[i];
+        const size_t rows = (size_t)d.batch * (greedy ? g : 2 * g);
+        P.U = (long long)rows * P.I <= 2ll * kWarps * sms ? 1 : P.I <= 64 ? 2 : P.I <= 256 ? 4 : 8;
+        P.units = (P.I + P.U - 1) / P.U;
+        auto up = [](size_t x) { return (x + 255) / 256 * 256; };
+        P.off_mass = up(rows * P.units * sizeof(float2));
+        P.off_stat = P.off_mass + (P.phases > 1 && !greedy ? up((size_t)d.batch * P.units * sizeof(float)) : 0);
+        P.off_a = P.off_stat + up(d.batch * sizeof(float4));
+        P.off_ticket = P.off_a + up(d.batch * sizeof(int));
+        P.bytes = P.off_ticket + 256;
     }
     return P;
 }
 
-AcceptPlan plan_accept(const cs_accept_dims& d, int n_draft, bool greedy, bool with_cluster) {
-    return plan_accept_rows(d, n_draft + 1, n_draft, greedy, with_cluster);
+// The scratch of a call, wherever its rows lie.
+size_t workspace_bytes(const cs_accept_dims& d, int n, bool tree, bool greedy) {
+    const size_t a = plan_accept(d, n, tree, greedy, true).bytes, b = plan_accept(d, n, tree, greedy, false).bytes;
+    return a > b ? a : b;
 }
 
-template <typename T, bool G>
-cs_status launch_typed(AcceptParams p, const AcceptPlan& P, bool tree, cudaStream_t stream) {
-    // both kernels are programmatic dependents of the kernel before them:
-    // each may start early and waits (griddepcontrol.wait) before it reads
-    // what that kernel wrote
+// Every kernel of a call is a programmatic dependent of the kernel before it:
+// it may start early and waits (griddepcontrol.wait) before it reads what
+// that kernel wrote.
+template <typename Kern, typename Params>
+cudaError_t launch_after(Kern kern, unsigned gx, unsigned gy, int threads, int cluster, cudaStream_t stream,
+                         const Params& p) {
     cudaLaunchAttribute attrs[2];
     attrs[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attrs[0].val.programmaticStreamSerializationAllowed = 1;
-    cudaError_t e;
-    {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)P.grid1, 1, 1);
-        cfg.blockDim = dim3(kThreads, 1, 1);
-        cfg.stream = stream;
-        cfg.attrs = attrs;
-        cfg.numAttrs = 1;
-        e = cudaLaunchKernelEx(&cfg, accept_stats_kernel<T, G>, p);
-        if (e != cudaSuccess) return cuda_fail(e, "accept_stats_kernel launch");
-    }
-    if (G) {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((p.B + kWarps - 1) / kWarps, 1, 1);
-        cfg.blockDim = dim3(kThreads, 1, 1);
-        cfg.stream = stream;
-        cfg.attrs = attrs;
-        cfg.numAttrs = 1;
-        e = cudaLaunchKernelEx(&cfg, tree ? tree_greedy_kernel<T> : accept_greedy_kernel<T>, p);
-        if (e != cudaSuccess) return cuda_fail(e, "greedy acceptance kernel launch");
-        return CS_OK;
-    }
-    auto kern = tree ? tree_draw_kernel<T> : accept_draw_kernel<T>;
-    if (P.cluster > 8) {
-        e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-        if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(non-portable cluster)");
-    }
     attrs[1].id = cudaLaunchAttributeClusterDimension;
-    attrs[1].val.clusterDim.x = P.cluster;
+    attrs[1].val.clusterDim.x = cluster;
     attrs[1].val.clusterDim.y = 1;
     attrs[1].val.clusterDim.z = 1;
-    for (int b0 = 0; b0 < p.B; b0 += 65535) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(gx, gy, 1);
+    cfg.blockDim = dim3(threads, 1, 1);
+    cfg.stream = stream;
+    cfg.attrs = attrs;
+    cfg.numAttrs = cluster > 1 ? 2 : 1;
+    return cudaLaunchKernelEx(&cfg, kern, p);
+}
+
+template <typename T, bool G>
+cs_status launch_typed(StatsParams sp, TestParams tp, WalkParams p, const AcceptPlan& P, bool tree, void* workspace,
+                       cudaStream_t stream) {
+    uint8_t* ws = static_cast<uint8_t*>(workspace);
+    const Decided dec{reinterpret_cast<int*>(ws + P.off_a), reinterpret_cast<float4*>(ws + P.off_stat)};
+    Phase ph{};
+    ph.units = P.units;
+    ph.U = P.U;
+    ph.part = reinterpret_cast<float2*>(ws);
+    ph.ticket = reinterpret_cast<unsigned*>(ws + P.off_ticket);
+    sp.by_units.set(P.units);
+    sp.stat = dec.stat;
+    sp.mass = reinterpret_cast<float*>(ws + P.off_mass);
+    const int fill = 2 * current_sm_count();   // two CTAs an SM (the kernel's launch bounds)
+    for (int i = 0; i < P.phases; ++i) {
+        const int g = P.start[i + 1] - P.start[i];
+        const bool last = i + 1 == P.phases;
+        ph.p0 = P.start[i];
+        ph.t_rows = g;
+        ph.R = G ? g : tree ? 2 * g : last ? 2 * g - 1 : 2 * g;
+        ph.undecided = i ? dec.a : nullptr;
+        sp.ph = ph;
+        sp.mass_lo = i ? P.start[i - 1] : 0;
+        sp.mass_hi = ph.p0;
+        sp.by_R.set(ph.R);
+        const long long ctas = ((long long)sp.B * ph.R * ph.units + kWarps - 1) / kWarps;
+        const unsigned grid = (unsigned)(ctas < fill ? ctas : fill);
+        cudaError_t e = launch_after(i ? accept_stats_kernel<T, G, true> : accept_stats_kernel<T, G, false>, grid, 1,
+                                     kThreads, 1, stream, sp);
+        if (e != cudaSuccess) return cuda_fail(e, "accept_stats_kernel launch");
+        if (P.phases == 1) break;
+        tp.ph = ph;
+        tp.dec = dec;
+        e = launch_after(accept_test_kernel<T, G>, (unsigned)(sp.B + kWarps - 1) / kWarps, 1, kThreads, 1, stream, tp);
+        if (e != cudaSuccess) return cuda_fail(e, "accept_test_kernel launch");
+        if (last && !G) {   // the masses of the pairs that the last phase decided
+            sp.ph.p0 = sp.n;
+            sp.ph.t_rows = sp.ph.R = 0;
+            sp.ph.undecided = dec.a;
+            sp.mass_lo = ph.p0;
+            sp.mass_hi = sp.n - 1;
+            sp.by_R.set(0);
+            e = launch_after(accept_stats_kernel<T, G, true>, grid, 1, kThreads, 1, stream, sp);
+            if (e != cudaSuccess) return cuda_fail(e, "accept_stats_kernel launch");
+        }
+    }
+    if (P.phases > 1) ph.undecided = dec.a;
+    p.mass = sp.mass;
+    p.reverse = true;
+    p.ph = ph;
+    p.dec = dec;
+    for (int b0 = 0; b0 < sp.B; b0 += 65535) {
         p.b_base = b0;
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(P.cluster, p.B - b0 < 65535 ? p.B - b0 : 65535, 1);
-        cfg.blockDim = dim3(kDrawThreads, 1, 1);
-        cfg.stream = stream;
-        cfg.attrs = attrs;
-        cfg.numAttrs = 2;
-        e = cudaLaunchKernelEx(&cfg, kern, p);
-        if (e != cudaSuccess) return cuda_fail(e, "acceptance draw kernel launch");
+        const cudaError_t e = launch_after(P.phases ? accept_walk_kernel<T, G, false> : accept_walk_kernel<T, G, true>, P.cluster, sp.B - b0 < 65535 ? sp.B - b0 : 65535,
+                                           P.threads, P.cluster, stream, p);
+        if (e != cudaSuccess) return cuda_fail(e, "accept_walk_kernel launch");
     }
     return CS_OK;
+}
+
+cs_status launch_accept(const cs_accept_dims& d, const void* target, const void* draft, const int32_t* parents,
+                        const int32_t* tokens, const float* uniforms, int n, float temperature, int32_t* out_tokens,
+                        int32_t* out_path, int32_t* out_n, void* workspace, cudaStream_t stream) {
+    const bool greedy = temperature == 0.f, tree = parents != nullptr;
+    const size_t esz = d.logit_dtype == CS_F32 ? 4 : 2;
+    const bool aligned = (size_t)d.vocab * esz % 16 == 0 &&
+                         ((reinterpret_cast<uintptr_t>(target) | reinterpret_cast<uintptr_t>(draft)) & 15) == 0;
+    const AcceptPlan P = plan_accept(d, n, tree, greedy, aligned);
+    const double c = temperature > 0.f ? 1.4426950408889634 / (double)temperature : 0.0;
+    StatsParams sp{};
+    sp.target = target;
+    sp.draft = draft;
+    sp.parents = parents;
+    sp.B = d.batch;
+    sp.V = d.vocab;
+    sp.n = n;
+    sp.d_rows = tree ? n : n - 1;
+    sp.I = P.I;
+    sp.c_hi = (float)c;
+    sp.c_lo = (float)(c - (double)sp.c_hi);
+    TestParams tp{};
+    tp.target = target;
+    tp.draft = draft;
+    tp.tokens = tokens;
+    tp.uniforms = uniforms;
+    tp.B = d.batch;
+    tp.V = d.vocab;
+    tp.n = n;
+    tp.c_hi = sp.c_hi;
+    tp.c_lo = sp.c_lo;
+    WalkParams p{};
+    p.target = target;
+    p.draft = draft;
+    p.tokens = tokens;
+    p.uniforms = uniforms;
+    p.parents = parents;
+    p.out_tokens = out_tokens;
+    p.out_n = out_n;
+    p.out_path = out_path;
+    p.B = d.batch;
+    p.V = d.vocab;
+    p.n = n;
+    p.d_rows = sp.d_rows;
+    p.I = P.I;
+    p.blocks = P.blocks;
+    p.per = P.per;
+    p.look = P.look;
+    p.c_hi = sp.c_hi;
+    p.c_lo = sp.c_lo;
+    if (d.logit_dtype == CS_F32)
+        return greedy ? launch_typed<float, true>(sp, tp, p, P, tree, workspace, stream)
+                      : launch_typed<float, false>(sp, tp, p, P, tree, workspace, stream);
+    return greedy ? launch_typed<__nv_bfloat16, true>(sp, tp, p, P, tree, workspace, stream)
+                  : launch_typed<__nv_bfloat16, false>(sp, tp, p, P, tree, workspace, stream);
 }
 
 }  // namespace
 
 size_t accept_workspace_bytes(const cs_accept_dims& d, int n_draft, float temperature) {
-    if (temperature == 0.f) return plan_accept(d, n_draft, true, false).bytes;
-    return plan_accept(d, n_draft, false, false).bytes;
+    return workspace_bytes(d, n_draft + 1, false, temperature == 0.f);
 }
 
 size_t accept_workspace_bytes_any(const cs_accept_dims& d, int n_draft) {
-    const size_t a = plan_accept(d, n_draft, true, false).bytes;
-    const size_t b = plan_accept(d, n_draft, false, false).bytes;
+    const size_t a = workspace_bytes(d, n_draft + 1, false, true);
+    const size_t b = workspace_bytes(d, n_draft + 1, false, false);
     return a > b ? a : b;
 }
 
@@ -1305,40 +1057,13 @@ cs_status launch_spec_accept(const cs_accept_dims& d, const void* target, const 
                              const int32_t* tokens, const float* uniforms, int n_draft,
                              float temperature, int32_t* out_tokens, int32_t* out_n,
                              void* workspace, cudaStream_t stream) {
-    const bool greedy = temperature == 0.f;
-    const AcceptPlan P = plan_accept(d, n_draft, greedy, true);
-    AcceptParams p{};
-    p.target = target;
-    p.draft = draft;
-    p.tokens = tokens;
-    p.uniforms = uniforms;
-    p.out_tokens = out_tokens;
-    p.out_n = out_n;
-    p.B = d.batch;
-    p.V = d.vocab;
-    p.k = n_draft;
-    p.n_t = n_draft + 1;
-    p.d_rows = n_draft;
-    p.R = P.R;
-    p.I = P.I;
-    p.N = P.N;
-    p.W = P.W;
-    p.J = P.J;
-    p.slice = P.slice;
-    const double c = temperature > 0.f ? 1.4426950408889634 / (double)temperature : 0.0;
-    p.c_hi = (float)c;
-    p.c_lo = (float)(c - (double)p.c_hi);
-    p.part = static_cast<float2*>(workspace);
-    p.cnt = reinterpret_cast<int*>(static_cast<uint8_t*>(workspace) + P.off_cnt);
-    if (d.logit_dtype == CS_F32)
-        return greedy ? launch_typed<float, true>(p, P, false, stream) : launch_typed<float, false>(p, P, false, stream);
-    return greedy ? launch_typed<__nv_bfloat16, true>(p, P, false, stream)
-                  : launch_typed<__nv_bfloat16, false>(p, P, false, stream);
+    return launch_accept(d, target, draft, nullptr, tokens, uniforms, n_draft + 1, temperature, out_tokens, nullptr,
+                         out_n, workspace, stream);
 }
 
 size_t tree_accept_workspace_bytes(const cs_accept_dims& d, int n_nodes) {
-    const size_t a = plan_accept_rows(d, n_nodes, n_nodes, true, false).bytes;
-    const size_t b = plan_accept_rows(d, n_nodes, n_nodes, false, false).bytes;
+    const size_t a = workspace_bytes(d, n_nodes, true, true);
+    const size_t b = workspace_bytes(d, n_nodes, true, false);
     return a > b ? a : b;
 }
 
@@ -1346,37 +1071,8 @@ cs_status launch_tree_accept(const cs_accept_dims& d, const void* target, const 
                              const int32_t* parents, const int32_t* tokens, const float* uniforms, int n_nodes,
                              float temperature, int32_t* out_tokens, int32_t* out_path, int32_t* out_n,
                              void* workspace, cudaStream_t stream) {
-    const bool greedy = temperature == 0.f;
-    const AcceptPlan P = plan_accept_rows(d, n_nodes, n_nodes, greedy, true);
-    AcceptParams p{};
-    p.target = target;
-    p.draft = draft;
-    p.tokens = tokens;
-    p.uniforms = uniforms;
-    p.out_tokens = out_tokens;
-    p.out_n = out_n;
-    p.parents = parents;
-    p.out_path = out_path;
-    p.B = d.batch;
-    p.V = d.vocab;
-    p.k = n_nodes - 1;
-    p.n_t = n_nodes;
-    p.d_rows = n_nodes;
-    p.R = P.R;
-    p.I = P.I;
-    p.N = P.N;
-    p.W = P.W;
-    p.J = P.J;
-    p.slice = P.slice;
-    const double c = temperature > 0.f ? 1.4426950408889634 / (double)temperature : 0.0;
-    p.c_hi = (float)c;
-    p.c_lo = (float)(c - (double)p.c_hi);
-    p.part = static_cast<float2*>(workspace);
-    p.cnt = reinterpret_cast<int*>(static_cast<uint8_t*>(workspace) + P.off_cnt);
-    if (d.logit_dtype == CS_F32)
-        return greedy ? launch_typed<float, true>(p, P, true, stream) : launch_typed<float, false>(p, P, true, stream);
-    return greedy ? launch_typed<__nv_bfloat16, true>(p, P, true, stream)
-                  : launch_typed<__nv_bfloat16, false>(p, P, true, stream);
+    return launch_accept(d, target, draft, parents, tokens, uniforms, n_nodes, temperature, out_tokens, out_path,
+                         out_n, workspace, stream);
 }
 
 }  // namespace cs
