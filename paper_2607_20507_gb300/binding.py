@@ -4,11 +4,15 @@ Every step of the draft-and-verify path runs in the library's CUDA kernels;
 this module checks tensor dtypes, shapes and devices, passes raw device
 pointers and the current CUDA stream through ctypes, and turns a non-OK
 status into an exception.  It never computes any part of the method and has
-no CPU fallback: if the library is missing, every call raises.
+no CPU fallback: if the library is missing, every call raises.  The calls
+of a step go through the compiled module ``_marshal``, which does the same
+checks and passes on what it does not take to the code here.
 """
 from __future__ import annotations
 
 import ctypes
+import importlib.machinery
+import importlib.util
 import os
 import threading
 
@@ -64,6 +68,8 @@ def library_path() -> str:
 def load_library(path: str | None = None):
     """Load libcachespec.so (built in-tree by ``__graft_entry__.build()``).  Raises if absent."""
     global _lib
+    if _lib is not None and path is None:
+        return _lib
     with _lock:
         if _lib is not None and path is None:
             return _lib
@@ -125,6 +131,35 @@ def load_library(path: str | None = None):
         return lib
 
 
+_fast = None
+
+
+def _load_fast():
+    """The compiled marshalling module, beside the library.  Raises if absent."""
+    global _fast
+    load_library()
+    with _lock:
+        if _fast is None:
+            if not os.path.exists(_build.MARSHAL):
+                raise RuntimeError(f"{os.path.basename(_build.MARSHAL)} not found at {_build.MARSHAL}; build it with "
+                                   "`python -c 'import __graft_entry__ as g; g.build()'`")
+            name = __package__ + "._marshal"
+            loader = importlib.machinery.ExtensionFileLoader(name, _build.MARSHAL)
+            mod = importlib.util.module_from_spec(importlib.util.spec_from_file_location(name, _build.MARSHAL,
+                                                                                         loader=loader))
+            loader.exec_module(mod)
+            mod.use_workspaces(lambda kind, index, n: _cached_workspace(kind, torch.device("cuda", index), n))
+            _fast = mod
+    return _fast
+
+
+def _done(r):
+    """A result of the marshalling module; a status (an int) raises."""
+    if type(r) is int:
+        _check(load_library(), r)
+    return r
+
+
 def _check(lib, status: int) -> None:
     if status != CS_OK:
         raise CacheSpecError(status, lib.cs_last_error().decode(errors="replace"))
@@ -134,11 +169,21 @@ def _ptr(t: torch.Tensor | None) -> int | None:
     return None if t is None else t.data_ptr()
 
 
+# The current stream's handle without a torch.cuda.Stream object around it
+# (2 us a call less on the host).
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream(device: torch.device) -> int:
+    if _raw_stream is not None and device.index is not None:
+        return _raw_stream(device.index)
     return torch.cuda.current_stream(device).cuda_stream
 
 
 def _need(t: torch.Tensor, name: str, dtype: torch.dtype, ndim: int, device) -> None:
+    if (isinstance(t, torch.Tensor) and t.dtype is dtype and t.dim() == ndim and t.is_cuda and t.is_contiguous()
+            and (device is None or t.device == device)):
+        return
     if not isinstance(t, torch.Tensor):
         raise TypeError(f"{name} must be a torch.Tensor")
     if t.dtype != dtype:
@@ -158,21 +203,24 @@ def attn_dims(q: torch.Tensor, k_pages: torch.Tensor, page_table: torch.Tensor,
     return AttnDims(B, Hq, Hkv, D, ps, page_table.shape[1], P, float(sm_scale))
 
 
-# Workspaces handed out by this module, one per (device, size).  The kernels
+# Workspaces handed out by this module, one per (kind, device, size).  The kernels
 # leave a workspace ready for the next call, so calls ordered on one stream
 # may share it.
 _workspaces: dict = {}
 
 
-def verify_attention_workspace(dims: AttnDims, n_draft: int, device) -> torch.Tensor:
-    lib = load_library()
-    n = lib.cs_verify_attention_workspace_bytes(ctypes.byref(dims), int(n_draft))
-    key = (str(device), n)
+def _cached_workspace(kind: str, device, n: int) -> torch.Tensor:
+    key = (kind, device, n)
     ws = _workspaces.get(key)
     if ws is None:
         ws = torch.zeros(max(n, 256), dtype=torch.uint8, device=device)
         _workspaces[key] = ws
     return ws
+
+
+def verify_attention_workspace(dims: AttnDims, n_draft: int, device) -> torch.Tensor:
+    n = load_library().cs_verify_attention_workspace_bytes(ctypes.byref(dims), int(n_draft))
+    return _cached_workspace("attn", device, n)
 
 
 def cs_verify_attention_workspace_bytes(q, k_pages, page_table, n_draft, sm_scale=0.0) -> int:
@@ -184,6 +232,10 @@ def cs_verify_attention_workspace_bytes(q, k_pages, page_table, n_draft, sm_scal
 def cs_verify_attention(q, k_pages, v_pages, page_table, ctx_lens, n_draft, out=None,
                         workspace=None, sm_scale: float = 0.0, stream: int | None = None):
     """Verify attention; returns ``out`` (bf16 [B, k+1, Hq, D]).  See include/cachespec.h."""
+    r = (_fast or _load_fast()).verify_attention(q, k_pages, v_pages, page_table, ctx_lens, n_draft, out, workspace,
+                                                 sm_scale, stream)
+    if r is not None:
+        return _done(r)
     lib = load_library()
     dev = q.device
     _need(q, "q", torch.bfloat16, 4, dev)
@@ -202,29 +254,28 @@ def cs_verify_attention(q, k_pages, v_pages, page_table, ctx_lens, n_draft, out=
         _need(out, "out", torch.bfloat16, 4, dev)
     if workspace is None:
         workspace = verify_attention_workspace(d, n_draft, dev)
-    st = lib.cs_verify_attention(ctypes.byref(d), _ptr(q), _ptr(k_pages), _ptr(v_pages),
-                                 _ptr(page_table), _ptr(ctx_lens), int(n_draft), _ptr(out),
-                                 _ptr(workspace), workspace.numel() * workspace.element_size(),
+    st = lib.cs_verify_attention(ctypes.byref(d), q.data_ptr(), k_pages.data_ptr(), v_pages.data_ptr(),
+                                 page_table.data_ptr(), ctx_lens.data_ptr(), int(n_draft), out.data_ptr(),
+                                 workspace.data_ptr(), workspace.nbytes,
                                  _stream(dev) if stream is None else stream)
-    _check(lib, st)
+    if st:
+        _check(lib, st)
     return out
 
 
 def spec_accept_workspace(dims: AcceptDims, n_draft: int, device) -> torch.Tensor:
-    lib = load_library()
-    n = lib.cs_spec_accept_workspace_bytes(ctypes.byref(dims), int(n_draft))
-    key = ("accept", str(device), n)
-    ws = _workspaces.get(key)
-    if ws is None:
-        ws = torch.zeros(max(n, 256), dtype=torch.uint8, device=device)
-        _workspaces[key] = ws
-    return ws
+    n = load_library().cs_spec_accept_workspace_bytes(ctypes.byref(dims), int(n_draft))
+    return _cached_workspace("accept", device, n)
 
 
 def cs_spec_accept(target_logits, draft_logits, draft_tokens, uniforms, temperature,
                    out_tokens=None, out_n_accepted=None, workspace=None,
                    stream: int | None = None):
     """Speculative acceptance; returns (out_tokens [B, k+1], n_accepted [B]).  See include/cachespec.h."""
+    r = (_fast or _load_fast()).spec_accept(target_logits, draft_logits, draft_tokens, uniforms, temperature, out_tokens,
+                                            out_n_accepted, workspace, stream)
+    if r is not None:
+        return _done(r)
     lib = load_library()
     dev = target_logits.device
     if target_logits.dtype not in (torch.float32, torch.bfloat16):
@@ -240,26 +291,32 @@ def cs_spec_accept(target_logits, draft_logits, draft_tokens, uniforms, temperat
     _need(draft_tokens, "draft_tokens", torch.int32, 2, dev)
     _need(uniforms, "uniforms", torch.float32, 2, dev)
     if out_tokens is None:
-        out_tokens = torch.empty((B, k + 1), dtype=torch.int32, device=dev)
+        out_tokens = draft_tokens.new_empty((B, k + 1))
+    else:
+        _need(out_tokens, "out_tokens", torch.int32, 2, dev)
     if out_n_accepted is None:
-        out_n_accepted = torch.empty((B,), dtype=torch.int32, device=dev)
-    _need(out_tokens, "out_tokens", torch.int32, 2, dev)
-    _need(out_n_accepted, "out_n_accepted", torch.int32, 1, dev)
+        out_n_accepted = draft_tokens.new_empty((B,))
+    else:
+        _need(out_n_accepted, "out_n_accepted", torch.int32, 1, dev)
     d = AcceptDims(B, V, CS_F32 if dtype == torch.float32 else CS_BF16)
     if workspace is None:
         workspace = spec_accept_workspace(d, k, dev)
-    st = lib.cs_spec_accept(ctypes.byref(d), _ptr(target_logits), _ptr(draft_logits),
-                            _ptr(draft_tokens), _ptr(uniforms), int(k), float(temperature),
-                            _ptr(out_tokens), _ptr(out_n_accepted), _ptr(workspace),
-                            workspace.numel() * workspace.element_size(),
-                            _stream(dev) if stream is None else stream)
-    _check(lib, st)
+    st = lib.cs_spec_accept(ctypes.byref(d), target_logits.data_ptr(), _ptr(draft_logits),
+                            draft_tokens.data_ptr(), uniforms.data_ptr(), int(k), float(temperature),
+                            out_tokens.data_ptr(), out_n_accepted.data_ptr(), workspace.data_ptr(),
+                            workspace.nbytes, _stream(dev) if stream is None else stream)
+    if st:
+        _check(lib, st)
     return out_tokens, out_n_accepted
 
 
 def cs_kv_append(new_k, new_v, k_pages, v_pages, page_table, ctx_lens, stream: int | None = None):
     """Append the K/V rows of the newest positions into the page pools (in place).
     new_k / new_v bf16 [B, n_new, Hkv, D]; pools [P, Hkv, ps, D].  See include/cachespec.h."""
+    r = (_fast or _load_fast()).kv_append(new_k, new_v, k_pages, v_pages, page_table, ctx_lens, stream)
+    if r is not None:
+        _done(r)
+        return
     lib = load_library()
     dev = k_pages.device
     _need(new_k, "new_k", torch.bfloat16, 4, dev)
@@ -273,20 +330,27 @@ def cs_kv_append(new_k, new_v, k_pages, v_pages, page_table, ctx_lens, stream: i
     if tuple(new_v.shape) != tuple(new_k.shape) or Hkv2 != Hkv or D2 != D or k_pages.shape != v_pages.shape:
         raise ValueError("new rows and pools do not match")
     d = AttnDims(B, Hkv, Hkv, D, ps, page_table.shape[1], P, 0.0)
-    st = lib.cs_kv_append(ctypes.byref(d), _ptr(new_k), _ptr(new_v), _ptr(k_pages), _ptr(v_pages),
-                          _ptr(page_table), _ptr(ctx_lens), int(n_new), _stream(dev) if stream is None else stream)
-    _check(lib, st)
+    st = lib.cs_kv_append(ctypes.byref(d), new_k.data_ptr(), new_v.data_ptr(), k_pages.data_ptr(), v_pages.data_ptr(),
+                          page_table.data_ptr(), ctx_lens.data_ptr(), int(n_new),
+                          _stream(dev) if stream is None else stream)
+    if st:
+        _check(lib, st)
 
 
 def cs_kv_commit(ctx_lens, n_accepted, n_draft: int, stream: int | None = None):
     """Keep the accepted prefix: ctx_lens <- max(0, ctx_lens - k + n_accepted), in place."""
+    r = (_fast or _load_fast()).kv_commit(ctx_lens, n_accepted, n_draft, stream)
+    if r is not None:
+        _done(r)
+        return
     lib = load_library()
     dev = ctx_lens.device
     _need(ctx_lens, "ctx_lens", torch.int32, 1, dev)
     _need(n_accepted, "n_accepted", torch.int32, 1, dev)
-    st = lib.cs_kv_commit(int(ctx_lens.shape[0]), _ptr(ctx_lens), _ptr(n_accepted), int(n_draft),
+    st = lib.cs_kv_commit(int(ctx_lens.shape[0]), ctx_lens.data_ptr(), n_accepted.data_ptr(), int(n_draft),
                           _stream(dev) if stream is None else stream)
-    _check(lib, st)
+    if st:
+        _check(lib, st)
 
 
 def cs_route_norms(centroids, inv_norms=None, stream: int | None = None):
@@ -298,15 +362,20 @@ def cs_route_norms(centroids, inv_norms=None, stream: int | None = None):
     if inv_norms is None:
         inv_norms = torch.empty((N,), dtype=torch.float32, device=dev)
     _need(inv_norms, "inv_norms", torch.float32, 1, dev)
-    st = lib.cs_route_norms(int(N), int(d), _ptr(centroids) if N else None, _ptr(inv_norms) if N else None,
+    st = lib.cs_route_norms(int(N), int(d), centroids.data_ptr() if N else None, inv_norms.data_ptr() if N else None,
                             _stream(dev) if stream is None else stream)
-    _check(lib, st)
+    if st:
+        _check(lib, st)
     return inv_norms
 
 
 def cs_route(emb, centroids, inv_norms, tau, out_group=None, out_best=None, out_score=None, workspace=None,
              stream: int | None = None):
     """Batched semantic routing; returns (group [B], best [B], score [B]).  See include/cachespec.h."""
+    if out_group is None and out_best is None and out_score is None:
+        r = (_fast or _load_fast()).route(emb, centroids, inv_norms, tau, workspace, stream)
+        if r is not None:
+            return _done(r)
     lib = load_library()
     dev = emb.device
     _need(emb, "emb", torch.bfloat16, 2, dev)
@@ -316,21 +385,18 @@ def cs_route(emb, centroids, inv_norms, tau, out_group=None, out_best=None, out_
     N = centroids.shape[0]
     if N and centroids.shape[1] != d:
         raise ValueError("emb and centroids differ in width")
-    out_group = torch.empty((B,), dtype=torch.int32, device=dev) if out_group is None else out_group
-    out_best = torch.empty((B,), dtype=torch.int32, device=dev) if out_best is None else out_best
-    out_score = torch.empty((B,), dtype=torch.float32, device=dev) if out_score is None else out_score
+    out_group = inv_norms.new_empty((B,), dtype=torch.int32) if out_group is None else out_group
+    out_best = inv_norms.new_empty((B,), dtype=torch.int32) if out_best is None else out_best
+    out_score = inv_norms.new_empty((B,)) if out_score is None else out_score
     dims = RouteDims(B, N, d)
     if workspace is None:
-        n = lib.cs_route_workspace_bytes(ctypes.byref(dims))
-        key = ("route", str(dev), n)
-        workspace = _workspaces.get(key)
-        if workspace is None:
-            workspace = torch.zeros(max(n, 256), dtype=torch.uint8, device=dev)
-            _workspaces[key] = workspace
-    st = lib.cs_route(ctypes.byref(dims), _ptr(emb), _ptr(centroids) if N else None, _ptr(inv_norms) if N else None,
-                      float(tau), _ptr(out_group), _ptr(out_best), _ptr(out_score), _ptr(workspace),
-                      workspace.numel() * workspace.element_size(), _stream(dev) if stream is None else stream)
-    _check(lib, st)
+        workspace = _cached_workspace("route", dev, lib.cs_route_workspace_bytes(ctypes.byref(dims)))
+    st = lib.cs_route(ctypes.byref(dims), emb.data_ptr(), centroids.data_ptr() if N else None,
+                      inv_norms.data_ptr() if N else None,
+                      float(tau), out_group.data_ptr(), out_best.data_ptr(), out_score.data_ptr(), workspace.data_ptr(),
+                      workspace.nbytes, _stream(dev) if stream is None else stream)
+    if st:
+        _check(lib, st)
     return out_group, out_best, out_score
 
 
@@ -338,6 +404,9 @@ def cs_sample(logits, uniforms, temperature, out_tokens=None, workspace=None,
               stream: int | None = None):
     """Draft-side sampling, one token per row of ``logits`` [B, V]; returns out_tokens [B].
     See include/cachespec.h."""
+    r = (_fast or _load_fast()).sample(logits, uniforms, temperature, out_tokens, workspace, stream)
+    if r is not None:
+        return _done(r)
     lib = load_library()
     dev = logits.device
     if logits.dtype not in (torch.float32, torch.bfloat16):
@@ -346,36 +415,29 @@ def cs_sample(logits, uniforms, temperature, out_tokens=None, workspace=None,
     B, V = logits.shape
     _need(uniforms, "uniforms", torch.float32, 1, dev)
     if out_tokens is None:
-        out_tokens = torch.empty((B,), dtype=torch.int32, device=dev)
-    _need(out_tokens, "out_tokens", torch.int32, 1, dev)
+        out_tokens = uniforms.new_empty((B,), dtype=torch.int32)
+    else:
+        _need(out_tokens, "out_tokens", torch.int32, 1, dev)
     d = AcceptDims(B, V, CS_F32 if logits.dtype == torch.float32 else CS_BF16)
     if workspace is None:
-        n = lib.cs_sample_workspace_bytes(ctypes.byref(d))
-        key = ("sample", str(dev), n)
-        workspace = _workspaces.get(key)
-        if workspace is None:
-            workspace = torch.zeros(max(n, 256), dtype=torch.uint8, device=dev)
-            _workspaces[key] = workspace
-    st = lib.cs_sample(ctypes.byref(d), _ptr(logits), _ptr(uniforms), float(temperature), _ptr(out_tokens),
-                       _ptr(workspace), workspace.numel() * workspace.element_size(),
+        workspace = _cached_workspace("sample", dev, lib.cs_sample_workspace_bytes(ctypes.byref(d)))
+    st = lib.cs_sample(ctypes.byref(d), logits.data_ptr(), uniforms.data_ptr(), float(temperature),
+                       out_tokens.data_ptr(),
+                       workspace.data_ptr(), workspace.nbytes,
                        _stream(dev) if stream is None else stream)
-    _check(lib, st)
+    if st:
+        _check(lib, st)
     return out_tokens
-
-
-def _cached_workspace(kind: str, device, n: int) -> torch.Tensor:
-    key = (kind, str(device), n)
-    ws = _workspaces.get(key)
-    if ws is None:
-        ws = torch.zeros(max(n, 256), dtype=torch.uint8, device=device)
-        _workspaces[key] = ws
-    return ws
 
 
 def cs_tree_verify_attention(q, k_pages, v_pages, page_table, ctx_lens, parents, out=None, workspace=None,
                              sm_scale: float = 0.0, stream: int | None = None):
     """Token-tree verify attention; q / out bf16 [B, n, Hq, D], parents int32 [B, n].
     Returns ``out``.  See include/cachespec.h."""
+    r = (_fast or _load_fast()).tree_verify_attention(q, k_pages, v_pages, page_table, ctx_lens, parents, out, workspace,
+                                                      sm_scale, stream)
+    if r is not None:
+        return _done(r)
     lib = load_library()
     dev = q.device
     _need(q, "q", torch.bfloat16, 4, dev)
@@ -392,15 +454,17 @@ def cs_tree_verify_attention(q, k_pages, v_pages, page_table, ctx_lens, parents,
     d = attn_dims(q, k_pages, page_table, sm_scale)
     if out is None:
         out = torch.empty_like(q)
-    _need(out, "out", torch.bfloat16, 4, dev)
+    else:
+        _need(out, "out", torch.bfloat16, 4, dev)
     if workspace is None:
         workspace = _cached_workspace("tree_attn", dev,
                                       lib.cs_tree_verify_attention_workspace_bytes(ctypes.byref(d), int(n)))
-    st = lib.cs_tree_verify_attention(ctypes.byref(d), _ptr(q), _ptr(k_pages), _ptr(v_pages), _ptr(page_table),
-                                      _ptr(ctx_lens), _ptr(parents), int(n), _ptr(out), _ptr(workspace),
-                                      workspace.numel() * workspace.element_size(),
+    st = lib.cs_tree_verify_attention(ctypes.byref(d), q.data_ptr(), k_pages.data_ptr(), v_pages.data_ptr(),
+                                      page_table.data_ptr(), ctx_lens.data_ptr(), parents.data_ptr(), int(n),
+                                      out.data_ptr(), workspace.data_ptr(), workspace.nbytes,
                                       _stream(dev) if stream is None else stream)
-    _check(lib, st)
+    if st:
+        _check(lib, st)
     return out
 
 
@@ -408,6 +472,10 @@ def cs_tree_accept(target_logits, draft_logits, parents, node_tokens, uniforms, 
                    out_path=None, out_n_accepted=None, workspace=None, stream: int | None = None):
     """Token-tree acceptance walk; target / draft logits [B, n, V], parents / node_tokens int32 [B, n],
     uniforms fp32 [B, n].  Returns (tokens [B, n], path [B, n], n_accepted [B]).  See include/cachespec.h."""
+    r = (_fast or _load_fast()).tree_accept(target_logits, draft_logits, parents, node_tokens, uniforms, temperature,
+                                            out_tokens, out_path, out_n_accepted, workspace, stream)
+    if r is not None:
+        return _done(r)
     lib = load_library()
     dev = target_logits.device
     if target_logits.dtype not in (torch.float32, torch.bfloat16):
@@ -424,26 +492,38 @@ def cs_tree_accept(target_logits, draft_logits, parents, node_tokens, uniforms, 
         if tuple(t.shape) != (B, n):
             raise ValueError(f"{name} must be [{B}, {n}]")
     _need(uniforms, "uniforms", torch.float32, 2, dev)
-    out_tokens = torch.empty((B, n), dtype=torch.int32, device=dev) if out_tokens is None else out_tokens
-    out_path = torch.empty((B, n), dtype=torch.int32, device=dev) if out_path is None else out_path
-    out_n_accepted = torch.empty((B,), dtype=torch.int32, device=dev) if out_n_accepted is None else out_n_accepted
-    _need(out_tokens, "out_tokens", torch.int32, 2, dev)
-    _need(out_path, "out_path", torch.int32, 2, dev)
-    _need(out_n_accepted, "out_n_accepted", torch.int32, 1, dev)
+    if out_tokens is None:
+        out_tokens = parents.new_empty((B, n))
+    else:
+        _need(out_tokens, "out_tokens", torch.int32, 2, dev)
+    if out_path is None:
+        out_path = parents.new_empty((B, n))
+    else:
+        _need(out_path, "out_path", torch.int32, 2, dev)
+    if out_n_accepted is None:
+        out_n_accepted = parents.new_empty((B,))
+    else:
+        _need(out_n_accepted, "out_n_accepted", torch.int32, 1, dev)
     d = AcceptDims(B, V, CS_F32 if dtype == torch.float32 else CS_BF16)
     if workspace is None:
         workspace = _cached_workspace("tree_accept", dev, lib.cs_tree_accept_workspace_bytes(ctypes.byref(d), int(n)))
-    st = lib.cs_tree_accept(ctypes.byref(d), _ptr(target_logits), _ptr(draft_logits), _ptr(parents),
-                            _ptr(node_tokens), _ptr(uniforms), int(n), float(temperature), _ptr(out_tokens),
-                            _ptr(out_path), _ptr(out_n_accepted), _ptr(workspace),
-                            workspace.numel() * workspace.element_size(), _stream(dev) if stream is None else stream)
-    _check(lib, st)
+    st = lib.cs_tree_accept(ctypes.byref(d), target_logits.data_ptr(), _ptr(draft_logits), parents.data_ptr(),
+                            node_tokens.data_ptr(), uniforms.data_ptr(), int(n), float(temperature),
+                            out_tokens.data_ptr(),
+                            out_path.data_ptr(), out_n_accepted.data_ptr(), workspace.data_ptr(),
+                            workspace.nbytes, _stream(dev) if stream is None else stream)
+    if st:
+        _check(lib, st)
     return out_tokens, out_path, out_n_accepted
 
 
 def cs_kv_commit_tree(k_pages, v_pages, page_table, ctx_lens, path, n_accepted, stream: int | None = None):
     """Move the accepted tree path's K/V rows next to the root and shorten ctx_lens (in place);
     path int32 [B, n] and n_accepted [B] as returned by cs_tree_accept."""
+    r = (_fast or _load_fast()).kv_commit_tree(k_pages, v_pages, page_table, ctx_lens, path, n_accepted, stream)
+    if r is not None:
+        _done(r)
+        return
     lib = load_library()
     dev = k_pages.device
     _need(k_pages, "k_pages", torch.bfloat16, 4, dev)
@@ -457,9 +537,11 @@ def cs_kv_commit_tree(k_pages, v_pages, page_table, ctx_lens, path, n_accepted, 
     P, Hkv, ps, D = k_pages.shape
     B, n = path.shape
     d = AttnDims(B, Hkv, Hkv, D, ps, page_table.shape[1], P, 0.0)
-    st = lib.cs_kv_commit_tree(ctypes.byref(d), _ptr(k_pages), _ptr(v_pages), _ptr(page_table), _ptr(ctx_lens),
-                               _ptr(path), _ptr(n_accepted), int(n), _stream(dev) if stream is None else stream)
-    _check(lib, st)
+    st = lib.cs_kv_commit_tree(ctypes.byref(d), k_pages.data_ptr(), v_pages.data_ptr(), page_table.data_ptr(),
+                               ctx_lens.data_ptr(), path.data_ptr(), n_accepted.data_ptr(), int(n),
+                               _stream(dev) if stream is None else stream)
+    if st:
+        _check(lib, st)
 
 
 def cs_verify_attention_noalloc(q, k_pages, v_pages, page_table, ctx_lens, n_draft, out=None,
@@ -476,11 +558,13 @@ def cs_verify_attention_noalloc(q, k_pages, v_pages, page_table, ctx_lens, n_dra
     d = attn_dims(q, k_pages, page_table, sm_scale)
     if out is None:
         out = torch.empty_like(q)
-    _need(out, "out", torch.bfloat16, 4, dev)
-    st = lib.cs_verify_attention_noalloc(ctypes.byref(d), _ptr(q), _ptr(k_pages), _ptr(v_pages),
-                                         _ptr(page_table), _ptr(ctx_lens), int(n_draft), _ptr(out),
+    else:
+        _need(out, "out", torch.bfloat16, 4, dev)
+    st = lib.cs_verify_attention_noalloc(ctypes.byref(d), q.data_ptr(), k_pages.data_ptr(), v_pages.data_ptr(),
+                                         page_table.data_ptr(), ctx_lens.data_ptr(), int(n_draft), out.data_ptr(),
                                          _stream(dev) if stream is None else stream)
-    _check(lib, st)
+    if st:
+        _check(lib, st)
     return out
 
 

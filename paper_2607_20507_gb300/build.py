@@ -1,4 +1,5 @@
-"""Builds libcachespec.so in-tree for sm_103a (nvcc, one -gencode, parallel TUs).
+"""Builds libcachespec.so in-tree for sm_103a (nvcc, one -gencode, parallel TUs)
+and the binding's marshalling module beside it (g++, against the installed torch).
 
 ``python -m paper_2607_20507_gb300.build [--force] [--ptxas-v]``
 """
@@ -8,6 +9,7 @@ import concurrent.futures
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
@@ -15,6 +17,7 @@ CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 BUILD_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libcachespec.so")
+MARSHAL = os.path.join(HERE, "_marshal.so")
 SOURCES = ["capi.cu", "verify_attention.cu", "spec_accept.cu", "noalloc.cu", "kv_cache.cu", "route.cu", "selftest.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
@@ -32,10 +35,39 @@ def _inputs() -> list[str]:
 
 
 def is_stale() -> bool:
-    if not os.path.exists(LIB):
+    if not os.path.exists(LIB) or not os.path.exists(MARSHAL):
         return True
-    t = os.path.getmtime(LIB)
+    t = min(os.path.getmtime(LIB), os.path.getmtime(MARSHAL))
     return any(os.path.getmtime(f) > t for f in _inputs())
+
+
+def _run(cmd: list[str], what: str) -> str:
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode != 0:
+        raise RuntimeError(f"{what} failed:\n{r.stdout}\n{r.stderr}")
+    return r.stdout + r.stderr
+
+
+def _compile_marshal() -> str:
+    import torch
+    home = os.path.dirname(torch.__file__)
+    cuda = os.path.join(os.environ.get("CUDA_HOME", "/usr/local/cuda"), "include")
+    obj = os.path.join(BUILD_DIR, "marshal.o")
+    _run(["g++", "-O2", "-std=c++17", "-fPIC", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+          "-I", INCLUDE, "-I", os.path.join(home, "include"),
+          "-I", os.path.join(home, "include", "torch", "csrc", "api", "include"),
+          "-I", sysconfig.get_paths()["include"], "-I", cuda,
+          "-c", os.path.join(CSRC, "marshal.cpp"), "-o", obj], "g++ marshal.cpp")
+    return obj
+
+
+def _link_marshal(obj: str) -> None:
+    import torch
+    libs = os.path.join(os.path.dirname(torch.__file__), "lib")
+    tmp = MARSHAL + f".tmp{os.getpid()}"
+    _run(["g++", "-shared", "-o", tmp, obj, "-L", libs, "-L", HERE, "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10",
+          "-lc10_cuda", "-l:" + os.path.basename(LIB), "-Wl,-rpath,$ORIGIN", "-Wl,-rpath," + libs], "marshal link")
+    os.replace(tmp, MARSHAL)
 
 
 def build(force: bool = False, ptxas_verbose: bool = False, quiet: bool = True) -> str:
@@ -50,12 +82,10 @@ def build(force: bool = False, ptxas_verbose: bool = False, quiet: bool = True) 
     def compile_one(src: str) -> tuple[str, str]:
         obj = os.path.join(BUILD_DIR, src.replace(".cu", ".o"))
         cmd = [_nvcc(), *flags, "-c", os.path.join(CSRC, src), "-o", obj]
-        r = subprocess.run(cmd, capture_output=True, text=True)
-        if r.returncode != 0:
-            raise RuntimeError(f"nvcc failed for {src}:\n{r.stdout}\n{r.stderr}")
-        return obj, r.stdout + r.stderr
+        return obj, _run(cmd, f"nvcc {src}")
 
-    with concurrent.futures.ThreadPoolExecutor(max_workers=len(SOURCES)) as ex:
+    with concurrent.futures.ThreadPoolExecutor(max_workers=len(SOURCES) + 1) as ex:
+        marshal = ex.submit(_compile_marshal)
         results = list(ex.map(compile_one, SOURCES))
     if ptxas_verbose or not quiet:
         for _, log in results:
@@ -63,10 +93,9 @@ def build(force: bool = False, ptxas_verbose: bool = False, quiet: bool = True) 
                 print(log, file=sys.stderr)
     tmp = LIB + f".tmp{os.getpid()}"
     cmd = [_nvcc(), "-shared", *ARCH, "-o", tmp, *[o for o, _ in results]]
-    r = subprocess.run(cmd, capture_output=True, text=True)
-    if r.returncode != 0:
-        raise RuntimeError(f"link failed:\n{r.stdout}\n{r.stderr}")
+    _run(cmd, "link")
     os.replace(tmp, LIB)
+    _link_marshal(marshal.result())
     return LIB
 
 

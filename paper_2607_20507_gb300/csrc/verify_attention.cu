@@ -1237,8 +1237,18 @@ cs_status launch_verify_attention(const cs_attn_dims& d, const AttnPlan& pl, con
         p.tc_vstages = tc_v_stages(pl.n_rows);
         p.tc_q_half = tc_q_half_bytes(pl.n_rows);
         const int smem_bytes = tc_smem_bytes(pl.n_rows);
-        cudaError_t e = cudaFuncSetAttribute(tk_fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
-        if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(verify_attention_tc_kernel)");
+        cudaError_t e = cudaSuccess;
+        {
+            static int attr_smem[2][3][64] = {};   // the limit set so far
+            int dev = 0;
+            e = cudaGetDevice(&dev);
+            if (e != cudaSuccess) return cuda_fail(e, "cudaGetDevice");
+            if (dev < 0 || dev >= 64 || attr_smem[pl.tree][ti][dev] < smem_bytes) {
+                e = cudaFuncSetAttribute(tk_fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
+                if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(verify_attention_tc_kernel)");
+                if (dev >= 0 && dev < 64) attr_smem[pl.tree][ti][dev] = smem_bytes;
+            }
+        }
         for (int b0 = 0; b0 < d.batch; b0 += kMaxBatchPerLaunch) {
             p.b_base = b0;
             p.n_batch = d.batch - b0 < kMaxBatchPerLaunch ? d.batch - b0 : kMaxBatchPerLaunch;

@@ -1,0 +1,63 @@
+"""The binding's compiled marshalling: given outputs, workspaces and streams
+are used, and an argument that a call does not take raises what the Python
+checks raise."""
+import pytest
+import torch
+
+from paper_2607_20507_gb300 import binding
+from paper_2607_20507_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+DEV = "cuda:0"
+
+
+def inputs():
+    w = W.Workload(94, "binding", batch=3, n_draft=3, vocab=3001, logit_dtype="bf16", draft_sigma=0.7,
+                   temperatures=(0.8,), n_q_heads=16, n_kv_heads=4, head_dim=128, ctx=("uniform", 40, 400), page_size=16)
+    a, c = W.attention_inputs(w, DEV), W.accept_inputs(w, 0.8, DEV)
+    return ([a[k] for k in ("q", "k_pages", "v_pages", "page_table", "ctx_lens")],
+            [c[k] for k in ("target", "draft", "draft_tokens", "uniforms")])
+
+
+def test_given_outputs_workspace_and_stream():
+    a, c = inputs()
+    expect, (tok, n) = binding.cs_verify_attention(*a, 3), binding.cs_spec_accept(*c, 0.8)
+    out = torch.empty_like(a[0])
+    ws = torch.zeros(binding.cs_verify_attention_workspace_bytes(a[0], a[1], a[3], 3), dtype=torch.uint8, device=DEV)
+    side = torch.cuda.Stream()
+    side.wait_stream(torch.cuda.current_stream())
+    assert binding.cs_verify_attention(*a, 3, out=out, workspace=ws, stream=side.cuda_stream) is out
+    t2, n2 = torch.empty_like(tok), torch.empty_like(n)
+    r = binding.cs_spec_accept(*c, 0.8, out_tokens=t2, out_n_accepted=n2, stream=side.cuda_stream)
+    side.synchronize()
+    torch.cuda.synchronize()
+    assert r[0].data_ptr() == t2.data_ptr() and r[1].data_ptr() == n2.data_ptr()
+    assert torch.equal(out, expect) and torch.equal(t2, tok) and torch.equal(n2, n)
+    with torch.cuda.stream(side):   # the current stream
+        again = binding.cs_verify_attention(*a, 3, sm_scale=0)
+    side.synchronize()
+    assert torch.equal(again, expect)
+
+
+def test_refusals():
+    a, c = inputs()
+    for i, bad in ((0, a[0].float()), (0, a[0].transpose(1, 2)), (1, a[1].cpu()), (3, a[3].long()), (4, a[4][None])):
+        with pytest.raises((TypeError, ValueError)):
+            binding.cs_verify_attention(*a[:i], bad, *a[i + 1:], 3)
+    with pytest.raises(ValueError, match="n_draft"):
+        binding.cs_verify_attention(*a, 2)
+    with pytest.raises(ValueError, match="same shape"):
+        binding.cs_verify_attention(a[0], a[1], a[2][:-1].contiguous(), *a[3:], 3)
+    with pytest.raises(binding.CacheSpecError) as e:
+        binding.cs_verify_attention(*a, 3, workspace=torch.zeros(256, dtype=torch.uint8, device=DEV))
+    assert e.value.status == binding.CS_ERR_WORKSPACE
+    with pytest.raises(binding.CacheSpecError) as e:
+        binding.cs_spec_accept(*c, -1)
+    assert e.value.status == binding.CS_ERR_INVALID_ARG
+    with pytest.raises(ValueError):
+        binding.cs_spec_accept(c[0], c[1][:, :2].contiguous(), *c[2:], 0.8)
+    with pytest.raises(TypeError):
+        binding.cs_sample(c[0][:, 0].contiguous().half(), c[3][:, 0].contiguous(), 1.0)
+    with pytest.raises(TypeError):
+        binding.cs_kv_commit(a[4].long(), a[4], 3)
