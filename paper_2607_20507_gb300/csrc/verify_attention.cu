@@ -83,11 +83,11 @@ struct AttnParams {
     int* part_span;              // [2 * grid] span (b * n_vh + h) of each partial slot, -1 if unused
     int* status;
     int Hq, Hkv, G, R, n_rows, ps, box_t, max_pages, row_warps;
+    int P;                       // pages of the pool
     int n_rb;                    // row blocks per KV head (n_rows rows each)
     int n_vh;                    // Hkv * n_rb spans per request ("virtual heads")
     int n_rows_all;              // R * G query rows per KV head
     int tc_stages, tc_vstages;   // tcgen05 kernel: K and V ring depths
-    int tc_q_half;               // tcgen05 kernel: bytes between query dim halves
     int b_base, n_batch;         // requests [b_base, b_base + n_batch) in this launch
     int span_x;                  // work units charged to each span's start (see tiles_before)
     float scale_log2;            // sm_scale * log2(e)
@@ -941,6 +941,9 @@ verify_attention_merge_cut_kernel(const AttnParams p, int n_slots) {
 
 #include "verify_attention_tc.cuh"
 
+// 8-key groups of a pool (the tcgen05 form addresses them by a 32-bit coordinate)
+long long tc_groups(const cs_attn_dims& d) { return (long long)d.num_pages * d.n_kv_heads * (d.page_size / 8); }
+
 PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
     static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
     if (!fn) {
@@ -954,9 +957,7 @@ PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
     return fn;
 }
 
-// halves: dim halves per box (2: [half][keys][64 dims] per page piece; 1: one
-// half per box, for tiles laid out [half][64 keys][64 dims])
-cs_status encode_pool_map(CUtensorMap* map, const void* pool, const cs_attn_dims& d, int box_t, int halves = 2) {
+cs_status encode_pool_map(CUtensorMap* map, const void* pool, const cs_attn_dims& d, int box_t) {
     auto enc = tensor_map_encoder();
     if (!enc) return fail(CS_ERR_CUDA, "cuTensorMapEncodeTiled is not available from the driver");
     // (64 dims, keys, 2 dim halves, heads, pages): one box holds both halves
@@ -965,13 +966,32 @@ cs_status encode_pool_map(CUtensorMap* map, const void* pool, const cs_attn_dims
                                 (cuuint64_t)d.num_pages};
     const cuuint64_t row = (cuuint64_t)d.head_dim * 2;
     const cuuint64_t strides[4] = {row, 128, row * d.page_size, row * d.page_size * d.n_kv_heads};
-    const cuuint32_t box[5] = {64, (cuuint32_t)box_t, (cuuint32_t)halves, 1, 1};
+    const cuuint32_t box[5] = {64, (cuuint32_t)box_t, 2, 1, 1};
     const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
     const CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(pool), dims,
                            strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                            CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) return fail(CS_ERR_CUDA, "cuTensorMapEncodeTiled failed (CUresult %d)", (int)r);
+    return CS_OK;
+}
+
+// The same pool as 8-key groups, for the tcgen05 form: (64 dims, 8 keys, 2 dim
+// halves, groups), a (page, head)'s groups side by side, so a box of box_t
+// keys lands as [group][half][8 keys][64 dims] and a tile of several boxes has
+// its groups at one stride: one MMA covers its 64 keys.
+cs_status encode_group_map(CUtensorMap* map, const void* pool, const cs_attn_dims& d, int box_t) {
+    auto enc = tensor_map_encoder();
+    if (!enc) return fail(CS_ERR_CUDA, "cuTensorMapEncodeTiled is not available from the driver");
+    const cuuint64_t dims[4] = {64, 8, 2, (cuuint64_t)tc_groups(d)};
+    const cuuint64_t row = (cuuint64_t)d.head_dim * 2;
+    const cuuint64_t strides[3] = {row, 128, row * 8};
+    const cuuint32_t box[4] = {64, 8, 2, (cuuint32_t)(box_t / 8)};
+    const cuuint32_t estr[4] = {1, 1, 1, 1};
+    const CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(pool), dims, strides, box, estr,
+                           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                           CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS) return fail(CS_ERR_CUDA, "cuTensorMapEncodeTiled (groups) failed (CUresult %d)", (int)r);
     return CS_OK;
 }
 
@@ -1005,10 +1025,10 @@ int tc_resident_per_sm() {
     }
     if (!cache[dev]) {
         int n = 0;
-        if (cudaFuncSetAttribute(verify_attention_tc_kernel<false, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 tc_smem_bytes(kTcRows)) != cudaSuccess ||
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, verify_attention_tc_kernel<false, 16>, kTcThreads,
-                                                          tc_smem_bytes(kTcRows)) != cudaSuccess)
+        if (cudaFuncSetAttribute(verify_attention_tc_kernel<false, 16, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 tc_smem_bytes()) != cudaSuccess ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, verify_attention_tc_kernel<false, 16, false>, kTcThreads,
+                                                          tc_smem_bytes()) != cudaSuccess)
             n = 0;
         cudaGetLastError();
         cache[dev] = n + 1;
@@ -1128,8 +1148,7 @@ AttnPlan plan_attention(const cs_attn_dims& d, int rows, bool tree, int sm_count
         tc_rows = ((rows + tc_rb - 1) / tc_rb) * pl.group;
     }
     pl.tc = allow_tc && tc_rows > kTcMinRows && tc_rows <= kTcRows && d.page_size >= 16 && rows <= 256 &&
-            pl.group <= 256 &&
-            tc_resident_per_sm() >= 1;
+            pl.group <= 256 && tc_resident_per_sm() >= 1;
     if (pl.tc) {
         pl.n_rb = tc_rb;
         pl.n_rows = tc_rows;
@@ -1173,12 +1192,6 @@ cs_status launch_verify_attention(const cs_attn_dims& d, const AttnPlan& pl, con
     if (pl.tree != (parents != nullptr))
         return fail(CS_ERR_INVALID_ARG, "tree plan and parent array do not match");
     const int box_t = d.page_size < kTileT ? d.page_size : kTileT;
-    CUtensorMap tk, tv;
-    cs_status st = encode_pool_map(&tk, k_pages, d, box_t);
-    if (st != CS_OK) return st;
-    st = encode_pool_map(&tv, v_pages, d, box_t);
-    if (st != CS_OK) return st;
-
     uint8_t* ws = static_cast<uint8_t*>(workspace);
     AttnParams p{};
     p.q = static_cast<const __nv_bfloat16*>(q);
@@ -1196,6 +1209,7 @@ cs_status launch_verify_attention(const cs_attn_dims& d, const AttnPlan& pl, con
     p.R = pl.rows;
     p.n_rows = pl.n_rows;
     p.ps = d.page_size;
+    p.P = d.num_pages;
     p.box_t = box_t;
     p.max_pages = d.max_pages_per_seq;
     p.row_warps = pl.row_warps;
@@ -1219,27 +1233,37 @@ cs_status launch_verify_attention(const cs_attn_dims& d, const AttnPlan& pl, con
         return launch_verify_attention(d, alt, q, k_pages, v_pages, page_table, ctx_lens, parents, out, workspace,
                                        stream);
     }
+    CUtensorMap tk, tv;
     if (pl.tc) {
+        // Pages of 16 or 32 keys in 8-key groups up to 64 query rows: k = 8 (36
+        // rows), context 4096, at B = 256 740 us in pieces and 699 in groups, 35
+        // rows at B = 64 68.4 and 66.7.  With more rows the pieces are the
+        // faster: 68 rows 209 and 217 us, 128 rows 257 and 268 (72 rows: 1722 and
+        // 1718).
+        const bool groups = pl.n_rows <= 64 && box_t < kTileT && tc_groups(d) <= 0x7fffffffLL;
         CUtensorMap tq;
+        cs_status st = groups ? encode_group_map(&tk, k_pages, d, box_t) : encode_pool_map(&tk, k_pages, d, box_t);
+        if (st != CS_OK) return st;
+        st = groups ? encode_group_map(&tv, v_pages, d, box_t) : encode_pool_map(&tv, v_pages, d, box_t);
+        if (st != CS_OK) return st;
         st = encode_q_map(&tq, q, d, pl.rows, pl.n_rows / pl.group);
         if (st != CS_OK) return st;
-        // one box per page piece with both dim halves, as for the other form
-
         using TcKern = void (*)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const AttnParams);
-        static const TcKern tc_kerns[2][3] = {
-            {verify_attention_tc_kernel<false, 16>, verify_attention_tc_kernel<false, 32>,
-             verify_attention_tc_kernel<false, 64>},
-            {verify_attention_tc_kernel<true, 16>, verify_attention_tc_kernel<true, 32>,
-             verify_attention_tc_kernel<true, 64>}};
-        const int ti = box_t == 16 ? 0 : box_t == 32 ? 1 : 2;
+        static const TcKern tc_kerns[2][5] = {
+            {verify_attention_tc_kernel<false, 16, false>, verify_attention_tc_kernel<false, 32, false>,
+             verify_attention_tc_kernel<false, 64, false>, verify_attention_tc_kernel<false, 16, true>,
+             verify_attention_tc_kernel<false, 32, true>},
+            {verify_attention_tc_kernel<true, 16, false>, verify_attention_tc_kernel<true, 32, false>,
+             verify_attention_tc_kernel<true, 64, false>, verify_attention_tc_kernel<true, 16, true>,
+             verify_attention_tc_kernel<true, 32, true>}};
+        const int ti = (box_t == 16 ? 0 : box_t == 32 ? 1 : 2) + (groups ? 3 : 0);
         const TcKern tk_fn = tc_kerns[pl.tree][ti];
-        p.tc_stages = tc_k_stages(pl.n_rows);
-        p.tc_vstages = tc_v_stages(pl.n_rows);
-        p.tc_q_half = tc_q_half_bytes(pl.n_rows);
-        const int smem_bytes = tc_smem_bytes(pl.n_rows);
+        p.tc_stages = tc_k_stages();
+        p.tc_vstages = tc_v_stages();
+        const int smem_bytes = tc_smem_bytes();
         cudaError_t e = cudaSuccess;
         {
-            static int attr_smem[2][3][64] = {};   // the limit set so far
+            static int attr_smem[2][5][64] = {};   // the limit set so far
             int dev = 0;
             e = cudaGetDevice(&dev);
             if (e != cudaSuccess) return cuda_fail(e, "cudaGetDevice");
@@ -1259,6 +1283,10 @@ cs_status launch_verify_attention(const cs_attn_dims& d, const AttnPlan& pl, con
         }
         return CS_OK;
     }
+    cs_status st = encode_pool_map(&tk, k_pages, d, box_t);
+    if (st != CS_OK) return st;
+    st = encode_pool_map(&tv, v_pages, d, box_t);
+    if (st != CS_OK) return st;
     // kernels by (key split, tree, box size 8/16/32/64 keys)
     using Kern = void (*)(const CUtensorMap, const CUtensorMap, const AttnParams);
     static const Kern kerns[2][2][4] = {

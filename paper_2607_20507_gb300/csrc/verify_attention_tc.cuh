@@ -16,14 +16,13 @@
 // (with them on SMSPs 0 and 1 the kernel ran 7-15% slower):
 //   warp 2  K producer: the span's query rows (one 4-D box per dim half into
 //           one buffer, refilled once the previous span's rows have been
-//           copied into tensor memory; each half as many 128-byte rows as
-//           the span has: the MMA's 128-row window runs on into whatever
-//           follows, which only feeds padded rows) and the K tiles of the
-//           range through the K ring, one box per page piece with both dim
+//           copied into tensor memory; the MMA's 128 rows, of which no copy
+//           writes those past the span's: they stay zero) and the K tiles of
+//           the range through the K ring, one box per page piece with both dim
 //           halves (contiguous 256-byte rows: a per-half box of 128-byte rows
 //           kept the SM's copy engine saturated at two thirds of the
-//           bandwidth), so a tile lands as [piece][dim half][keys][128 B],
-//           128-byte swizzle;
+//           bandwidth), 128-byte swizzle; a tile lands as [piece][dim half]
+//           [keys][128 B] or, up to 64 query rows, as 8-key groups (TcTile);
 //           beside each stage it leaves whether the tile opens or closes a
 //           piece;
 //   warp 3  V producer: the V tiles through the V ring, the same way.  The
@@ -34,9 +33,9 @@
 //   warp 0  QK issuer (the whole warp waits, one elected lane issues): at
 //           a piece's start the query rows from shared into tensor memory
 //           (tcgen05.cp, one buffer per span parity), then per tile
-//           S_t = Q K_t^T into tensor memory (M = 128 padded rows, per page
-//           piece N = its keys, Q from tensor memory, K a K-major
-//           shared-memory operand, 8 steps of 16 dims) as soon as K_t has
+//           S_t = Q K_t^T into tensor memory (M = 128 padded rows, N = the
+//           keys of a page piece or of the tile, Q from tensor memory, K a
+//           K-major shared-memory operand, 8 steps of 16 dims) as soon as K_t has
 //           landed and one of four S buffers is free -- up to four tiles
 //           ahead of the softmax.  It also allocates the tensor memory (512
 //           columns: four S/P buffers of 64, O in 128, two query buffers of
@@ -44,9 +43,7 @@
 //   warp 1  PV issuer: O += P_t V_t (N = 128 dims, 8 steps of 16 keys: 4
 //           with P_hi, 4 with P_lo) as soon as the softmax releases P_t and
 //           V_t has landed, with P read from tensor memory and V, as stored
-//           in bf16, an MN-major operand (per 16 keys, the rows of one page
-//           piece) whose two dim halves lie one piece half apart; in a span's
-//           last tile it first zeroes the V rows past L_b (their slots may
+//           in bf16, an MN-major operand; in a span's last tile it first zeroes the V rows past L_b (their slots may
 //           hold any bits);
 //   warps 4-11 softmax and epilogue, one warp per 16 tensor-memory lanes
 //           (query rows; warp 4+q lanes 32q..32q+15, warp 8+q lanes
@@ -83,26 +80,30 @@ constexpr int kTcBarBytes = 512;
 constexpr int kTcFixedSmem = kTcBarBytes + (kMaxBatchPerLaunch + 1) * 8 + kMaxBatchPerLaunch * 4 + 1024;
 constexpr int kTcSmemLimit = 232448 - 2560;        // opt-in shared memory per block, less the static part
 
-// Bytes between the two dim halves of a span's query rows (1024-aligned).
-__host__ __device__ constexpr int tc_q_half_bytes(int rows) { return (rows * 128 + 1023) / 1024 * 1024; }
+// One dim half of a span's query rows: the MMA's 128 rows, those past the
+// span's zero.  (The padded rows of S, and of P, which is written over it,
+// are then zeros too.  With whatever followed the rows in their place the
+// tensor pipe drew the card to its power limit: 1380 W, the clock down to
+// 1790-1960 MHz, against 990 W and 2070 MHz without the MMAs.)
+constexpr int kTcQHalfBytes = kTcRows * 128;
 // 16 KB tile stages (one K or one V tile each) that fit beside the query
-// buffer of `rows` rows, split between the K ring (a third: K is released
+// buffer, split between the K ring (a third: K is released
 // as soon as its QK is done) and the V ring (the rest: V waits for the
 // softmax).
-__host__ __device__ constexpr int tc_tile_stages(int rows) {
-    return (kTcSmemLimit - kTcFixedSmem - 2 * tc_q_half_bytes(rows)) / kTensorTileBytes;
+__host__ __device__ constexpr int tc_tile_stages() {
+    return (kTcSmemLimit - kTcFixedSmem - 2 * kTcQHalfBytes) / kTensorTileBytes;
 }
-__host__ __device__ constexpr int tc_k_stages(int rows) {
-    return (tc_tile_stages(rows) + 1) / 3 < 2 ? 2
-           : (tc_tile_stages(rows) + 1) / 3 > kTcMaxK ? kTcMaxK : (tc_tile_stages(rows) + 1) / 3;
+__host__ __device__ constexpr int tc_k_stages() {
+    return (tc_tile_stages() + 1) / 3 < 2 ? 2
+           : (tc_tile_stages() + 1) / 3 > kTcMaxK ? kTcMaxK : (tc_tile_stages() + 1) / 3;
 }
-__host__ __device__ constexpr int tc_v_stages(int rows) {
-    return tc_tile_stages(rows) - tc_k_stages(rows) > kTcMaxV ? kTcMaxV : tc_tile_stages(rows) - tc_k_stages(rows);
+__host__ __device__ constexpr int tc_v_stages() {
+    return tc_tile_stages() - tc_k_stages() > kTcMaxV ? kTcMaxV : tc_tile_stages() - tc_k_stages();
 }
-__host__ __device__ constexpr int tc_smem_bytes(int rows) {
-    return 2 * tc_q_half_bytes(rows) + (tc_k_stages(rows) + tc_v_stages(rows)) * kTensorTileBytes + kTcFixedSmem;
+__host__ __device__ constexpr int tc_smem_bytes() {
+    return 2 * kTcQHalfBytes + (tc_k_stages() + tc_v_stages()) * kTensorTileBytes + kTcFixedSmem;
 }
-static_assert(tc_k_stages(kTcRows) >= 2 && tc_v_stages(kTcRows) >= 4, "rings too shallow for 128 query rows");
+static_assert(tc_k_stages() >= 2 && tc_v_stages() >= 4, "rings too shallow");
 static_assert((2 * kTcMaxK + 2 * kTcMaxV + 4 + 3 * kTcSBuf + 1) * 8 <= kTcBarBytes, "barrier block too small");
 constexpr float kTcRescale = 8.f;                  // log2 growth of the max that forces a rescale of O
 
@@ -112,13 +113,36 @@ __device__ __forceinline__ uint64_t tc_sw128_desc(uint32_t addr) {
            (2ull << 61);
 }
 
-// MN-major, 128-byte swizzle, for a V page piece [dim half][keys][128 B]:
-// 8-key groups 1024 bytes apart (stride), the two 64-dim halves
-// `half_bytes` apart (leading offset)
-__device__ __forceinline__ uint64_t tc_mn_desc(uint32_t addr, uint32_t half_bytes) {
-    return (uint64_t)((addr >> 4) & 0x3FFF) | ((uint64_t)(half_bytes >> 4) << 16) |
-           ((uint64_t)(1024 >> 4) << 32) | (1ull << 46) | (2ull << 61);
-}
+// How a 64-key tile of K or V lies in shared memory, by what one TMA box of
+// kBoxT keys (a page piece) leaves: [dim half][keys][128 B], or, kGroups,
+// [8-key group][dim half][8 keys][128 B].  Groups have one stride through the
+// tile, whatever its pieces, so one MMA takes its 64 keys (780 cycles a tile
+// for QK and PV back to back, against 890 and 940 with 32 and 16 keys an MMA).
+template <int kBoxT, bool kGroups>
+struct TcTile {
+    static constexpr int kN = kGroups ? kTileT : kBoxT;                    // keys of a QK MMA
+    static constexpr uint32_t kPiece = kBoxT * 256u;                       // bytes of a page piece
+    static constexpr uint32_t kGroup = kGroups ? 2048u : 1024u;            // from an 8-key group to the next
+    static constexpr uint32_t kHalf = kGroups ? 1024u : kBoxT * 128u;      // from a dim half to the other
+    // K, K-major, 128-byte swizzle
+    static __device__ __forceinline__ uint64_t k_desc(uint32_t addr) {
+        return (uint64_t)((addr >> 4) & 0x3FFF) | ((uint64_t)1 << 16) | ((uint64_t)(kGroup >> 4) << 32) | (1ull << 46) |
+               (2ull << 61);
+    }
+    // V, MN-major, 128-byte swizzle: 8-key groups (stride), dim halves (leading offset)
+    static __device__ __forceinline__ uint64_t v_desc(uint32_t addr) {
+        return (uint64_t)((addr >> 4) & 0x3FFF) | ((uint64_t)(kHalf >> 4) << 16) | ((uint64_t)(kGroup >> 4) << 32) |
+               (1ull << 46) | (2ull << 61);
+    }
+    // offset of keys 16 kk .. 16 kk + 15 of V
+    static __host__ __device__ constexpr uint32_t v_step(int kk) {
+        return kGroups ? 2u * kk * kGroup : ((16 * kk) / kBoxT) * kPiece + ((16 * kk) % kBoxT) * 128u;
+    }
+    // the key of 128-byte row r
+    static __device__ __forceinline__ int key_of(int r) {
+        return kGroups ? (r >> 4) * 8 + (r & 7) : (r / (2 * kBoxT)) * kBoxT + r % kBoxT;
+    }
+};
 
 // kind::f16 instruction descriptor: fp32 D, M = 128, N = n, A and B both
 // bf16 (f16 = false) or both fp16; b_mn: B is MN-major (its N index contiguous)
@@ -262,18 +286,17 @@ __device__ __forceinline__ bool tc_wait(uint64_t* bar, uint32_t parity, volatile
 }
 
 
-template <bool kTree, int kBoxT>
+template <bool kTree, int kBoxT, bool kGroups>
 __global__ void __launch_bounds__(kTcThreads, 1)
 verify_attention_tc_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_constant__ CUtensorMap tmap_v,
                            const __grid_constant__ CUtensorMap tmap_q, const AttnParams p) {
     constexpr int kPieces = kTileT / kBoxT;
-    constexpr uint32_t kPieceBytes = (uint32_t)kBoxT * 256u;   // bytes of one page piece of K (or of V)
-    constexpr uint32_t kPieceHalf = (uint32_t)kBoxT * 128u;    // one dim half of a page piece
+    using Tile = TcTile<kBoxT, kGroups>;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const int SK = p.tc_stages, SV = p.tc_vstages;          // K and V ring depths
-    const int qh = p.tc_q_half;                             // bytes between the dim halves of a span's rows
-    uint8_t* sq = smem;                                     // [2 halves][rows][128 B]: one span's query rows
+    constexpr int qh = kTcQHalfBytes;                       // bytes between the dim halves of a span's rows
+    uint8_t* sq = smem;                                     // [2 halves][128 rows][128 B]: one span's query rows, then zeros
     uint8_t* sk = smem + 2 * qh;                            // [K stage][half][64 keys][128 B]
     uint8_t* sv = sk + SK * kTensorTileBytes;               // [V stage][half][64 keys][128 B]
     uint64_t* bars = reinterpret_cast<uint64_t*>(sv + SV * kTensorTileBytes);
@@ -337,6 +360,13 @@ verify_attention_tc_kernel(const __grid_constant__ CUtensorMap tmap_k, const __g
         }
         mbar_init(o_free, n_live);
         fence_barrier_init();
+    }
+    // the padded query rows, which no copy writes
+    {
+        const int pad = (kTcRows - p.n_rows) * 8;   // 16-byte pieces of a half
+        for (int i = threadIdx.x; i < 2 * pad; i += kTcThreads)
+            reinterpret_cast<uint4*>(sq + (i >= pad ? qh : 0))[p.n_rows * 8 + (i >= pad ? i - pad : i)] = make_uint4(0, 0, 0, 0);
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the tensor core reads them next
     }
     // a programmatic dependent of the kernel before it (inputs are read
     // below); the merge kernel may start once every CTA is past this point
@@ -473,15 +503,21 @@ verify_attention_tc_kernel(const __grid_constant__ CUtensorMap tmap_k, const __g
             if (lane == 0) {
                 if (k_side) s_info[st] = (c.first ? 1 : 0) | (c.last ? 2 : 0);
                 else s_keys[st] = max(0, min(kTileT, c.L - c.ts));
-                mbar_arrive_expect_tx(&fullb[st], (uint32_t)c.valid * kPieceBytes);
+                mbar_arrive_expect_tx(&fullb[st], (uint32_t)c.valid * Tile::kPiece);
             }
             __syncwarp();
             if (lane < c.valid) {
-                // one box per page piece, both dim halves: [half][kBoxT keys][128 B]
-                // (page sizes are powers of two)
-                const uint32_t dst = smem_u32(ring + st * kTensorTileBytes) + (uint32_t)lane * kPieceBytes;
+                // one box per page piece, both dim halves (page sizes are powers of two)
+                const uint32_t dst = smem_u32(ring + st * kTensorTileBytes) + (uint32_t)lane * Tile::kPiece;
                 const int slot = (c.ts + lane * kBoxT) & (p.ps - 1);
-                tma_load_5d(dst, tmap, &fullb[st], 0, slot, 0, c.h, c.page);
+                if (kGroups) {
+                    // (a page outside the pool reads as zeros, from in front of it)
+                    const int group = (unsigned)c.page < (unsigned)p.P
+                                          ? (c.page * p.Hkv + c.h) * (p.ps >> 3) + (slot >> 3) : -(kBoxT >> 3);
+                    tma_load_4d(dst, tmap, &fullb[st], 0, 0, 0, group);
+                } else {
+                    tma_load_5d(dst, tmap, &fullb[st], 0, slot, 0, c.h, c.page);
+                }
             }
             if (jt + 1 < n_tiles) prepare(jt + 1);
         }
@@ -508,10 +544,10 @@ verify_attention_tc_kernel(const __grid_constant__ CUtensorMap tmap_k, const __g
         // carry).
         const bool qk_warp = warp == kTcQkWarp;
         // QK and PV both bf16: P enters as two bf16 terms (hi + lo) against V as stored
-        constexpr uint32_t id_s = tc_idesc(kBoxT, false, false), id_o = tc_idesc(kD, true, false);
+        constexpr uint32_t id_s = tc_idesc(Tile::kN, false, false), id_o = tc_idesc(kD, true, false);
         const uint64_t dq0 = tc_sw128_desc(smem_u32(sq));
         const uint64_t qhalf16 = (uint64_t)qh >> 4;
-        const uint64_t dk0 = tc_sw128_desc(smem_u32(sk)), dv0 = tc_mn_desc(smem_u32(sv), kPieceHalf);
+        const uint64_t dk0 = Tile::k_desc(smem_u32(sk)), dv0 = Tile::v_desc(smem_u32(sv));
         int span = -1, pv_piece = 0;
         Cursor cur = locate(f0, s_prefix, s_len, nb, p.n_vh);   // the PV warp's own view of the pieces
         uint64_t* last_bar = nullptr;   // the warp's latest commit: completes after all its MMAs
@@ -549,15 +585,13 @@ verify_attention_tc_kernel(const __grid_constant__ CUtensorMap tmap_k, const __g
                             tc_cp_128x256b(tq + ks * 8, dq0 + (ks >> 2) * qhalf16 + (uint64_t)((ks & 3) * 2));
                         tc_commit(q_cp);   // the producer may refill the query buffer
                     }
-                    // per page piece (N = kBoxT keys, S columns pc*kBoxT..), 8
-                    // steps of 16 dims
+                    // the keys of an MMA, 8 steps of 16 dims
 #pragma unroll
-                    for (int pc = 0; pc < kPieces; ++pc) {
+                    for (int pc = 0; pc < kTileT / Tile::kN; ++pc) {
 #pragma unroll
                         for (int ks = 0; ks < kD / 16; ++ks) {
-                            const uint64_t ko =
-                                (uint64_t)(((pc * kPieceBytes + (ks >> 2) * kPieceHalf) >> 4) + (ks & 3) * 2);
-                            tc_mma_ts(tmem + sb * 64 + pc * kBoxT, tq + ks * 8, dk + ko, id_s, ks > 0 ? 1u : 0u);
+                            const uint64_t ko = (uint64_t)(((pc * Tile::kPiece + (ks >> 2) * Tile::kHalf) >> 4) + (ks & 3) * 2);
+                            tc_mma_ts(tmem + sb * 64 + pc * Tile::kN, tq + ks * 8, dk + ko, id_s, ks > 0 ? 1u : 0u);
                         }
                     }
                     tc_commit(&s_full[sb]);
@@ -580,15 +614,13 @@ verify_attention_tc_kernel(const __grid_constant__ CUtensorMap tmap_k, const __g
                     ++pv_piece;
                 }
                 // a span's last tile: the slots past L_b may hold any bits (NaN
-                // included) and P is 0 there, so their V rows are zeroed (128-byte
-                // row r of the tile, [piece][half][kBoxT keys], holds key
-                // (r / (2 kBoxT)) kBoxT + r % kBoxT)
+                // included) and P is 0 there, so their V rows are zeroed
                 const int keys = s_keys[st];
                 if (keys < kTileT) {
                     uint4* vt = reinterpret_cast<uint4*>(sv + st * kTensorTileBytes);
                     for (int i = lane; i < kTensorTileBytes / 16; i += 32) {
                         const int r = i >> 3;
-                        if ((r / (2 * kBoxT)) * kBoxT + r % kBoxT >= keys) vt[i] = make_uint4(0, 0, 0, 0);
+                        if (Tile::key_of(r) >= keys) vt[i] = make_uint4(0, 0, 0, 0);
                     }
                     // generic writes the tensor core reads next
                     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -599,15 +631,15 @@ verify_attention_tc_kernel(const __grid_constant__ CUtensorMap tmap_k, const __g
                 // the buffer), 4 with P_lo (columns 32..63), both dim halves per step
                 const uint64_t dv = dv0 + (uint64_t)((st * kTensorTileBytes) >> 4);
                 if (elect_one()) {
-                    // keys 16kk..16kk+15: rows (16kk) % kBoxT.. of page piece 16kk / kBoxT
+                    // keys 16kk..16kk+15
 #pragma unroll
                     for (int kk = 0; kk < kTileT / 16; ++kk) {
-                        const uint64_t vk = dv + (uint64_t)((((16 * kk) / kBoxT) * kPieceBytes + ((16 * kk) % kBoxT) * 128) >> 4);
+                        const uint64_t vk = dv + (uint64_t)(Tile::v_step(kk) >> 4);
                         tc_mma_ts(tmem + kTcOCol, tmem + sb * 64 + kk * 8, vk, id_o, (first && kk == 0) ? 0u : 1u);
                     }
 #pragma unroll
                     for (int kk = 0; kk < kTileT / 16; ++kk) {
-                        const uint64_t vk = dv + (uint64_t)((((16 * kk) / kBoxT) * kPieceBytes + ((16 * kk) % kBoxT) * 128) >> 4);
+                        const uint64_t vk = dv + (uint64_t)(Tile::v_step(kk) >> 4);
                         tc_mma_ts(tmem + kTcOCol, tmem + sb * 64 + 32 + kk * 8, vk, id_o, 1u);
                     }
                     tc_commit(&o_ready[sb]);
