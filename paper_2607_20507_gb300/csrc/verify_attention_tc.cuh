@@ -411,8 +411,7 @@ verify_attention_tc_kernel(const __grid_constant__ CUtensorMap tmap_k, const __g
     const uint32_t tmem = s_tmem;
 
     const long long W = s_prefix[nb];
-    const long long g_need = (W + kMinTilesPerCta - 1) / kMinTilesPerCta;
-    const int Gc = (int)(g_need < (long long)gridDim.x ? (g_need > 0 ? g_need : 1) : gridDim.x);
+    const int Gc = (int)(W < (long long)gridDim.x ? (W > 0 ? W : 1) : gridDim.x);
     const int cta = blockIdx.x;
     const long long U = W + (long long)p.span_x * p.n_vh * nb;
     long long f0 = tiles_before(unit_start(cta, U, Gc), s_prefix, s_len, nb, p.n_vh, p.span_x);
