@@ -218,4 +218,13 @@ __device__ __forceinline__ float bf16_bits_to_float(uint32_t bits16) {
     return __uint_as_float(bits16 << 16);
 }
 
+// Programmatic dependent launch: a kernel may start while the one before it
+// in the stream runs; every CTA waits here, before it reads what an earlier
+// kernel wrote or overwrites what one reads (a no-op when the kernel was
+// launched without the attribute).
+__device__ __forceinline__ void wait_prior_grid() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void allow_dependent_launch() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 }  // namespace cs

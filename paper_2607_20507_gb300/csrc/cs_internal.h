@@ -17,6 +17,24 @@ cs_status cuda_fail(cudaError_t e, const char* what);
 // Streaming multiprocessors of the current device (cached per device).
 int current_sm_count();
 
+// A launch that may start while the kernel before it in the stream runs
+// (the kernel waits with griddepcontrol.wait before it reads its inputs).
+template <typename... Args, typename... Params>
+cudaError_t launch_dependent(void (*kern)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
+                             Args... args) {
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
 // ------------------------------------------------------------- attention
 struct AttnPlan {
     int group;        // G = Hq / Hkv

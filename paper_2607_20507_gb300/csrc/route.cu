@@ -145,6 +145,8 @@ route_gemm_kernel(const __grid_constant__ CUtensorMap tmap_e, const __grid_const
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     if (threadIdx.x == 0) {
+        tma_prefetch_desc(&tmap_e);
+        tma_prefetch_desc(&tmap_c);
         mbar_init(a_full, 1);
         mbar_init(a_free, 1);
         for (int i = 0; i < 2; ++i) {
@@ -162,11 +164,11 @@ route_gemm_kernel(const __grid_constant__ CUtensorMap tmap_e, const __grid_const
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = s_tmem;
+    wait_prior_grid();
+    allow_dependent_launch();
 
     if (warp == 0 && lane == 0) {
         // ---------------------------------------------------------- TMA
-        tma_prefetch_desc(&tmap_e);
-        tma_prefetch_desc(&tmap_c);
         int s = 0, cur_m = -1;
         uint32_t use = 0, a_loads = 0;
         bool ok = true;
@@ -343,6 +345,8 @@ __global__ void __launch_bounds__(256) route_merge_kernel(const __nv_bfloat16* e
                                                            float tau, int32_t* out_group, int32_t* out_best,
                                                            float* out_score) {
     const int b = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    wait_prior_grid();
+    allow_dependent_launch();
     if (b >= B) return;
     float ss = 0.f;
     for (int k = lane; k < d; k += 32) {
@@ -476,14 +480,12 @@ cs_status launch_route(const cs_route_dims& d, const RoutePlan& pl, const void* 
         p.inv_norm_c = inv_norms;
         p.status = reinterpret_cast<int*>(ws);
         p.part = reinterpret_cast<float2*>(ws + 256);
-        route_gemm_kernel<<<pl.grid, kRThreads, smem, stream>>>(te, tc, p);
-        e = cudaGetLastError();
+        e = launch_dependent(route_gemm_kernel, dim3(pl.grid), dim3(kRThreads), smem, stream, te, tc, p);
         if (e != cudaSuccess) return cuda_fail(e, "route_gemm_kernel launch");
     }
-    route_merge_kernel<<<(d.batch + 7) / 8, 256, 0, stream>>>(
-        static_cast<const __nv_bfloat16*>(emb), reinterpret_cast<const float2*>(ws + 256), d.batch, d.dim,
-        pl.n_tiles, pl.items, pl.grid, pl.seg_slots, tau, out_group, out_best, out_score);
-    e = cudaGetLastError();
+    e = launch_dependent(route_merge_kernel, dim3((d.batch + 7) / 8), dim3(256), 0, stream,
+                         static_cast<const __nv_bfloat16*>(emb), reinterpret_cast<const float2*>(ws + 256), d.batch,
+                         d.dim, pl.n_tiles, pl.items, pl.grid, pl.seg_slots, tau, out_group, out_best, out_score);
     if (e != cudaSuccess) return cuda_fail(e, "route_merge_kernel launch");
     return CS_OK;
 }

@@ -258,14 +258,6 @@ __device__ __noinline__ long long div_nn(long long x, long long d) {
     return x / d;
 }
 
-// Programmatic dependent launch: each kernel may start while the one before
-// it runs; it waits here before reading what that kernel wrote (a no-op
-// when it was launched without the attribute).
-__device__ __forceinline__ void wait_prior_grid() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void allow_dependent_launch() {
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
-
 // ------------------------------------------------------------ kernel 1
 // Largest of the logits of one lane's vectors (bf16: packed maxima, one
 // instruction per pair).

@@ -1035,24 +1035,6 @@ int tc_resident_per_sm() {
 
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
-// A launch that may start while the kernel before it in the stream runs
-// (the kernel waits with griddepcontrol.wait before it reads its inputs).
-template <typename... Args, typename... Params>
-cudaError_t launch_dependent(void (*kern)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
-                             Args... args) {
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = block;
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = stream;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, args...);
-}
-
 // The split merge as a programmatic dependent of the main kernel: it may
 // start early and waits (griddepcontrol.wait) before it reads the partials.
 // The form with the smaller grid: per span (spans x 8-row chunks; few

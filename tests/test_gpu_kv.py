@@ -101,3 +101,31 @@ def test_one_step_chained_through_the_c_abi():
     tie = am < 1e-5                              # accept tests within the near-tie band
     assert (n_gpu[~tie] == en[~tie]).all()
     np.testing.assert_array_equal(lens.cpu().numpy(), oracle.kv_commit(inp["ctx_lens"].cpu().numpy(), n_gpu, k))
+
+
+@pytest.mark.parametrize("n,H,ps,kind", [(64, 1, 8, "path"), (9, 3, 16, "path"), (34, 8, 16, "aliased"),
+                                         (64, 40, 16, "path"), (20, 2, 16, "any"), (1, 8, 16, "path")])
+def test_tree_commit_parity(n, H, ps, kind):
+    """Long and short paths, more columns than a block has threads, a page that
+    appears twice in a table, and nodes in any order (bytes are bytes)."""
+    B = 5
+    kp, vp, pt, L, _, _ = setup(B, n, H, ps, 200 // ps, seed=n * 13 + H)
+    rng = np.random.default_rng(n + H)
+    path = np.full((B, n), -1, np.int32)
+    na = np.zeros(B, np.int32)
+    for b in range(B):
+        na[b] = rng.integers(0, n) if b else n - 1
+        nodes = rng.permutation(np.arange(1, n))[:na[b]]
+        path[b, :na[b]] = nodes if kind == "any" else np.sort(nodes)
+    if kind == "any":      # any order, but no source before the first key
+        L[:] = torch.clamp(L, min=2 * n)
+    if kind == "aliased":
+        pt[:, 1::2] = pt[:, 0::2][:, :pt[:, 1::2].shape[1]]
+    gk, gv, lens = kp.to(DEV), vp.to(DEV), L.to(DEV)
+    binding.cs_kv_commit_tree(gk, gv, pt.to(DEV), lens, torch.from_numpy(path).to(DEV), torch.from_numpy(na).to(DEV))
+    torch.cuda.synchronize()
+    ok, ov = bits(kp).copy(), bits(vp).copy()
+    exp = oracle.kv_commit_tree(ok, ov, pt.numpy(), L.numpy(), path, na, n)
+    np.testing.assert_array_equal(lens.cpu().numpy(), exp)
+    np.testing.assert_array_equal(bits(gk.cpu()), ok)
+    np.testing.assert_array_equal(bits(gv.cpu()), ov)
