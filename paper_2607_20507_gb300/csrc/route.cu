@@ -8,12 +8,21 @@
 // (the B x N score matrix never reaches memory):
 //   route_gemm_kernel: a CTA owns 128 requests (MMA M) and a contiguous range
 //     of 128-group tiles.  Warp 0 loads the CTA's embedding rows once (one TMA
-//     box per 64-dim chunk, 128-byte swizzle, kept in shared memory) and
-//     streams the centroid chunks through a 6-slot TMA ring; warp 1 issues
-//     tcgen05.mma from one thread (M = 128, N = 128, K = 16 per instruction,
-//     fp32 accumulators in tensor memory, two buffers); warps 4-7 take one
-//     row each per thread, scale each dot product by the centroid's inverse
-//     norm and keep the running maximum and its lowest index.
+//     box per 64 dims, 128-byte swizzle, kept in shared memory) and streams
+//     the centroids through a TMA ring, 128 dims a stage; warp 1 issues
+//     tcgen05.mma (M = 128, N = 128, K = 16 per instruction, fp32 accumulators
+//     in tensor memory, two buffers); warps 4-11 take one row and half a
+//     tile's columns each per thread, scale each dot product by the
+//     centroid's inverse norm and keep the running maximum and its lowest
+//     index.
+//     What bounds it: a tile is 24 MMAs of 64 cycles at 384 dims, and the two
+//     issuing warps and the epilogue have to keep below that.  Both issuing
+//     warps run their loops with all lanes and elect one to issue: a lone lane
+//     beside 31 parked at the block barrier took 450 cycles for each 64 dims
+//     without its MMAs (a tile 4140 cycles; loads or none made no
+//     difference).  1024 requests, 16384 groups, 384 dims, both kernels in a
+//     captured graph: 23.8 us so, 17.7 as it is; a further 1024 requests 14.6
+//     and 9.5.
 //   route_merge_kernel: one warp per request folds the CTAs' partials (score
 //     first, then lower index), applies the request's own inverse norm and
 //     the threshold.
@@ -29,27 +38,28 @@ namespace {
 
 constexpr int kRM = 128;                  // requests per tile (MMA M)
 constexpr int kRN = 128;                  // groups per tile (MMA N)
-constexpr int kKC = 64;                   // dims per chunk: one 128-byte swizzle row
-constexpr int kChunkBytes = kRM * 128;    // 128 rows x 64 dims x 2 B
-constexpr int kMaxSlots = 12;             // centroid-chunk ring, at most
-constexpr int kRThreads = 256;            // warp 0 TMA, warp 1 MMA, warp 2 TMEM, warps 4-7 epilogue
+constexpr int kKC = 64;                   // dims per box: one 128-byte swizzle row
+constexpr int kBoxBytes = kRM * 128;      // 128 rows x 64 dims x 2 B
+constexpr int kStageBoxes = 2;            // boxes of 128 groups a ring stage holds
+constexpr int kMaxSlots = 6;              // ring stages, at most
+constexpr int kEpiWarps = 8;              // two to a quarter of the rows, 64 columns of a tile each
+constexpr int kRThreads = 128 + kEpiWarps * 32;   // warp 0 TMA, warp 1 MMA, warp 2 TMEM, warps 4-11 epilogue
 constexpr int kRTmemCols = 2 * kRN;
-constexpr int kRBarBytes = 256;
-constexpr int kRStaticSmem = 2 * kRN * 4 + 64;   // inverse-norm double buffer, TMEM address
-constexpr int kRSmemLimit = 232448;              // opt-in shared memory per block on sm_103a
+constexpr int kRSmemLimit = 232448;       // opt-in shared memory per block on sm_103a
+constexpr int kRTailBytes = 256 /*barriers*/ + 2 * kRN * 4 /*inverse norms*/ + kRM * 8 /*column halves*/ + 16;
 
-__host__ __device__ constexpr int route_slots(int n_chunks) {
-    return (kRSmemLimit - kRStaticSmem - 1024 - kRBarBytes - n_chunks * kChunkBytes) / kChunkBytes < kMaxSlots
-               ? (kRSmemLimit - kRStaticSmem - 1024 - kRBarBytes - n_chunks * kChunkBytes) / kChunkBytes
+__host__ __device__ constexpr int route_slots(int n_boxes) {
+    return (kRSmemLimit - kRTailBytes - n_boxes * kBoxBytes) / (kStageBoxes * kBoxBytes) < kMaxSlots
+               ? (kRSmemLimit - kRTailBytes - n_boxes * kBoxBytes) / (kStageBoxes * kBoxBytes)
                : kMaxSlots;
 }
-__host__ __device__ constexpr int route_smem_bytes(int n_chunks) {
-    return 1024 + n_chunks * kChunkBytes + route_slots(n_chunks) * kChunkBytes + kRBarBytes;
+__host__ __device__ constexpr int route_smem_bytes(int n_boxes) {
+    return (n_boxes + route_slots(n_boxes) * kStageBoxes) * kBoxBytes + kRTailBytes;
 }
-static_assert(route_slots(kMaxRouteDim / kKC) >= 6, "ring too shallow for the widest embedding");
+static_assert(route_slots(kMaxRouteDim / kKC) >= 4, "ring too shallow for the widest embedding");
 
 struct RouteParams {
-    int B, N, d, n_chunks, n_tiles, slots, grid, seg_slots;
+    int B, N, n_boxes, n_tiles, slots, grid, seg_slots;
     long long items;              // m_tiles * n_tiles work items, split evenly over the grid
     const float* inv_norm_c;      // [N]
     float2* part;                 // [m_tiles, seg_slots, 128]: (max of dot * inv_norm_c, index as int bits)
@@ -92,17 +102,32 @@ __device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity) {
     return done != 0;
 }
 
-// Spins (no suspend) on the phase; about one second at most, then records
-// the timeout in the status word and returns false.
+// One lane of the (converged) warp.
+__device__ __forceinline__ bool route_elect() {
+    uint32_t r;
+    asm volatile(
+        "{\n\t.reg .pred P;\n\telect.sync _|P, 0xffffffff;\n\tselp.u32 %0, 1, 0, P;\n\t}\n"
+        : "=r"(r));
+    return r != 0;
+}
+
+// The whole warp spins (no suspend) on the phase; about one second at most,
+// then records the timeout in the status word.  The result is the same in
+// every lane, so that no lane leaves a loop while another still issues.
 __device__ __forceinline__ bool wait_bar(uint64_t* bar, uint32_t parity, int* status) {
-    if (mbar_test(bar, parity)) return true;
-    const uint64_t t0 = global_timer_ns();
-    for (uint32_t it = 0; it < (1u << 28); ++it) {
-        if (mbar_test(bar, parity)) return true;
-        if ((it & 1023u) == 1023u && global_timer_ns() - t0 > 1000000000ull) break;
+    if (__all_sync(0xffffffffu, mbar_test(bar, parity))) return true;
+    uint64_t t0 = 0;
+    bool done = false;
+    for (uint32_t it = 0; it < (1u << 28) && !done; ++it) {
+        done = mbar_test(bar, parity);
+        if ((it & 1023u) == 1023u) {
+            const uint64_t now = global_timer_ns();
+            if (t0 == 0) t0 = now;
+            else if (now - t0 > 1000000000ull) break;
+        }
     }
-    atomicOr(status, CS_DEVICE_WAIT_TIMEOUT);
-    return false;
+    if (!done) atomicOr(status, CS_DEVICE_WAIT_TIMEOUT);
+    return __all_sync(0xffffffffu, done);
 }
 
 __device__ __forceinline__ void umma_commit(uint64_t* bar) {
@@ -110,36 +135,54 @@ __device__ __forceinline__ void umma_commit(uint64_t* bar) {
                  : "memory");
 }
 
-__device__ __forceinline__ void epi_bar_sync() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
+// 32 columns of this warp's 32 rows.
+__device__ __forceinline__ void tmem_ld32(uint32_t (&r)[32], uint32_t addr) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
+        "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
+          "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
+          "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+        : "r"(addr));
+}
+
+// The epilogue warps of one column half (ids 1, 2), and all of them (id 3).
+__device__ __forceinline__ void epi_half_sync(int half) {
+    asm volatile("bar.sync %0, %1;" ::"r"(1 + half), "n"(kEpiWarps * 16) : "memory");
+}
+__device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 3, %0;" ::"n"(kEpiWarps * 32) : "memory"); }
 
 // Persistent: CTA c owns the work items [c*I/G, (c+1)*I/G) of the m-major
 // sequence (request tile m, group tile t).  The request tile stays resident
-// in shared memory while t advances and is reloaded when m changes.
+// in shared memory while t advances and is reloaded when m changes: its
+// boxes come with the first group tile's, each on that stage's barrier.
 __global__ void __launch_bounds__(kRThreads, 1)
 route_gemm_kernel(const __grid_constant__ CUtensorMap tmap_e, const __grid_constant__ CUtensorMap tmap_c,
                   const RouteParams p) {
-    extern __shared__ uint8_t smem_raw[];
-    __shared__ __align__(16) float s_inv[2 * kRN];
-    __shared__ uint32_t s_tmem;
-    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    extern __shared__ __align__(1024) uint8_t smem[];
     const int slots = p.slots;
-    uint8_t* sa = smem;                                   // [n_chunks][128 rows][128 B]
-    uint8_t* sb = smem + p.n_chunks * kChunkBytes;        // [slots][128 groups][128 B]
-    uint64_t* bars = reinterpret_cast<uint64_t*>(sb + slots * kChunkBytes);
-    uint64_t* a_full = bars;
-    uint64_t* a_free = bars + 1;
-    uint64_t* d_full = bars + 2;             // [2]
-    uint64_t* d_free = bars + 4;             // [2]
-    uint64_t* mma_done = bars + 6;
-    uint64_t* full = bars + 7;               // [slots]
+    uint8_t* sa = smem;                                   // [n_boxes][128 rows][128 B]
+    uint8_t* sb = smem + p.n_boxes * kBoxBytes;           // [slots][2 boxes][128 groups][128 B]
+    uint8_t* tail = sb + slots * kStageBoxes * kBoxBytes;
+    uint64_t* a_free = reinterpret_cast<uint64_t*>(tail);
+    uint64_t* d_full = a_free + 1;           // [2]
+    uint64_t* d_free = a_free + 3;           // [2]
+    uint64_t* mma_done = a_free + 5;
+    uint64_t* full = a_free + 6;             // [slots]
     uint64_t* empty = full + kMaxSlots;      // [slots]
+    float* s_inv = reinterpret_cast<float*>(tail + 256);                   // [2][128]
+    float2* s_half = reinterpret_cast<float2*>(tail + 256 + 2 * kRN * 4);   // [128]
+    uint32_t* s_tmem = reinterpret_cast<uint32_t*>(tail + 256 + 2 * kRN * 4 + kRM * 8);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const long long it0 = (long long)blockIdx.x * p.items / p.grid;
     const long long it1 = (long long)(blockIdx.x + 1) * p.items / p.grid;
     const int nt = (int)(it1 - it0);
+    int m = (int)(it0 / p.n_tiles), t = (int)(it0 - (long long)m * p.n_tiles);   // the current item
+    const int n_kc = (p.n_boxes + kStageBoxes - 1) / kStageBoxes;               // stages a tile
     if (warp == 2) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)),
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(s_tmem)),
                      "n"(kRTmemCols)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -147,11 +190,10 @@ route_gemm_kernel(const __grid_constant__ CUtensorMap tmap_e, const __grid_const
     if (threadIdx.x == 0) {
         tma_prefetch_desc(&tmap_e);
         tma_prefetch_desc(&tmap_c);
-        mbar_init(a_full, 1);
         mbar_init(a_free, 1);
         for (int i = 0; i < 2; ++i) {
             mbar_init(&d_full[i], 1);
-            mbar_init(&d_free[i], 4);
+            mbar_init(&d_free[i], kEpiWarps);
         }
         mbar_init(mma_done, 1);
         for (int i = 0; i < slots; ++i) {
@@ -163,172 +205,192 @@ route_gemm_kernel(const __grid_constant__ CUtensorMap tmap_e, const __grid_const
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const uint32_t tmem = s_tmem;
+    const uint32_t tmem = *s_tmem;
     wait_prior_grid();
     allow_dependent_launch();
 
-    if (warp == 0 && lane == 0) {
+    if (warp == 0) {
         // ---------------------------------------------------------- TMA
-        int s = 0, cur_m = -1;
+        const uint32_t a_base = smem_u32(sa), b_base = smem_u32(sb);
+        int s = 0;
         uint32_t use = 0, a_loads = 0;
-        bool ok = true;
-        for (long long it = it0; it < it1 && ok; ++it) {
-            const int m = (int)(it / p.n_tiles), t = (int)(it - (long long)m * p.n_tiles);
-            if (m != cur_m) {
-                if (a_loads > 0 && !wait_bar(a_free, (a_loads - 1) & 1, p.status)) break;
-                mbar_arrive_expect_tx(a_full, (uint32_t)(p.n_chunks * kChunkBytes));
-                for (int kc = 0; kc < p.n_chunks; ++kc)
-                    tma_load_2d(smem_u32(sa + kc * kChunkBytes), &tmap_e, a_full, kc * kKC, m * kRM);
-                ++a_loads;
-                cur_m = m;
-            }
-            for (int kc = 0; kc < p.n_chunks; ++kc) {
+        bool ok = true, new_m = true;
+        for (int tl = 0; tl < nt && ok; ++tl) {
+            if (new_m && a_loads > 0 && !wait_bar(a_free, (a_loads - 1) & 1, p.status)) break;
+            for (int kc = 0; kc < n_kc; ++kc) {
                 if (use > 0 && !wait_bar(&empty[s], (use - 1) & 1, p.status)) {
                     ok = false;
                     break;
                 }
-                mbar_arrive_expect_tx(&full[s], (uint32_t)kChunkBytes);
-                tma_load_2d(smem_u32(sb + s * kChunkBytes), &tmap_c, &full[s], kc * kKC, t * kRN);
+                if (route_elect()) {
+                    const int k0 = kc * kStageBoxes, nb = min(kStageBoxes, p.n_boxes - k0);
+                    mbar_arrive_expect_tx(&full[s], (uint32_t)(nb * kBoxBytes) << (new_m ? 1 : 0));
+                    for (int k = k0; k < k0 + nb; ++k) {
+                        if (new_m) tma_load_2d(a_base + k * kBoxBytes, &tmap_e, &full[s], k * kKC, m * kRM);
+                        tma_load_2d(b_base + (s * kStageBoxes + k - k0) * kBoxBytes, &tmap_c, &full[s], k * kKC,
+                                    t * kRN);
+                    }
+                }
+                __syncwarp();
                 if (++s == slots) {
                     s = 0;
                     ++use;
                 }
             }
+            a_loads += new_m ? 1 : 0;
+            new_m = ++t == p.n_tiles;
+            if (new_m) {
+                t = 0;
+                ++m;
+            }
         }
-        // no copy in flight at exit: the last fill of every slot and the last
-        // request tile have landed
-        const long long total = (long long)nt * p.n_chunks;
+        // no copy in flight at exit: the last fill of every slot has landed
+        const long long total = (long long)nt * n_kc;
         for (long long f = total > slots ? total - slots : 0; f < total; ++f)
             if (!mbar_wait_bounded(&full[f % slots], (uint32_t)(f / slots) & 1))
                 atomicOr(p.status, CS_DEVICE_WAIT_TIMEOUT);
-        if (a_loads > 0 && !mbar_wait_bounded(a_full, (a_loads - 1) & 1)) atomicOr(p.status, CS_DEVICE_WAIT_TIMEOUT);
-    } else if (warp == 1 && lane == 0) {
+    } else if (warp == 1) {
         // ---------------------------------------------------------- MMA
-        int s = 0, cur_m = -1;
-        uint32_t use = 0, a_loads = 0;
+        const uint64_t da0 = sw128_desc(smem_u32(sa)), db0 = sw128_desc(smem_u32(sb));
+        int s = 0;
+        uint32_t use = 0;
         bool ok = true;
         for (int tl = 0; tl < nt && ok; ++tl) {
-            const int m = (int)((it0 + tl) / p.n_tiles);
-            if (m != cur_m) {
-                if (a_loads > 0) umma_commit(a_free);   // the previous request tile may be overwritten
-                if (!wait_bar(a_full, a_loads & 1, p.status)) break;
-                ++a_loads;
-                cur_m = m;
-            }
             const int db = tl & 1;
             if (tl >= 2 && !wait_bar(&d_free[db], (uint32_t)((tl >> 1) - 1) & 1, p.status)) break;
-            for (int kc = 0; kc < p.n_chunks; ++kc) {
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const uint32_t td = tmem + db * kRN;
+            const bool last_of_m = ++t == p.n_tiles;
+            if (last_of_m) t = 0;
+            for (int kc = 0; kc < n_kc; ++kc) {
                 if (!wait_bar(&full[s], use & 1, p.status)) {
                     ok = false;
                     break;
                 }
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint32_t a0 = smem_u32(sa + kc * kChunkBytes), b0 = smem_u32(sb + s * kChunkBytes);
+                // descriptors advance by whole boxes and 32-byte steps (addresses
+                // stay below 256 KB: the 14-bit start field cannot carry)
+                const uint64_t da = da0 + (uint64_t)((kc * kStageBoxes * kBoxBytes) >> 4);
+                const uint64_t dbs = db0 + (uint64_t)((s * kStageBoxes * kBoxBytes) >> 4);
+                const int nb = p.n_boxes - kc * kStageBoxes;
+                if (route_elect()) {
 #pragma unroll
-                for (int ks = 0; ks < kKC / 16; ++ks) {
-                    const uint32_t acc = (kc > 0 || ks > 0) ? 1u : 0u;
-                    asm volatile(
-                        "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %4, 0;\n\t"
-                        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, q;\n\t}\n" ::"r"(tmem + db * kRN),
-                        "l"(sw128_desc(a0 + ks * 32)), "l"(sw128_desc(b0 + ks * 32)), "r"(route_idesc()), "r"(acc)
-                        : "memory");
+                    for (int k = 0; k < kStageBoxes; ++k) {
+                        if (k >= nb) break;
+#pragma unroll
+                        for (int ks = 0; ks < kKC / 16; ++ks) {
+                            const uint32_t acc = (kc > 0 || k > 0 || ks > 0) ? 1u : 0u;
+                            const uint64_t off = (uint64_t)((k * kBoxBytes) >> 4) + ks * 2;
+                            asm volatile(
+                                "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %4, 0;\n\t"
+                                "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, q;\n\t}\n" ::"r"(td),
+                                "l"(da + off), "l"(dbs + off), "r"(route_idesc()), "r"(acc)
+                                : "memory");
+                        }
+                    }
+                    umma_commit(&empty[s]);
+                    if (kc == n_kc - 1) {
+                        umma_commit(&d_full[db]);
+                        if (last_of_m) umma_commit(a_free);   // the request tile may be overwritten
+                    }
                 }
-                umma_commit(&empty[s]);
+                __syncwarp();
                 if (++s == slots) {
                     s = 0;
                     ++use;
                 }
             }
-            if (ok) umma_commit(&d_full[db]);
         }
-        umma_commit(mma_done);
+        if (route_elect()) umma_commit(mma_done);
+        __syncwarp();
         if (!mbar_wait_bounded(mma_done, 0)) atomicOr(p.status, CS_DEVICE_WAIT_TIMEOUT);
     } else if (warp >= 4) {
         // ------------------------------------------------------ epilogue
-        const int sub = warp & 3;
+        const int sub = warp & 3, half = (warp - 4) >> 2;
         const int row = sub * 32 + lane;
-        const uint32_t t_lane = tmem + ((uint32_t)(sub * 32) << 16);
+        const uint32_t t_lane = tmem + ((uint32_t)(sub * 32) << 16) + half * (kRN / 2);
         const float kNaN = __int_as_float(0x7fffffff);   // excluded by fmaxf and by ==
-        auto inv_of = [&](long long it) {
-            const int t = (int)(it % p.n_tiles);
-            const int j = t * kRN + row;
-            return j < p.N ? __ldg(p.inv_norm_c + j) : kNaN;
+        // this thread's share of the half's 64 inverse norms (warps 0 and 1 of it)
+        const int col = half * (kRN / 2) + row;
+        const bool loads = row < kRN / 2;
+        auto inv_of = [&](int tile) {
+            const int j = tile * kRN + col;
+            return loads && j < p.N ? __ldg(p.inv_norm_c + j) : kNaN;
         };
-        auto flush = [&](int m, float best, int idx) {
+        float best = kNegInf;
+        int idx = -1;
+        auto flush = [&]() {
+            if (half == 1) s_half[row] = make_float2(best, __int_as_float(idx));
+            epi_sync();
             const int b = m * kRM + row;
-            if (b < p.B) {
+            if (half == 0 && b < p.B) {
+                const float2 o = s_half[row];
+                const int oi = __float_as_int(o.y);
+                if (oi >= 0 && (idx < 0 || o.x > best || (o.x == best && oi < idx))) {
+                    best = o.x;
+                    idx = oi;
+                }
                 const int slot = blockIdx.x - route_owner((long long)m * p.n_tiles, p.items, p.grid);
                 p.part[((size_t)m * p.seg_slots + slot) * kRM + row] = make_float2(best, __int_as_float(idx));
             }
+            epi_sync();
         };
-        float inv_next = nt > 0 ? inv_of(it0) : 0.f;
-        float best = kNegInf;
-        int idx = -1, cur_m = nt > 0 ? (int)(it0 / p.n_tiles) : -1;
+        float inv_next = nt > 0 ? inv_of(t) : 0.f;
         bool dead = false;
         for (int tl = 0; tl < nt; ++tl) {
-            const long long it = it0 + tl;
-            const int m = (int)(it / p.n_tiles), t = (int)(it - (long long)m * p.n_tiles);
-            if (m != cur_m) {
-                flush(cur_m, best, idx);
+            const int db = tl & 1;
+            float* inv = s_inv + db * kRN;
+            if (loads) inv[col] = inv_next;
+            epi_half_sync(half);
+            const int tile = t;
+            const bool last_of_m = ++t == p.n_tiles;
+            if (last_of_m) t = 0;
+            if (tl + 1 < nt) inv_next = inv_of(t);
+            // after a timed-out wait the warp keeps taking part in the named
+            // barriers but skips the rest
+            if (!dead && !wait_bar(&d_full[db], (uint32_t)(tl >> 1) & 1, p.status)) dead = true;
+            if (!dead) {
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                uint32_t r[2][32];
+                tmem_ld32(r[0], t_lane + db * kRN);
+                tmem_ld32(r[1], t_lane + db * kRN + 32);
+                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&d_free[db]);
+#pragma unroll
+                for (int c = 0; c < 2; ++c) {
+                    const float4* sv = reinterpret_cast<const float4*>(inv + half * (kRN / 2) + c * 32);
+                    float sc[32];
+                    float mx = kNegInf;
+#pragma unroll
+                    for (int q4 = 0; q4 < 8; ++q4) {
+                        const float4 v = sv[q4];
+                        sc[4 * q4 + 0] = __uint_as_float(r[c][4 * q4 + 0]) * v.x;
+                        sc[4 * q4 + 1] = __uint_as_float(r[c][4 * q4 + 1]) * v.y;
+                        sc[4 * q4 + 2] = __uint_as_float(r[c][4 * q4 + 2]) * v.z;
+                        sc[4 * q4 + 3] = __uint_as_float(r[c][4 * q4 + 3]) * v.w;
+                        mx = fmaxf(mx, fmaxf(fmaxf(sc[4 * q4], sc[4 * q4 + 1]), fmaxf(sc[4 * q4 + 2], sc[4 * q4 + 3])));
+                    }
+                    // ascending group ids and a strict > across chunks keep the
+                    // lowest id of the maximum; inside the chunk, its first hit
+                    if (mx > best) {
+                        int e0 = 31;
+#pragma unroll
+                        for (int e = 31; e >= 0; --e)
+                            if (sc[e] == mx) e0 = e;
+                        best = mx;
+                        idx = tile * kRN + half * (kRN / 2) + c * 32 + e0;
+                    }
+                }
+            }
+            if (last_of_m || tl == nt - 1) {
+                flush();
                 best = kNegInf;
                 idx = -1;
-                cur_m = m;
+                ++m;
             }
-            const int db = tl & 1;
-            s_inv[db * kRN + row] = inv_next;
-            epi_bar_sync();
-            if (tl + 1 < nt) inv_next = inv_of(it + 1);
-            // after a timed-out wait the warp keeps taking part in the named
-            // barrier (every epilogue warp passes it nt times) but skips the rest
-            int ok = 0;
-            if (lane == 0 && !dead) ok = wait_bar(&d_full[db], (uint32_t)(tl >> 1) & 1, p.status) ? 1 : 0;
-            ok = __shfl_sync(0xffffffffu, ok, 0);
-            if (!ok) {
-                dead = true;
-                continue;
-            }
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-#pragma unroll 1
-            for (int c0 = 0; c0 < kRN; c0 += 32) {
-                uint32_t r[32];
-                asm volatile(
-                    "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-                    "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-                    : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-                      "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
-                      "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]),
-                      "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]),
-                      "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-                    : "r"(t_lane + db * kRN + c0));
-                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                const float4* sv = reinterpret_cast<const float4*>(s_inv + db * kRN + c0);
-                float sc[32];
-                float mx = kNegInf;
-#pragma unroll
-                for (int q4 = 0; q4 < 8; ++q4) {
-                    const float4 v = sv[q4];
-                    sc[4 * q4 + 0] = __uint_as_float(r[4 * q4 + 0]) * v.x;
-                    sc[4 * q4 + 1] = __uint_as_float(r[4 * q4 + 1]) * v.y;
-                    sc[4 * q4 + 2] = __uint_as_float(r[4 * q4 + 2]) * v.z;
-                    sc[4 * q4 + 3] = __uint_as_float(r[4 * q4 + 3]) * v.w;
-                    mx = fmaxf(mx, fmaxf(fmaxf(sc[4 * q4], sc[4 * q4 + 1]), fmaxf(sc[4 * q4 + 2], sc[4 * q4 + 3])));
-                }
-                // ascending group ids and a strict > across chunks keep the
-                // lowest id of the maximum; inside the chunk, its first hit
-                if (mx > best) {
-                    int e0 = 31;
-#pragma unroll
-                    for (int e = 31; e >= 0; --e)
-                        if (sc[e] == mx) e0 = e;
-                    best = mx;
-                    idx = t * kRN + c0 + e0;
-                }
-            }
-            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&d_free[db]);
         }
-        if (cur_m >= 0) flush(cur_m, best, idx);
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
@@ -345,14 +407,24 @@ __global__ void __launch_bounds__(256) route_merge_kernel(const __nv_bfloat16* e
                                                            float tau, int32_t* out_group, int32_t* out_best,
                                                            float* out_score) {
     const int b = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    // the embeddings were complete before any CTA of the GEMM kernel let this
+    // one start; without groups there is no such kernel in between
+    if (n_tiles == 0) wait_prior_grid();
+    float ss = 0.f;
+    if (b < B) {
+        __nv_bfloat16 e[kMaxRouteDim / 32];
+#pragma unroll
+        for (int j = 0; j < kMaxRouteDim / 32; ++j)
+            e[j] = lane + 32 * j < d ? emb[(size_t)b * d + lane + 32 * j] : __float2bfloat16(0.f);
+#pragma unroll
+        for (int j = 0; j < kMaxRouteDim / 32; ++j) {
+            const float x = __bfloat162float(e[j]);
+            ss = fmaf(x, x, ss);
+        }
+    }
     wait_prior_grid();
     allow_dependent_launch();
     if (b >= B) return;
-    float ss = 0.f;
-    for (int k = lane; k < d; k += 32) {
-        const float e = __bfloat162float(emb[(size_t)b * d + k]);
-        ss = fmaf(e, e, ss);
-    }
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, off);
     float best = kNegInf;
@@ -457,8 +529,8 @@ cs_status launch_route(const cs_route_dims& d, const RoutePlan& pl, const void* 
         if (st != CS_OK) return st;
         st = encode_rows_map(&tc, centroids, d.n_groups, d.dim);
         if (st != CS_OK) return st;
-        const int n_chunks = d.dim / kKC;
-        const int smem = route_smem_bytes(n_chunks);
+        const int n_boxes = d.dim / kKC;
+        const int smem = route_smem_bytes(n_boxes);
         static int attr_smem[64] = {};
         int dev = 0;
         cudaGetDevice(&dev);
@@ -470,10 +542,9 @@ cs_status launch_route(const cs_route_dims& d, const RoutePlan& pl, const void* 
         RouteParams p{};
         p.B = d.batch;
         p.N = d.n_groups;
-        p.d = d.dim;
-        p.n_chunks = n_chunks;
+        p.n_boxes = n_boxes;
         p.n_tiles = pl.n_tiles;
-        p.slots = route_slots(n_chunks);
+        p.slots = route_slots(n_boxes);
         p.grid = pl.grid;
         p.seg_slots = pl.seg_slots;
         p.items = pl.items;
