@@ -7,9 +7,10 @@
 // The scores are one GEMM, E C^T, with the arg max fused into its epilogue
 // (the B x N score matrix never reaches memory):
 //   route_gemm_kernel: a CTA owns 128 requests (MMA M) and a contiguous range
-//     of 128-group tiles.  Warp 0 loads the CTA's embedding rows once (one TMA
-//     box per 64 dims, 128-byte swizzle, kept in shared memory) and streams
-//     the centroids through a TMA ring, 128 dims a stage; warp 1 issues
+//     of 128-group tiles.  Warp 0 streams the CTA's embedding rows, once, and
+//     the centroids through a TMA ring, 128 dims a stage (a box per 64 dims,
+//     128-byte swizzle); warp 1 copies the embedding rows to tensor memory as
+//     they land (up to 192 columns), where every MMA reads them, and issues
 //     tcgen05.mma (M = 128, N = 128, K = 16 per instruction, fp32 accumulators
 //     in tensor memory, two buffers); warps 4-11 take one row and half a
 //     tile's columns each per thread, scale each dot product by the
@@ -21,8 +22,8 @@
 //     beside 31 parked at the block barrier took 450 cycles for each 64 dims
 //     without its MMAs (a tile 4140 cycles; loads or none made no
 //     difference).  1024 requests, 16384 groups, 384 dims, both kernels in a
-//     captured graph: 23.8 us so, 17.7 as it is; a further 1024 requests 14.6
-//     and 9.5.
+//     captured graph: 23.8 us so, 17.1 as it is; a further 1024 requests 14.6
+//     and 8.2.
 //   route_merge_kernel: one warp per request folds the CTAs' partials (score
 //     first, then lower index), applies the request's own inverse norm and
 //     the threshold.
@@ -41,25 +42,19 @@ constexpr int kRN = 128;                  // groups per tile (MMA N)
 constexpr int kKC = 64;                   // dims per box: one 128-byte swizzle row
 constexpr int kBoxBytes = kRM * 128;      // 128 rows x 64 dims x 2 B
 constexpr int kStageBoxes = 2;            // boxes of 128 groups a ring stage holds
-constexpr int kMaxSlots = 6;              // ring stages, at most
+constexpr int kStageBytes = kStageBoxes * kBoxBytes;
+constexpr int kSlots = 7;                 // ring stages
 constexpr int kEpiWarps = 8;              // two to a quarter of the rows, 64 columns of a tile each
 constexpr int kRThreads = 128 + kEpiWarps * 32;   // warp 0 TMA, warp 1 MMA, warp 2 TMEM, warps 4-11 epilogue
-constexpr int kRTmemCols = 2 * kRN;
-constexpr int kRSmemLimit = 232448;       // opt-in shared memory per block on sm_103a
+constexpr int kRACol = 2 * kRN;           // tensor memory: two accumulators, then the request tile
+constexpr int kRTmemCols = 512;
 constexpr int kRTailBytes = 256 /*barriers*/ + 2 * kRN * 4 /*inverse norms*/ + kRM * 8 /*column halves*/ + 16;
-
-__host__ __device__ constexpr int route_slots(int n_boxes) {
-    return (kRSmemLimit - kRTailBytes - n_boxes * kBoxBytes) / (kStageBoxes * kBoxBytes) < kMaxSlots
-               ? (kRSmemLimit - kRTailBytes - n_boxes * kBoxBytes) / (kStageBoxes * kBoxBytes)
-               : kMaxSlots;
-}
-__host__ __device__ constexpr int route_smem_bytes(int n_boxes) {
-    return (n_boxes + route_slots(n_boxes) * kStageBoxes) * kBoxBytes + kRTailBytes;
-}
-static_assert(route_slots(kMaxRouteDim / kKC) >= 4, "ring too shallow for the widest embedding");
+constexpr int kRSmemBytes = kSlots * kStageBytes + kRTailBytes;
+static_assert(kRSmemBytes <= 232448, "shared memory per block on sm_103a");
+static_assert(kRACol + kMaxRouteDim / 2 <= kRTmemCols, "tensor memory");
 
 struct RouteParams {
-    int B, N, n_boxes, n_tiles, slots, grid, seg_slots;
+    int B, N, n_boxes, n_tiles, grid, seg_slots;
     long long items;              // m_tiles * n_tiles work items, split evenly over the grid
     const float* inv_norm_c;      // [N]
     float2* part;                 // [m_tiles, seg_slots, 128]: (max of dot * inv_norm_c, index as int bits)
@@ -102,13 +97,12 @@ __device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity) {
     return done != 0;
 }
 
-// One lane of the (converged) warp.
-__device__ __forceinline__ bool route_elect() {
-    uint32_t r;
+__device__ __forceinline__ void tc_mma_ss(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
     asm volatile(
-        "{\n\t.reg .pred P;\n\telect.sync _|P, 0xffffffff;\n\tselp.u32 %0, 1, 0, P;\n\t}\n"
-        : "=r"(r));
-    return r != 0;
+        "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, q;\n\t}\n" ::"r"(d),
+        "l"(a), "l"(b), "r"(idesc), "r"(acc)
+        : "memory");
 }
 
 // The whole warp spins (no suspend) on the phase; about one second at most,
@@ -128,11 +122,6 @@ __device__ __forceinline__ bool wait_bar(uint64_t* bar, uint32_t parity, int* st
     }
     if (!done) atomicOr(status, CS_DEVICE_WAIT_TIMEOUT);
     return __all_sync(0xffffffffu, done);
-}
-
-__device__ __forceinline__ void umma_commit(uint64_t* bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
-                 : "memory");
 }
 
 // 32 columns of this warp's 32 rows.
@@ -155,22 +144,23 @@ __device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 3, %0;" ::"n
 
 // Persistent: CTA c owns the work items [c*I/G, (c+1)*I/G) of the m-major
 // sequence (request tile m, group tile t).  The request tile stays resident
-// in shared memory while t advances and is reloaded when m changes: its
-// boxes come with the first group tile's, each on that stage's barrier.
+// in tensor memory while t advances and is reloaded when m changes: a stage
+// of its dims comes before each stage of the first group tile's.  (Read from
+// shared memory, an MMA of 128 x 128 x 16 moves 8 KB of operands in the 64
+// cycles it takes, all that shared memory has: 46.1 us for 4096 requests and
+// 16384 groups of 384 dims, 41.7 from tensor memory; 1024 requests 17.8 and
+// 17.1.  The stream of centroids is the next bound: 98 KB a tile, 1.2 us.)
 __global__ void __launch_bounds__(kRThreads, 1)
 route_gemm_kernel(const __grid_constant__ CUtensorMap tmap_e, const __grid_constant__ CUtensorMap tmap_c,
                   const RouteParams p) {
     extern __shared__ __align__(1024) uint8_t smem[];
-    const int slots = p.slots;
-    uint8_t* sa = smem;                                   // [n_boxes][128 rows][128 B]
-    uint8_t* sb = smem + p.n_boxes * kBoxBytes;           // [slots][2 boxes][128 groups][128 B]
-    uint8_t* tail = sb + slots * kStageBoxes * kBoxBytes;
+    uint8_t* tail = smem + kSlots * kStageBytes;          // after the ring: [kSlots][2 boxes][128 rows][128 B]
     uint64_t* a_free = reinterpret_cast<uint64_t*>(tail);
     uint64_t* d_full = a_free + 1;           // [2]
     uint64_t* d_free = a_free + 3;           // [2]
     uint64_t* mma_done = a_free + 5;
-    uint64_t* full = a_free + 6;             // [slots]
-    uint64_t* empty = full + kMaxSlots;      // [slots]
+    uint64_t* full = a_free + 6;             // [kSlots]
+    uint64_t* empty = full + kSlots;         // [kSlots]
     float* s_inv = reinterpret_cast<float*>(tail + 256);                   // [2][128]
     float2* s_half = reinterpret_cast<float2*>(tail + 256 + 2 * kRN * 4);   // [128]
     uint32_t* s_tmem = reinterpret_cast<uint32_t*>(tail + 256 + 2 * kRN * 4 + kRM * 8);
@@ -196,7 +186,7 @@ route_gemm_kernel(const __grid_constant__ CUtensorMap tmap_e, const __grid_const
             mbar_init(&d_free[i], kEpiWarps);
         }
         mbar_init(mma_done, 1);
-        for (int i = 0; i < slots; ++i) {
+        for (int i = 0; i < kSlots; ++i) {
             mbar_init(&full[i], 1);
             mbar_init(&empty[i], 1);
         }
@@ -211,33 +201,32 @@ route_gemm_kernel(const __grid_constant__ CUtensorMap tmap_e, const __grid_const
 
     if (warp == 0) {
         // ---------------------------------------------------------- TMA
-        const uint32_t a_base = smem_u32(sa), b_base = smem_u32(sb);
+        const uint32_t base = smem_u32(smem);
         int s = 0;
-        uint32_t use = 0, a_loads = 0;
+        uint32_t use = 0;
+        long long fills = 0;
         bool ok = true, new_m = true;
-        for (int tl = 0; tl < nt && ok; ++tl) {
-            if (new_m && a_loads > 0 && !wait_bar(a_free, (a_loads - 1) & 1, p.status)) break;
-            for (int kc = 0; kc < n_kc; ++kc) {
-                if (use > 0 && !wait_bar(&empty[s], (use - 1) & 1, p.status)) {
-                    ok = false;
-                    break;
-                }
-                if (route_elect()) {
-                    const int k0 = kc * kStageBoxes, nb = min(kStageBoxes, p.n_boxes - k0);
-                    mbar_arrive_expect_tx(&full[s], (uint32_t)(nb * kBoxBytes) << (new_m ? 1 : 0));
-                    for (int k = k0; k < k0 + nb; ++k) {
-                        if (new_m) tma_load_2d(a_base + k * kBoxBytes, &tmap_e, &full[s], k * kKC, m * kRM);
-                        tma_load_2d(b_base + (s * kStageBoxes + k - k0) * kBoxBytes, &tmap_c, &full[s], k * kKC,
-                                    t * kRN);
-                    }
-                }
-                __syncwarp();
-                if (++s == slots) {
-                    s = 0;
-                    ++use;
-                }
+        auto load = [&](const CUtensorMap* map, int kc, int row0) {
+            if (use > 0 && !wait_bar(&empty[s], (use - 1) & 1, p.status)) return false;
+            if (elect_one()) {
+                const int k0 = kc * kStageBoxes, nb = min(kStageBoxes, p.n_boxes - k0);
+                mbar_arrive_expect_tx(&full[s], (uint32_t)(nb * kBoxBytes));
+                for (int k = 0; k < nb; ++k)
+                    tma_load_2d(base + s * kStageBytes + k * kBoxBytes, map, &full[s], (k0 + k) * kKC, row0);
             }
-            a_loads += new_m ? 1 : 0;
+            __syncwarp();
+            ++fills;
+            if (++s == kSlots) {
+                s = 0;
+                ++use;
+            }
+            return true;
+        };
+        for (int tl = 0; tl < nt && ok; ++tl) {
+            for (int kc = 0; kc < n_kc && ok; ++kc) {
+                if (new_m) ok = load(&tmap_e, kc, m * kRM);
+                ok = ok && load(&tmap_c, kc, t * kRN);
+            }
             new_m = ++t == p.n_tiles;
             if (new_m) {
                 t = 0;
@@ -245,63 +234,96 @@ route_gemm_kernel(const __grid_constant__ CUtensorMap tmap_e, const __grid_const
             }
         }
         // no copy in flight at exit: the last fill of every slot has landed
-        const long long total = (long long)nt * n_kc;
-        for (long long f = total > slots ? total - slots : 0; f < total; ++f)
-            if (!mbar_wait_bounded(&full[f % slots], (uint32_t)(f / slots) & 1))
+        for (long long f = fills > kSlots ? fills - kSlots : 0; f < fills; ++f)
+            if (!mbar_wait_bounded(&full[f % kSlots], (uint32_t)(f / kSlots) & 1))
                 atomicOr(p.status, CS_DEVICE_WAIT_TIMEOUT);
     } else if (warp == 1) {
         // ---------------------------------------------------------- MMA
-        const uint64_t da0 = sw128_desc(smem_u32(sa)), db0 = sw128_desc(smem_u32(sb));
+        const uint64_t d0 = sw128_desc(smem_u32(smem));
+        const uint32_t ta = tmem + kRACol;
         int s = 0;
-        uint32_t use = 0;
-        bool ok = true;
+        uint32_t use = 0, a_loads = 0;
+        bool ok = true, new_m = true;
+        auto advance = [&] {
+            if (++s == kSlots) {
+                s = 0;
+                ++use;
+            }
+        };
         for (int tl = 0; tl < nt && ok; ++tl) {
             const int db = tl & 1;
             if (tl >= 2 && !wait_bar(&d_free[db], (uint32_t)((tl >> 1) - 1) & 1, p.status)) break;
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            // the MMAs of the previous request tile are done with its rows
+            if (new_m && a_loads > 0 && !wait_bar(a_free, (a_loads - 1) & 1, p.status)) break;
             const uint32_t td = tmem + db * kRN;
             const bool last_of_m = ++t == p.n_tiles;
             if (last_of_m) t = 0;
-            for (int kc = 0; kc < n_kc; ++kc) {
-                if (!wait_bar(&full[s], use & 1, p.status)) {
-                    ok = false;
-                    break;
-                }
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                // descriptors advance by whole boxes and 32-byte steps (addresses
-                // stay below 256 KB: the 14-bit start field cannot carry)
-                const uint64_t da = da0 + (uint64_t)((kc * kStageBoxes * kBoxBytes) >> 4);
-                const uint64_t dbs = db0 + (uint64_t)((s * kStageBoxes * kBoxBytes) >> 4);
-                const int nb = p.n_boxes - kc * kStageBoxes;
-                if (route_elect()) {
-#pragma unroll
-                    for (int k = 0; k < kStageBoxes; ++k) {
-                        if (k >= nb) break;
-#pragma unroll
-                        for (int ks = 0; ks < kKC / 16; ++ks) {
-                            const uint32_t acc = (kc > 0 || k > 0 || ks > 0) ? 1u : 0u;
-                            const uint64_t off = (uint64_t)((k * kBoxBytes) >> 4) + ks * 2;
-                            asm volatile(
-                                "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %4, 0;\n\t"
-                                "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, q;\n\t}\n" ::"r"(td),
-                                "l"(da + off), "l"(dbs + off), "r"(route_idesc()), "r"(acc)
-                                : "memory");
+            if (new_m) {
+                // the request tile's first group tile reads its rows from the
+                // ring and leaves them in tensor memory for the next ones
+                for (int kc = 0; kc < n_kc; ++kc) {
+                    const int nb = p.n_boxes - kc * kStageBoxes;   // boxes left; a stage holds two at most
+                    const int sa = s;
+                    if (!(ok = wait_bar(&full[s], use & 1, p.status))) break;
+                    advance();
+                    if (!(ok = wait_bar(&full[s], use & 1, p.status))) break;
+                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                    if (elect_one()) {
+                        const uint64_t da = d0 + (uint64_t)((sa * kStageBytes) >> 4);
+                        const uint64_t ds = d0 + (uint64_t)((s * kStageBytes) >> 4);
+                        const uint32_t tk = ta + kc * kStageBoxes * (kKC / 2);
+                        const int steps = min(nb, kStageBoxes) * (kKC / 16);
+#pragma unroll 1
+                        for (int i = 0; i < steps; ++i) {
+                            const uint64_t off = (uint64_t)(((i >> 2) * kBoxBytes) >> 4) + (i & 3) * 2;
+                            tc_mma_ss(td, da + off, ds + off, route_idesc(), (kc > 0 || i > 0) ? 1u : 0u);
                         }
+                        if (tl + 1 < nt) {
+#pragma unroll 1
+                            for (int i = 0; i < steps; ++i)
+                                tc_cp_128x256b(tk + i * 8, da + (uint64_t)(((i >> 2) * kBoxBytes) >> 4) + (i & 3) * 2);
+                        }
+                        tc_commit(&empty[sa]);
+                        tc_commit(&empty[s]);
                     }
-                    umma_commit(&empty[s]);
-                    if (kc == n_kc - 1) {
-                        umma_commit(&d_full[db]);
-                        if (last_of_m) umma_commit(a_free);   // the request tile may be overwritten
-                    }
+                    __syncwarp();
+                    advance();
                 }
-                __syncwarp();
-                if (++s == slots) {
-                    s = 0;
-                    ++use;
+            } else {
+                for (int kc = 0; kc < n_kc; ++kc) {
+                    const int nb = p.n_boxes - kc * kStageBoxes;
+                    if (!(ok = wait_bar(&full[s], use & 1, p.status))) break;
+                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                    if (elect_one()) {
+                        // descriptors advance by whole boxes and 32-byte steps (addresses
+                        // stay below 256 KB: the 14-bit start field cannot carry)
+                        const uint64_t ds = d0 + (uint64_t)((s * kStageBytes) >> 4);
+                        const uint32_t tk = ta + kc * kStageBoxes * (kKC / 2);
+#pragma unroll
+                        for (int k = 0; k < kStageBoxes; ++k) {
+                            if (k >= nb) break;
+#pragma unroll
+                            for (int ks = 0; ks < kKC / 16; ++ks)
+                                tc_mma_ts(td, tk + k * (kKC / 2) + ks * 8,
+                                          ds + (uint64_t)((k * kBoxBytes) >> 4) + ks * 2, route_idesc(),
+                                          (kc > 0 || k > 0 || ks > 0) ? 1u : 0u);
+                        }
+                        tc_commit(&empty[s]);
+                    }
+                    __syncwarp();
+                    advance();
                 }
             }
+            if (!ok) break;
+            if (elect_one()) {
+                tc_commit(&d_full[db]);
+                if (last_of_m) tc_commit(a_free);
+            }
+            __syncwarp();
+            a_loads += new_m ? 1 : 0;
+            new_m = last_of_m;
         }
-        if (route_elect()) umma_commit(mma_done);
+        if (elect_one()) tc_commit(mma_done);
         __syncwarp();
         if (!mbar_wait_bounded(mma_done, 0)) atomicOr(p.status, CS_DEVICE_WAIT_TIMEOUT);
     } else if (warp >= 4) {
@@ -348,7 +370,11 @@ route_gemm_kernel(const __grid_constant__ CUtensorMap tmap_e, const __grid_const
             if (tl + 1 < nt) inv_next = inv_of(t);
             // after a timed-out wait the warp keeps taking part in the named
             // barriers but skips the rest
-            if (!dead && !wait_bar(&d_full[db], (uint32_t)(tl >> 1) & 1, p.status)) dead = true;
+            // (a suspended wait: sixteen polling warps cost the issuing warps 10%)
+            if (!dead && !__all_sync(0xffffffffu, mbar_wait_bounded(&d_full[db], (uint32_t)(tl >> 1) & 1))) {
+                atomicOr(p.status, CS_DEVICE_WAIT_TIMEOUT);
+                dead = true;
+            }
             if (!dead) {
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 uint32_t r[2][32];
@@ -529,29 +555,26 @@ cs_status launch_route(const cs_route_dims& d, const RoutePlan& pl, const void* 
         if (st != CS_OK) return st;
         st = encode_rows_map(&tc, centroids, d.n_groups, d.dim);
         if (st != CS_OK) return st;
-        const int n_boxes = d.dim / kKC;
-        const int smem = route_smem_bytes(n_boxes);
-        static int attr_smem[64] = {};
+        static bool attr_set[64] = {};
         int dev = 0;
         cudaGetDevice(&dev);
-        if (dev < 0 || dev >= 64 || attr_smem[dev] < smem) {
-            e = cudaFuncSetAttribute(route_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (dev < 0 || dev >= 64 || !attr_set[dev]) {
+            e = cudaFuncSetAttribute(route_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kRSmemBytes);
             if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(route_gemm_kernel)");
-            if (dev >= 0 && dev < 64) attr_smem[dev] = smem;
+            if (dev >= 0 && dev < 64) attr_set[dev] = true;
         }
         RouteParams p{};
         p.B = d.batch;
         p.N = d.n_groups;
-        p.n_boxes = n_boxes;
+        p.n_boxes = d.dim / kKC;
         p.n_tiles = pl.n_tiles;
-        p.slots = route_slots(n_boxes);
         p.grid = pl.grid;
         p.seg_slots = pl.seg_slots;
         p.items = pl.items;
         p.inv_norm_c = inv_norms;
         p.status = reinterpret_cast<int*>(ws);
         p.part = reinterpret_cast<float2*>(ws + 256);
-        e = launch_dependent(route_gemm_kernel, dim3(pl.grid), dim3(kRThreads), smem, stream, te, tc, p);
+        e = launch_dependent(route_gemm_kernel, dim3(pl.grid), dim3(kRThreads), kRSmemBytes, stream, te, tc, p);
         if (e != cudaSuccess) return cuda_fail(e, "route_gemm_kernel launch");
     }
     e = launch_dependent(route_merge_kernel, dim3((d.batch + 7) / 8), dim3(256), 0, stream,

@@ -131,3 +131,13 @@ def test_device_status_is_clear_after_a_call():
     ws = torch.zeros(binding.load_library().cs_route_workspace_bytes(dims), dtype=torch.uint8, device=DEV)
     binding.cs_route(e, c, inv, 0.85, workspace=ws)
     assert binding.cs_read_device_status(ws) == 0
+
+
+@pytest.mark.parametrize("B,N,d", [(700, 5000, 320), (4100, 700, 64), (2900, 1000, 384)])
+def test_blocks_that_change_request_tile(B, N, d):
+    """More tile pairs than blocks: a block's range crosses from one request
+    tile to the next (once or several times), with one to three ring stages a
+    tile and a half-filled last one."""
+    g = torch.Generator().manual_seed(B)
+    emb, cent = torch.randn(B, d, generator=g), torch.randn(N, d, generator=g)
+    check(emb.to(torch.bfloat16), cent.to(torch.bfloat16), 0.2)
