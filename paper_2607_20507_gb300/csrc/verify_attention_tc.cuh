@@ -672,14 +672,18 @@ verify_attention_tc_kernel(const __grid_constant__ CUtensorMap tmap_k, const __g
 #pragma unroll
                 for (int e = 0; e < 32; ++e) s[e] = kNegInf;
             } else if (kTree) {
+                // a tile wholly before node 0 is wholly visible (64
+                // requests, 44 rows: 135.9 us with the mask on every tile, 133.4)
                 const int d = ts - tree_base;
-                const uint64_t pre = d >= 0 ? 0ull : (d <= -64 ? ~0ull : (1ull << -d) - 1ull);
-                const uint64_t live = span_L - ts >= 64 ? ~0ull : (1ull << max(span_L - ts, 0)) - 1ull;
-                const uint64_t tr = d >= 64 ? 0ull : (d >= 0 ? anc >> d : (d <= -64 ? 0ull : anc << -d));
-                const uint32_t vis = (uint32_t)(((pre | tr) & live) >> kb);
+                if (d > -64) {
+                    const uint64_t pre = d >= 0 ? 0ull : (1ull << -d) - 1ull;
+                    const uint64_t live = span_L - ts >= 64 ? ~0ull : (1ull << max(span_L - ts, 0)) - 1ull;
+                    const uint64_t tr = d >= 64 ? 0ull : (d >= 0 ? anc >> d : anc << -d);
+                    const uint32_t vis = (uint32_t)(((pre | tr) & live) >> kb);
 #pragma unroll
-                for (int e = 0; e < 32; ++e)
-                    if (!((vis >> e) & 1u)) s[e] = kNegInf;
+                    for (int e = 0; e < 32; ++e)
+                        if (!((vis >> e) & 1u)) s[e] = kNegInf;
+                }
             } else {
                 const int lim_t = lim - ts - kb;   // keys e < lim_t of this half are visible
                 if (lim_t < 32) {
