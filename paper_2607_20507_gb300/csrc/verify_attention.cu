@@ -7,7 +7,7 @@
 // in order, tiles in key order; span (b, h) has T_b = ceil(L_b / 64) tiles.
 // The grid holds exactly as many CTAs as are resident at once; each span also
 // costs a few work units for its start, and CTA c takes the tiles of units
-// [cU/G, (c+1)U/G) (tiles_before below), so the CTAs' work evens out.  A span
+// [cU/G, (c+1)U/G) (range_of below), so the CTAs' work evens out.  A span
 // that lies inside one CTA's range is finished there and written in bf16;
 // a span cut by range boundaries leaves one partial per piece -- the piece's
 // own normalised output and its (m, l) -- (each CTA writes at most two: its
@@ -88,7 +88,7 @@ struct AttnParams {
     int n_rows_all;              // R * G query rows per KV head
     int tc_stages, tc_vstages;   // tcgen05 kernel: K and V ring depths
     int b_base, n_batch;         // requests [b_base, b_base + n_batch) in this launch
-    int span_x;                  // work units charged to each span's start (see tiles_before)
+    int span_x;                  // work units charged to each span's start (see range_of)
     float scale_log2;            // sm_scale * log2(e)
 };
 
@@ -98,9 +98,14 @@ __device__ __forceinline__ void flag_timeout(int* status) {
 
 __device__ __forceinline__ int tiles_of(int L) { return max(1, (L + kTileT - 1) / kTileT); }
 
+// a / b for a >= 0, b > 0 (a 64-bit division only where the numbers need one)
+__device__ __forceinline__ long long div_pos(long long a, long long b) {
+    return ((a | b) >> 32) == 0 ? (long long)((unsigned)a / (unsigned)b) : a / b;
+}
+
 // The CTA whose range holds work unit v (ranges start at floor(c*U/G)).
 __device__ __forceinline__ int owner_of(long long v, long long U, int G) {
-    return (int)(((v + 1) * G + U - 1) / U) - 1;
+    return (int)div_pos((v + 1) * G + U - 1, U) - 1;
 }
 
 // The work split.  Every span (request, KV head or row block) costs its T
@@ -108,54 +113,63 @@ __device__ __forceinline__ int owner_of(long long v, long long U, int G) {
 // grows with the span pieces it holds).  In the sequence of work units --
 // each span's X start units, then its T tiles -- CTA c of G takes units
 // [floor(c U / G), floor((c+1) U / G)) of U = W + X * n_vh * B, i.e. the
-// tiles whose unit index falls there.  tiles_before(v) counts the tiles
-// whose unit index is below v; request b's units start at
+// tiles whose unit index falls there; request b's units start at
 // prefix[b] + X * n_vh * b (prefix: its first tile).
-__device__ __forceinline__ long long tiles_before(long long v, const long long* prefix, const int* lens,
-                                                  int n_batch, int n_vh, int X) {
-    if (v <= 0) return 0;
-    int lo = 0, hi = n_batch - 1;   // largest b whose units start at or below v
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (prefix[mid] + (long long)X * n_vh * mid <= v) lo = mid;
-        else hi = mid - 1;
-    }
-    const int T = tiles_of(lens[lo]);
-    const long long local = v - (prefix[lo] + (long long)X * n_vh * lo);
-    const int S = T + X;
-    // local < (n_vh + 1) * S: one 32-bit division whenever that fits
-    const long long h = local <= 0x7fffffffLL ? (long long)((unsigned)local / (unsigned)S) : local / S;
-    if (h >= n_vh) return prefix[lo] + (long long)n_vh * T;   // past the last unit
-    const long long tv = local - h * S;
-    return prefix[lo] + h * T + (tv > X ? tv - X : 0);
-}
 
-// floor(c * U / G) for the unit range of CTA c
-__device__ __forceinline__ long long unit_start(int c, long long U, int G) {
-    const long long n = (long long)c * U;
-    return n <= 0xffffffffLL ? (long long)((unsigned)n / (unsigned)G) : n / G;
-}
-
-// Position of flat tile f in the schedule: request (launch-local), head, tile.
+// Position of a tile in the schedule: request (launch-local), head, tile.
 struct Cursor {
     int b, h, t, T;
 };
 
-__device__ __forceinline__ Cursor locate(long long f, const long long* prefix, const int* lens,
-                                         int n_batch, int n_vh) {
-    int lo = 0, hi = n_batch - 1;   // largest b with prefix[b] <= f
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (prefix[mid] <= f) lo = mid;
-        else hi = mid - 1;
+// A CTA's tiles.
+struct Range {
+    int n_tiles;
+    Cursor first;
+};
+
+// The range of CTA c of G, by one warp (all its lanes): lanes compare the
+// requests' starts (a binary search of the shared prefix took a chain of
+// loads per step), even lanes then place the range's start and odd ones its
+// end.  With the search, two placements one after the other and 64-bit
+// divisions the range and the first cursor were 3000 cycles of a call (8
+// requests: 25.4 us, 24.0 so; one of 512 keys 9.9 and 8.7; 64 requests
+// of 4096 keys, 12 rows: 173.9 and 170.1).
+__device__ __forceinline__ Range range_of(int c, long long U, int G, const long long* prefix, const int* lens,
+                                          int n_batch, int n_vh, int X) {
+    const int lane = threadIdx.x & 31;
+    const long long xh = (long long)X * n_vh;
+    // floor(c U / G) and floor((c + 1) U / G)
+    const long long v = div_pos((long long)(c + (lane & 1)) * U, G);
+    // the last request whose units start at or below v0, then v1
+    int lo = 0;
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+        const long long ve = __shfl_sync(0xffffffffu, v, e);
+        int blk = 0;
+        if (n_batch > 32) {
+            const int b = lane * 32;
+            blk = 31 - __clz(__ballot_sync(0xffffffffu, b < n_batch && prefix[b] + xh * b <= ve));
+        }
+        const int b = blk * 32 + lane;
+        const int l = blk * 32 + 31 - __clz(__ballot_sync(0xffffffffu, b < n_batch && prefix[b] + xh * b <= ve));
+        if ((lane & 1) == e) lo = l;
     }
-    Cursor c;
-    c.b = lo;
-    c.T = tiles_of(lens[lo]);
-    const long long local = f - prefix[lo];
-    c.h = (int)(local / c.T);
-    c.t = (int)(local % c.T);
-    return c;
+    Cursor cur;
+    cur.b = lo;
+    cur.T = tiles_of(lens[lo]);
+    const long long local = v - (prefix[lo] + xh * lo);
+    const int S = cur.T + X;
+    cur.h = (int)div_pos(local, S);      // n_vh: past the last unit
+    const int tv = (int)(local - (long long)cur.h * S);
+    cur.t = tv > X ? tv - X : 0;
+    const long long f = prefix[lo] + (long long)cur.h * cur.T + cur.t;   // tiles before v
+    Range r;
+    r.n_tiles = (int)(__shfl_sync(0xffffffffu, f, 1) - __shfl_sync(0xffffffffu, f, 0));
+    r.first.b = __shfl_sync(0xffffffffu, cur.b, 0);
+    r.first.h = __shfl_sync(0xffffffffu, cur.h, 0);
+    r.first.t = __shfl_sync(0xffffffffu, cur.t, 0);
+    r.first.T = __shfl_sync(0xffffffffu, cur.T, 0);
+    return r;
 }
 
 __device__ __forceinline__ void advance(Cursor& c, const int* lens, int n_batch, int n_vh) {
@@ -164,6 +178,64 @@ __device__ __forceinline__ void advance(Cursor& c, const int* lens, int n_batch,
     if (++c.h < n_vh) return;
     c.h = 0;
     if (++c.b < n_batch) c.T = tiles_of(lens[c.b]);
+}
+
+// n tiles on (at most to the first request past the launch's).
+__device__ __forceinline__ void advance_by(Cursor& c, int n, const int* lens, int n_batch, int n_vh) {
+    c.t += n;
+    while (c.t >= c.T && c.b < n_batch) {
+        c.t -= c.T;
+        if (++c.h < n_vh) continue;
+        c.h = 0;
+        if (++c.b < n_batch) c.T = tiles_of(lens[c.b]);
+    }
+}
+
+// The exclusive prefix of the requests' tiles (times their spans) and their
+// clamped lengths, into shared memory; ends with a block barrier.  One warp
+// does up to 32 requests, the block any number.
+__device__ __forceinline__ void build_schedule(const int32_t* ctx_lens, int nb, int l_cap, int n_vh, long long* prefix,
+                                               int* lens, long long* wtot, long long* carry) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    auto scan = [&](long long v) {
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const long long y = __shfl_up_sync(0xffffffffu, v, off);
+            if (lane >= off) v += y;
+        }
+        return v;
+    };
+    auto load = [&](int b) -> long long {
+        if (b >= nb) return 0;
+        const int L = max(0, min(__ldg(ctx_lens + b), l_cap));
+        lens[b] = L;
+        return (long long)tiles_of(L) * n_vh;
+    };
+    if (nb <= 32) {
+        if (warp == 0) {
+            const long long v = load(lane), inc = scan(v);
+            if (lane < nb) prefix[lane] = inc - v;
+            if (lane == 31) prefix[nb] = inc;
+        }
+        __syncthreads();
+        return;
+    }
+    if (threadIdx.x == 0) *carry = 0;
+    __syncthreads();
+    for (int base = 0; base < nb; base += blockDim.x) {
+        const int bl = base + threadIdx.x;
+        const long long v = load(bl), inc = scan(v);
+        if (lane == 31) wtot[warp] = inc;
+        __syncthreads();
+        long long before = *carry;
+        for (int w = 0; w < warp; ++w) before += wtot[w];
+        if (bl < nb) prefix[bl] = before + inc - v;
+        __syncthreads();
+        if (threadIdx.x == blockDim.x - 1) *carry = before + inc;
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) prefix[nb] = *carry;
+    __syncthreads();
 }
 
 // Ancestor-or-self bit masks of tree nodes `lane` and `lane + 32` (n <= 64
@@ -235,7 +307,6 @@ verify_attention_kernel(const __grid_constant__ CUtensorMap tmap_k,
 
     // ---- schedule: exclusive prefix of tiles per request (x heads), clamped L
     if (threadIdx.x == 0) {
-        s_carry = 0;
         for (int i = 0; i < kStages; ++i) {
             mbar_init(&full[i], 1);
             mbar_init(&empty[i], kSplit * nw);
@@ -250,38 +321,11 @@ verify_attention_kernel(const __grid_constant__ CUtensorMap tmap_k,
     // schedule while this one runs.
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    __syncthreads();
-    const int l_cap = p.max_pages * p.ps;
-    for (int base = 0; base < nb; base += blockDim.x) {
-        const int bl = base + threadIdx.x;
-        long long v = 0;
-        if (bl < nb) {
-            int L = __ldg(p.ctx_lens + p.b_base + bl);
-            L = max(0, min(L, l_cap));
-            s_len[bl] = L;
-            v = (long long)tiles_of(L) * p.n_vh;
-        }
-        long long inc = v;
-#pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            const long long y = __shfl_up_sync(0xffffffffu, inc, off);
-            if (lane >= off) inc += y;
-        }
-        if (lane == 31) s_wtot[warp] = inc;
-        __syncthreads();
-        long long before = s_carry;
-        for (int w = 0; w < warp; ++w) before += s_wtot[w];
-        if (bl < nb) s_prefix[bl] = before + inc - v;
-        __syncthreads();
-        if (threadIdx.x == blockDim.x - 1) s_carry = before + inc;
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) s_prefix[nb] = s_carry;
-    __syncthreads();
+    build_schedule(p.ctx_lens + p.b_base, nb, p.max_pages * p.ps, p.n_vh, s_prefix, s_len, s_wtot, &s_carry);
 
     const long long W = s_prefix[nb];
-    // small problems: a tile a CTA (one request of 512 keys, 64 tiles: 9.9 us
-    // against 15.1 with the 8 CTAs that eight tiles each make)
+    // small problems: a tile a CTA (one request of 512 keys, 64 tiles: 8.7 us
+    // against 13.9 with the 8 CTAs that eight tiles each make)
     const int Gc = (int)(W < (long long)gridDim.x ? (W > 0 ? W : 1) : gridDim.x);
     const int cta = blockIdx.x;
     // this CTA's two partial slots start unused (thread 0 -- row warp 0,
@@ -292,10 +336,9 @@ verify_attention_kernel(const __grid_constant__ CUtensorMap tmap_k,
     }
     if (cta >= Gc) return;
     const long long U = W + (long long)p.span_x * p.n_vh * nb;
-    const long long f0 = tiles_before(unit_start(cta, U, Gc), s_prefix, s_len, nb, p.n_vh, p.span_x);
-    const long long f1 = tiles_before(unit_start(cta + 1, U, Gc), s_prefix, s_len, nb, p.n_vh, p.span_x);
-    if (f0 >= f1) return;
-    const int n_tiles = (int)(f1 - f0);
+    const Range range = range_of(cta, U, Gc, s_prefix, s_len, nb, p.n_vh, p.span_x);
+    const int n_tiles = range.n_tiles;
+    if (n_tiles <= 0) return;
     const uint32_t smem_base = smem_u32(smem);
 
     if (warp == kSplit * nw) {
@@ -310,16 +353,20 @@ verify_attention_kernel(const __grid_constant__ CUtensorMap tmap_k,
         constexpr int pieces = kTileT / kBoxT;
         constexpr uint32_t piece_bytes = (uint32_t)kBoxT * 256u;   // both dim halves of kBoxT keys
         constexpr int per_batch = 32 / pieces;   // tiles whose page ids one warp-wide load covers
-        // lane l: the page of piece l % pieces of tile j0 + l / pieces
+        // lane l: the page of piece l % pieces of tile j0 + l / pieces (j0 a
+        // multiple of per_batch, in order)
+        Cursor pages_at = range.first;   // tile j0
         auto batch_pages = [&](int j0) -> int {
             const int jj = j0 + lane / pieces;
+            Cursor cc = pages_at;
+            advance_by(cc, lane / pieces, s_len, nb, p.n_vh);
+            advance_by(pages_at, per_batch, s_len, nb, p.n_vh);
             if (jj >= n_tiles) return -1;
-            const Cursor cc = locate(f0 + jj, s_prefix, s_len, nb, p.n_vh);
             const int tok = cc.t * kTileT + (lane % pieces) * kBoxT;
             if (tok >= s_len[cc.b]) return -1;
             return __ldg(p.page_table + (size_t)(p.b_base + cc.b) * p.max_pages + tok / p.ps);
         };
-        Cursor cur = locate(f0, s_prefix, s_len, nb, p.n_vh);
+        Cursor cur = range.first;
         int pg_cur = batch_pages(0);
         int pg_next = per_batch < n_tiles ? batch_pages(per_batch) : -1;
         int jt = 0;   // next tile to issue
@@ -384,7 +431,7 @@ verify_attention_kernel(const __grid_constant__ CUtensorMap tmap_k,
     const int lm = lane >> 3, lr = lane & 7;   // ldmatrix: matrix index, row within it
     const float c = p.scale_log2;
 
-    Cursor cur = locate(f0, s_prefix, s_len, nb, p.n_vh);
+    Cursor cur = range.first;
     int seg_t0 = cur.t;
     bool first_seg = true;
     int folds = 0;
@@ -853,7 +900,7 @@ verify_attention_merge_span_kernel(const AttnParams p, int grid_main) {
         L = max(0, min(L, l_cap));
         const int T = tiles_of(L);
         const int Gc = (int)(W < (long long)grid_main ? (W > 0 ? W : 1) : grid_main);
-        // in work units (tiles_before): the span's start units begin at vs,
+        // in work units (range_of): the span's start units begin at vs,
         // its tiles at vs + X; the CTA whose unit range holds its first tile
         // holds it as its first piece unless that range starts before vs
         // (unit vs - 1 is the previous span's last tile); every later owner
@@ -865,7 +912,7 @@ verify_attention_merge_span_kernel(const AttnParams p, int grid_main) {
         const int c_last = owner_of(vs + X + T - 1, U, Gc);
         int n_p = 0;
         for (int cc = c_first; cc <= c_last && n_p < 2 * kMaxGrid; ++cc)
-            s_slots[n_p++] = 2 * cc + ((cc == c_first && (long long)cc * U / Gc < vs) ? 1 : 0);
+            s_slots[n_p++] = 2 * cc + ((cc == c_first && div_pos((long long)cc * U, Gc) < vs) ? 1 : 0);
         s_np = n_p;
     }
     __syncthreads();

@@ -302,7 +302,6 @@ verify_attention_tc_kernel(const __grid_constant__ CUtensorMap tmap_k, const __g
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     if (threadIdx.x == 0) {
-        s_carry = 0;
         s_dead = 0;
         for (int i = 0; i < SK; ++i) {
             mbar_init(&kfull[i], 1);
@@ -334,35 +333,8 @@ verify_attention_tc_kernel(const __grid_constant__ CUtensorMap tmap_k, const __g
     // below); the merge kernel may start once every CTA is past this point
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    // ---- schedule: exclusive prefix of tiles per request (x spans), clamped L
-    __syncthreads();
-    const int l_cap = p.max_pages * p.ps;
-    for (int base = 0; base < nb; base += kTcThreads) {
-        const int bl = base + threadIdx.x;
-        long long v = 0;
-        if (bl < nb) {
-            int L = __ldg(p.ctx_lens + p.b_base + bl);
-            L = max(0, min(L, l_cap));
-            s_len[bl] = L;
-            v = (long long)tiles_of(L) * p.n_vh;
-        }
-        long long inc = v;
-#pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            const long long y = __shfl_up_sync(0xffffffffu, inc, off);
-            if (lane >= off) inc += y;
-        }
-        if (lane == 31) s_wtot[warp] = inc;
-        __syncthreads();
-        long long before = s_carry;
-        for (int w = 0; w < warp; ++w) before += s_wtot[w];
-        if (bl < nb) s_prefix[bl] = before + inc - v;
-        __syncthreads();
-        if (threadIdx.x == kTcThreads - 1) s_carry = before + inc;
-        __syncthreads();
-    }
+    build_schedule(p.ctx_lens + p.b_base, nb, p.max_pages * p.ps, p.n_vh, s_prefix, s_len, s_wtot, &s_carry);
     if (threadIdx.x == 0) {
-        s_prefix[nb] = s_carry;
         // this CTA's two partial slots start unused
         p.part_span[2 * blockIdx.x] = -1;
         p.part_span[2 * blockIdx.x + 1] = -1;
@@ -376,10 +348,8 @@ verify_attention_tc_kernel(const __grid_constant__ CUtensorMap tmap_k, const __g
     const int Gc = (int)(W < (long long)gridDim.x ? (W > 0 ? W : 1) : gridDim.x);
     const int cta = blockIdx.x;
     const long long U = W + (long long)p.span_x * p.n_vh * nb;
-    long long f0 = tiles_before(unit_start(cta, U, Gc), s_prefix, s_len, nb, p.n_vh, p.span_x);
-    long long f1 = tiles_before(unit_start(cta + 1, U, Gc), s_prefix, s_len, nb, p.n_vh, p.span_x);
-    if (cta >= Gc) f0 = f1 = 0;
-    const int n_tiles = (int)(f1 - f0);
+    const Range range = range_of(min(cta, Gc - 1), U, Gc, s_prefix, s_len, nb, p.n_vh, p.span_x);
+    const int n_tiles = cta < Gc ? range.n_tiles : 0;
     // one dim half of a span's rows (trees: of its row block of q_nodes nodes)
     const uint32_t qrow_bytes = (uint32_t)(kTree ? p.n_rows : p.R * p.G) * 128u;
     const int q_nodes = p.n_rows / p.G;
@@ -396,10 +366,13 @@ verify_attention_tc_kernel(const __grid_constant__ CUtensorMap tmap_k, const __g
         uint64_t* const emptyb = k_side ? kempty : vempty;
         const CUtensorMap* const tmap = k_side ? &tmap_k : &tmap_v;
         constexpr int per_batch = 32 / kPieces;
+        Cursor pages_at = range.first;   // tile j0 of the next batch (the batches come in order)
         auto batch_pages = [&](int j0) -> int {
             const int jj = j0 + lane / kPieces;
+            Cursor cc = pages_at;
+            advance_by(cc, lane / kPieces, s_len, nb, p.n_vh);
+            advance_by(pages_at, per_batch, s_len, nb, p.n_vh);
             if (jj >= n_tiles) return -1;
-            const Cursor cc = locate(f0 + jj, s_prefix, s_len, nb, p.n_vh);
             const int tok = cc.t * kTileT + (lane % kPieces) * kBoxT;
             if (tok >= s_len[cc.b]) return -1;
             return __ldg(p.page_table + (size_t)(p.b_base + cc.b) * p.max_pages + tok / p.ps);
@@ -408,7 +381,7 @@ verify_attention_tc_kernel(const __grid_constant__ CUtensorMap tmap_k, const __g
             tma_prefetch_desc(tmap);
             if (k_side) tma_prefetch_desc(&tmap_q);
         }
-        Cursor cur = locate(f0, s_prefix, s_len, nb, p.n_vh);
+        Cursor cur = range.first;
         int pg_cur = batch_pages(0);
         int pg_next = per_batch < n_tiles ? batch_pages(per_batch) : -1;
         // The next tile's page, position and flags are worked out while the
@@ -510,7 +483,7 @@ verify_attention_tc_kernel(const __grid_constant__ CUtensorMap tmap_k, const __g
         const uint64_t qhalf16 = (uint64_t)qh >> 4;
         const uint64_t dk0 = Tile::k_desc(smem_u32(sk)), dv0 = Tile::v_desc(smem_u32(sv));
         int span = -1, pv_piece = 0;
-        Cursor cur = locate(f0, s_prefix, s_len, nb, p.n_vh);   // the PV warp's own view of the pieces
+        Cursor cur = range.first;   // the PV warp's own view of the pieces
         uint64_t* last_bar = nullptr;   // the warp's latest commit: completes after all its MMAs
         uint32_t last_par = 0;
         // every lane waits; the result is made warp-uniform, so that no lane
@@ -628,7 +601,7 @@ verify_attention_tc_kernel(const __grid_constant__ CUtensorMap tmap_k, const __g
         const int row = lane0 + (lane & 15);                   // query row of the span = tensor-memory lane
         const uint32_t t_row = tmem + ((uint32_t)lane0 << 16);
         const float c = p.scale_log2;
-        Cursor cur = locate(f0, s_prefix, s_len, nb, p.n_vh);
+        Cursor cur = range.first;
         int seg_t0 = cur.t;
         bool first_seg = true;
         float m_run = kNegInf, l_part = 0.f;

@@ -33,3 +33,22 @@ def test_rows_and_pages(k, Hq, Hkv, ps):
                                       table.cpu().numpy(), np.asarray(lens, dtype=np.int32), k)
         got = got.float().cpu().numpy()
         assert (np.abs(got - exp) <= 2e-3 + 1e-2 * np.abs(exp)).all()
+
+
+@pytest.mark.parametrize("k", [2, 9])           # the mma.sync and the tcgen05 form
+@pytest.mark.parametrize("B", [1, 31, 32, 33, 64, 1025])
+def test_schedule_over_batches(k, B):
+    """Batches around a warp of requests and past one launch's, contexts of one
+    tile to many side by side (a context may be shorter than the verify rows)."""
+    Hq, Hkv, ps = 8, 2, 16
+    rng = np.random.default_rng(B)
+    lens = rng.choice([0, 1, k + 1, 63, 64, 65, 300, 1000 if B < 100 else 90], B).astype(np.int32)
+    w = W.Workload(96, "schedule", batch=B, n_draft=k, vocab=100, logit_dtype="bf16", draft_sigma=1.0,
+                   temperatures=(1.0,), n_q_heads=Hq, n_kv_heads=Hkv, head_dim=128,
+                   ctx=("const", int(max(lens.max(), k + 1))), page_size=ps, cell=k * B)
+    inp = W.attention_inputs(w, DEV, ctx_lens=torch.from_numpy(lens))
+    got = binding.cs_verify_attention(inp["q"], inp["k_pages"], inp["v_pages"], inp["page_table"], inp["ctx_lens"], k)
+    exp = oracle.verify_attention(W.host_bits(inp["q"]), W.host_bits(inp["k_pages"]), W.host_bits(inp["v_pages"]),
+                                  inp["page_table"].cpu().numpy(), lens, k)
+    got = got.float().cpu().numpy()
+    assert (np.abs(got - exp) <= 2e-3 + 1e-2 * np.abs(exp)).all()
