@@ -324,8 +324,8 @@ verify_attention_kernel(const __grid_constant__ CUtensorMap tmap_k,
     build_schedule(p.ctx_lens + p.b_base, nb, p.max_pages * p.ps, p.n_vh, s_prefix, s_len, s_wtot, &s_carry);
 
     const long long W = s_prefix[nb];
-    // small problems: a tile a CTA (one request of 512 keys, 64 tiles: 8.7 us
-    // against 13.9 with the 8 CTAs that eight tiles each make)
+    // small problems: a tile a CTA (one request of 512 keys, 64 tiles: 15.1 us
+    // with the 8 CTAs that eight tiles each make, 9.9 with 64)
     const int Gc = (int)(W < (long long)gridDim.x ? (W > 0 ? W : 1) : gridDim.x);
     const int cta = blockIdx.x;
     // this CTA's two partial slots start unused (thread 0 -- row warp 0,
@@ -766,13 +766,20 @@ constexpr int kMergePieces = 8;                  // pieces of a row merged in on
 constexpr int kMergePiecesCut = 4;               // the same for the register-capped per-CTA form
 constexpr int kMergeWin = 64;                    // slots read ahead of CTA c's first slot
 
-// the convex combination of one row's pieces (slots[0..n_p)), by one warp.
+// The partial slots of a span's pieces: slot0 in CTA c, then the first slot of
+// each CTA after it.
+struct Pieces {
+    int c, slot0, n;
+    __device__ __forceinline__ size_t slot(int j) const { return (size_t)(j == 0 ? slot0 : 2 * (c + j)); }
+};
+
+// the convex combination of one row's pieces, by one warp.
 // Up to kPieces pieces (the usual case) take one round trip: every
 // piece's (m, l) and this lane's four output columns of every piece are
 // requested together; more pieces go through the general loop.
 template <int kPieces>
-__device__ __forceinline__ void merge_row(const AttnParams& p, const int* slots, int n_p, int bl, int h, int row,
-                                          int lane) {
+__device__ __forceinline__ void merge_row(const AttnParams& p, const Pieces& pc, int bl, int h, int row, int lane) {
+    const int n_p = pc.n;
     const int bg = p.b_base + bl;
     const int head = h / p.n_rb, rbase = (h - head * p.n_rb) * p.n_rows;
     if (row >= p.n_rows || rbase + row >= p.n_rows_all) return;
@@ -780,12 +787,12 @@ __device__ __forceinline__ void merge_row(const AttnParams& p, const int* slots,
     if (n_p <= kPieces) {
         float4 v[kPieces];
         float2 ml = make_float2(kNegInf, 0.f);   // lane q < n_p: piece q
-        if (lane < n_p) ml = __ldcg(&p.part_ml[(size_t)slots[lane] * p.n_rows + row]);
+        if (lane < n_p) ml = __ldcg(&p.part_ml[pc.slot(lane) * p.n_rows + row]);
 #pragma unroll
         for (int j = 0; j < kPieces; ++j) {
             v[j] = make_float4(0.f, 0.f, 0.f, 0.f);
             if (j < n_p)
-                v[j] = __ldcg(reinterpret_cast<const float4*>(p.part_o + ((size_t)slots[j] * p.n_rows + row) * kD +
+                v[j] = __ldcg(reinterpret_cast<const float4*>(p.part_o + (pc.slot(j) * p.n_rows + row) * kD +
                                                               lane * 4));
         }
         float M = ml.x;
@@ -811,13 +818,13 @@ __device__ __forceinline__ void merge_row(const AttnParams& p, const int* slots,
         }
     } else {
         float M = kNegInf;
-        for (int q = lane; q < n_p; q += 32) M = fmaxf(M, __ldcg(&p.part_ml[(size_t)slots[q] * p.n_rows + row]).x);
+        for (int q = lane; q < n_p; q += 32) M = fmaxf(M, __ldcg(&p.part_ml[pc.slot(q) * p.n_rows + row]).x);
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, off));
         float lsum = 0.f;
         if (M != kNegInf)
             for (int q = lane; q < n_p; q += 32) {
-                const float2 ml = __ldcg(&p.part_ml[(size_t)slots[q] * p.n_rows + row]);
+                const float2 ml = __ldcg(&p.part_ml[pc.slot(q) * p.n_rows + row]);
                 if (ml.x != kNegInf) lsum = fmaf(ml.y, ex2(ml.x - M), lsum);
             }
 #pragma unroll
@@ -826,7 +833,7 @@ __device__ __forceinline__ void merge_row(const AttnParams& p, const int* slots,
         for (int q0 = 0; q0 < n_p && inv > 0.f; q0 += 32) {
             float wq = 0.f;   // the weight of piece q0 + lane
             if (q0 + lane < n_p) {
-                const float2 ml = __ldcg(&p.part_ml[(size_t)slots[q0 + lane] * p.n_rows + row]);
+                const float2 ml = __ldcg(&p.part_ml[pc.slot(q0 + lane) * p.n_rows + row]);
                 wq = ml.x == kNegInf ? 0.f : ml.y * ex2(ml.x - M) * inv;
             }
             const int nq = min(32, n_p - q0);
@@ -837,7 +844,7 @@ __device__ __forceinline__ void merge_row(const AttnParams& p, const int* slots,
                 for (int j = 0; j < kPieces; ++j) {
                     const bool ok = qq + j < nq;
                     wgt[j] = __shfl_sync(0xffffffffu, wq, (qq + j) & 31);
-                    const size_t sl = (size_t)slots[q0 + (ok ? qq + j : 0)];
+                    const size_t sl = pc.slot(q0 + (ok ? qq + j : 0));
                     v[j] = ok ? __ldcg(reinterpret_cast<const float4*>(p.part_o + (sl * p.n_rows + row) * kD + lane * 4))
                               : make_float4(0.f, 0.f, 0.f, 0.f);
                     if (!ok) wgt[j] = 0.f;
@@ -860,12 +867,11 @@ __device__ __forceinline__ void merge_row(const AttnParams& p, const int* slots,
     *reinterpret_cast<uint2*>(dst) = pk;
 }
 
-// grid (span h, request bl, 8-row chunk)
+// grid (span h, request bl, row chunk: rows 8 z + warp, and 8 gridDim.z on)
 __global__ void __launch_bounds__(kMergeThreads)
 verify_attention_merge_span_kernel(const AttnParams p, int grid_main) {
     __shared__ long long s_red[2][kMergeThreads / 32];
-    __shared__ int s_slots[2 * kMaxGrid];
-    __shared__ int s_np;
+    __shared__ Pieces s_pieces;
     const int h = blockIdx.x, bl = blockIdx.y;
     const int nb = p.n_batch;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -910,13 +916,12 @@ verify_attention_merge_span_kernel(const AttnParams p, int grid_main) {
         const long long vs = bf + (long long)X * p.n_vh * bl + (long long)h * (T + X);
         const int c_first = owner_of(vs + X, U, Gc);
         const int c_last = owner_of(vs + X + T - 1, U, Gc);
-        int n_p = 0;
-        for (int cc = c_first; cc <= c_last && n_p < 2 * kMaxGrid; ++cc)
-            s_slots[n_p++] = 2 * cc + ((cc == c_first && div_pos((long long)cc * U, Gc) < vs) ? 1 : 0);
-        s_np = n_p;
+        s_pieces.c = c_first;
+        s_pieces.slot0 = 2 * c_first + (div_pos((long long)c_first * U, Gc) < vs ? 1 : 0);
+        s_pieces.n = c_last - c_first + 1;
     }
     __syncthreads();
-    const int n_p = s_np;
+    const Pieces pc = s_pieces;
     // everything above depends only on the context lengths; the pieces are
     // the main kernel's output.  Every CTA waits, even one with nothing to
     // merge, so that this grid never completes before the main kernel (a
@@ -924,16 +929,17 @@ verify_attention_merge_span_kernel(const AttnParams p, int grid_main) {
     // next kernel of the stream start.
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    if (n_p <= 1) return;   // written whole by the main kernel
-    merge_row<kMergePieces>(p, s_slots, n_p, bl, h, blockIdx.z * kMergeRows + warp, lane);
+    if (pc.n <= 1) return;   // written whole by the main kernel
+    for (int row = blockIdx.z * kMergeRows + warp; row < p.n_rows; row += gridDim.z * kMergeRows)
+        merge_row<kMergePieces>(p, pc, bl, h, row, lane);
 }
 
 // grid (main-kernel CTA c, 8-row chunk)
 __global__ void __launch_bounds__(kMergeThreads, kMergePerSm)
 verify_attention_merge_cut_kernel(const AttnParams p, int n_slots) {
     __shared__ int s_win[2 + kMergeWin];   // slots 2c-2 .. 2c+kMergeWin-1
-    __shared__ int s_slots[2 * kMaxGrid];
-    __shared__ int s_np, s_span;
+    __shared__ Pieces s_pieces;
+    __shared__ int s_span;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // the slot list is the main kernel's output.  Every CTA waits, even one
     // with nothing to merge, so that this grid never completes before the
@@ -966,21 +972,24 @@ verify_attention_merge_cut_kernel(const AttnParams p, int n_slots) {
         }
         int n_p = 0;
         if (id >= 0) {
-            s_slots[n_p++] = r0;
+            n_p = 1;
             // the following CTAs' first pieces, while the span goes on
-            for (int cc = c + 1; 2 * cc < n_slots && n_p < 2 * kMaxGrid; ++cc) {
+            for (int cc = c + 1; 2 * cc < n_slots; ++cc) {
                 if (span_at(2 * cc) != id) break;
-                s_slots[n_p++] = 2 * cc;
+                ++n_p;
                 if (span_at(2 * cc + 1) >= 0) break;   // CTA cc has a later piece: the span ends here
             }
         }
-        s_np = n_p;
+        s_pieces.c = c;
+        s_pieces.slot0 = r0;
+        s_pieces.n = n_p;
         s_span = id;
     }
     __syncthreads();
-    const int n_p = s_np, id = s_span;
-    if (n_p <= 1) return;   // no cut span starts here (a single piece cannot occur)
-    merge_row<kMergePiecesCut>(p, s_slots, n_p, id / p.n_vh, id % p.n_vh, blockIdx.y * kMergeRows + warp, lane);
+    const Pieces pc = s_pieces;
+    const int id = s_span;
+    if (pc.n <= 1) return;   // no cut span starts here (a single piece cannot occur)
+    merge_row<kMergePiecesCut>(p, pc, id / p.n_vh, id % p.n_vh, blockIdx.y * kMergeRows + warp, lane);
 }
 
 #include "verify_attention_tc.cuh"
@@ -1097,7 +1106,11 @@ cudaError_t launch_merge(const AttnParams& p, const AttnPlan& pl, cudaStream_t s
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
     if ((long long)p.n_vh * p.n_batch <= (long long)pl.grid) {
-        cfg.gridDim = dim3(p.n_vh, p.n_batch, chunks);
+        // in one wave (three CTAs an SM): more rows a CTA instead of a second
+        // one (8 requests of 34 nodes, 128 spans of 68 rows: 49.4
+        // us for the attention in three waves, 48.0 so)
+        const int room = 3 * current_sm_count() / (p.n_vh * p.n_batch);
+        cfg.gridDim = dim3(p.n_vh, p.n_batch, room < 1 ? 1 : room < (int)chunks ? room : chunks);
         return cudaLaunchKernelEx(&cfg, verify_attention_merge_span_kernel, p, (int)pl.grid);
     }
     cfg.gridDim = dim3((unsigned)pl.grid, chunks, 1);
