@@ -148,6 +148,33 @@ __device__ __forceinline__ int walk_locate(const DrawRow<T>& d, int j, int V, fl
     return warp_max_int(last);
 }
 
+// A sum and its rounding error (h the nearest float to h + l).
+struct Sum2 {
+    float h, l;
+};
+
+__device__ __forceinline__ Sum2 add2(Sum2 a, Sum2 b) {
+    const float s = a.h + b.h, bb = s - a.h;
+    const float e = ((a.h - (s - bb)) + (b.h - bb)) + (a.l + b.l);
+    const float h = s + e;
+    return {h, e - (h - s)};
+}
+
+__device__ __forceinline__ Sum2 shfl2(Sum2 v, int src) {
+    return {__shfl_sync(0xffffffffu, v.h, src), __shfl_sync(0xffffffffu, v.l, src)};
+}
+
+// Inclusive scan of the warp's values.
+__device__ __forceinline__ Sum2 warp_incl_scan2(float x, int lane) {
+    Sum2 v = {x, 0.f};
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const Sum2 y = {__shfl_up_sync(0xffffffffu, v.h, off), __shfl_up_sync(0xffffffffu, v.l, off)};
+        if (lane >= off) v = add2(v, y);
+    }
+    return v;
+}
+
 // Writes v to the same shared-memory address of CTA `rank` of the cluster.
 __device__ __forceinline__ void st_cluster_f2(float2* local, uint32_t rank, float2 v) {
     uint32_t remote;
@@ -527,25 +554,33 @@ __global__ void __launch_bounds__(kWalkMaxThreads, 2) accept_walk_kernel(const W
                 const float x = f.x == kNegInf ? 0.f : f.y * ex2_scaled(f.x - d.mt, p.c_hi, p.c_lo);
                 return x > 0x1p-120f ? x : 0.f;   // a unit that counts has a weight that is not flushed
             };
-            float Z = 0.f;
+            // the CDF over the units and the draw's place in it as pairs of
+            // floats: a token of 1e-6 of the mass is 16 roundings of a float
+            // sum (against 64 bits 14 of 5872 draws moved to the next token,
+            // 4 with pairs; in doubles 256 rows of 128256 took 1.5 us longer)
+            const float x0 = mass(lane);
+            const Sum2 incl0 = warp_incl_scan2(x0, lane);
+            Sum2 Z = shfl2(incl0, 31);
 #pragma unroll 1
-            for (int l0 = 0; l0 < p.ph.units; l0 += 32)
-                Z += __shfl_sync(0xffffffffu, warp_incl_scan(mass(l0 + lane), lane), 31);
-            const float t = uk * Z;
-            float run = 0.f;
+            for (int l0 = 32; l0 < p.ph.units; l0 += 32) Z = add2(Z, shfl2(warp_incl_scan2(mass(l0 + lane), lane), 31));
+            // u Z, less the units passed
+            const float tp = uk * Z.h;
+            Sum2 rest = add2({tp, 0.f}, {fmaf(uk, Z.h, -tp), uk * Z.l});
             int at = -1, last = -1;
 #pragma unroll 1
             for (int l0 = 0; l0 < p.ph.units && at < 0; l0 += 32) {
-                const float x = mass(l0 + lane);
-                const float incl = warp_incl_scan(x, lane);
-                const unsigned hit = __ballot_sync(0xffffffffu, x > 0.f && run + incl > t);
+                const float x = l0 > 0 ? mass(l0 + lane) : x0;
+                const Sum2 incl = l0 > 0 ? warp_incl_scan2(x, lane) : incl0;
+                const Sum2 past = add2(incl, {-rest.h, -rest.l});
+                const unsigned hit = __ballot_sync(0xffffffffu, x > 0.f && past.h > 0.f);
                 const unsigned any = __ballot_sync(0xffffffffu, x > 0.f);
                 if (hit) {
                     at = l0 + __ffs(hit) - 1;
-                    tt = t - (run + __shfl_sync(0xffffffffu, incl - x, at - l0));
+                    tt = __shfl_sync(0xffffffffu, add2({x, 0.f}, {-past.h, -past.l}).h, at - l0);
                 }
                 if (any) last = l0 + 31 - __clz((int)any);
-                run += __shfl_sync(0xffffffffu, incl, 31);
+                const Sum2 end = shfl2(incl, 31);
+                rest = add2(rest, {-end.h, -end.l});
             }
             if (at < 0) at = last;   // past the total through rounding: the last positive unit (tt: its end)
             if (at >= 0) {           // (no mass at all: the residual is empty up to rounding, drawn from p below)
