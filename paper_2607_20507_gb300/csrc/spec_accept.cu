@@ -93,6 +93,7 @@ struct StatsParams {
     int mass_lo, mass_hi;
     const float4* stat;       // [B] statistics of the pair
     float* mass;              // [B, units]
+    long long share, extra;   // phase 0: units of a warp, and how many warps take one more
     FastDiv by_units, by_R;
 };
 
@@ -463,12 +464,47 @@ __global__ void __launch_bounds__(kThreads, 2) accept_stats_kernel(const StatsPa
     __shared__ uint16_t s_list[kLater ? kMaxPhased : 1];   // undecided requests from the front, decided from the back
     __shared__ int s_wcount[2][kWarps];
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int I = p.I, V = p.V, R = p.ph.R, t_rows = p.ph.t_rows, p0 = p.ph.p0, units = p.ph.units, U = p.ph.U;
+    const T* rp = nullptr;   // row, items and partial of the unit whose items are being loaded
+    int item = 0, end = 0, at = 0;
+    long long slot = 0;
+    bool skip = false, drafted = false;
+    auto open_unit = [&](long long x) {
+        const long long row = p.by_units.div(x);
+        const int u = (int)(x - row * units);
+        const int idx = (int)p.by_R.div(row), r = (int)(row - (long long)idx * R);
+        const int b = kLater ? s_list[idx] : idx;
+        at = p0 + (r < t_rows ? r : r - t_rows);   // the row's node
+        drafted = r >= t_rows;
+        rp = !drafted ? static_cast<const T*>(p.target) + ((size_t)b * p.n + at) * V
+                      : static_cast<const T*>(p.draft) + ((size_t)b * p.d_rows + at) * V;
+        item = u * U;
+        end = min(item + U, I);
+        slot = ((long long)b * R + r) * units + u;
+    };
+    // tree: the draft row of a node without children is never used
+    auto set_skip = [&]() {
+        if (!kLater && !kGreedy && p.parents) {
+            const int b = (int)p.by_R.div(p.by_units.div(slot));
+            skip = drafted && !((tree_child_mask(p.parents + (size_t)b * p.n, p.n, lane) >> at) & 1ull);
+        }
+    };
+    // phase 0 knows its shares before it reads anything, and works them out
+    // before the wait, with no division (after it, with two: 15.0 us a call of
+    // B = 8, k = 5, V = 128256, 14.2 so).  The warps with one unit more are
+    // spread over the CTAs.
+    long long unit = 0, hi = 0;
+    if (!kLater) {
+        const long long w = (long long)wid * gridDim.x + blockIdx.x;
+        unit = w * p.share + min(w, p.extra);
+        hi = unit + p.share + (w < p.extra ? 1 : 0);
+        if (unit < hi) open_unit(unit);
+    }
     // launched as a programmatic dependent of the kernel before it: its
     // inputs are read only past this wait, and the next kernel (which
     // reads some inputs before its own wait) only starts after it
     wait_prior_grid();
     allow_dependent_launch();
-    const int I = p.I, V = p.V, R = p.ph.R, t_rows = p.ph.t_rows, p0 = p.ph.p0, units = p.ph.units, U = p.ph.U;
     int requests = p.B, massed = 0;
     if (kLater) {
         requests = 0;
@@ -499,29 +535,11 @@ __global__ void __launch_bounds__(kThreads, 2) accept_stats_kernel(const StatsPa
     }
     // contiguous shares; of a later phase the last quarter goes by the counter
     const int W = (int)gridDim.x * kWarps, w = (int)blockIdx.x * kWarps + wid;
-    const long long N = (long long)requests * R * units, fixed = kLater ? N - N / 4 : N;
-    long long unit = div_nn(w * fixed, W);
-    const long long hi = div_nn((w + 1) * fixed, W);
-
-    const T* rp = nullptr;   // row, items and partial of the unit whose items are being loaded
-    int item = 0, end = 0;
-    long long slot = 0;
-    bool skip = false;
-    auto open_unit = [&](long long x) {
-        const long long row = p.by_units.div(x);
-        const int u = (int)(x - row * units);
-        const int idx = (int)p.by_R.div(row), r = (int)(row - (long long)idx * R);
-        const int b = kLater ? s_list[idx] : idx;
-        const int at = p0 + (r < t_rows ? r : r - t_rows);   // the row's node
-        rp = r < t_rows ? static_cast<const T*>(p.target) + ((size_t)b * p.n + at) * V
-                        : static_cast<const T*>(p.draft) + ((size_t)b * p.d_rows + at) * V;
-        item = u * U;
-        end = min(item + U, I);
-        slot = ((long long)b * R + r) * units + u;
-        // tree: the draft row of a node without children is never used
-        if (!kLater && !kGreedy && p.parents)
-            skip = r >= t_rows && !((tree_child_mask(p.parents + (size_t)b * p.n, p.n, lane) >> at) & 1ull);
-    };
+    const long long N = (long long)requests * R * units, fixed = N - N / 4;
+    if (kLater) {
+        unit = div_nn(w * fixed, W);
+        hi = div_nn((w + 1) * fixed, W);
+    }
     // One item into registers: lane l holds vectors u*32 + l; entries past
     // the row's end, and skipped rows, read as -inf.
     auto load = [&](uint4 (&v)[kVecs]) {
@@ -562,7 +580,8 @@ __global__ void __launch_bounds__(kThreads, 2) accept_stats_kernel(const StatsPa
         if (unit >= N) return;
         if (lane == 0) next = atomicAdd(p.ph.ticket, 1u);
     }
-    open_unit(unit);
+    if (kLater) open_unit(unit);
+    else set_skip();
 
     float m = kNegInf, s = 0.f;            // sampling: lane's running (max, sum)
     int id = INT_MAX;                      // greedy: lane's lowest id of the max (m)
@@ -580,7 +599,10 @@ __global__ void __launch_bounds__(kThreads, 2) accept_stats_kernel(const StatsPa
             } else {
                 more = unit < hi;
             }
-            if (more) open_unit(unit);
+            if (more) {
+                open_unit(unit);
+                set_skip();
+            }
         }
         if (more) load(nxt);
         // a ticket ahead from the share's last unit on
@@ -944,6 +966,8 @@ cs_status launch_typed(StatsParams sp, TestParams tp, WalkParams p, const Accept
         sp.by_R.set(ph.R);
         const long long ctas = ((long long)sp.B * ph.R * ph.units + kWarps - 1) / kWarps;
         const unsigned grid = (unsigned)(ctas < fill ? ctas : fill);
+        sp.share = (long long)sp.B * ph.R * ph.units / ((long long)grid * kWarps);
+        sp.extra = (long long)sp.B * ph.R * ph.units % ((long long)grid * kWarps);
         cudaError_t e = launch_after(i ? accept_stats_kernel<T, G, true> : accept_stats_kernel<T, G, false>, grid, 1,
                                      kThreads, 1, stream, sp);
         if (e != cudaSuccess) return cuda_fail(e, "accept_stats_kernel launch");
