@@ -24,9 +24,9 @@ deliberately slow baseline; rank 0 only).
 from __future__ import annotations
 
 import argparse
+import ctypes
 import hashlib
 import json
-import math
 import os
 import statistics
 import subprocess
@@ -55,6 +55,7 @@ KERNEL_SOURCES = {
                          "paper_2607_20507_gb300/csrc/verify_attention_tc.cuh",
                          "paper_2607_20507_gb300/csrc/cs_device.cuh"),
     "spec_accept": ("paper_2607_20507_gb300/csrc/spec_accept.cu",
+                    "paper_2607_20507_gb300/csrc/spec_accept_walk.cuh",
                     "paper_2607_20507_gb300/csrc/cs_device.cuh"),
 }
 
@@ -237,6 +238,22 @@ def capture(fn):
     return gr
 
 
+def kernel_launches(fn) -> int:
+    """Kernels that one call of fn launches: the kernel nodes of its graph."""
+    gr = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(gr):
+        fn()
+    driver, graph, n = ctypes.CDLL("libcuda.so.1"), ctypes.c_void_p(gr.raw_cuda_graph()), ctypes.c_size_t()
+    if driver.cuGraphGetNodes(graph, None, ctypes.byref(n)) != 0:
+        raise RuntimeError("cuGraphGetNodes failed")
+    nodes, kind, kernels = (ctypes.c_void_p * n.value)(), ctypes.c_int(), 0
+    driver.cuGraphGetNodes(graph, nodes, ctypes.byref(n))
+    for node in nodes:
+        driver.cuGraphNodeGetType(ctypes.c_void_p(node), ctypes.byref(kind))
+        kernels += kind.value == 0   # CU_GRAPH_NODE_TYPE_KERNEL
+    return kernels
+
+
 def flushed_times(gr, steps, flush, stream) -> list[float]:
     """Seconds of `steps` replays of graph `gr`, the L2 flushed before each
     (outside the events)."""
@@ -283,12 +300,13 @@ def kernel_figures(w, T, lens, n_acc, t_attn, t_acc, hbm_peak) -> dict:
                              "frac": round(ab / m_attn / 1e9 / hbm_peak, 4),
                              "frac_of_nominal_8tbs": round(ab / m_attn / 1e9 / NOMINAL_HBM_GBS, 4),
                              "tflops": round(attention_flops(lens, w) / m_attn / 1e12, 1)},
-        # the acceptance kernels read every row once (all positions in parallel);
-        # `needed_bytes` (rows 0..a) is what a rejection-ordered pass would touch
-        "spec_accept": {"us": round(1e6 * m_acc, 2), "bytes": acc_full, "gbs": round(acc_full / m_acc / 1e9, 1),
-                        "frac": round(acc_full / m_acc / 1e9 / hbm_peak, 4),
-                        "frac_of_nominal_8tbs": round(acc_full / m_acc / 1e9 / NOMINAL_HBM_GBS, 4),
-                        "needed_bytes": acc_need, "mean_accepted": round(float(n_acc.mean()), 4)},
+        # `bytes`: rows 0..a of every request, which the accept tests and the draw
+        # cannot do without; `all_rows_bytes`: every row once, as a call reads
+        # them that is too short for phases
+        "spec_accept": {"us": round(1e6 * m_acc, 2), "bytes": acc_need, "gbs": round(acc_need / m_acc / 1e9, 1),
+                        "frac": round(acc_need / m_acc / 1e9 / hbm_peak, 4),
+                        "frac_of_nominal_8tbs": round(acc_need / m_acc / 1e9 / NOMINAL_HBM_GBS, 4),
+                        "all_rows_bytes": acc_full, "mean_accepted": round(float(n_acc.mean()), 4)},
     }
 
 
@@ -361,6 +379,7 @@ def run_gb300(args) -> dict | None:
     # replay it.  Each call is also captured on its own, to time the two
     # calls' shares of the step.
     g_step, g_attn, g_acc = capture(step), capture(attention), capture(accept)
+    launches = kernel_launches(step)
 
     # warm-up: at least W steps and about a second of work, with clocks sampled
     sampler = ClockSampler(local)
@@ -598,10 +617,10 @@ def run_gb300(args) -> dict | None:
                             "context lengths, target and draft logits, draft tokens and uniforms; the two "
                             "C-ABI calls; device->host read of the emitted tokens and counts.  The paged KV "
                             "cache stays resident on the device (serving state, not a per-step input)"},
-            # per step: the verify-attention kernel and its split merge (one pair per
-            # 1024-request slice), the acceptance statistics kernel and the draw
-            # kernel (one launch per 65535 requests)
-            "gpu_launches": args.steps * (2 * math.ceil(B / 1024) + 1 + math.ceil(B / 65535)),
+            # per step: the verify-attention kernel and its split merge, and the
+            # acceptance kernels (statistics and tests by phase, the walk), counted
+            # as the kernel nodes of the captured step
+            "gpu_launches": args.steps * launches,
             "clocks": sampler.summary() | {"window": f"warm-up (>= {args.warmup_seconds:g} s) and the timed steps"},
         }
     if world > 1:
@@ -762,8 +781,8 @@ def run_reference(args) -> dict | None:
 def run_sweep(args) -> None:
     """The sweep's cells at B >= 64 (one JSON line each): verify attention over
     k x B at context 4096, and the acceptance over k x B x V at draft sigma
-    1.0 (the sigma changes how many positions are accepted, not the bytes the
-    kernels read).  Each cell: inputs generated on the device, the C-ABI call
+    1.0 (the sigma changes how many positions are accepted, and with them the
+    bytes that have to be read).  Each cell: inputs generated on the device, the C-ABI call
     captured in a CUDA graph, 5 untimed replays, then the median of `steps`
     replays with the L2 flushed before each (outside the events)."""
     from paper_2607_20507_gb300 import binding
@@ -826,7 +845,7 @@ def run_sweep(args) -> None:
         us = median_us(lambda: binding.cs_spec_accept(acc["target"], acc["draft"], acc["draft_tokens"],
                                                       acc["uniforms"], T, ot, on))
         n_acc = on.cpu().numpy()
-        line("spec_accept", w, us, accept_bytes(n_acc, w, T)[1], {"mean_accepted": float(n_acc.mean())})
+        line("spec_accept", w, us, accept_bytes(n_acc, w, T)[0], {"mean_accepted": float(n_acc.mean())})
         del acc, ot, on
         torch.cuda.empty_cache()
 
