@@ -164,13 +164,21 @@ __device__ __forceinline__ Sum2 shfl2(Sum2 v, int src) {
     return {__shfl_sync(0xffffffffu, v.h, src), __shfl_sync(0xffffffffu, v.l, src)};
 }
 
-// Inclusive scan of the warp's values.
-__device__ __forceinline__ Sum2 warp_incl_scan2(float x, int lane) {
-    Sum2 v = {x, 0.f};
+__device__ __forceinline__ Sum2 sub2(Sum2 a, Sum2 b) { return add2(a, {-b.h, -b.l}); }
+
+// u times a sum.
+__device__ __forceinline__ Sum2 scale2(float u, Sum2 z) {
+    const float p = u * z.h;
+    return add2({p, 0.f}, {fmaf(u, z.h, -p), u * z.l});
+}
+
+// Inclusive scan of the warp's values (out of line: one copy of its steps to
+// fetch; lanes below a step's distance add zero).
+__device__ __noinline__ Sum2 warp_incl_scan2(Sum2 v, int lane) {
 #pragma unroll
     for (int off = 1; off < 32; off <<= 1) {
-        const Sum2 y = {__shfl_up_sync(0xffffffffu, v.h, off), __shfl_up_sync(0xffffffffu, v.l, off)};
-        if (lane >= off) v = add2(v, y);
+        const float h = __shfl_up_sync(0xffffffffu, v.h, off), l = __shfl_up_sync(0xffffffffu, v.l, off);
+        v = add2(v, {lane >= off ? h : 0.f, lane >= off ? l : 0.f});
     }
     return v;
 }
@@ -559,28 +567,26 @@ __global__ void __launch_bounds__(kWalkMaxThreads, 2) accept_walk_kernel(const W
             // sum (against 64 bits 14 of 5872 draws moved to the next token,
             // 4 with pairs; in doubles 256 rows of 128256 took 1.5 us longer)
             const float x0 = mass(lane);
-            const Sum2 incl0 = warp_incl_scan2(x0, lane);
+            const Sum2 incl0 = warp_incl_scan2({x0, 0.f}, lane);
             Sum2 Z = shfl2(incl0, 31);
 #pragma unroll 1
-            for (int l0 = 32; l0 < p.ph.units; l0 += 32) Z = add2(Z, shfl2(warp_incl_scan2(mass(l0 + lane), lane), 31));
+            for (int l0 = 32; l0 < p.ph.units; l0 += 32) Z = add2(Z, shfl2(warp_incl_scan2({mass(l0 + lane), 0.f}, lane), 31));
             // u Z, less the units passed
-            const float tp = uk * Z.h;
-            Sum2 rest = add2({tp, 0.f}, {fmaf(uk, Z.h, -tp), uk * Z.l});
+            Sum2 rest = scale2(uk, Z);
             int at = -1, last = -1;
 #pragma unroll 1
             for (int l0 = 0; l0 < p.ph.units && at < 0; l0 += 32) {
                 const float x = l0 > 0 ? mass(l0 + lane) : x0;
-                const Sum2 incl = l0 > 0 ? warp_incl_scan2(x, lane) : incl0;
-                const Sum2 past = add2(incl, {-rest.h, -rest.l});
+                const Sum2 incl = l0 > 0 ? warp_incl_scan2({x, 0.f}, lane) : incl0;
+                const Sum2 past = sub2(incl, rest);
                 const unsigned hit = __ballot_sync(0xffffffffu, x > 0.f && past.h > 0.f);
                 const unsigned any = __ballot_sync(0xffffffffu, x > 0.f);
                 if (hit) {
                     at = l0 + __ffs(hit) - 1;
-                    tt = __shfl_sync(0xffffffffu, add2({x, 0.f}, {-past.h, -past.l}).h, at - l0);
+                    tt = __shfl_sync(0xffffffffu, sub2({x, 0.f}, past).h, at - l0);
                 }
                 if (any) last = l0 + 31 - __clz((int)any);
-                const Sum2 end = shfl2(incl, 31);
-                rest = add2(rest, {-end.h, -end.l});
+                rest = sub2(rest, shfl2(incl, 31));
             }
             if (at < 0) at = last;   // past the total through rounding: the last positive unit (tt: its end)
             if (at >= 0) {           // (no mass at all: the residual is empty up to rounding, drawn from p below)
@@ -616,17 +622,15 @@ __global__ void __launch_bounds__(kWalkMaxThreads, 2) accept_walk_kernel(const W
                 break;
             }
             const float x = swap_mass();
-            const float incl = warp_incl_scan(x, lane);
-            const float Z = __shfl_sync(0xffffffffu, incl, 31);
-            if (Z > 0.f || !residual) {
+            const Sum2 incl = warp_incl_scan2({x, 0.f}, lane), Z = shfl2(incl, 31);
+            if (Z.h > 0.f || !residual) {
                 // the CTA whose cell holds u Z (past the total through rounding: the last positive mass)
-                const float t = uk * Z;
-                const unsigned own = __ballot_sync(0xffffffffu, x > 0.f && incl > t);
+                const Sum2 past = sub2(incl, scale2(uk, Z));
+                const unsigned own = __ballot_sync(0xffffffffu, x > 0.f && past.h > 0.f);
                 const unsigned pos = __ballot_sync(0xffffffffu, x > 0.f);
                 const int owner = own ? __ffs(own) - 1 : pos ? 31 - __clz((int)pos) : 0;
-                const float before = __shfl_sync(0xffffffffu, incl - x, owner);
                 mine = (int)rank == owner;
-                if (own) tt = t - before;
+                if (own) tt = __shfl_sync(0xffffffffu, sub2({x, 0.f}, past).h, owner);
                 break;
             }
             residual = false;   // no positive residual (p == q up to rounding): draw from p instead
