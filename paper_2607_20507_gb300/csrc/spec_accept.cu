@@ -456,7 +456,11 @@ __device__ __forceinline__ float item_masses(const DrawRow<T>& d, int i0, int i1
 // of the units goes to whichever warp is free, by a counter (a short phase
 // dealt out in equal shares ended 20-30% after its mean).  A warp keeps the next item in flight
 // while it reduces the current one, across units.
-template <typename T, bool kGreedy, bool kLater>
+// kShort, phase 0 of a call with few items a warp: one copy of the reduction,
+// the items changing registers, where two copies in turn save that (7% of a
+// long call): 16 requests, k = 5, V = 128256 22.3 us a call and 21.3 so, 8 from
+// a flushed L2 24.8 and 24.3.
+template <typename T, bool kGreedy, bool kLater, bool kShort>
 __global__ void __launch_bounds__(kThreads, 2) accept_stats_kernel(const StatsParams p) {
     constexpr int kPer = 16 / (int)sizeof(T);
     constexpr int kItem = kItemBytes / (int)sizeof(T);
@@ -632,8 +636,13 @@ __global__ void __launch_bounds__(kThreads, 2) accept_stats_kernel(const StatsPa
     for (;;) {
         step(va, vb);
         if (!more) break;
-        step(vb, va);
-        if (!more) break;
+        if (kShort) {
+#pragma unroll
+            for (int u = 0; u < kVecs; ++u) va[u] = vb[u];
+        } else {
+            step(vb, va);
+            if (!more) break;
+        }
     }
 }
 
@@ -857,14 +866,18 @@ AcceptPlan plan_accept(const cs_accept_dims& d, int n, bool tree, bool greedy, b
         // The first phase takes the positions of about 30 us, every later one
         // twice as many as were read before it, and what is left over when it
         // is less than 15 us joins the last.  A phase costs about 8 us (its
-        // test, two hand-offs, an uneven end), so a call under 45 us is read
-        // at once.  B = 256, k = 8, V = 128256, bf16: 140 us with 1.9 of 8
+        // test, two hand-offs, an uneven end), so a call under 60 us is read
+        // at once (in two phases a call of 45 us, B = 64, k = 8, V = 128256,
+        // took 81 us from a flushed L2 and at once 71; one of 50 us, B = 512,
+        // k = 4, V = 32000, 94 and 87; one of 85 us, B = 256, k = 16, V = 32000,
+        // 94 and 112).  B = 256, k = 8, V = 128256, bf16: 140 us with 1.9 of 8
         // drafts accepted and 198 with 7.5 (at once: 208 and 201); B = 64,
         // k = 4, V = 151936 at once 46 us, in two phases 58.
-        constexpr double kPhaseUs = 30.0;
+        constexpr double kPhaseUs = 30.0, kPhasedUs = 60.0;
         P.phases = 1;
         long long g = (long long)(kPhaseUs / pos_us) + 1;
-        while (!tree && d.batch <= kMaxPhased && P.phases < kMaxPhases && g < n && (n - g) * pos_us >= kPhaseUs / 2) {
+        while (!tree && n * pos_us >= kPhasedUs && d.batch <= kMaxPhased && P.phases < kMaxPhases && g < n &&
+               (n - g) * pos_us >= kPhaseUs / 2) {
             P.start[P.phases++] = (int)g;
             g *= 2;
         }
@@ -968,8 +981,10 @@ cs_status launch_typed(StatsParams sp, TestParams tp, WalkParams p, const Accept
         const unsigned grid = (unsigned)(ctas < fill ? ctas : fill);
         sp.share = (long long)sp.B * ph.R * ph.units / ((long long)grid * kWarps);
         sp.extra = (long long)sp.B * ph.R * ph.units % ((long long)grid * kWarps);
-        cudaError_t e = launch_after(i ? accept_stats_kernel<T, G, true> : accept_stats_kernel<T, G, false>, grid, 1,
-                                     kThreads, 1, stream, sp);
+        auto* const stats = i ? accept_stats_kernel<T, G, true, false>
+                              : sp.share * ph.U < 8 ? accept_stats_kernel<T, G, false, true>
+                                                    : accept_stats_kernel<T, G, false, false>;
+        cudaError_t e = launch_after(stats, grid, 1, kThreads, 1, stream, sp);
         if (e != cudaSuccess) return cuda_fail(e, "accept_stats_kernel launch");
         if (P.phases == 1) break;
         tp.ph = ph;
@@ -983,7 +998,7 @@ cs_status launch_typed(StatsParams sp, TestParams tp, WalkParams p, const Accept
             sp.mass_lo = ph.p0;
             sp.mass_hi = sp.n - 1;
             sp.by_R.set(0);
-            e = launch_after(accept_stats_kernel<T, G, true>, grid, 1, kThreads, 1, stream, sp);
+            e = launch_after(accept_stats_kernel<T, G, true, false>, grid, 1, kThreads, 1, stream, sp);
             if (e != cudaSuccess) return cuda_fail(e, "accept_stats_kernel launch");
         }
     }
