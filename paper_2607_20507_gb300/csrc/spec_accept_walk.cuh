@@ -70,6 +70,12 @@ __device__ __forceinline__ void load_run(const DrawRow<T>& d, int j, int V, int 
             r.t[u] = __ldg(reinterpret_cast<const uint4*>(d.rt + at) + u);
             r.d[u] = __ldg(reinterpret_cast<const uint4*>(d.rd + at) + u);
         }
+    } else if (d.same && whole_vectors(d.rt, V)) {
+#pragma unroll
+        for (int u = 0; u < kRunVecs; ++u) {
+            r.t[u] = load_or_ninf(d.rt, at + u * kPer, V);
+            r.d[u] = load_or_ninf(d.rd, at + u * kPer, V);
+        }
     } else {
         uint4 t[2 * kRunVecs];
         load_slow(d.rt, at, kPer, kRunVecs, V, t);

@@ -73,7 +73,7 @@ def test_phases_with_every_first_rejection_and_empty_residuals():
     assert (n == np.arange(B) % 10).all()
 
 
-@pytest.mark.parametrize("V", [1, 2, 9, 511, 513, 1025, 2049, 4097])
+@pytest.mark.parametrize("V", [1, 2, 8, 9, 511, 513, 1025, 1032, 2040, 2049, 4097, 4104])
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 def test_vocabularies_around_a_block(V, dtype):
     for T in (0.0, 0.9):
