@@ -82,26 +82,36 @@ bool stream_of(PyObject* o, c10::Device dev, cs_stream_t* s) {
 enum Kind { kAttn, kTreeAttn, kAccept, kTreeAccept, kSample, kRoute };
 const char* const kKinds[] = {"attn", "tree_attn", "accept", "tree_accept", "sample", "route"};
 
+// Scratch of a call; `hold` is the kept workspace it lies in.
+struct Scratch {
+    void* ptr = nullptr;
+    size_t bytes = 0;
+    at::Tensor hold;
+};
+
 // The caller's workspace, or the one that binding.py keeps for the size.
-bool workspace(PyObject* o, Kind kind, c10::Device dev, size_t bytes, void** ptr, size_t* size) {
+// Asking binding.py runs Python code, in which another thread may come here:
+// nothing of the map is held meanwhile.
+bool workspace(PyObject* o, Kind kind, c10::Device dev, size_t bytes, Scratch* w) {
     if (o != Py_None) {
         if (!THPVariable_CheckExact(o)) return false;
-        const at::Tensor& t = THPVariable_Unpack(o);
-        *ptr = t.data_ptr();
-        *size = t.nbytes();
-        return true;
+        w->hold = THPVariable_Unpack(o);
+    } else {
+        static auto* kept = new std::map<std::tuple<int, int, size_t>, at::Tensor>;   // under the interpreter lock
+        const std::tuple<int, int, size_t> key{(int)kind, (int)dev.index(), bytes};
+        const auto it = kept->find(key);
+        if (it != kept->end()) {
+            w->hold = it->second;
+        } else {
+            PyObject* r = PyObject_CallFunction(g_workspace_of, "sin", kKinds[kind], (int)dev.index(), (Py_ssize_t)bytes);
+            if (!r) throw python_error();
+            w->hold = THPVariable_Unpack(r);
+            Py_DECREF(r);
+            kept->emplace(key, w->hold);   // (a reference: binding.py owns the workspace)
+        }
     }
-    static auto* kept = new std::map<std::tuple<int, int, size_t>, at::Tensor>;   // under the interpreter lock
-    if (kept->size() >= 64) kept->clear();   // (references only: binding.py owns the workspaces)
-    at::Tensor& t = (*kept)[{(int)kind, (int)dev.index(), bytes}];
-    if (!t.defined()) {
-        PyObject* r = PyObject_CallFunction(g_workspace_of, "sin", kKinds[kind], (int)dev.index(), (Py_ssize_t)bytes);
-        if (!r) throw python_error();
-        t = THPVariable_Unpack(r);
-        Py_DECREF(r);
-    }
-    *ptr = t.data_ptr();
-    *size = t.nbytes();
+    w->ptr = w->hold.data_ptr();
+    w->bytes = w->hold.nbytes();
     return true;
 }
 
@@ -154,19 +164,19 @@ PyObject* attention(PyObject* const* a, bool tree) {
     if (a[6] != Py_None && !need(a[6], at::kBFloat16, 4, dev, &o)) Py_RETURN_NONE;
     const cs_attn_dims d{(int32_t)q->size(0), (int32_t)q->size(2), (int32_t)k->size(1), (int32_t)q->size(3),
                          (int32_t)k->size(2), (int32_t)table->size(1), (int32_t)k->size(0), scale};
-    void* ws;
+    Scratch ws;
     size_t bytes = 0;
     if (a[7] == Py_None)
         bytes = tree ? cs_tree_verify_attention_workspace_bytes(&d, (int32_t)rows)
                      : cs_verify_attention_workspace_bytes(&d, n_draft);
-    if (!workspace(a[7], tree ? kTreeAttn : kAttn, dev, bytes, &ws, &bytes)) Py_RETURN_NONE;
+    if (!workspace(a[7], tree ? kTreeAttn : kAttn, dev, bytes, &ws)) Py_RETURN_NONE;
     const at::Tensor out = a[6] == Py_None ? at::empty_like(*q) : *o;
     const int32_t *tp = (const int32_t*)table->data_ptr(), *lp = (const int32_t*)lens->data_ptr();
     const cs_status st =
         tree ? cs_tree_verify_attention(&d, q->data_ptr(), k->data_ptr(), v->data_ptr(), tp, lp,
-                                        (const int32_t*)par->data_ptr(), (int32_t)rows, out.data_ptr(), ws, bytes, s)
+                                        (const int32_t*)par->data_ptr(), (int32_t)rows, out.data_ptr(), ws.ptr, ws.bytes, s)
              : cs_verify_attention(&d, q->data_ptr(), k->data_ptr(), v->data_ptr(), tp, lp, n_draft, out.data_ptr(),
-                                   ws, bytes, s);
+                                   ws.ptr, ws.bytes, s);
     if (st != CS_OK) return status(st);
     return a[6] == Py_None ? THPVariable_Wrap(out) : Py_NewRef(a[6]);
 }
@@ -194,15 +204,15 @@ CALL(spec_accept, 9)
         Py_RETURN_NONE;
     const cs_accept_dims d{(int32_t)B, (int32_t)V, t->scalar_type() == at::kFloat ? CS_F32 : CS_BF16};
     at::Tensor tokens, count;
-    void* ws;
-    size_t bytes = a[7] == Py_None ? cs_spec_accept_workspace_bytes(&d, (int32_t)k) : 0;
+    Scratch ws;
+    const size_t bytes = a[7] == Py_None ? cs_spec_accept_workspace_bytes(&d, (int32_t)k) : 0;
     if (!output(a[5], {B, k + 1}, dev, &tokens) || !output(a[6], {B}, dev, &count) ||
-        !workspace(a[7], kAccept, dev, bytes, &ws, &bytes))
+        !workspace(a[7], kAccept, dev, bytes, &ws))
         Py_RETURN_NONE;
     const cs_status st =
         cs_spec_accept(&d, t->data_ptr(), q ? q->data_ptr() : nullptr, (const int32_t*)x->data_ptr(),
                        (const float*)u->data_ptr(), (int32_t)k, T, (int32_t*)tokens.data_ptr(),
-                       (int32_t*)count.data_ptr(), ws, bytes, s);
+                       (int32_t*)count.data_ptr(), ws.ptr, ws.bytes, s);
     return st != CS_OK ? status(st) : pair(tokens, count);
 CALL_END
 
@@ -221,15 +231,15 @@ CALL(tree_accept, 11)
         if (y->size(0) != B || y->size(1) != n) Py_RETURN_NONE;
     const cs_accept_dims d{(int32_t)B, (int32_t)t->size(2), t->scalar_type() == at::kFloat ? CS_F32 : CS_BF16};
     at::Tensor tokens, path, count;
-    void* ws;
-    size_t bytes = a[9] == Py_None ? cs_tree_accept_workspace_bytes(&d, (int32_t)n) : 0;
+    Scratch ws;
+    const size_t bytes = a[9] == Py_None ? cs_tree_accept_workspace_bytes(&d, (int32_t)n) : 0;
     if (!output(a[6], {B, n}, dev, &tokens) || !output(a[7], {B, n}, dev, &path) || !output(a[8], {B}, dev, &count) ||
-        !workspace(a[9], kTreeAccept, dev, bytes, &ws, &bytes))
+        !workspace(a[9], kTreeAccept, dev, bytes, &ws))
         Py_RETURN_NONE;
     const cs_status st =
         cs_tree_accept(&d, t->data_ptr(), q ? q->data_ptr() : nullptr, (const int32_t*)par->data_ptr(),
                        (const int32_t*)x->data_ptr(), (const float*)u->data_ptr(), (int32_t)n, T,
-                       (int32_t*)tokens.data_ptr(), (int32_t*)path.data_ptr(), (int32_t*)count.data_ptr(), ws, bytes, s);
+                       (int32_t*)tokens.data_ptr(), (int32_t*)path.data_ptr(), (int32_t*)count.data_ptr(), ws.ptr, ws.bytes, s);
     if (st != CS_OK) return status(st);
     return Py_BuildValue("(NNN)", THPVariable_Wrap(tokens), THPVariable_Wrap(path), THPVariable_Wrap(count));
 CALL_END
@@ -245,11 +255,11 @@ CALL(sample, 6)
         Py_RETURN_NONE;
     const cs_accept_dims d{(int32_t)z->size(0), (int32_t)z->size(1), z->scalar_type() == at::kFloat ? CS_F32 : CS_BF16};
     at::Tensor tokens;
-    void* ws;
-    size_t bytes = a[4] == Py_None ? cs_sample_workspace_bytes(&d) : 0;
-    if (!output(a[3], {z->size(0)}, dev, &tokens) || !workspace(a[4], kSample, dev, bytes, &ws, &bytes)) Py_RETURN_NONE;
-    const cs_status st = cs_sample(&d, z->data_ptr(), (const float*)u->data_ptr(), T, (int32_t*)tokens.data_ptr(), ws,
-                                   bytes, s);
+    Scratch ws;
+    const size_t bytes = a[4] == Py_None ? cs_sample_workspace_bytes(&d) : 0;
+    if (!output(a[3], {z->size(0)}, dev, &tokens) || !workspace(a[4], kSample, dev, bytes, &ws)) Py_RETURN_NONE;
+    const cs_status st = cs_sample(&d, z->data_ptr(), (const float*)u->data_ptr(), T, (int32_t*)tokens.data_ptr(), ws.ptr,
+                                   ws.bytes, s);
     return st != CS_OK ? status(st) : THPVariable_Wrap(tokens);
 CALL_END
 
@@ -265,14 +275,14 @@ CALL(route, 6)
         Py_RETURN_NONE;
     const int64_t B = e->size(0);
     const cs_route_dims d{(int32_t)B, (int32_t)c->size(0), (int32_t)e->size(1)};
-    void* ws;
-    size_t bytes = a[4] == Py_None ? cs_route_workspace_bytes(&d) : 0;
-    if (!workspace(a[4], kRoute, dev, bytes, &ws, &bytes)) Py_RETURN_NONE;
+    Scratch ws;
+    const size_t bytes = a[4] == Py_None ? cs_route_workspace_bytes(&d) : 0;
+    if (!workspace(a[4], kRoute, dev, bytes, &ws)) Py_RETURN_NONE;
     const at::Tensor group = ints({B}, dev), best = ints({B}, dev),
                      score = at::empty({B}, at::TensorOptions(at::kFloat).device(dev));
     const cs_status st = cs_route(&d, e->data_ptr(), c->data_ptr(), (const float*)inv->data_ptr(), tau,
-                                  (int32_t*)group.data_ptr(), (int32_t*)best.data_ptr(), (float*)score.data_ptr(), ws,
-                                  bytes, s);
+                                  (int32_t*)group.data_ptr(), (int32_t*)best.data_ptr(), (float*)score.data_ptr(), ws.ptr,
+                                  ws.bytes, s);
     if (st != CS_OK) return status(st);
     return Py_BuildValue("(NNN)", THPVariable_Wrap(group), THPVariable_Wrap(best), THPVariable_Wrap(score));
 CALL_END

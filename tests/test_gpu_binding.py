@@ -1,6 +1,10 @@
 """The binding's compiled marshalling: given outputs, workspaces and streams
 are used, and an argument that a call does not take raises what the Python
 checks raise."""
+import random
+import sys
+import threading
+
 import pytest
 import torch
 
@@ -61,3 +65,44 @@ def test_refusals():
         binding.cs_sample(c[0][:, 0].contiguous().half(), c[3][:, 0].contiguous(), 1.0)
     with pytest.raises(TypeError):
         binding.cs_kv_commit(a[4].long(), a[4], 3)
+
+
+def run_threads(works):
+    """Each callable in a thread of its own; the first exception is raised here."""
+    errors = []
+
+    def guarded(f):
+        try:
+            f()
+        except BaseException as e:   # noqa: BLE001
+            errors.append(e)
+
+    threads = [threading.Thread(target=guarded, args=(f,)) for f in works]
+    before = sys.getswitchinterval()
+    sys.setswitchinterval(1e-6)
+    try:
+        for t in threads:
+            t.start()
+        for t in threads:
+            t.join()
+    finally:
+        sys.setswitchinterval(before)
+    if errors:
+        raise errors[0]
+
+
+def test_more_workspaces_than_one_thread_can_keep():
+    """Over a hundred default workspaces of different sizes, taken by three threads at a time."""
+    z = torch.randn((120, 128256), device=DEV).to(torch.bfloat16)
+    u = torch.zeros((120,), device=DEV)
+    top = (z == z.max(dim=1, keepdim=True).values).int().argmax(dim=1).int()   # the lowest of equal ids
+    torch.cuda.synchronize()
+
+    def work(seed):
+        sizes = list(range(1, 121))
+        random.Random(seed).shuffle(sizes)
+        got = [(b, binding.cs_sample(z[:b], u[:b], 0.0)) for b in sizes]
+        for b, t in got:
+            assert torch.equal(t, top[:b]), b
+
+    run_threads([lambda s=s: work(s) for s in range(3)])
