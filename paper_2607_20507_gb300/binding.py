@@ -210,6 +210,9 @@ _workspaces: dict = {}
 
 
 def _cached_workspace(kind: str, device, n: int) -> torch.Tensor:
+    device = torch.device(device)   # "cuda:0", "cuda" and the device itself are one key
+    if device.index is None and device.type == "cuda":
+        device = torch.device("cuda", torch.cuda.current_device())
     key = (kind, device, n)
     ws = _workspaces.get(key)
     if ws is None:

@@ -106,3 +106,13 @@ def test_more_workspaces_than_one_thread_can_keep():
             assert torch.equal(t, top[:b]), b
 
     run_threads([lambda s=s: work(s) for s in range(3)])
+
+
+def test_default_workspace_by_any_name_of_its_device():
+    """A caller reads the status of its default calls from the workspace that they use."""
+    a, c = inputs()
+    d = binding.attn_dims(a[0], a[1], a[3])
+    binding.cs_verify_attention(*a, 3)
+    ws = [binding.verify_attention_workspace(d, 3, dev) for dev in (DEV, "cuda", torch.device(DEV), a[0].device)]
+    assert len({w.data_ptr() for w in ws}) == 1
+    assert torch.count_nonzero(ws[0]).item() > 0 and binding.cs_read_device_status(ws[0]) == 0
