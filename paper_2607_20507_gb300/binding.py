@@ -10,6 +10,7 @@ checks and passes on what it does not take to the code here.
 """
 from __future__ import annotations
 
+import contextlib
 import ctypes
 import importlib.machinery
 import importlib.util
@@ -148,7 +149,7 @@ def _load_fast():
             mod = importlib.util.module_from_spec(importlib.util.spec_from_file_location(name, _build.MARSHAL,
                                                                                          loader=loader))
             loader.exec_module(mod)
-            mod.use_workspaces(lambda kind, index, n: _cached_workspace(kind, torch.device("cuda", index), n))
+            mod.use_workspaces(lambda kind, index, n, stream: _workspace_of(kind, torch.device("cuda", index), n, stream))
             _fast = mod
     return _fast
 
@@ -203,25 +204,55 @@ def attn_dims(q: torch.Tensor, k_pages: torch.Tensor, page_table: torch.Tensor,
     return AttnDims(B, Hq, Hkv, D, ps, page_table.shape[1], P, float(sm_scale))
 
 
-# Workspaces handed out by this module, one per (kind, device, size).  The kernels
-# leave a workspace ready for the next call, so calls ordered on one stream
-# may share it.
+# Workspaces handed out by this module, one per (kind, device, stream, size): the
+# kernels leave a workspace ready for the next call, so calls ordered on one
+# stream may share it, and calls on two streams may not.  They stay for the
+# process's life (a captured graph holds their addresses).
 _workspaces: dict = {}
+_WITH_STATUS = ("attn", "tree_attn", "route")   # whose first word has to start at zero
 
 
-def _cached_workspace(kind: str, device, n: int) -> torch.Tensor:
+def _made_on(stream: int, device):
+    """The context in which a new workspace's memory, and its zero fill, are ordered with the calls on ``stream``."""
+    if device.type != "cuda" or stream == _stream(device):
+        return contextlib.nullcontext()
+    if stream in (0, 1):   # the legacy default stream's two handles
+        return torch.cuda.stream(torch.cuda.default_stream(device))
+    return torch.cuda.stream(torch.cuda.ExternalStream(stream, device=device))
+
+
+def _workspace_of(kind: str, device, n: int, stream: int | None = None):
+    """(workspace, whether it is the stream's own)"""
     device = torch.device(device)   # "cuda:0", "cuda" and the device itself are one key
     if device.index is None and device.type == "cuda":
         device = torch.device("cuda", torch.cuda.current_device())
-    key = (kind, device, n)
+    here = _stream(device) if device.type == "cuda" else 0
+    if stream is None:
+        stream = here
+    else:   # as ctypes takes it
+        stream = (stream if isinstance(stream, ctypes.c_void_p) else ctypes.c_void_p(stream)).value or 0
+    key = (kind, device, stream, n)
     ws = _workspaces.get(key)
-    if ws is None:
-        ws = torch.zeros(max(n, 256), dtype=torch.uint8, device=device)
-        _workspaces[key] = ws
-    return ws
+    if ws is not None:
+        return ws, True
+    if kind in _WITH_STATUS and stream == here and device.type == "cuda" and torch.cuda.is_current_stream_capturing():
+        # a zero fill would become a part of the graph, so a captured call takes
+        # the workspace of the calls before the capture (with whose stream the
+        # graph's replays have to be ordered)
+        for (k, d, _, m), ws in list(_workspaces.items()):
+            if (k, d, m) == (kind, device, n):
+                return ws, False
+    with _made_on(stream, device):
+        ws = (torch.zeros if kind in _WITH_STATUS else torch.empty)(max(n, 256), dtype=torch.uint8, device=device)
+    return _workspaces.setdefault(key, ws), True
+
+
+def _cached_workspace(kind: str, device, n: int, stream: int | None = None) -> torch.Tensor:
+    return _workspace_of(kind, device, n, stream)[0]
 
 
 def verify_attention_workspace(dims: AttnDims, n_draft: int, device) -> torch.Tensor:
+    """The default workspace of the current stream's calls."""
     n = load_library().cs_verify_attention_workspace_bytes(ctypes.byref(dims), int(n_draft))
     return _cached_workspace("attn", device, n)
 
@@ -256,7 +287,8 @@ def cs_verify_attention(q, k_pages, v_pages, page_table, ctx_lens, n_draft, out=
     else:
         _need(out, "out", torch.bfloat16, 4, dev)
     if workspace is None:
-        workspace = verify_attention_workspace(d, n_draft, dev)
+        workspace = _cached_workspace("attn", dev, lib.cs_verify_attention_workspace_bytes(ctypes.byref(d), int(n_draft)),
+                                      stream)
     st = lib.cs_verify_attention(ctypes.byref(d), q.data_ptr(), k_pages.data_ptr(), v_pages.data_ptr(),
                                  page_table.data_ptr(), ctx_lens.data_ptr(), int(n_draft), out.data_ptr(),
                                  workspace.data_ptr(), workspace.nbytes,
@@ -267,6 +299,7 @@ def cs_verify_attention(q, k_pages, v_pages, page_table, ctx_lens, n_draft, out=
 
 
 def spec_accept_workspace(dims: AcceptDims, n_draft: int, device) -> torch.Tensor:
+    """The default workspace of the current stream's calls."""
     n = load_library().cs_spec_accept_workspace_bytes(ctypes.byref(dims), int(n_draft))
     return _cached_workspace("accept", device, n)
 
@@ -303,7 +336,7 @@ def cs_spec_accept(target_logits, draft_logits, draft_tokens, uniforms, temperat
         _need(out_n_accepted, "out_n_accepted", torch.int32, 1, dev)
     d = AcceptDims(B, V, CS_F32 if dtype == torch.float32 else CS_BF16)
     if workspace is None:
-        workspace = spec_accept_workspace(d, k, dev)
+        workspace = _cached_workspace("accept", dev, lib.cs_spec_accept_workspace_bytes(ctypes.byref(d), int(k)), stream)
     st = lib.cs_spec_accept(ctypes.byref(d), target_logits.data_ptr(), _ptr(draft_logits),
                             draft_tokens.data_ptr(), uniforms.data_ptr(), int(k), float(temperature),
                             out_tokens.data_ptr(), out_n_accepted.data_ptr(), workspace.data_ptr(),
@@ -393,7 +426,7 @@ def cs_route(emb, centroids, inv_norms, tau, out_group=None, out_best=None, out_
     out_score = inv_norms.new_empty((B,)) if out_score is None else out_score
     dims = RouteDims(B, N, d)
     if workspace is None:
-        workspace = _cached_workspace("route", dev, lib.cs_route_workspace_bytes(ctypes.byref(dims)))
+        workspace = _cached_workspace("route", dev, lib.cs_route_workspace_bytes(ctypes.byref(dims)), stream)
     st = lib.cs_route(ctypes.byref(dims), emb.data_ptr(), centroids.data_ptr() if N else None,
                       inv_norms.data_ptr() if N else None,
                       float(tau), out_group.data_ptr(), out_best.data_ptr(), out_score.data_ptr(), workspace.data_ptr(),
@@ -423,7 +456,7 @@ def cs_sample(logits, uniforms, temperature, out_tokens=None, workspace=None,
         _need(out_tokens, "out_tokens", torch.int32, 1, dev)
     d = AcceptDims(B, V, CS_F32 if logits.dtype == torch.float32 else CS_BF16)
     if workspace is None:
-        workspace = _cached_workspace("sample", dev, lib.cs_sample_workspace_bytes(ctypes.byref(d)))
+        workspace = _cached_workspace("sample", dev, lib.cs_sample_workspace_bytes(ctypes.byref(d)), stream)
     st = lib.cs_sample(ctypes.byref(d), logits.data_ptr(), uniforms.data_ptr(), float(temperature),
                        out_tokens.data_ptr(),
                        workspace.data_ptr(), workspace.nbytes,
@@ -461,7 +494,7 @@ def cs_tree_verify_attention(q, k_pages, v_pages, page_table, ctx_lens, parents,
         _need(out, "out", torch.bfloat16, 4, dev)
     if workspace is None:
         workspace = _cached_workspace("tree_attn", dev,
-                                      lib.cs_tree_verify_attention_workspace_bytes(ctypes.byref(d), int(n)))
+                                      lib.cs_tree_verify_attention_workspace_bytes(ctypes.byref(d), int(n)), stream)
     st = lib.cs_tree_verify_attention(ctypes.byref(d), q.data_ptr(), k_pages.data_ptr(), v_pages.data_ptr(),
                                       page_table.data_ptr(), ctx_lens.data_ptr(), parents.data_ptr(), int(n),
                                       out.data_ptr(), workspace.data_ptr(), workspace.nbytes,
@@ -509,7 +542,8 @@ def cs_tree_accept(target_logits, draft_logits, parents, node_tokens, uniforms, 
         _need(out_n_accepted, "out_n_accepted", torch.int32, 1, dev)
     d = AcceptDims(B, V, CS_F32 if dtype == torch.float32 else CS_BF16)
     if workspace is None:
-        workspace = _cached_workspace("tree_accept", dev, lib.cs_tree_accept_workspace_bytes(ctypes.byref(d), int(n)))
+        workspace = _cached_workspace("tree_accept", dev, lib.cs_tree_accept_workspace_bytes(ctypes.byref(d), int(n)),
+                                      stream)
     st = lib.cs_tree_accept(ctypes.byref(d), target_logits.data_ptr(), _ptr(draft_logits), parents.data_ptr(),
                             node_tokens.data_ptr(), uniforms.data_ptr(), int(n), float(temperature),
                             out_tokens.data_ptr(),

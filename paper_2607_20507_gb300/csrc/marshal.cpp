@@ -24,7 +24,7 @@
 
 namespace {
 
-// binding._cached_workspace(kind, device_index, bytes) -> Tensor
+// binding._workspace_of(kind, device_index, bytes, stream) -> (Tensor, whether to keep it)
 PyObject* g_workspace_of = nullptr;
 
 // A device tensor of the given type and rank, contiguous, on the device of
@@ -89,25 +89,27 @@ struct Scratch {
     at::Tensor hold;
 };
 
-// The caller's workspace, or the one that binding.py keeps for the size.
+// The caller's workspace, or the one that binding.py keeps for the size and the stream.
 // Asking binding.py runs Python code, in which another thread may come here:
 // nothing of the map is held meanwhile.
-bool workspace(PyObject* o, Kind kind, c10::Device dev, size_t bytes, Scratch* w) {
+bool workspace(PyObject* o, Kind kind, c10::Device dev, size_t bytes, cs_stream_t s, Scratch* w) {
     if (o != Py_None) {
         if (!THPVariable_CheckExact(o)) return false;
         w->hold = THPVariable_Unpack(o);
     } else {
-        static auto* kept = new std::map<std::tuple<int, int, size_t>, at::Tensor>;   // under the interpreter lock
-        const std::tuple<int, int, size_t> key{(int)kind, (int)dev.index(), bytes};
+        using Key = std::tuple<int, int, size_t, cs_stream_t>;
+        static auto* kept = new std::map<Key, at::Tensor>;   // under the interpreter lock
+        const Key key{(int)kind, (int)dev.index(), bytes, s};
         const auto it = kept->find(key);
         if (it != kept->end()) {
             w->hold = it->second;
         } else {
-            PyObject* r = PyObject_CallFunction(g_workspace_of, "sin", kKinds[kind], (int)dev.index(), (Py_ssize_t)bytes);
+            PyObject* r = PyObject_CallFunction(g_workspace_of, "sinK", kKinds[kind], (int)dev.index(), (Py_ssize_t)bytes,
+                                                (unsigned long long)reinterpret_cast<uintptr_t>(s));
             if (!r) throw python_error();
-            w->hold = THPVariable_Unpack(r);
+            w->hold = THPVariable_Unpack(PyTuple_GET_ITEM(r, 0));
+            if (PyTuple_GET_ITEM(r, 1) == Py_True) kept->emplace(key, w->hold);   // (binding.py owns the workspace)
             Py_DECREF(r);
-            kept->emplace(key, w->hold);   // (a reference: binding.py owns the workspace)
         }
     }
     w->ptr = w->hold.data_ptr();
@@ -169,7 +171,7 @@ PyObject* attention(PyObject* const* a, bool tree) {
     if (a[7] == Py_None)
         bytes = tree ? cs_tree_verify_attention_workspace_bytes(&d, (int32_t)rows)
                      : cs_verify_attention_workspace_bytes(&d, n_draft);
-    if (!workspace(a[7], tree ? kTreeAttn : kAttn, dev, bytes, &ws)) Py_RETURN_NONE;
+    if (!workspace(a[7], tree ? kTreeAttn : kAttn, dev, bytes, s, &ws)) Py_RETURN_NONE;
     const at::Tensor out = a[6] == Py_None ? at::empty_like(*q) : *o;
     const int32_t *tp = (const int32_t*)table->data_ptr(), *lp = (const int32_t*)lens->data_ptr();
     const cs_status st =
@@ -207,7 +209,7 @@ CALL(spec_accept, 9)
     Scratch ws;
     const size_t bytes = a[7] == Py_None ? cs_spec_accept_workspace_bytes(&d, (int32_t)k) : 0;
     if (!output(a[5], {B, k + 1}, dev, &tokens) || !output(a[6], {B}, dev, &count) ||
-        !workspace(a[7], kAccept, dev, bytes, &ws))
+        !workspace(a[7], kAccept, dev, bytes, s, &ws))
         Py_RETURN_NONE;
     const cs_status st =
         cs_spec_accept(&d, t->data_ptr(), q ? q->data_ptr() : nullptr, (const int32_t*)x->data_ptr(),
@@ -234,7 +236,7 @@ CALL(tree_accept, 11)
     Scratch ws;
     const size_t bytes = a[9] == Py_None ? cs_tree_accept_workspace_bytes(&d, (int32_t)n) : 0;
     if (!output(a[6], {B, n}, dev, &tokens) || !output(a[7], {B, n}, dev, &path) || !output(a[8], {B}, dev, &count) ||
-        !workspace(a[9], kTreeAccept, dev, bytes, &ws))
+        !workspace(a[9], kTreeAccept, dev, bytes, s, &ws))
         Py_RETURN_NONE;
     const cs_status st =
         cs_tree_accept(&d, t->data_ptr(), q ? q->data_ptr() : nullptr, (const int32_t*)par->data_ptr(),
@@ -257,7 +259,7 @@ CALL(sample, 6)
     at::Tensor tokens;
     Scratch ws;
     const size_t bytes = a[4] == Py_None ? cs_sample_workspace_bytes(&d) : 0;
-    if (!output(a[3], {z->size(0)}, dev, &tokens) || !workspace(a[4], kSample, dev, bytes, &ws)) Py_RETURN_NONE;
+    if (!output(a[3], {z->size(0)}, dev, &tokens) || !workspace(a[4], kSample, dev, bytes, s, &ws)) Py_RETURN_NONE;
     const cs_status st = cs_sample(&d, z->data_ptr(), (const float*)u->data_ptr(), T, (int32_t*)tokens.data_ptr(), ws.ptr,
                                    ws.bytes, s);
     return st != CS_OK ? status(st) : THPVariable_Wrap(tokens);
@@ -277,7 +279,7 @@ CALL(route, 6)
     const cs_route_dims d{(int32_t)B, (int32_t)c->size(0), (int32_t)e->size(1)};
     Scratch ws;
     const size_t bytes = a[4] == Py_None ? cs_route_workspace_bytes(&d) : 0;
-    if (!workspace(a[4], kRoute, dev, bytes, &ws)) Py_RETURN_NONE;
+    if (!workspace(a[4], kRoute, dev, bytes, s, &ws)) Py_RETURN_NONE;
     const at::Tensor group = ints({B}, dev), best = ints({B}, dev),
                      score = at::empty({B}, at::TensorOptions(at::kFloat).device(dev));
     const cs_status st = cs_route(&d, e->data_ptr(), c->data_ptr(), (const float*)inv->data_ptr(), tau,

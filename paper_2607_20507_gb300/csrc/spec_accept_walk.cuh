@@ -290,9 +290,11 @@ __global__ void __launch_bounds__(kWalkMaxThreads, 2) accept_walk_kernel(const W
         node = depth = p.ph.p0;
         have = (p.ph.t_rows < 64 ? (1ull << p.ph.t_rows) - 1ull : ~0ull) << p.ph.p0;
         if (p.ph.undecided) {
-            const int a = __ldcg(p.dec.a + b);
+            // (every request is decided: the calls read in phases end with one more
+            // test; the bounds are for a workspace that another call writes at the
+            // same time, whose tokens are undefined but whose reads are not)
+            const int a = max(0, min(__ldcg(p.dec.a + b), n - 1));
             const float4 st = __ldcg(p.dec.stat + b);
-            // (every request is: the calls read in phases end with one more test)
             decided = true;
             node = depth = a;
             kappa = a + 1 < n ? 1.f : 0.f;

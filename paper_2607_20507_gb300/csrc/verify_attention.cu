@@ -970,6 +970,8 @@ verify_attention_merge_cut_kernel(const AttnParams p, int n_slots) {
                 r0 = 2 * c;
             }
         }
+        // (an id of another call's, in a workspace that it writes at the same time, is no span here)
+        if (id >= p.n_vh * p.n_batch) id = -1;
         int n_p = 0;
         if (id >= 0) {
             n_p = 1;

@@ -8,6 +8,7 @@ import threading
 import pytest
 import torch
 
+import bench
 from paper_2607_20507_gb300 import binding
 from paper_2607_20507_gb300 import workloads as W
 
@@ -116,3 +117,81 @@ def test_default_workspace_by_any_name_of_its_device():
     ws = [binding.verify_attention_workspace(d, 3, dev) for dev in (DEV, "cuda", torch.device(DEV), a[0].device)]
     assert len({w.data_ptr() for w in ws}) == 1
     assert torch.count_nonzero(ws[0]).item() > 0 and binding.cs_read_device_status(ws[0]) == 0
+
+
+def test_two_streams_share_nothing():
+    """The same calls on two streams, with nothing between them, on different inputs: as one after the other.
+    The acceptance is long enough to be read in phases, whose decisions are in the workspace."""
+    def case(seed):
+        kw = dict(vocab=128256, logit_dtype="bf16", draft_sigma=0.7, temperatures=(0.8,), n_q_heads=16, n_kv_heads=4,
+                  head_dim=128, page_size=16)
+        wa = W.Workload(95, "streams", batch=40, n_draft=8, ctx=("uniform", 100, 3000), cell=seed, **kw)
+        wc = W.Workload(95, "streams", batch=160, n_draft=8, ctx=("const", 64), cell=seed, **kw)
+        a, c = W.attention_inputs(wa, DEV), W.accept_inputs(wc, 0.8, DEV)
+        r = W.route_inputs(W.RouteWorkload(30, "streams", 300, 2000, 384), DEV, seed=seed)
+        return ([a[k] for k in ("q", "k_pages", "v_pages", "page_table", "ctx_lens")],
+                [c[k] for k in ("target", "draft", "draft_tokens", "uniforms")],
+                (r["emb"], r["centroids"], binding.cs_route_norms(r["centroids"])))
+
+    def calls(x):
+        a, c, r = x
+        return (binding.cs_verify_attention(*a, 8), *binding.cs_spec_accept(*c, 0.8),
+                binding.cs_sample(c[0][:, 0].contiguous(), c[3][:, 0].contiguous(), 0.8),
+                *binding.cs_route(*r, W.ROUTE_TAU))
+
+    x = [case(s) for s in (1, 2)]
+    expect = [calls(v) for v in x]
+    torch.cuda.synchronize()
+    streams = [torch.cuda.Stream() for _ in x]
+    got = [[], []]
+    for _ in range(12):
+        for i, s in enumerate(streams):
+            with torch.cuda.stream(s):
+                got[i].append(calls(x[i]))
+    torch.cuda.synchronize()
+    for i in range(2):
+        for g in got[i]:
+            for u, v in zip(g, expect[i]):
+                assert torch.equal(u, v)
+
+
+def test_capture_adds_no_fill():
+    """Captured after the same calls, with default workspaces: the calls' own kernels and nothing else."""
+    a, c = inputs()
+    r = W.route_inputs(W.RouteWorkload(30, "capture", 70, 300, 128), DEV, seed=2)
+    route = (r["emb"], r["centroids"], binding.cs_route_norms(r["centroids"]))
+    z, u = c[0][:, 0].contiguous(), c[3][:, 0].contiguous()
+
+    def step():
+        return (binding.cs_verify_attention(*a, 3), *binding.cs_spec_accept(*c, 0.8), binding.cs_sample(z, u, 0.8),
+                *binding.cs_route(*route, W.ROUTE_TAU))
+
+    expect = step()
+    assert bench.kernel_launches(step) == 8   # two each
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        got = step()
+    for _ in range(3):
+        g.replay()
+    torch.cuda.synchronize()
+    for x, y in zip(got, expect):
+        assert torch.equal(x, y)
+
+
+def test_new_workspace_is_filled_on_its_stream():
+    """With the current stream busy, the zero fill of a new workspace does not come after the call that uses it."""
+    a, c = inputs()
+    a = [a[0][:2].contiguous(), *a[1:3], a[3][:2].contiguous(), a[4][:2].contiguous()]
+    expect = binding.cs_verify_attention(*a, 3)
+    d = binding.attn_dims(a[0], a[1], a[3])
+    out, side = torch.empty_like(expect), torch.cuda.Stream()
+    torch.cuda.synchronize()
+    torch.cuda._sleep(100_000_000)   # about 50 ms
+    binding.cs_verify_attention(*a, 3, out=out, stream=side.cuda_stream)
+    with torch.cuda.stream(side):
+        ws = binding.verify_attention_workspace(d, 3, DEV)
+        early = ws.clone()
+        assert torch.equal(out, expect)
+    torch.cuda.synchronize()
+    assert torch.count_nonzero(early).item() > 0 and torch.equal(ws, early)
+    assert ws.data_ptr() != binding.verify_attention_workspace(d, 3, DEV).data_ptr()
