@@ -39,7 +39,10 @@
  *     frees or synchronises (except the status reads cs_read_device_status
  *     and cs_verify_attention_noalloc_status, which say so).
  *   - Calls are asynchronous on `stream` (a cudaStream_t; NULL is the legacy
- *     default stream) and return once the work is enqueued.
+ *     default stream) and return once the work is enqueued.  Any host threads
+ *     may call; the kernels of one call follow each other on its stream with
+ *     none of another call's between them, so calls of several threads on one
+ *     stream are ordered in the sense that sharing a workspace asks for.
  *   - Arguments are checked on the host before anything is enqueued; a bad
  *     argument returns an error code and enqueues nothing.  Values that live
  *     in device memory (context lengths, page ids, token ids) cannot be

@@ -7,6 +7,9 @@
 #include <stdio.h>
 #include <string.h>
 
+#include <atomic>
+#include <new>
+
 #include "cs_internal.h"
 
 namespace cs {
@@ -19,6 +22,39 @@ bool aligned(const void* p, size_t a) { return (reinterpret_cast<uintptr_t>(p) %
 
 bool pow2_page(int ps) {
     return ps == 8 || ps == 16 || ps == 32 || ps == 64 || ps == 128 || ps == 256;
+}
+
+// The turns of the streams seen so far.  A thread that blocks in a launch (the
+// stream's queue is full) holds no other stream's turn, so each stream has its
+// own; an entry stays (streams are few, and their handles come again).
+struct Turn {
+    int dev;
+    cudaStream_t stream;
+    Turn* next;
+    std::recursive_mutex m;
+};
+std::atomic<Turn*> g_turns{nullptr};
+std::mutex g_new_turn;
+std::recursive_mutex g_any_turn;   // a stream's for which there was no memory
+
+std::recursive_mutex& turn_of(cudaStream_t stream) {
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess) cudaGetLastError();
+    auto find = [&]() -> Turn* {
+        Turn* t = g_turns.load(std::memory_order_acquire);
+        while (t && (t->stream != stream || t->dev != dev)) t = t->next;
+        return t;
+    };
+    if (Turn* t = find()) return t->m;
+    std::lock_guard<std::mutex> lock(g_new_turn);
+    if (Turn* t = find()) return t->m;
+    Turn* t = new (std::nothrow) Turn;
+    if (!t) return g_any_turn;
+    t->dev = dev;
+    t->stream = stream;
+    t->next = g_turns.load(std::memory_order_relaxed);
+    g_turns.store(t, std::memory_order_release);
+    return t->m;
 }
 
 // Geometry checks shared by the chain and tree attention calls.
@@ -117,6 +153,8 @@ cs_status check_sample(const cs_accept_dims* d, float temperature) {
 }
 }  // namespace
 
+StreamTurn::StreamTurn(cudaStream_t stream) : turn_(turn_of(stream)) { turn_.lock(); }
+
 cs_status fail(cs_status st, const char* fmt, ...) {
     va_list ap;
     va_start(ap, fmt);
@@ -170,6 +208,7 @@ cs_status cs_verify_attention(const cs_attn_dims* dims, const void* q, const voi
         return fail(CS_ERR_WORKSPACE, "workspace of %zu bytes given, %zu needed", workspace_bytes,
                     plan.bytes);
     if (!aligned(workspace, 256)) return fail(CS_ERR_INVALID_ARG, "workspace must be 256-byte aligned");
+    const StreamTurn turn(reinterpret_cast<cudaStream_t>(stream));
     return launch_verify_attention(*dims, plan, q, k_pages, v_pages, page_table, ctx_lens, nullptr, out,
                                    workspace, reinterpret_cast<cudaStream_t>(stream));
 }
@@ -194,6 +233,7 @@ cs_status cs_tree_verify_attention(const cs_attn_dims* dims, const void* q, cons
     if (!workspace || workspace_bytes < plan.bytes)
         return fail(CS_ERR_WORKSPACE, "workspace of %zu bytes given, %zu needed", workspace_bytes, plan.bytes);
     if (!aligned(workspace, 256)) return fail(CS_ERR_INVALID_ARG, "workspace must be 256-byte aligned");
+    const StreamTurn turn(reinterpret_cast<cudaStream_t>(stream));
     return launch_verify_attention(*dims, plan, q, k_pages, v_pages, page_table, ctx_lens, parents, out,
                                    workspace, reinterpret_cast<cudaStream_t>(stream));
 }
@@ -228,6 +268,7 @@ cs_status cs_tree_accept(const cs_accept_dims* dims, const void* target_logits, 
     if (!workspace || workspace_bytes < need)
         return fail(CS_ERR_WORKSPACE, "workspace of %zu bytes given, %zu needed", workspace_bytes, need);
     if (!aligned(workspace, 256)) return fail(CS_ERR_INVALID_ARG, "workspace must be 256-byte aligned");
+    const StreamTurn turn(reinterpret_cast<cudaStream_t>(stream));
     return launch_tree_accept(*dims, target_logits, temperature > 0.f ? draft_logits : nullptr, parents, node_tokens,
                               uniforms, n_nodes, temperature, out_tokens, out_path, out_n_accepted, workspace,
                               reinterpret_cast<cudaStream_t>(stream));
@@ -284,6 +325,7 @@ cs_status cs_spec_accept(const cs_accept_dims* dims, const void* target_logits,
     if (!workspace || workspace_bytes < need)
         return fail(CS_ERR_WORKSPACE, "workspace of %zu bytes given, %zu needed", workspace_bytes, need);
     if (!aligned(workspace, 256)) return fail(CS_ERR_INVALID_ARG, "workspace must be 256-byte aligned");
+    const StreamTurn turn(reinterpret_cast<cudaStream_t>(stream));
     return launch_spec_accept(*dims, target_logits, temperature > 0.f ? draft_logits : nullptr,
                               draft_tokens, uniforms, n_draft, temperature, out_tokens,
                               out_n_accepted, workspace, reinterpret_cast<cudaStream_t>(stream));
@@ -359,6 +401,7 @@ cs_status cs_route(const cs_route_dims* dims, const void* emb, const void* centr
     if (!workspace || workspace_bytes < pl.bytes)
         return fail(CS_ERR_WORKSPACE, "workspace of %zu bytes given, %zu needed", workspace_bytes, pl.bytes);
     if (!aligned(workspace, 256)) return fail(CS_ERR_INVALID_ARG, "workspace must be 256-byte aligned");
+    const StreamTurn turn(reinterpret_cast<cudaStream_t>(stream));
     return launch_route(*dims, pl, emb, centroids, inv_norms, tau, out_group, out_best, out_score, workspace,
                         reinterpret_cast<cudaStream_t>(stream));
 }
@@ -385,6 +428,7 @@ cs_status cs_sample(const cs_accept_dims* dims, const void* logits, const float*
     if (!aligned(workspace, 256)) return fail(CS_ERR_INVALID_ARG, "workspace must be 256-byte aligned");
     // the acceptance path with no drafted positions: every request decides
     // a = 0 and draws its token from p_0 (or takes its argmax when T == 0)
+    const StreamTurn turn(reinterpret_cast<cudaStream_t>(stream));
     return launch_spec_accept(*dims, logits, nullptr, nullptr, uniforms, 0, temperature, out_tokens,
                               nullptr, workspace, reinterpret_cast<cudaStream_t>(stream));
 }

@@ -6,6 +6,8 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include <mutex>
+
 #include "cachespec.h"
 
 namespace cs {
@@ -16,6 +18,19 @@ cs_status cuda_fail(cudaError_t e, const char* what);
 
 // Streaming multiprocessors of the current device (cached per device).
 int current_sm_count();
+
+// Holds `stream` for the launches of one call, so that the calls of several
+// threads on one stream follow each other whole: they may share a workspace.
+class StreamTurn {
+public:
+    explicit StreamTurn(cudaStream_t stream);
+    ~StreamTurn() { turn_.unlock(); }
+    StreamTurn(const StreamTurn&) = delete;
+    StreamTurn& operator=(const StreamTurn&) = delete;
+
+private:
+    std::recursive_mutex& turn_;
+};
 
 // A launch that may start while the kernel before it in the stream runs
 // (the kernel waits with griddepcontrol.wait before it reads its inputs).

@@ -117,20 +117,33 @@ bool workspace(PyObject* o, Kind kind, c10::Device dev, size_t bytes, cs_stream_
     return true;
 }
 
+// The interpreter lock is not held while outputs are allocated and the library
+// launches: an allocation or a launch that waits for the device stops this
+// thread only, and a host callback that the device waits for may need the lock.
+template <typename F>
+cs_status launch(F call) {
+    struct Unlocked {
+        PyThreadState* const held = PyEval_SaveThread();
+        ~Unlocked() { PyEval_RestoreThread(held); }
+    } unlocked;
+    return call();
+}
+
 at::Tensor ints(at::IntArrayRef shape, c10::Device dev) { return at::empty(shape, at::TensorOptions(at::kInt).device(dev)); }
 
 PyObject* status(cs_status st) { return PyLong_FromLong(st); }
 
-// The given output, checked, or a new one; `mine` holds a new one.
-bool output(PyObject* o, at::IntArrayRef shape, c10::Device dev, at::Tensor* t) {
-    if (o == Py_None) {
-        *t = ints(shape, dev);
-        return true;
-    }
+// The given output, checked; none given leaves `t` undefined, for make().
+bool output(PyObject* o, int ndim, c10::Device dev, at::Tensor* t) {
+    if (o == Py_None) return true;
     const at::Tensor* x;
-    if (!need(o, at::kInt, (int)shape.size(), dev, &x)) return false;
+    if (!need(o, at::kInt, ndim, dev, &x)) return false;
     *t = *x;
     return true;
+}
+
+void make(at::Tensor* t, at::IntArrayRef shape, c10::Device dev) {
+    if (!t->defined()) *t = ints(shape, dev);
 }
 
 PyObject* pair(const at::Tensor& a, const at::Tensor& b) {
@@ -172,13 +185,16 @@ PyObject* attention(PyObject* const* a, bool tree) {
         bytes = tree ? cs_tree_verify_attention_workspace_bytes(&d, (int32_t)rows)
                      : cs_verify_attention_workspace_bytes(&d, n_draft);
     if (!workspace(a[7], tree ? kTreeAttn : kAttn, dev, bytes, s, &ws)) Py_RETURN_NONE;
-    const at::Tensor out = a[6] == Py_None ? at::empty_like(*q) : *o;
+    at::Tensor out;
     const int32_t *tp = (const int32_t*)table->data_ptr(), *lp = (const int32_t*)lens->data_ptr();
-    const cs_status st =
-        tree ? cs_tree_verify_attention(&d, q->data_ptr(), k->data_ptr(), v->data_ptr(), tp, lp,
-                                        (const int32_t*)par->data_ptr(), (int32_t)rows, out.data_ptr(), ws.ptr, ws.bytes, s)
-             : cs_verify_attention(&d, q->data_ptr(), k->data_ptr(), v->data_ptr(), tp, lp, n_draft, out.data_ptr(),
-                                   ws.ptr, ws.bytes, s);
+    const cs_status st = launch([&] {
+        out = a[6] == Py_None ? at::empty_like(*q) : *o;
+        return tree ? cs_tree_verify_attention(&d, q->data_ptr(), k->data_ptr(), v->data_ptr(), tp, lp,
+                                               (const int32_t*)par->data_ptr(), (int32_t)rows, out.data_ptr(), ws.ptr,
+                                               ws.bytes, s)
+                    : cs_verify_attention(&d, q->data_ptr(), k->data_ptr(), v->data_ptr(), tp, lp, n_draft,
+                                          out.data_ptr(), ws.ptr, ws.bytes, s);
+    });
     if (st != CS_OK) return status(st);
     return a[6] == Py_None ? THPVariable_Wrap(out) : Py_NewRef(a[6]);
 }
@@ -208,13 +224,16 @@ CALL(spec_accept, 9)
     at::Tensor tokens, count;
     Scratch ws;
     const size_t bytes = a[7] == Py_None ? cs_spec_accept_workspace_bytes(&d, (int32_t)k) : 0;
-    if (!output(a[5], {B, k + 1}, dev, &tokens) || !output(a[6], {B}, dev, &count) ||
+    if (!output(a[5], 2, dev, &tokens) || !output(a[6], 1, dev, &count) ||
         !workspace(a[7], kAccept, dev, bytes, s, &ws))
         Py_RETURN_NONE;
-    const cs_status st =
-        cs_spec_accept(&d, t->data_ptr(), q ? q->data_ptr() : nullptr, (const int32_t*)x->data_ptr(),
-                       (const float*)u->data_ptr(), (int32_t)k, T, (int32_t*)tokens.data_ptr(),
-                       (int32_t*)count.data_ptr(), ws.ptr, ws.bytes, s);
+    const cs_status st = launch([&] {
+        make(&tokens, {B, k + 1}, dev);
+        make(&count, {B}, dev);
+        return cs_spec_accept(&d, t->data_ptr(), q ? q->data_ptr() : nullptr, (const int32_t*)x->data_ptr(),
+                              (const float*)u->data_ptr(), (int32_t)k, T, (int32_t*)tokens.data_ptr(),
+                              (int32_t*)count.data_ptr(), ws.ptr, ws.bytes, s);
+    });
     return st != CS_OK ? status(st) : pair(tokens, count);
 CALL_END
 
@@ -235,13 +254,18 @@ CALL(tree_accept, 11)
     at::Tensor tokens, path, count;
     Scratch ws;
     const size_t bytes = a[9] == Py_None ? cs_tree_accept_workspace_bytes(&d, (int32_t)n) : 0;
-    if (!output(a[6], {B, n}, dev, &tokens) || !output(a[7], {B, n}, dev, &path) || !output(a[8], {B}, dev, &count) ||
+    if (!output(a[6], 2, dev, &tokens) || !output(a[7], 2, dev, &path) || !output(a[8], 1, dev, &count) ||
         !workspace(a[9], kTreeAccept, dev, bytes, s, &ws))
         Py_RETURN_NONE;
-    const cs_status st =
-        cs_tree_accept(&d, t->data_ptr(), q ? q->data_ptr() : nullptr, (const int32_t*)par->data_ptr(),
-                       (const int32_t*)x->data_ptr(), (const float*)u->data_ptr(), (int32_t)n, T,
-                       (int32_t*)tokens.data_ptr(), (int32_t*)path.data_ptr(), (int32_t*)count.data_ptr(), ws.ptr, ws.bytes, s);
+    const cs_status st = launch([&] {
+        make(&tokens, {B, n}, dev);
+        make(&path, {B, n}, dev);
+        make(&count, {B}, dev);
+        return cs_tree_accept(&d, t->data_ptr(), q ? q->data_ptr() : nullptr, (const int32_t*)par->data_ptr(),
+                              (const int32_t*)x->data_ptr(), (const float*)u->data_ptr(), (int32_t)n, T,
+                              (int32_t*)tokens.data_ptr(), (int32_t*)path.data_ptr(), (int32_t*)count.data_ptr(),
+                              ws.ptr, ws.bytes, s);
+    });
     if (st != CS_OK) return status(st);
     return Py_BuildValue("(NNN)", THPVariable_Wrap(tokens), THPVariable_Wrap(path), THPVariable_Wrap(count));
 CALL_END
@@ -259,9 +283,12 @@ CALL(sample, 6)
     at::Tensor tokens;
     Scratch ws;
     const size_t bytes = a[4] == Py_None ? cs_sample_workspace_bytes(&d) : 0;
-    if (!output(a[3], {z->size(0)}, dev, &tokens) || !workspace(a[4], kSample, dev, bytes, s, &ws)) Py_RETURN_NONE;
-    const cs_status st = cs_sample(&d, z->data_ptr(), (const float*)u->data_ptr(), T, (int32_t*)tokens.data_ptr(), ws.ptr,
-                                   ws.bytes, s);
+    if (!output(a[3], 1, dev, &tokens) || !workspace(a[4], kSample, dev, bytes, s, &ws)) Py_RETURN_NONE;
+    const cs_status st = launch([&] {
+        make(&tokens, {z->size(0)}, dev);
+        return cs_sample(&d, z->data_ptr(), (const float*)u->data_ptr(), T, (int32_t*)tokens.data_ptr(), ws.ptr,
+                         ws.bytes, s);
+    });
     return st != CS_OK ? status(st) : THPVariable_Wrap(tokens);
 CALL_END
 
@@ -280,11 +307,15 @@ CALL(route, 6)
     Scratch ws;
     const size_t bytes = a[4] == Py_None ? cs_route_workspace_bytes(&d) : 0;
     if (!workspace(a[4], kRoute, dev, bytes, s, &ws)) Py_RETURN_NONE;
-    const at::Tensor group = ints({B}, dev), best = ints({B}, dev),
-                     score = at::empty({B}, at::TensorOptions(at::kFloat).device(dev));
-    const cs_status st = cs_route(&d, e->data_ptr(), c->data_ptr(), (const float*)inv->data_ptr(), tau,
-                                  (int32_t*)group.data_ptr(), (int32_t*)best.data_ptr(), (float*)score.data_ptr(), ws.ptr,
-                                  ws.bytes, s);
+    at::Tensor group, best, score;
+    const cs_status st = launch([&] {
+        make(&group, {B}, dev);
+        make(&best, {B}, dev);
+        score = at::empty({B}, at::TensorOptions(at::kFloat).device(dev));
+        return cs_route(&d, e->data_ptr(), c->data_ptr(), (const float*)inv->data_ptr(), tau,
+                        (int32_t*)group.data_ptr(), (int32_t*)best.data_ptr(), (float*)score.data_ptr(), ws.ptr,
+                        ws.bytes, s);
+    });
     if (st != CS_OK) return status(st);
     return Py_BuildValue("(NNN)", THPVariable_Wrap(group), THPVariable_Wrap(best), THPVariable_Wrap(score));
 CALL_END
@@ -302,9 +333,11 @@ CALL(kv_append, 7)
     const int32_t hkv = (int32_t)k->size(1);
     const cs_attn_dims d{(int32_t)nk->size(0), hkv, hkv, (int32_t)k->size(3), (int32_t)k->size(2),
                          (int32_t)table->size(1), (int32_t)k->size(0), 0.f};
-    const cs_status st = cs_kv_append(&d, nk->data_ptr(), nv->data_ptr(), k->data_ptr(), v->data_ptr(),
-                                      (const int32_t*)table->data_ptr(), (const int32_t*)lens->data_ptr(),
-                                      (int32_t)nk->size(1), s);
+    const cs_status st = launch([&] {
+        return cs_kv_append(&d, nk->data_ptr(), nv->data_ptr(), k->data_ptr(), v->data_ptr(),
+                            (const int32_t*)table->data_ptr(), (const int32_t*)lens->data_ptr(), (int32_t)nk->size(1),
+                            s);
+    });
     if (st != CS_OK) return status(st);
     Py_RETURN_TRUE;
 CALL_END
@@ -318,7 +351,9 @@ CALL(kv_commit, 4)
     if (!first(a[0], at::kInt, 1, &dev, &lens) || !need(a[1], at::kInt, 1, dev, &n) || !small_int(a[2], &k) ||
         !stream_of(a[3], dev, &s))
         Py_RETURN_NONE;
-    const cs_status st = cs_kv_commit((int32_t)lens->size(0), (int32_t*)lens->data_ptr(), (const int32_t*)n->data_ptr(), k, s);
+    const cs_status st = launch([&] {
+        return cs_kv_commit((int32_t)lens->size(0), (int32_t*)lens->data_ptr(), (const int32_t*)n->data_ptr(), k, s);
+    });
     if (st != CS_OK) return status(st);
     Py_RETURN_TRUE;
 CALL_END
@@ -336,9 +371,11 @@ CALL(kv_commit_tree, 7)
     const int32_t hkv = (int32_t)k->size(1);
     const cs_attn_dims d{(int32_t)path->size(0), hkv, hkv, (int32_t)k->size(3), (int32_t)k->size(2),
                          (int32_t)table->size(1), (int32_t)k->size(0), 0.f};
-    const cs_status st = cs_kv_commit_tree(&d, k->data_ptr(), v->data_ptr(), (const int32_t*)table->data_ptr(),
-                                           (int32_t*)lens->data_ptr(), (const int32_t*)path->data_ptr(),
-                                           (const int32_t*)n->data_ptr(), (int32_t)path->size(1), s);
+    const cs_status st = launch([&] {
+        return cs_kv_commit_tree(&d, k->data_ptr(), v->data_ptr(), (const int32_t*)table->data_ptr(),
+                                 (int32_t*)lens->data_ptr(), (const int32_t*)path->data_ptr(),
+                                 (const int32_t*)n->data_ptr(), (int32_t)path->size(1), s);
+    });
     if (st != CS_OK) return status(st);
     Py_RETURN_TRUE;
 CALL_END

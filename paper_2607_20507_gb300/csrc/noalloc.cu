@@ -69,6 +69,7 @@ extern "C" cs_status cs_verify_attention_noalloc(const cs_attn_dims* dims, const
     void* scratch = nullptr;
     cs_status st = scratch_address(&scratch);
     if (st != CS_OK) return st;
+    const cs::StreamTurn turn(reinterpret_cast<cudaStream_t>(stream));   // the clearing belongs to the call
     // The status word must start at zero: clear it, so that a failed or
     // interrupted call cannot leak into this one.
     cudaError_t e = cudaMemsetAsync(scratch, 0, 256, reinterpret_cast<cudaStream_t>(stream));

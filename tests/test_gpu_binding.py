@@ -4,6 +4,7 @@ checks raise."""
 import random
 import sys
 import threading
+import time
 
 import pytest
 import torch
@@ -195,3 +196,54 @@ def test_new_workspace_is_filled_on_its_stream():
     torch.cuda.synchronize()
     assert torch.count_nonzero(early).item() > 0 and torch.equal(ws, early)
     assert ws.data_ptr() != binding.verify_attention_workspace(d, 3, DEV).data_ptr()
+
+
+def test_other_threads_run_while_a_launch_waits():
+    """The stream is busy for about a second and its queue fills up: the launching thread waits, the others do not."""
+    lens, n = torch.zeros((4,), dtype=torch.int32, device=DEV), torch.zeros((4,), dtype=torch.int32, device=DEV)
+    binding.cs_kv_commit(lens, n, 3)
+    torch.cuda.synchronize()
+    gaps, stop = [], threading.Event()
+
+    def tick():
+        t = time.perf_counter()
+        while not stop.is_set():
+            time.sleep(0.002)
+            now = time.perf_counter()
+            gaps.append(now - t)
+            t = now
+
+    ticker = threading.Thread(target=tick)
+    ticker.start()
+    try:
+        torch.cuda._sleep(2_000_000_000)
+        t0 = time.perf_counter()
+        for _ in range(8192):
+            binding.cs_kv_commit(lens, n, 3)
+        waited = time.perf_counter() - t0
+    finally:
+        stop.set()
+        ticker.join()
+    torch.cuda.synchronize()
+    assert waited > 0.3, "the queue did not fill up"
+    assert max(gaps) < 0.5 * waited
+
+
+def test_threads_on_one_stream_share_its_workspace():
+    """Calls of one shape from four threads on the same stream, each of several kernels: as one after the other."""
+    w = W.Workload(96, "threads", batch=96, n_draft=8, vocab=128256, logit_dtype="bf16", draft_sigma=0.7,
+                   temperatures=(0.8,), n_q_heads=16, n_kv_heads=4, head_dim=128, ctx=("const", 64), page_size=16)
+    x = []
+    for seed in range(4):
+        c = W.accept_inputs(w.with_(cell=seed), 0.8, DEV)
+        x.append([c[k] for k in ("target", "draft", "draft_tokens", "uniforms")])
+    expect = [binding.cs_spec_accept(*c, 0.8) for c in x]
+    torch.cuda.synchronize()
+
+    def work(i):
+        got = [binding.cs_spec_accept(*x[i], 0.8) for _ in range(40)]
+        torch.cuda.synchronize()
+        for tok, n in got:
+            assert torch.equal(tok, expect[i][0]) and torch.equal(n, expect[i][1])
+
+    run_threads([lambda i=i: work(i) for i in range(4)])
