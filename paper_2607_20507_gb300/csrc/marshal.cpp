@@ -76,7 +76,9 @@ bool stream_of(PyObject* o, c10::Device dev, cs_stream_t* s) {
     }
     if (!PyLong_CheckExact(o)) return false;
     *s = static_cast<cs_stream_t>(PyLong_AsVoidPtr(o));
-    return !PyErr_Occurred();
+    if (!PyErr_Occurred()) return true;
+    PyErr_Clear();   // (more than a handle: binding.py passes on its low bits)
+    return false;
 }
 
 enum Kind { kAttn, kTreeAttn, kAccept, kTreeAccept, kSample, kRoute };

@@ -69,6 +69,16 @@ def test_refusals():
         binding.cs_kv_commit(a[4].long(), a[4], 3)
 
 
+def test_stream_of_more_than_a_handle():
+    """Its low 64 bits count, as in every ctypes call (here 0: the default stream)."""
+    lens, n = torch.tensor([9, 5], dtype=torch.int32, device=DEV), torch.tensor([1, 0], dtype=torch.int32, device=DEV)
+    binding.cs_kv_commit(lens, n, 3, stream=1 << 70)
+    assert lens.tolist() == [7, 2]
+    z, u = torch.randn((2, 1000), device=DEV), torch.zeros((2,), device=DEV)
+    t = binding.cs_sample(z, u, 0.0, stream=1 << 70)
+    assert torch.equal(t, z.argmax(dim=1).int())
+
+
 def run_threads(works):
     """Each callable in a thread of its own; the first exception is raised here."""
     errors = []
