@@ -221,7 +221,9 @@ __device__ __forceinline__ float bf16_bits_to_float(uint32_t bits16) {
 // Programmatic dependent launch: a kernel may start while the one before it
 // in the stream runs; every CTA waits here, before it reads what an earlier
 // kernel wrote or overwrites what one reads (a no-op when the kernel was
-// launched without the attribute).
+// launched without the attribute).  What is read past it may have been written
+// while this kernel was resident, so no load here is a non-coherent one, which
+// takes memory that does not change during the kernel.
 __device__ __forceinline__ void wait_prior_grid() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void allow_dependent_launch() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

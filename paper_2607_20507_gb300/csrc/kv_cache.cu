@@ -57,12 +57,12 @@ __global__ void __launch_bounds__(kAppendThreads) kv_append_kernel(const AppendP
     const int i = (int)(bi % p.n_new);
     const int b = (int)(bi / p.n_new);
     const size_t src = (size_t)r * kRowThreads + c;
-    int L = __ldg(p.ctx_lens + b);
-    const uint4 k = __ldg(p.new_k + src), v = __ldg(p.new_v + src);
+    int L = __ldcg(p.ctx_lens + b);
+    const uint4 k = __ldcg(p.new_k + src), v = __ldcg(p.new_v + src);
     L = max(0, min(L, p.max_pages * p.ps));
     const int pos = L - p.n_new + i;          // key position of verify row i
     if (pos < 0) return;                      // the context cannot hold this row
-    const int page = __ldg(p.page_table + (size_t)b * p.max_pages + pos / p.ps);
+    const int page = __ldcg(p.page_table + (size_t)b * p.max_pages + pos / p.ps);
     if (page < 0 || page >= p.P) return;      // no such page: nothing is written
     const size_t dst = (((size_t)page * p.Hkv + h) * p.ps + pos % p.ps) * kRowThreads + c;
     p.k_pages[dst] = k;
@@ -75,7 +75,7 @@ __global__ void kv_commit_kernel(int32_t* ctx_lens, const int32_t* n_accepted, i
     allow_dependent_launch();
     if (b >= batch) return;
     // rows kept: the prefix, the verify input token and the accepted drafts
-    const int L = ctx_lens[b] - n_draft + __ldg(n_accepted + b);
+    const int L = __ldcg(ctx_lens + b) - n_draft + __ldcg(n_accepted + b);
     ctx_lens[b] = L > 0 ? L : 0;
 }
 
@@ -103,15 +103,15 @@ __global__ void __launch_bounds__(kCommitMaxThreads) kv_commit_tree_kernel(const
     wait_prior_grid();
     allow_dependent_launch();
     const int32_t* table = p.page_table + (size_t)b * p.max_pages;
-    const int L = max(0, min(p.ctx_lens[b], p.max_pages * p.ps));
-    const int a = max(0, min(__ldg(p.n_accepted + b), p.n - 1));
+    const int L = max(0, min(__ldcg(p.ctx_lens + b), p.max_pages * p.ps));
+    const int a = max(0, min(__ldcg(p.n_accepted + b), p.n - 1));
     const int base = L - p.n;
     if (tid < p.n) {
-        const int node = __ldg(p.path + (size_t)b * p.n + tid);
+        const int node = __ldcg(p.path + (size_t)b * p.n + tid);
         const int src = base + node, dst = base + 1 + tid;
         long long sr = -1, dr = -1;
         if (tid < a && node >= 1 && node < p.n && src != dst && src >= 0 && dst >= 0) {
-            const int sp = __ldg(table + src / p.ps), dp = __ldg(table + dst / p.ps);
+            const int sp = __ldcg(table + src / p.ps), dp = __ldcg(table + dst / p.ps);
             if (sp >= 0 && sp < p.P && dp >= 0 && dp < p.P) {
                 sr = (long long)sp * p.Hkv * p.ps + src % p.ps;
                 dr = (long long)dp * p.Hkv * p.ps + dst % p.ps;

@@ -337,7 +337,7 @@ route_gemm_kernel(const __grid_constant__ CUtensorMap tmap_e, const __grid_const
         const bool loads = row < kRN / 2;
         auto inv_of = [&](int tile) {
             const int j = tile * kRN + col;
-            return loads && j < p.N ? __ldg(p.inv_norm_c + j) : kNaN;
+            return loads && j < p.N ? p.inv_norm_c[j] : kNaN;
         };
         float best = kNegInf;
         int idx = -1;

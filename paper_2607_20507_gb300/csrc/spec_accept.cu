@@ -100,7 +100,7 @@ struct StatsParams {
 // ------------------------------------------------------------ small helpers
 __device__ __forceinline__ uint4 ld_stream(const void* p) {
     uint4 v;
-    asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];"
+    asm volatile("ld.global.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];"
                  : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
                  : "l"(p));
     return v;
@@ -135,9 +135,9 @@ __device__ __forceinline__ uint4 load16_any(const T* row, int start, int V) {
         for (int e = 0; e < kPer; ++e) v.t[e] = start + e >= 0 && start + e < V ? row[start + e] : (T)kNegInf;
         return v.q;
     }
-    const uint4 lo = __ldg(reinterpret_cast<const uint4*>(row + a));
+    const uint4 lo = *reinterpret_cast<const uint4*>(row + a);
     if (off == 0) return lo;
-    const uint4 hi = __ldg(reinterpret_cast<const uint4*>(row + a) + 1);
+    const uint4 hi = reinterpret_cast<const uint4*>(row + a)[1];
     uint32_t w[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
     if (off & 8) {
 #pragma unroll
@@ -264,7 +264,7 @@ __device__ __forceinline__ uint64_t tree_child_mask(const int32_t* par, int n, i
     for (int h = 0; h < 2; ++h) {
         const int c = lane + 32 * h;
         if (c > 0 && c < n) {
-            const int q = __ldg(par + c);
+            const int q = par[c];
             if (q >= 0 && q < c) m |= 1ull << q;
         }
     }
@@ -428,8 +428,8 @@ __device__ __forceinline__ float item_masses(const DrawRow<T>& d, int i0, int i1
         if (base >= 0 && base + kHalf <= V && d.same) {
 #pragma unroll
             for (int u = 0; u < kN; ++u) {
-                t[u] = __ldg(reinterpret_cast<const uint4*>(d.rt + at + u * 32 * kPer));
-                q[u] = __ldg(reinterpret_cast<const uint4*>(d.rd + at + u * 32 * kPer));
+                t[u] = *reinterpret_cast<const uint4*>(d.rt + at + u * 32 * kPer);
+                q[u] = *reinterpret_cast<const uint4*>(d.rd + at + u * 32 * kPer);
             }
         } else if (d.same && whole_vectors(d.rt, V)) {
 #pragma unroll
@@ -753,9 +753,9 @@ __global__ void __launch_bounds__(kThreads) accept_test_kernel(const TestParams 
     int x = -1;
     float zt = kNegInf, zd = 0.f, u = 1.f;
     if (b < p.B && lane < tests) {
-        x = __ldg(p.tokens + (size_t)b * (p.n - 1) + p0 + lane);
+        x = p.tokens[(size_t)b * (p.n - 1) + p0 + lane];
         if (!kGreedy) {
-            u = __ldg(p.uniforms + (size_t)b * p.n + p0 + lane);
+            u = p.uniforms[(size_t)b * p.n + p0 + lane];
             if (x >= 0 && x < p.V) {
                 zt = to_f(static_cast<const T*>(p.target)[((size_t)b * p.n + p0 + lane) * p.V + x]);
                 zd = to_f(static_cast<const T*>(p.draft)[((size_t)b * (p.n - 1) + p0 + lane) * p.V + x]);

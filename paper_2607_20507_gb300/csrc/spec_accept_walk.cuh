@@ -67,8 +67,8 @@ __device__ __forceinline__ void load_run(const DrawRow<T>& d, int j, int V, int 
     if (base >= 0 && base + kBlock <= V && d.same) {
 #pragma unroll
         for (int u = 0; u < kRunVecs; ++u) {
-            r.t[u] = __ldg(reinterpret_cast<const uint4*>(d.rt + at) + u);
-            r.d[u] = __ldg(reinterpret_cast<const uint4*>(d.rd + at) + u);
+            r.t[u] = reinterpret_cast<const uint4*>(d.rt + at)[u];
+            r.d[u] = reinterpret_cast<const uint4*>(d.rd + at)[u];
         }
     } else if (d.same && whole_vectors(d.rt, V)) {
 #pragma unroll
@@ -246,14 +246,14 @@ __global__ void __launch_bounds__(kWalkMaxThreads, 2) accept_walk_kernel(const W
     int par = -1, tok = -1;
     if (tid < n) {
         if (tree) {
-            const int q = tid > 0 ? __ldg(p.parents + (size_t)b * n + tid) : -1;
+            const int q = tid > 0 ? p.parents[(size_t)b * n + tid] : -1;
             par = q >= 0 && q < tid ? q : -1;
-            tok = __ldg(p.tokens + (size_t)b * n + tid);
+            tok = p.tokens[(size_t)b * n + tid];
         } else if (tid > 0) {
             par = tid - 1;
-            tok = __ldg(p.tokens + (size_t)b * (n - 1) + tid - 1);
+            tok = p.tokens[(size_t)b * (n - 1) + tid - 1];
         }
-        if (!kGreedy) s_u[tid] = __ldg(p.uniforms + (size_t)b * n + tid);
+        if (!kGreedy) s_u[tid] = p.uniforms[(size_t)b * n + tid];
         s_tok[tid] = tok;
         s_kids[tid] = tree || tid + 1 == n ? 0ull : 1ull << (tid + 1);
     }

@@ -207,7 +207,7 @@ __device__ __forceinline__ void build_schedule(const int32_t* ctx_lens, int nb, 
     };
     auto load = [&](int b) -> long long {
         if (b >= nb) return 0;
-        const int L = max(0, min(__ldg(ctx_lens + b), l_cap));
+        const int L = max(0, min(__ldcg(ctx_lens + b), l_cap));
         lens[b] = L;
         return (long long)tiles_of(L) * n_vh;
     };
@@ -247,11 +247,11 @@ __device__ __forceinline__ void tree_ancestor_masks(const int32_t* par, int n, i
     const int c0 = lane, c1 = lane + 32;
     int j0 = -1, j1 = -1;
     if (c0 > 0 && c0 < n) {
-        const int q = __ldg(par + c0);
+        const int q = par[c0];
         j0 = (q >= 0 && q < c0) ? q : -1;
     }
     if (c1 < n) {
-        const int q = __ldg(par + c1);
+        const int q = par[c1];
         j1 = (q >= 0 && q < c1) ? q : -1;
     }
     m0 = c0 < n ? (1ull << c0) : 0ull;
@@ -364,7 +364,7 @@ verify_attention_kernel(const __grid_constant__ CUtensorMap tmap_k,
             if (jj >= n_tiles) return -1;
             const int tok = cc.t * kTileT + (lane % pieces) * kBoxT;
             if (tok >= s_len[cc.b]) return -1;
-            return __ldg(p.page_table + (size_t)(p.b_base + cc.b) * p.max_pages + tok / p.ps);
+            return p.page_table[(size_t)(p.b_base + cc.b) * p.max_pages + tok / p.ps];
         };
         Cursor cur = range.first;
         int pg_cur = batch_pages(0);
@@ -463,8 +463,8 @@ verify_attention_kernel(const __grid_constant__ CUtensorMap tmap_k,
 #pragma unroll
             for (int kk = 0; kk < 8; ++kk) {
                 const int col = kk * 16 + tq * 2;
-                qa[kk][k] = qr ? __ldg(reinterpret_cast<const uint32_t*>(qr + col)) : 0u;
-                qa[kk][2 + k] = qr ? __ldg(reinterpret_cast<const uint32_t*>(qr + col + 8)) : 0u;
+                qa[kk][k] = qr ? *reinterpret_cast<const uint32_t*>(qr + col) : 0u;
+                qa[kk][2 + k] = qr ? *reinterpret_cast<const uint32_t*>(qr + col + 8) : 0u;
             }
         }
 #pragma unroll
@@ -880,7 +880,7 @@ verify_attention_merge_span_kernel(const AttnParams p, int grid_main) {
     // tiles before request bl, and in total (x spans)
     long long before = 0, total = 0;
     for (int b = threadIdx.x; b < nb; b += kMergeThreads) {
-        int L = __ldg(p.ctx_lens + p.b_base + b);
+        int L = __ldcg(p.ctx_lens + p.b_base + b);
         L = max(0, min(L, l_cap));
         const long long v = (long long)tiles_of(L) * p.n_vh;
         total += v;
@@ -902,7 +902,7 @@ verify_attention_merge_span_kernel(const AttnParams p, int grid_main) {
             bf += s_red[0][w];
             W += s_red[1][w];
         }
-        int L = __ldg(p.ctx_lens + p.b_base + bl);
+        int L = __ldcg(p.ctx_lens + p.b_base + bl);
         L = max(0, min(L, l_cap));
         const int T = tiles_of(L);
         const int Gc = (int)(W < (long long)grid_main ? (W > 0 ? W : 1) : grid_main);

@@ -375,7 +375,7 @@ verify_attention_tc_kernel(const __grid_constant__ CUtensorMap tmap_k, const __g
             if (jj >= n_tiles) return -1;
             const int tok = cc.t * kTileT + (lane % kPieces) * kBoxT;
             if (tok >= s_len[cc.b]) return -1;
-            return __ldg(p.page_table + (size_t)(p.b_base + cc.b) * p.max_pages + tok / p.ps);
+            return p.page_table[(size_t)(p.b_base + cc.b) * p.max_pages + tok / p.ps];
         };
         if (lane == 0) {
             tma_prefetch_desc(tmap);
