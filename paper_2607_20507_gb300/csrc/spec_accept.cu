@@ -925,9 +925,15 @@ AcceptPlan plan_accept(const cs_accept_dims& d, int n, bool tree, bool greedy, b
         if (n > 1) P.threads = 64;
     }
     P.look = 1;
-    const int block = 32 * kWalkVecs * 16 / esz, most = kWalkSegs * kRunVecs / kWalkVecs;
+    // A long row takes more CTAs, 512 blocks each; where the device has no
+    // cluster of that many, the largest one holds up to twice that a CTA.
+    constexpr int kRowBlocks = 512, kMostBlocks = kWalkSegs * kRunVecs / kWalkVecs;
+    static_assert((CS_MAX_VOCAB * 4ll + 12 + kWalkVecs * 512 - 1) / (kWalkVecs * 512) <= 8 * kMostBlocks,
+                  "a portable cluster holds the longest row, at any alignment");
+    const int block = 32 * kWalkVecs * 16 / esz;
     P.blocks = (int)(((long long)d.vocab + (aligned ? 0 : 16 / esz - 1) + block - 1) / block);
-    const int need = (P.blocks + most - 1) / most;
+    int need = (P.blocks + kRowBlocks - 1) / kRowBlocks;
+    if (need > max_cluster_size()) need = max_cluster_size();
     if (c < need) c = need;
     if (c > P.blocks) c = P.blocks;
     P.cluster = c;

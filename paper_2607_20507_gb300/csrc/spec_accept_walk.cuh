@@ -31,7 +31,7 @@ constexpr int kWalkBatch = 17;                 // nodes of one round, at most
 constexpr int kWalkRows = 2 * kWalkBatch;
 constexpr int kWalkVecs = 4;                   // streaming: 16-byte vectors per lane per block (2 KB of a row)
 constexpr int kRunVecs = 2;                    // draw: contiguous vectors per lane per block (1 KB of a row)
-constexpr int kWalkSegs = 1024;                // draw blocks of one row per CTA, at most
+constexpr int kWalkSegs = 2050;                // draw blocks of one row per CTA, at most
 
 struct WalkParams {
     const void* target;       // [B, n, V]

@@ -92,6 +92,25 @@ def test_vocabularies_of_many_blocks(dtype, V):
         assert ((got == exp) | (margin < DRAW_TIE)).all()
 
 
+@pytest.mark.parametrize("V", [4194301, 4194302, 4194304])   # the last one is the largest that calls take
+@pytest.mark.parametrize("first", [0, 1])
+def test_largest_f32_vocabularies_at_any_alignment(V, first):
+    g = torch.Generator(device=DEV).manual_seed(V + first)
+    flat = torch.randn((first + 4 * V,), generator=g, device=DEV) * 3.0
+    z = flat[first:first + 2 * V].view(2, V)
+    u = torch.rand((2, 2), generator=g, device=DEV)
+    for T in (0.0, 0.8):
+        got = binding.cs_sample(z, u[:, 0].contiguous(), T).cpu().numpy()
+        exp, margin = oracle.sample(W.host_bits(z), u[:, 0].cpu().numpy(), T, with_margin=True)
+        assert ((got == exp) | (margin < DRAW_TIE)).all()
+    if V == 4194302:
+        z = flat[first:first + 3 * V].view(1, 3, V)
+        draft = (z[:, :2] + 0.5 * torch.randn((1, 2, V), generator=g, device=DEV)).contiguous()
+        inp = dict(target=z, draft=draft, draft_tokens=draft.argmax(dim=2).int(), uniforms=torch.rand((1, 3), generator=g, device=DEV))
+        for T in (0.0, 0.8):
+            compare(inp, T, f"V={V}")
+
+
 @pytest.mark.parametrize("B,branching,V,dtype,T", [
     (40, (3, 2, 2, 1), 32001, "bf16", 0.7),    # streamed, rows at every alignment
     (40, (3, 2, 2, 1), 32001, "bf16", 0.0),
