@@ -213,6 +213,11 @@ __device__ __forceinline__ uint64_t f2_sub(uint64_t a, uint64_t b) {
     return d;
 }
 
+// a / b for a >= 0, b > 0 (a 64-bit division only where the numbers need one)
+__device__ __forceinline__ long long div_pos(long long a, long long b) {
+    return ((a | b) >> 32) == 0 ? (long long)((unsigned)a / (unsigned)b) : a / b;
+}
+
 // bf16 bit pattern -> fp32 (exact).
 __device__ __forceinline__ float bf16_bits_to_float(uint32_t bits16) {
     return __uint_as_float(bits16 << 16);

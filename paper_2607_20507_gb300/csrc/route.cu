@@ -85,18 +85,6 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map
         : "memory");
 }
 
-__device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity) {
-    uint32_t done;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}\n"
-        : "=r"(done)
-        : "r"(smem_u32(bar)), "r"(parity)
-        : "memory");
-    return done != 0;
-}
-
 __device__ __forceinline__ void tc_mma_ss(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
     asm volatile(
         "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %4, 0;\n\t"
@@ -109,11 +97,11 @@ __device__ __forceinline__ void tc_mma_ss(uint32_t d, uint64_t a, uint64_t b, ui
 // then records the timeout in the status word.  The result is the same in
 // every lane, so that no lane leaves a loop while another still issues.
 __device__ __forceinline__ bool wait_bar(uint64_t* bar, uint32_t parity, int* status) {
-    if (__all_sync(0xffffffffu, mbar_test(bar, parity))) return true;
+    if (__all_sync(0xffffffffu, mbar_test_wait(bar, parity))) return true;
     uint64_t t0 = 0;
     bool done = false;
     for (uint32_t it = 0; it < (1u << 28) && !done; ++it) {
-        done = mbar_test(bar, parity);
+        done = mbar_test_wait(bar, parity);
         if ((it & 1023u) == 1023u) {
             const uint64_t now = global_timer_ns();
             if (t0 == 0) t0 = now;

@@ -273,13 +273,8 @@ __device__ __forceinline__ uint64_t tree_child_mask(const int32_t* par, int n, i
     return m;
 }
 
-// x / d for x >= 0, d > 0: one 32-bit division whenever both fit (every
-// realistic problem), the 64-bit routine otherwise.
-__device__ __noinline__ long long div_nn(long long x, long long d) {
-    if ((unsigned long long)x <= 0xffffffffull && (unsigned long long)d <= 0xffffffffull)
-        return (long long)((unsigned)x / (unsigned)d);
-    return x / d;
-}
+// Out of line: a phase's start has four of them.
+__device__ __noinline__ long long div_nn(long long x, long long d) { return div_pos(x, d); }
 
 // ------------------------------------------------------------ kernel 1
 // Largest of the logits of one lane's vectors (bf16: packed maxima, one
@@ -874,7 +869,7 @@ struct AcceptPlan {
     int I;                                     // items of a row
     int phases, start[kMaxPhases + 1];         // nodes [start[i], start[i+1]) are read in phase i (0: the walk streams)
     int units, U;                              // units of a row, items of a unit
-    int cluster, threads, blocks, per, look;   // the walk
+    int cluster, threads, blocks, per;   // the walk
     size_t off_mass, off_stat, off_a, off_ticket, bytes;
 };
 
@@ -924,7 +919,6 @@ AcceptPlan plan_accept(const cs_accept_dims& d, int n, bool tree, bool greedy, b
         c = 1;
         if (n > 1) P.threads = 64;
     }
-    P.look = 1;
     // A long row takes more CTAs, 512 blocks each; where the device has no
     // cluster of that many, the largest one holds up to twice that a CTA.
     constexpr int kRowBlocks = 512, kMostBlocks = kWalkSegs * kRunVecs / kWalkVecs;
@@ -1038,7 +1032,6 @@ cs_status launch_typed(StatsParams sp, TestParams tp, WalkParams p, const Accept
     }
     if (P.phases > 1) ph.undecided = dec.a;
     p.mass = sp.mass;
-    p.reverse = true;
     p.ph = ph;
     p.dec = dec;
     for (int b0 = 0; b0 < sp.B; b0 += 65535) {
@@ -1096,7 +1089,6 @@ cs_status launch_accept(const cs_accept_dims& d, const void* target, const void*
     p.I = P.I;
     p.blocks = P.blocks;
     p.per = P.per;
-    p.look = P.look;
     p.c_hi = sp.c_hi;
     p.c_lo = sp.c_lo;
     if (d.logit_dtype == CS_F32)

@@ -7,9 +7,9 @@
 // all of them run this kernel.
 //  * After accept_stats_kernel (kStream = false) the statistics of the rows
 //    are folded from its partials, or a phase's test has decided already.
-//  * kStream = true: no kernel has run before.  In a round the cluster streams
-//    the target and draft rows of the next undecided node, swaps the row
-//    statistics through distributed shared memory and walks on; the walk
+//  * kStream = true, trees: no kernel has run before.  In a round the cluster
+//    streams the target and draft rows of the next undecided node, swaps the
+//    row statistics through distributed shared memory and walks on; the walk
 //    usually stops early, and the rows past it are never read.
 // The draw: where the unit masses of the row (pair) are known they are the
 // CDF, and one CTA weighs the unit that holds the cell.  Otherwise the cluster
@@ -27,8 +27,6 @@
 
 constexpr int kWalkMaxThreads = 256;
 constexpr int kWalkMaxWarps = kWalkMaxThreads / 32;
-constexpr int kWalkBatch = 17;                 // nodes of one round, at most
-constexpr int kWalkRows = 2 * kWalkBatch;
 constexpr int kWalkVecs = 4;                   // streaming: 16-byte vectors per lane per block (2 KB of a row)
 constexpr int kRunVecs = 2;                    // draw: contiguous vectors per lane per block (1 KB of a row)
 constexpr int kWalkSegs = 2050;                // draw blocks of one row per CTA, at most
@@ -44,9 +42,7 @@ struct WalkParams {
     int32_t* out_path;        // tree [B, n]
     int B, V, n, d_rows;
     int I;                    // 4 KB items of a row (accept_stats_kernel's)
-    bool reverse;             // the last requests first
     int blocks, per;          // 2 KB blocks of a row, blocks of a row per CTA
-    int look;                 // nodes of a round
     Phase ph;                 // the last phase of accept_stats_kernel (R == 0: it did not run)
     Decided dec;              // what the earlier phases decided (read when ph.undecided is set),
     const float* mass;        // and [B, units] the draw masses of the units of the pair that decided
@@ -215,11 +211,8 @@ __global__ void __launch_bounds__(kWalkMaxThreads, 2) accept_walk_kernel(const W
     __shared__ float2 s_z[kMaxTreeNodes];                    // target / draft logit of node c's token in its parent's rows
     __shared__ int s_tok[kMaxTreeNodes], s_path[kMaxTreeNodes];
     __shared__ float s_u[kMaxTreeNodes];
-    __shared__ int s_rows[kWalkRows];                        // rows of the round, coded as in s_stat
-    __shared__ int s_list[kWalkBatch];                       // its nodes (tree)
-    __shared__ int s_count;                                  // how many rows
-    __shared__ float2 s_part[kWalkRows][kWalkMaxWarps];      // statistics per row and warp
-    __shared__ float2 s_x[2][kWalkRows][kMaxCluster];        // ... per row and CTA, by round parity
+    __shared__ float2 s_part[2][kWalkMaxWarps];              // a round's statistics per row (target, draft) and warp
+    __shared__ float2 s_x[2][2][kMaxCluster];                // ... per row and CTA, by round parity
     __shared__ float s_seg[kWalkSegs], s_cum[kWalkSegs];     // draw masses of the blocks and their running sum
     __shared__ float2 s_m[2][kMaxCluster];                   // draw mass per CTA
 
@@ -227,7 +220,7 @@ __global__ void __launch_bounds__(kWalkMaxThreads, 2) accept_walk_kernel(const W
     const uint32_t rank = cluster_rank(), n_ranks = cluster_size();
     // (the requests whose rows were read last come first: they are the
     // likeliest to be in L2 still)
-    const int b = p.b_base + (int)(p.reverse ? gridDim.y - 1 - blockIdx.y : blockIdx.y);
+    const int b = p.b_base + (int)(gridDim.y - 1 - blockIdx.y);
     const int n = p.n, V = p.V;
     const bool tree = p.parents != nullptr;
     const float2 empty = make_float2(kNegInf, kGreedy ? __int_as_float(INT_MAX) : 0.f);
@@ -384,39 +377,15 @@ __global__ void __launch_bounds__(kWalkMaxThreads, 2) accept_walk_kernel(const W
     }
     while (!stop) {
         if (kStream && !((have >> node) & 1ull)) {
-            // ---- a round: its nodes, breadth first from the current one
-            __syncthreads();   // s_kids complete; the last round's s_rows are no longer read
-            if (!tree) {
-                const int cnt = min(p.look, n - node);
-                const int rows = kGreedy ? cnt : 2 * cnt - (node + cnt == n ? 1 : 0);
-                if (tid < rows) s_rows[tid] = kGreedy ? 2 * (node + tid) : 2 * node + tid;
-                if (tid == 0) s_count = rows;
-            } else if (tid == 0) {
-                int cnt = 1, rows = 0;
-                s_list[0] = node;
-                for (int q = 0; q < cnt; ++q) {
-                    const int u = s_list[q];
-                    unsigned long long kids = s_kids[u];
-                    s_rows[rows++] = 2 * u;
-                    if (!kGreedy && kids) s_rows[rows++] = 2 * u + 1;   // a leaf's draft row is not read
-                    while (kids && cnt < p.look) {
-                        s_list[cnt++] = __ffsll((long long)kids) - 1;
-                        kids &= kids - 1;
-                    }
-                }
-                s_count = rows;
-            }
-            __syncthreads();
-            const int n_rows = s_count;
-            for (int r = 0; r < n_rows; ++r) have |= 1ull << (s_rows[r] >> 1);
+            // ---- a round: the rows of the current node (a leaf's draft row is not read)
+            __syncthreads();   // s_kids complete; the last round's s_part are no longer read
+            const int n_rows = kGreedy || !s_kids[node] ? 1 : 2;
+            have |= 1ull << node;
 
             // ---- row statistics: the flattened items of the rows, dealt over the warps
-            for (int r = lane; r < n_rows; r += 32) s_part[r][wid] = empty;
+            if (lane < n_rows) s_part[lane][wid] = empty;
             __syncwarp();
-            auto row_of = [&](int r) -> const T* {
-                const int code = s_rows[r];
-                return ((code & 1) ? draft : target) + (size_t)(code >> 1) * V;
-            };
+            auto row_of = [&](int r) -> const T* { return (r ? draft : target) + (size_t)node * V; };
             const int total = n_rows * nj;
             int idx = wid, r = nj > 0 ? wid / nj : 0, j = nj > 0 ? wid - r * nj : 0;
             uint4 cur[kWalkVecs], nxt[kWalkVecs];
@@ -470,7 +439,7 @@ __global__ void __launch_bounds__(kWalkMaxThreads, 2) accept_walk_kernel(const W
                 float2 f = lane < nw ? s_part[q][lane] : empty;
                 f = kGreedy ? warp_fold_argmax(f) : warp_fold_sum(f.x, f.y, p.c_hi, p.c_lo);
                 if (n_ranks == 1) {
-                    if (lane == 0) s_stat[s_rows[q]] = f;
+                    if (lane == 0) s_stat[2 * node + q] = f;
                 } else if (lane < (int)n_ranks) {
                     st_cluster_f2(&s_x[slot][q][rank], lane, f);
                 }
@@ -482,7 +451,7 @@ __global__ void __launch_bounds__(kWalkMaxThreads, 2) accept_walk_kernel(const W
                 for (int q = wid; q < n_rows; q += nw) {
                     float2 f = lane < (int)n_ranks ? s_x[slot][q][lane] : empty;
                     f = kGreedy ? warp_fold_argmax(f) : warp_fold_sum(f.x, f.y, p.c_hi, p.c_lo);
-                    if (lane == 0) s_stat[s_rows[q]] = f;
+                    if (lane == 0) s_stat[2 * node + q] = f;
                 }
             }
             __syncthreads();

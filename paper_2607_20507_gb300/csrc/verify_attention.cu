@@ -98,11 +98,6 @@ __device__ __forceinline__ void flag_timeout(int* status) {
 
 __device__ __forceinline__ int tiles_of(int L) { return max(1, (L + kTileT - 1) / kTileT); }
 
-// a / b for a >= 0, b > 0 (a 64-bit division only where the numbers need one)
-__device__ __forceinline__ long long div_pos(long long a, long long b) {
-    return ((a | b) >> 32) == 0 ? (long long)((unsigned)a / (unsigned)b) : a / b;
-}
-
 // The CTA whose range holds work unit v (ranges start at floor(c*U/G)).
 __device__ __forceinline__ int owner_of(long long v, long long U, int G) {
     return (int)div_pos((v + 1) * G + U - 1, U) - 1;
