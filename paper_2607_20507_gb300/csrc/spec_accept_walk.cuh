@@ -59,29 +59,8 @@ struct RunPair {   // one lane's run of a draw block: kRunVecs contiguous vector
 template <typename T>
 __device__ __forceinline__ void load_run(const DrawRow<T>& d, int j, int V, int lane, RunPair<T>& r) {
     constexpr int kPer = 16 / (int)sizeof(T), kBlock = 32 * kRunVecs * kPer;
-    const int base = j * kBlock - misaligned_by(d.rt), at = base + lane * kRunVecs * kPer;
-    if (base >= 0 && base + kBlock <= V && d.same) {
-#pragma unroll
-        for (int u = 0; u < kRunVecs; ++u) {
-            r.t[u] = reinterpret_cast<const uint4*>(d.rt + at)[u];
-            r.d[u] = reinterpret_cast<const uint4*>(d.rd + at)[u];
-        }
-    } else if (d.same && whole_vectors(d.rt, V)) {
-#pragma unroll
-        for (int u = 0; u < kRunVecs; ++u) {
-            r.t[u] = load_or_ninf(d.rt, at + u * kPer, V);
-            r.d[u] = load_or_ninf(d.rd, at + u * kPer, V);
-        }
-    } else {
-        uint4 t[2 * kRunVecs];
-        load_slow(d.rt, at, kPer, kRunVecs, V, t);
-        load_slow(d.rd, at, kPer, kRunVecs, V, t + kRunVecs);
-#pragma unroll
-        for (int u = 0; u < kRunVecs; ++u) {
-            r.t[u] = t[u];
-            r.d[u] = t[kRunVecs + u];
-        }
-    }
+    const int base = j * kBlock - misaligned_by(d.rt);
+    load_pair(d.rt, d.rd, d.same, base, kBlock, base + lane * kRunVecs * kPer, kPer, V, r.t, r.d);
 }
 
 template <typename T>
