@@ -928,7 +928,7 @@ AcceptPlan plan_accept(const cs_accept_dims& d, int n, bool tree, bool greedy, b
         P.phases = 1;
         long long g = (long long)(kPhaseUs / pos_us) + 1;
         while (!tree && n * pos_us >= kPhasedUs && d.batch <= kMaxPhased && P.phases < kMaxPhases && g < n &&
-               (n - g) * pos_us >= kPhaseUs / 2) {
+               (n - g - (greedy ? 0.0 : 0.5)) * pos_us >= kPhaseUs / 2) {   // (the last position has no draft row)
             P.start[P.phases++] = (int)g;
             g *= 2;
         }
@@ -1047,7 +1047,7 @@ cs_status launch_typed(StatsParams sp, TestParams tp, WalkParams p, const Accept
         tp.dec = dec;
         e = launch_after(accept_test_kernel<T, G>, (unsigned)(sp.B + kWarps - 1) / kWarps, 1, kThreads, 1, stream, tp);
         if (e != cudaSuccess) return cuda_fail(e, "accept_test_kernel launch");
-        if (last && !G) {   // the masses of the pairs that the last phase decided
+        if (last && !G && ph.p0 < sp.n - 1) {   // the masses of the pairs that the last phase decided
             sp.ph.p0 = sp.n;
             sp.ph.t_rows = sp.ph.R = 0;
             sp.ph.undecided = dec.a;

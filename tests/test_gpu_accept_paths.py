@@ -6,6 +6,7 @@ import numpy as np
 import pytest
 import torch
 
+import bench
 import oracle
 from paper_2607_20507_gb300 import binding
 from paper_2607_20507_gb300 import workloads as W
@@ -44,10 +45,11 @@ def compare(inp, T, what, sample=24):
     return n
 
 
-# one position of these calls takes 4 to 20 us at the copy bandwidth, so they
+# one position of these calls takes 4 to 32 us at the copy bandwidth, so they
 # are read in two to four phases
 @pytest.mark.parametrize("B,k,V,dtype,sigma,T", [
     (256, 8, 128256, "bf16", 0.7, 0.8),    # [0, 1], [2, 3], [4, 8]
+    (400, 1, 128256, "bf16", 0.7, 0.8),    # [0], [1]: a phase of nothing but the position without a draft
     (256, 8, 128256, "bf16", 0.7, 0.0),
     (128, 16, 128256, "bf16", 0.1, 1.0),   # four phases, most requests pass all of them
     (96, 12, 128257, "bf16", 0.7, 0.8),    # rows at every alignment
@@ -57,6 +59,17 @@ def compare(inp, T, what, sample=24):
 def test_positions_read_in_phases(B, k, V, dtype, sigma, T):
     n = compare(chain(B, k, V, dtype, sigma, T, cell=B + k), T, f"B={B} k={k} V={V} {dtype} T={T}")
     assert n.min() < n.max()
+
+
+@pytest.mark.parametrize("B,k,kernels", [
+    (256, 8, 8),   # three phases of a statistics and a test kernel, the last one's masses, the walk
+    (400, 1, 5),   # the second phase decides no pair: no masses
+])
+def test_every_launch_of_a_phased_call_has_work(B, k, kernels):
+    inp = chain(B, k, 128256, "bf16", 0.7, 0.8)
+    call = lambda: binding.cs_spec_accept(inp["target"], inp["draft"], inp["draft_tokens"], inp["uniforms"], 0.8)  # noqa: E731
+    call()
+    assert bench.kernel_launches(call) == kernels
 
 
 def test_phases_with_every_first_rejection_and_empty_residuals():
