@@ -18,6 +18,7 @@ INCLUDE = os.path.join(ROOT, "include")
 BUILD_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libcachespec.so")
 MARSHAL = os.path.join(HERE, "_marshal.so")
+AGAINST = os.path.join(BUILD_DIR, "marshal.against")
 SOURCES = ["capi.cu", "verify_attention.cu", "spec_accept.cu", "noalloc.cu", "kv_cache.cu", "route.cu", "selftest.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
@@ -34,9 +35,18 @@ def _inputs() -> list[str]:
     return files
 
 
+def _built_against() -> str:
+    """What the marshalling module's binary interface comes from."""
+    import torch
+    return f"python {sys.version}\ntorch {torch.__version__} {os.path.dirname(torch.__file__)}\n"
+
+
 def is_stale() -> bool:
-    if not os.path.exists(LIB) or not os.path.exists(MARSHAL):
+    if not os.path.exists(LIB) or not os.path.exists(MARSHAL) or not os.path.exists(AGAINST):
         return True
+    with open(AGAINST) as f:
+        if f.read() != _built_against():
+            return True
     t = min(os.path.getmtime(LIB), os.path.getmtime(MARSHAL))
     return any(os.path.getmtime(f) > t for f in _inputs())
 
@@ -68,6 +78,8 @@ def _link_marshal(obj: str) -> None:
     _run(["g++", "-shared", "-o", tmp, obj, "-L", libs, "-L", HERE, "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10",
           "-lc10_cuda", "-l:" + os.path.basename(LIB), "-Wl,-rpath,$ORIGIN", "-Wl,-rpath," + libs], "marshal link")
     os.replace(tmp, MARSHAL)
+    with open(AGAINST, "w") as f:
+        f.write(_built_against())
 
 
 def build(force: bool = False, ptxas_verbose: bool = False, quiet: bool = True) -> str:

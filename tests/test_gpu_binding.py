@@ -257,3 +257,79 @@ def test_threads_on_one_stream_share_its_workspace():
             assert torch.equal(tok, expect[i][0]) and torch.equal(n, expect[i][1])
 
     run_threads([lambda i=i: work(i) for i in range(4)])
+
+
+class Interpreted:
+    """In the marshalling module's place: takes nothing, so that binding.py's own checks run."""
+
+    def __getattr__(self, name):
+        return lambda *args: None
+
+
+def both_ways(monkeypatch, call):
+    """A call's result, or its exception's type, through the compiled marshalling and without it."""
+    got = []
+    for fast in (binding._load_fast(), Interpreted()):
+        with monkeypatch.context() as m:
+            m.setattr(binding, "_fast", fast)
+            try:
+                r = call()
+                got.append([t.clone() for t in (r if isinstance(r, tuple) else (r,)) if t is not None])
+            except Exception as e:   # noqa: BLE001
+                got.append((type(e), getattr(e, "status", None)))
+    return got
+
+
+def test_marshalling_does_what_the_checks_do(monkeypatch):
+    a, c = inputs()
+    tw = W.TreeWorkload(97, "ways", batch=3, branching=(2, 1), vocab=3001, logit_dtype="f32", draft_sigma=0.7,
+                        temperatures=(0.8,), n_q_heads=16, n_kv_heads=4, head_dim=128, ctx=("uniform", 40, 400),
+                        page_size=16)
+    ta, tc = W.tree_attention_inputs(tw, DEV), W.tree_accept_inputs(tw, 0.8, DEV)
+    tree = [tc[k] for k in ("target", "draft", "parents", "node_tokens", "uniforms")]
+    path, n = binding.cs_tree_accept(*tree, 0.8)[1:]
+    r = W.route_inputs(W.RouteWorkload(30, "ways", 5, 300, 128), DEV, seed=1)
+    route = (r["emb"], r["centroids"], binding.cs_route_norms(r["centroids"]))
+    rows = [torch.randn((3, 4, 4, 128), device=DEV).to(torch.bfloat16) for _ in range(2)]
+
+    def in_place(call, *written):
+        """Clones of what a call writes into copies of its arguments."""
+        def run():
+            x = [t.clone() for t in written]
+            call(*x)
+            return tuple(x)
+        return run
+
+    b = binding
+    good = [lambda: b.cs_verify_attention(*a, 3), lambda: b.cs_spec_accept(*c, 0.8),
+            lambda: b.cs_spec_accept(c[0], None, *c[2:], 0), lambda: b.cs_tree_accept(*tree, 0.8),
+            lambda: b.cs_tree_verify_attention(*[ta[k] for k in ("q", "k_pages", "v_pages", "page_table", "ctx_lens",
+                                                                 "parents")]),
+            lambda: b.cs_sample(c[0][:, 0].contiguous(), c[3][:, 0].contiguous(), 0.8),
+            lambda: b.cs_route(*route, W.ROUTE_TAU),
+            in_place(lambda k, v: b.cs_kv_append(*rows, k, v, a[3], a[4]), a[1], a[2]),
+            in_place(lambda x: b.cs_kv_commit(x, n, 3), a[4]),
+            in_place(lambda k, v, x: b.cs_kv_commit_tree(k, v, ta["page_table"], x, path, n), ta["k_pages"],
+                     ta["v_pages"], ta["ctx_lens"])]
+    for i, call in enumerate(good):
+        fast, slow = both_ways(monkeypatch, call)
+        assert len(fast) > 0 and len(fast) == len(slow), i
+        for x, y in zip(fast, slow):
+            assert isinstance(x, torch.Tensor) and x.dtype == y.dtype and torch.equal(x, y), i
+    bad = [lambda: b.cs_verify_attention(a[0].float(), *a[1:], 3), lambda: b.cs_verify_attention(*a, 2),
+           lambda: b.cs_verify_attention(*a, 3, sm_scale=float("nan")), lambda: b.cs_verify_attention(*a, "3"),
+           lambda: b.cs_verify_attention(*a, 3, out=torch.empty(1, device=DEV)),
+           lambda: b.cs_spec_accept(c[0], None, *c[2:], 0.8), lambda: b.cs_spec_accept(*c, float("inf")),
+           lambda: b.cs_spec_accept(*c, 0.8, out_tokens=c[3]),
+           lambda: b.cs_spec_accept(c[0], c[1].float(), *c[2:], 0.8), lambda: b.cs_spec_accept(*c, None),
+           lambda: b.cs_spec_accept(*c, 0.8, workspace=torch.zeros(256, dtype=torch.uint8, device=DEV)),
+           lambda: b.cs_tree_accept(*tree[:2], tree[2][:, 1:].contiguous(), *tree[3:], 0.8),
+           lambda: b.cs_sample(c[0], c[3], 0.8), lambda: b.cs_sample(c[0][:, 0], c[3][:, 0], 0.8),
+           lambda: b.cs_route(route[0], route[1][:, :64].contiguous(), route[2], 0.5),
+           lambda: b.cs_route(*route, float("nan")),
+           lambda: b.cs_kv_append(rows[0], rows[1][:2].contiguous(), a[1], a[2], a[3], a[4]),
+           lambda: b.cs_kv_commit(a[4], n, 17), lambda: b.cs_kv_commit(a[4].cpu(), n, 3),
+           lambda: b.cs_kv_commit_tree(ta["k_pages"], ta["v_pages"].float(), ta["page_table"], ta["ctx_lens"], path, n)]
+    for i, call in enumerate(bad):
+        fast, slow = both_ways(monkeypatch, call)
+        assert isinstance(fast, tuple) and fast == slow, (i, fast, slow)
