@@ -7,7 +7,6 @@
 #include <stdio.h>
 #include <string.h>
 
-#include <atomic>
 #include <new>
 
 #include "cs_internal.h"
@@ -16,7 +15,7 @@ namespace cs {
 
 namespace {
 thread_local char g_err[512] = "";
-int g_sms[64] = {0};
+std::atomic<int> g_sms[64];   // (threads launch at the same time)
 
 bool aligned(const void* p, size_t a) { return (reinterpret_cast<uintptr_t>(p) % a) == 0; }
 

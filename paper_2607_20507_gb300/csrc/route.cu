@@ -489,7 +489,7 @@ __global__ void __launch_bounds__(256) route_norms_kernel(const __nv_bfloat16* c
 }
 
 PFN_cuTensorMapEncodeTiled_v12000 route_encoder() {
-    static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
+    static std::atomic<PFN_cuTensorMapEncodeTiled_v12000> fn{nullptr};
     if (!fn) {
         void* ptr = nullptr;
         cudaDriverEntryPointQueryResult q;
@@ -543,7 +543,7 @@ cs_status launch_route(const cs_route_dims& d, const RoutePlan& pl, const void* 
         if (st != CS_OK) return st;
         st = encode_rows_map(&tc, centroids, d.n_groups, d.dim);
         if (st != CS_OK) return st;
-        static bool attr_set[64] = {};
+        static std::atomic<bool> attr_set[64];
         int dev = 0;
         cudaGetDevice(&dev);
         if (dev < 0 || dev >= 64 || !attr_set[dev]) {

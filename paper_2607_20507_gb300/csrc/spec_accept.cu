@@ -847,7 +847,7 @@ __device__ __forceinline__ void cluster_wait() {
 #include "spec_accept_walk.cuh"
 
 // ------------------------------------------------------------------- host
-int g_max_cluster[64] = {0};
+std::atomic<int> g_max_cluster[64];
 
 // The largest cluster (16, non-portable, or 8) the device schedules for the
 // walk kernel.

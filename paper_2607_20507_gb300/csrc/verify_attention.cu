@@ -995,7 +995,7 @@ verify_attention_merge_cut_kernel(const AttnParams p, int n_slots) {
 long long tc_groups(const cs_attn_dims& d) { return (long long)d.num_pages * d.n_kv_heads * (d.page_size / 8); }
 
 PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
-    static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
+    static std::atomic<PFN_cuTensorMapEncodeTiled_v12000> fn{nullptr};
     if (!fn) {
         void* ptr = nullptr;
         cudaDriverEntryPointQueryResult q;
@@ -1067,7 +1067,7 @@ cs_status encode_q_map(CUtensorMap* map, const void* q, const cs_attn_dims& d, i
 
 // CTAs per SM of the tcgen05 kernel (1 when its shared memory fits; cached).
 int tc_resident_per_sm() {
-    static int cache[64] = {};
+    static std::atomic<int> cache[64];
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) {
         cudaGetLastError();
@@ -1118,7 +1118,7 @@ cudaError_t launch_merge(const AttnParams& p, const AttnPlan& pl, cudaStream_t s
 template <bool kTree, int kSplit>
 int resident_per_sm(int threads) {
     // every box size instantiates the same code shape; the 16-key one stands for all
-    static int cache[64][kMaxRowWarps + 2] = {};
+    static std::atomic<int> cache[64][kMaxRowWarps + 2];
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) {
         cudaGetLastError();
@@ -1299,7 +1299,7 @@ cs_status launch_verify_attention(const cs_attn_dims& d, const AttnPlan& pl, con
         const int smem_bytes = tc_smem_bytes();
         cudaError_t e = cudaSuccess;
         {
-            static int attr_smem[2][5][64] = {};   // the limit set so far
+            static std::atomic<int> attr_smem[2][5][64];   // the limit set so far
             int dev = 0;
             e = cudaGetDevice(&dev);
             if (e != cudaSuccess) return cuda_fail(e, "cudaGetDevice");
@@ -1339,7 +1339,7 @@ cs_status launch_verify_attention(const cs_attn_dims& d, const AttnPlan& pl, con
     const Kern kern = kerns[si][pl.tree][bi];
     cudaError_t e = cudaSuccess;
     {
-        static bool attr_done[2][2][4][64] = {};
+        static std::atomic<bool> attr_done[2][2][4][64];
         int dev = 0;
         e = cudaGetDevice(&dev);
         if (e != cudaSuccess) return cuda_fail(e, "cudaGetDevice");
