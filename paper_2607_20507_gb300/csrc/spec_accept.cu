@@ -18,8 +18,8 @@
 //      masses of the CTAs' slices of the deciding row pair are swapped through
 //      distributed shared memory, and one warp of the CTA whose cell holds
 //      u_k * Z finds the token.  Greedy: the arg max of the deciding row.
-// A chain's rows past its first rejection are not needed, so a call whose
-// positions take long to read (plan_accept) reads them in phases: kernel 1 for
+// A chain's rows past its first rejection are not needed, so a call that
+// takes long to read (plan_accept) reads its positions in phases: kernel 1 for
 // the first positions of every request, accept_test_kernel for their tests,
 // kernel 1 for the next positions of the requests that are still undecided
 // (and for the draw masses of those just decided, whose rows are still in
@@ -907,6 +907,11 @@ AcceptPlan plan_accept(const cs_accept_dims& d, int n, bool tree, bool greedy, b
     const int esz = f32 ? 4 : 2, item = kItemBytes / esz, sms = current_sm_count();
     AcceptPlan P{};
     P.I = (int)(((long long)d.vocab + (aligned ? 0 : 16 / esz - 1) + item - 1) / item);
+    // The cluster: the CTAs of all requests in one wave (two an SM), a power
+    // of two (they pack a GPC; nine CTAs a request took 40 us where eight took
+    // 35, B = 32).
+    int c = 1;
+    while (2 * c <= max_cluster_size() && 2ll * c * d.batch <= 2 * sms) c *= 2;
     // one position of every request, in us at the copy bandwidth
     const double pos_us = (double)d.batch * d.vocab * esz * (greedy || n == 1 ? 1 : 2) / 6.5e6;
     // A tree whose nodes' rows take longer than a few rounds of the walk is
@@ -916,30 +921,43 @@ AcceptPlan plan_accept(const cs_accept_dims& d, int n, bool tree, bool greedy, b
     if (!stream) {
         // The first phase takes the positions of about 30 us, every later one
         // twice as many as were read before it, and what is left over when it
-        // is less than 15 us joins the last.  A phase costs about 8 us (its
-        // test, two hand-offs, an uneven end), so a call under 60 us is read
-        // at once (in two phases a call of 45 us, B = 64, k = 8, V = 128256,
-        // took 81 us from a flushed L2 and at once 71; one of 50 us, B = 512,
-        // k = 4, V = 32000, 94 and 87; one of 85 us, B = 256, k = 16, V = 32000,
-        // 94 and 112).  B = 256, k = 8, V = 128256, bf16: 140 us with 1.9 of 8
-        // drafts accepted and 198 with 7.5 (at once: 208 and 201); B = 64,
-        // k = 4, V = 151936 at once 46 us, in two phases 58.
-        constexpr double kPhaseUs = 30.0, kPhasedUs = 60.0;
+        // is less than 15 us joins the last.  The first split costs about 15 us
+        // (a test, hand-offs, an uneven end, the last masses), a further one 6,
+        // and a call whose drafts are nearly all accepted gets nothing for them.
+        // So a call is read in phases where that loses next to nothing (us with
+        // 0.95, 0.8 and 0.6 of the drafts accepted, V = 128256, bf16):
+        //  - a greedy call from 60 us on (it has no masses): B = 256, k = 8 94 and
+        //    59 with 0.95 and 0.7 accepted, at once 92 and 92;
+        //  - a sampled one from 60 us on where the walk would otherwise weigh more
+        //    than 300 KB of a row pair in one CTA, which takes about as long as a
+        //    split: B = 256, k = 3 94, 94, 94, at once 95, 101, 105 (B = 512, k = 8,
+        //    V = 32000, 128 KB: 118, 102, 93, at once 100, 106, 107);
+        //  - any other from 110 us on: B = 128, k = 8 (91 us) 115, 99, 89, at once
+        //    100, 104, 106; k = 11 (121 us) in two phases 134, 112, 92, in three 137,
+        //    108, 92, at once 127, 132, 133;
+        //  - in two phases up to 150 us, then in as many as there are: B = 128,
+        //    k = 16 (172 us) 180, 125, 99, in two 176, 134, 99, at once 175, 180, 181;
+        //    B = 256, k = 8 (182 us) 187, 158, 127, in two 184, 169, 143, at once 191,
+        //    200, 202.
+        // fp32 rows of the same bytes lie within 8% of these: B = 64, k = 8 (91 us)
+        // 109, 98, 90, at once 93, 99, 101; B = 64, k = 16 (172 us) 174, 127, 93, at once
+        // 166, 172, 172.
+        constexpr double kPhaseUs = 30.0, kShareBytes = 300e3;
+        const double call_us = n * pos_us;
+        const bool pays = greedy || 2.0 * d.vocab * esz / c > kShareBytes;
+        const int most = tree || d.batch > kMaxPhased || call_us < (pays ? 60.0 : 110.0) ? 1
+                         : greedy || call_us >= 150.0 ? kMaxPhases : 2;
         P.phases = 1;
-        long long g = (long long)(kPhaseUs / pos_us) + 1;
-        while (!tree && n * pos_us >= kPhasedUs && d.batch <= kMaxPhased && P.phases < kMaxPhases && g < n &&
+        long long g = most > 1 ? (long long)(kPhaseUs / pos_us) + 1 : n;
+        while (P.phases < most && g < n &&
                (n - g - (greedy ? 0.0 : 0.5)) * pos_us >= kPhaseUs / 2) {   // (the last position has no draft row)
             P.start[P.phases++] = (int)g;
             g *= 2;
         }
         P.start[P.phases] = n;
     }
-    // The cluster: the CTAs of all requests in one wave (two an SM), a power
-    // of two (they pack a GPC; nine CTAs a request took 40 us where eight took
-    // 35, B = 32); a streamed tree's at least four, for its rounds' latency.
+    // A streamed tree's cluster has at least four CTAs, for its rounds' latency.
     // Decided requests, the sampler and greedy calls have no slices to share.
-    int c = 1;
-    while (2 * c <= max_cluster_size() && 2 * c * d.batch <= 2 * sms) c *= 2;
     P.threads = kWalkMaxThreads;
     if (stream) {
         if (c < 4) c = 4;

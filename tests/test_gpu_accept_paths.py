@@ -45,16 +45,18 @@ def compare(inp, T, what, sample=24):
     return n
 
 
-# one position of these calls takes 4 to 32 us at the copy bandwidth, so they
-# are read in two to four phases
+# calls of 60 to 190 us at the copy bandwidth, read in two to four phases
 @pytest.mark.parametrize("B,k,V,dtype,sigma,T", [
     (256, 8, 128256, "bf16", 0.7, 0.8),    # [0, 1], [2, 3], [4, 8]
     (400, 1, 128256, "bf16", 0.7, 0.8),    # [0], [1]: a phase of nothing but the position without a draft
     (256, 8, 128256, "bf16", 0.7, 0.0),
     (128, 16, 128256, "bf16", 0.1, 1.0),   # four phases, most requests pass all of them
-    (96, 12, 128257, "bf16", 0.7, 0.8),    # rows at every alignment
+    (128, 11, 128256, "bf16", 0.5, 1.0),   # two phases
+    (160, 12, 128257, "bf16", 0.7, 0.8),   # rows at every alignment
+    (96, 12, 128257, "bf16", 0.7, 0.8),    # at once: 98 us
     (96, 16, 128257, "bf16", 0.7, 0.0),
     (97, 9, 100003, "f32", 1.0, 1.0),
+    (128, 3, 128256, "f32", 0.7, 0.8),     # from 60 us on: 513 KB of a row pair for a CTA of the walk
 ])
 def test_positions_read_in_phases(B, k, V, dtype, sigma, T):
     n = compare(chain(B, k, V, dtype, sigma, T, cell=B + k), T, f"B={B} k={k} V={V} {dtype} T={T}")
@@ -63,6 +65,8 @@ def test_positions_read_in_phases(B, k, V, dtype, sigma, T):
 
 @pytest.mark.parametrize("B,k,kernels", [
     (256, 8, 8),   # three phases of a statistics and a test kernel, the last one's masses, the walk
+    (128, 11, 6),  # two phases
+    (128, 8, 2),   # at once
     (400, 1, 5),   # the second phase decides no pair: no masses
 ])
 def test_every_launch_of_a_phased_call_has_work(B, k, kernels):
