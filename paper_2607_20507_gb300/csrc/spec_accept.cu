@@ -48,7 +48,8 @@ constexpr int kMaxCluster = 16;
 constexpr int kMaxTreeNodes = 64;
 constexpr int kMaxPhased = 4096;               // requests of a call whose positions are read in phases, at most
 
-// x / d for 0 <= x by a multiplication whenever x < 2^31: with
+// x / d for 0 <= x by a multiplication whenever x < 2^31 (division by an
+// invariant integer, Granlund and Montgomery 1994): with
 // s = ceil(log2 d) and mul = floor(2^(31+s) / d) + 1 < 2^32 + 1, the error of
 // x mul / 2^(31+s) over x / d is below x / 2^(31+s) < 1/d, too little to reach
 // the next whole number.

@@ -129,7 +129,8 @@ __device__ __forceinline__ int walk_locate(const DrawRow<T>& d, int j, int V, fl
     return warp_max_int(last);
 }
 
-// A sum and its rounding error (h the nearest float to h + l).
+// A sum and its rounding error (h the nearest float to h + l): the two-sum of
+// Knuth, kept as a double-length number as Dekker (1971) does.
 struct Sum2 {
     float h, l;
 };

@@ -259,8 +259,8 @@ verify_attention_tc_kernel(const __grid_constant__ CUtensorMap tmap_k, const __g
     const int SK = p.tc_stages, SV = p.tc_vstages;          // K and V ring depths
     constexpr int qh = kTcQHalfBytes;                       // bytes between the dim halves of a span's rows
     uint8_t* sq = smem;                                     // [2 halves][128 rows][128 B]: one span's query rows, then zeros
-    uint8_t* sk = smem + 2 * qh;                            // [K stage][half][64 keys][128 B]
-    uint8_t* sv = sk + SK * kTensorTileBytes;               // [V stage][half][64 keys][128 B]
+    uint8_t* sk = smem + 2 * qh;                            // [K stage][a tile, as TcTile lies]
+    uint8_t* sv = sk + SK * kTensorTileBytes;               // [V stage][the same]
     uint64_t* bars = reinterpret_cast<uint64_t*>(sv + SV * kTensorTileBytes);
     uint64_t* kfull = bars;                                 // [SK] K tile landed
     uint64_t* kempty = kfull + kTcMaxK;                     // [SK] K tile consumed (QK done)
