@@ -922,36 +922,41 @@ AcceptPlan plan_accept(const cs_accept_dims& d, int n, bool tree, bool greedy, b
     if (!stream) {
         // The first phase takes the positions of about 30 us, every later one
         // twice as many as were read before it, and what is left over when it
-        // is less than 15 us joins the last.  The first split costs about 15 us
-        // (a test, hand-offs, an uneven end, the last masses), a further one 6,
-        // and a call whose drafts are nearly all accepted gets nothing for them.
-        // So a call is read in phases where that loses next to nothing (us with
-        // 0.95, 0.8 and 0.6 of the drafts accepted, V = 128256, bf16):
-        //  - a greedy call from 60 us on (it has no masses): B = 256, k = 8 94 and
-        //    59 with 0.95 and 0.7 accepted, at once 92 and 92;
+        // is less than 15 us joins the last; 7.5 us are enough for the first
+        // split of a sampled call, which also takes the weighing from the walk
+        // (B = 256, k = 2, V = 128256, bf16 at once 75 to 86 us, in two phases 71 to
+        // 78; B = 160, fp32 99 to 116 and 82 to 91).
+        // The first split costs about 15 us (a test, hand-offs, an uneven end, the
+        // last masses), a further one 6, and a call whose drafts are nearly all
+        // accepted gets nothing for them.  So a call is read in phases where that
+        // loses next to nothing (us with 0.95, 0.8 and 0.6 of the drafts accepted,
+        // V = 128256, bf16):
+        //  - a greedy call from 60 us on (it has no masses): B = 256, k = 8 92 and
+        //    56 with 0.95 and 0.7 accepted, in three phases 94 and 59, at once 92 and 92;
         //  - a sampled one from 60 us on where the walk would otherwise weigh more
-        //    than 300 KB of a row pair in one CTA, which takes about as long as a
-        //    split: B = 256, k = 3 94, 94, 94, at once 95, 101, 105 (B = 512, k = 8,
-        //    V = 32000, 128 KB: 118, 102, 93, at once 100, 106, 107);
-        //  - any other from 110 us on: B = 128, k = 8 (91 us) 115, 99, 89, at once
-        //    100, 104, 106; k = 11 (121 us) in two phases 134, 112, 92, in three 137,
-        //    108, 92, at once 127, 132, 133;
-        //  - in two phases up to 150 us, then in as many as there are: B = 128,
-        //    k = 16 (172 us) 180, 125, 99, in two 176, 134, 99, at once 175, 180, 181;
-        //    B = 256, k = 8 (182 us) 187, 158, 127, in two 184, 169, 143, at once 191,
-        //    200, 202.
+        //    than 350 KB of a row pair in one CTA, which takes about as long as a
+        //    split: B = 256, k = 3 94, 94, 94, at once 95, 101, 105 (B = 64, k = 5,
+        //    V = 151936, fp32, 304 KB: 91 with 0.95, at once 78);
+        //  - any other from 100 us on: B = 128, k = 8 (91 us) 115, 99, 89, at once
+        //    100, 104, 106; k = 11 (121 us) in two phases 134, 112, 92, at once 127,
+        //    132, 133;
+        //  - in two phases up to 150 us, then in as many as there are: k = 11 in three
+        //    137, 108, 92; B = 128, k = 16 (172 us) in four 180, 125, 99, in two 176,
+        //    134, 99, at once 175, 180, 181; B = 256, k = 8 (182 us) in three 187, 158,
+        //    127, in two 184, 169, 143, at once 191, 200, 202.
         // fp32 rows of the same bytes lie within 8% of these: B = 64, k = 8 (91 us)
         // 109, 98, 90, at once 93, 99, 101; B = 64, k = 16 (172 us) 174, 127, 93, at once
         // 166, 172, 172.
-        constexpr double kPhaseUs = 30.0, kShareBytes = 300e3;
+        constexpr double kPhaseUs = 30.0, kShareBytes = 350e3;
         const double call_us = n * pos_us;
         const bool pays = greedy || 2.0 * d.vocab * esz / c > kShareBytes;
-        const int most = tree || d.batch > kMaxPhased || call_us < (pays ? 60.0 : 110.0) ? 1
-                         : greedy || call_us >= 150.0 ? kMaxPhases : 2;
+        const int most = tree || d.batch > kMaxPhased || call_us < (pays ? 60.0 : 100.0) ? 1
+                         : call_us < 150.0 ? 2 : kMaxPhases;
         P.phases = 1;
         long long g = most > 1 ? (long long)(kPhaseUs / pos_us) + 1 : n;
+        // (the last position has no draft row)
         while (P.phases < most && g < n &&
-               (n - g - (greedy ? 0.0 : 0.5)) * pos_us >= kPhaseUs / 2) {   // (the last position has no draft row)
+               (n - g - (greedy ? 0.0 : 0.5)) * pos_us >= (P.phases == 1 && !greedy ? kPhaseUs / 4 : kPhaseUs / 2)) {
             P.start[P.phases++] = (int)g;
             g *= 2;
         }

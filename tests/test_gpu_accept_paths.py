@@ -57,6 +57,7 @@ def compare(inp, T, what, sample=24):
     (96, 16, 128257, "bf16", 0.7, 0.0),
     (97, 9, 100003, "f32", 1.0, 1.0),
     (128, 3, 128256, "f32", 0.7, 0.8),     # from 60 us on: 513 KB of a row pair for a CTA of the walk
+    (256, 2, 128256, "bf16", 0.7, 0.8),    # [0, 1], [2]
 ])
 def test_positions_read_in_phases(B, k, V, dtype, sigma, T):
     n = compare(chain(B, k, V, dtype, sigma, T, cell=B + k), T, f"B={B} k={k} V={V} {dtype} T={T}")
@@ -67,6 +68,7 @@ def test_positions_read_in_phases(B, k, V, dtype, sigma, T):
     (256, 8, 8),   # three phases of a statistics and a test kernel, the last one's masses, the walk
     (128, 11, 6),  # two phases
     (128, 8, 2),   # at once
+    (256, 2, 5),   # a first split may leave the position without a draft alone
     (400, 1, 5),   # the second phase decides no pair: no masses
 ])
 def test_every_launch_of_a_phased_call_has_work(B, k, kernels):
